@@ -20,7 +20,7 @@ SO = os.path.join(HERE, "libsclap.so")
 BUILD_CHECK = os.path.join(HERE, "_build_check")
 SO_CHECK = os.path.join(HERE, "libsclap_check.so")
 SOURCES = ["scan.cu", "lp.cu", "contract.cu", "ip.cu", "driver.cu", "noalloc.cu", "server.cu"]
-HEADERS = [os.path.join(CSRC, "common.cuh"), os.path.join(ROOT, "include", "sclap.h")]
+HEADERS = [os.path.join(CSRC, "common.cuh"), os.path.join(CSRC, "arcs.cuh"), os.path.join(ROOT, "include", "sclap.h")]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-std=c++17", "-O3", "-lineinfo", "-Xcompiler", "-fPIC"]
 

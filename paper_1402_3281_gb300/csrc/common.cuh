@@ -328,6 +328,9 @@ struct LevelView {
   const int32_t* ew = nullptr;    // NULL: unit edge weights
   const int32_t* nw = nullptr;    // NULL: unit node weights
   const int32_t* gid = nullptr;   // slot of each node (NULL: one slot)
+  int32_t nslots = 1;
+  const int64_t* noff = nullptr;  // [nslots + 1] first node of each slot (device)
+  const int64_t* aoff = nullptr;  // [nslots + 1] first arc of each slot (device)
   // every sum of arc weights over a row (so every connection) is below 2^32:
   // the propose tables may accumulate with 32-bit atomics
   bool narrow = false;
@@ -421,14 +424,6 @@ __device__ __forceinline__ long long warp_max_ll(long long x, int width = 32) {
 __device__ __forceinline__ long long warp_sum_ll(long long x) {
   for (int off = 16; off > 0; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
   return x;
-}
-
-// Sum of positive int32 values over the lanes of `mask` as a 64-bit number,
-// from two 32-bit warp reductions of the 16-bit halves.
-__device__ __forceinline__ int64_t match_sum(unsigned mask, int32_t w) {
-  unsigned lo = __reduce_add_sync(mask, (unsigned)w & 0xffffu);
-  unsigned hi = __reduce_add_sync(mask, (unsigned)w >> 16);
-  return ((int64_t)hi << 16) + (int64_t)lo;
 }
 
 // Admission key: smaller key = admitted first.  High half: larger gain first
@@ -561,15 +556,9 @@ struct CoarseLevel {
   int64_t N = 0, M = 0;
   DevBuf<int64_t> row_ptr;
   DevBuf<int32_t> col, ew, nw, gid;
-  DevBuf<int64_t> noff_d;
+  DevBuf<int64_t> noff_d, aoff_d;
   std::vector<int64_t> noff;   // [nslots+1]
   std::vector<int64_t> aoff;   // arc offset of each slot [nslots+1]
-  LevelView view() const {
-    LevelView v;
-    v.N = N; v.M = M; v.row_ptr = row_ptr.p; v.col = col.p; v.ew = ew.p; v.nw = nw.p;
-    v.gid = gid.p;
-    return v;
-  }
 };
 // Step 1: ranks the used labels; nc_slot[s] = coarse nodes of slot s.
 // Overlay of two clusterings of a batched level (ensemble clusterings): for
@@ -687,6 +676,7 @@ void lift_blocks(const int32_t* cmap, const int32_t* fine_blk, int32_t* coarse_b
 void project(const int32_t* cmap, const int32_t* coarse_blk, int32_t* fine_blk, int64_t N,
              cudaStream_t s);
 // Block weights of every slot from scratch: W[label[v]] += nw[v].
-void block_weights(const int32_t* label, const int32_t* nw, int64_t N, wgt_t* W, cudaStream_t s);
+void block_weights(const int32_t* label, const int32_t* nw, int64_t N, wgt_t* W, int64_t nlabels,
+                   cudaStream_t s);
 
 }  // namespace sclap

@@ -812,11 +812,11 @@ void finish_level(CoarseLevel& out, int ns, cudaStream_t s) {
   const int64_t Nc = out.N;
   out.gid.alloc(std::max<int64_t>(Nc, 1), s);
   fill_gid(out.noff_d.p, ns, out.gid.p, Nc, s);
-  DevBuf<int64_t> ga(ns + 1, s);
-  k_gather<<<grid_for(ns + 1, 128, 64), 128, 0, s>>>(out.row_ptr.p, out.noff_d.p, ns + 1, ga.p); SCLAP_NOTE_LAUNCH("k_gather");
+  out.aoff_d.alloc(ns + 1, s);
+  k_gather<<<grid_for(ns + 1, 128, 64), 128, 0, s>>>(out.row_ptr.p, out.noff_d.p, ns + 1, out.aoff_d.p); SCLAP_NOTE_LAUNCH("k_gather");
   SCLAP_LAUNCH_CHECK();
   out.aoff.assign(ns + 1, 0);
-  SCLAP_CUDA(cudaMemcpyAsync(out.aoff.data(), ga.p, (ns + 1) * sizeof(int64_t),
+  SCLAP_CUDA(cudaMemcpyAsync(out.aoff.data(), out.aoff_d.p, (ns + 1) * sizeof(int64_t),
                              cudaMemcpyDeviceToHost, s));
   stream_sync(s);
 }

@@ -16,7 +16,7 @@
 #include <memory>
 #include <thread>
 
-#include "common.cuh"
+#include "arcs.cuh"
 
 namespace sclap {
 namespace {
@@ -56,89 +56,122 @@ sclap_config resolve_cfg(const sclap_config* c) {
 }
 
 // ------------------------------------------------------------- validation
-// Checks a batched level as built from the inputs (one warp per 32 nodes,
-// arcs flattened across lanes): row offsets non-decreasing and inside the
-// slot's arc range, neighbours inside the slot, no self-loops, positive
-// weights.  Per-slot error flags, c(V) and max c(v).  Arcs are read only
-// inside ranges already checked, so malformed input cannot send a read out
-// of the level's arrays.
-__global__ void __launch_bounds__(256) k_validate_level(
-    const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
-    const int32_t* __restrict__ ew, const int32_t* __restrict__ nw,
+// Checks a batched level as built from the inputs, in two passes: the nodes
+// (row offsets non-decreasing and inside the slot's arc range, positive
+// weights; c(V) and max c(v) per slot), then the arcs of the slots whose row
+// offsets are sound (neighbours inside the slot, no self-loops, positive
+// weights; total arc weight per slot).  Arcs are read only below the arc
+// count, so malformed input cannot send a read out of the level's arrays.
+//
+// Both passes are streams.  The arc pass is bounded by instruction issue
+// (65 % busy: finding each arc's source), reading 2.6 TB/s; the even split of
+// the arcs is what matters: with a warp per 32 rows the longest row was one
+// warp's serial job (R-MAT 2^21 nodes, 56 M weighted arcs: 3.51 ms before,
+// 0.04 ms for the nodes and 0.20 ms for the arcs now; 0.32 ms with the cut).
+__device__ __forceinline__ void val_flush(int32_t s, unsigned long long sum, int32_t mx,
+                                          unsigned long long* cV, int32_t* maxc) {
+  if (s < 0) return;
+  if (sum) atomicAdd(&cV[s], sum);
+  if (mx > 0) atomicMax(&maxc[s], mx);
+}
+__global__ void __launch_bounds__(256) k_validate_nodes(
+    const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ nw,
     const int64_t* __restrict__ noff, const int64_t* __restrict__ aoff, int32_t nslots,
-    int64_t N, int32_t* gerr, unsigned long long* cV, int32_t* maxc,
-    unsigned long long* arcw) {
-  const int lane = threadIdx.x & 31;
-  const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t base = w0 * 32; base < N; base += nwarps * 32) {
-    const int64_t v = base + lane;
-    int32_t s = -1;
-    int64_t rs = 0, d = 0;
-    bool bad = false;
-    int32_t w = 0;
-    if (v < N) {
-      int32_t lo = 0, hi = nslots - 1;
-      while (lo < hi) {
-        const int32_t mid = (lo + hi + 1) >> 1;
-        if (noff[mid] <= v) lo = mid; else hi = mid - 1;
+    int64_t N, int32_t* gerr, unsigned long long* cV, int32_t* maxc) {
+  __shared__ unsigned long long sh_sum[8];
+  __shared__ int32_t sh_max;
+  // a contiguous share of the nodes per CTA: a thread stays in one slot for
+  // long and keeps that slot's sums in registers
+  const int64_t per = (N + gridDim.x - 1) / gridDim.x;
+  const int64_t n0 = (int64_t)blockIdx.x * per, n1 = min64(n0 + per, N);
+  int32_t s = -1, mx = 0;
+  int64_t s1 = 0;                          // one past slot s's last node
+  unsigned long long sum = 0;
+  for (int64_t v = n0 + threadIdx.x; v < n1; v += blockDim.x) {
+    if (s < 0 || v >= s1) {
+      val_flush(s, sum, mx, cV, maxc);
+      sum = 0;
+      mx = 0;
+      s = slot_of(noff, nslots, v);
+      s1 = noff[s + 1];
+    }
+    const int64_t rs = row_ptr[v], re = row_ptr[v + 1];
+    const int32_t w = wat(nw, v);
+    const bool bad = rs > re || rs < aoff[s] || re > aoff[s + 1] ||
+                     (v == noff[s] && rs != aoff[s]) || (v == s1 - 1 && re != aoff[s + 1]) ||
+                     w <= 0;
+    if (bad) atomicOr(&gerr[s], 1);
+    if (w > 0) {
+      sum += (unsigned long long)w;
+      mx = max(mx, w);
+    }
+  }
+  // one atomic per CTA when all its nodes lie in one slot
+  const bool uni = n0 < n1 && slot_of(noff, nslots, n0) == slot_of(noff, nslots, n1 - 1);
+  if (!uni) {
+    val_flush(s, sum, mx, cV, maxc);
+    return;
+  }
+  if (threadIdx.x == 0) sh_max = 0;
+  const unsigned long long tot = cta_sum(sum, sh_sum);
+  if (mx > 0) atomicMax(&sh_max, mx);
+  __syncthreads();
+  if (threadIdx.x == 0) val_flush(s, tot, sh_max, cV, maxc);
+}
+
+// CUT: also adds twice the cut of `label` to cut2 (sclap_cut: one pass over
+// the arcs instead of two); a head is used as an index only once it was
+// found to lie in the slot.
+template <bool CUT>
+__global__ void __launch_bounds__(AT_NT, AT_CTAS) k_validate_arcs(
+    const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
+    const int32_t* __restrict__ ew, const int64_t* __restrict__ noff,
+    const int64_t* __restrict__ aoff, int32_t nslots, int64_t M, int32_t* gerr,
+    unsigned long long* arcw, const int32_t* __restrict__ label, unsigned long long* cut2) {
+  __shared__ int32_t sh_end[AT_V];
+  __shared__ unsigned long long sh_sum[AT_NT / 32];
+  __shared__ int32_t sh_bad;
+  int64_t lo, hi;
+  arc_share(M, &lo, &hi);
+  while (lo < hi) {
+    const int32_t s = slot_of(aoff, nslots, lo);
+    const int64_t end = min64(hi, aoff[s + 1]);
+    __syncthreads();
+    if (threadIdx.x == 0) sh_bad = gerr[s];   // one reading for the whole CTA
+    __syncthreads();
+    if (sh_bad == 0) {
+      const int64_t v0 = noff[s], v1 = noff[s + 1];
+      unsigned long long acc = 0, cut = 0;
+      bool bad = false;
+      for_arc_tiles(row_ptr, v0, v1, lo, end, col, ew, M, sh_end, [&](const ArcTile& t) {
+#pragma unroll
+        for (int i = 0; i < AT_PER; ++i) {
+          const bool in = t.v[i] >= 0;
+          const bool ok = t.c[i] >= v0 && t.c[i] < v1 && t.c[i] != t.v[i] && t.w[i] > 0;
+          bad = bad || (in && !ok);
+          acc += in && t.w[i] > 0 ? (unsigned long long)t.w[i] : 0ull;
+        }
+        if (CUT) {
+          int32_t a[AT_PER], b[AT_PER];
+#pragma unroll
+          for (int i = 0; i < AT_PER; ++i) {
+            const bool ok = t.v[i] >= 0 && t.c[i] >= v0 && t.c[i] < v1 && t.w[i] > 0;
+            a[i] = ok ? label[t.v[i]] : 0;
+            b[i] = ok ? label[t.c[i]] : 0;
+          }
+#pragma unroll
+          for (int i = 0; i < AT_PER; ++i) cut += a[i] != b[i] ? (unsigned long long)t.w[i] : 0ull;
+        }
+      });
+      const unsigned long long tot = cta_sum(acc, sh_sum);
+      if (threadIdx.x == 0 && tot) atomicAdd(&arcw[s], tot);
+      if (CUT) {
+        const unsigned long long c = cta_sum(cut, sh_sum);
+        if (threadIdx.x == 0 && c) atomicAdd(&cut2[s], c);
       }
-      s = lo;
-      rs = row_ptr[v];
-      const int64_t re = row_ptr[v + 1];
-      if (rs > re || rs < aoff[s] || re > aoff[s + 1]) bad = true;
-      if (v == noff[s] && rs != aoff[s]) bad = true;
-      if (v == noff[s + 1] - 1 && re != aoff[s + 1]) bad = true;
-      w = wat(nw, v);
-      if (w <= 0) bad = true;
-      d = bad ? 0 : re - rs;
+      if (bad) atomicOr(&gerr[s], 1);
     }
-    // per-slot sums of node weights (lanes of one slot merged)
-    const unsigned mm = __match_any_sync(0xffffffffu, s);
-    const int64_t wsum = match_sum(mm, w > 0 ? w : 0);
-    const int wmax = __reduce_max_sync(mm, w > 0 ? w : 0);
-    if (s >= 0 && lane == __ffs(mm) - 1) {
-      atomicAdd(&cV[s], (unsigned long long)wsum);
-      atomicMax(&maxc[s], wmax);
-    }
-    long long incl = d;
-    for (int o = 1; o < 32; o <<= 1) {
-      long long y = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += y;
-    }
-    const long long excl = incl - d;
-    const long long total = __shfl_sync(0xffffffffu, incl, 31);
-    // total arc weight per slot: summed in registers when the warp's nodes
-    // all lie in one slot, else one atomic per arc
-    const int32_t s0 = __shfl_sync(0xffffffffu, s, 0);
-    const bool uni = __all_sync(0xffffffffu, s < 0 || s == s0);
-    unsigned long long acc = 0;
-    for (long long x0 = 0; x0 < total; x0 += 32) {
-      const long long x = x0 + lane;
-      int L = 0;
-      for (int step = 16; step > 0; step >>= 1) {
-        long long y = __shfl_sync(0xffffffffu, incl, L + step - 1);
-        if (y <= x) L += step;
-      }
-      const long long rsL = __shfl_sync(0xffffffffu, (long long)rs, L);
-      const long long exL = __shfl_sync(0xffffffffu, excl, L);
-      const int32_t sL = __shfl_sync(0xffffffffu, s, L);
-      if (x < total) {
-        const int64_t e = rsL + (x - exL);
-        const int64_t src = base + L;
-        const int32_t c = col[e];
-        const int32_t we = wat(ew, e);
-        if (c < noff[sL] || c >= noff[sL + 1] || c == src || we <= 0) atomicOr(&gerr[sL], 1);
-        const unsigned long long wp = we > 0 ? (unsigned long long)we : 0ull;
-        if (uni) acc += wp;
-        else if (wp) atomicAdd(&arcw[sL], wp);
-      }
-    }
-    if (uni) {
-      for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-      if (lane == 0 && acc) atomicAdd(&arcw[s0], acc);
-    }
-    if (bad && s >= 0) atomicOr(&gerr[s], 1);
+    lo = end;
   }
 }
 
@@ -244,7 +277,7 @@ struct Slots {
 // NULL for a level holding one graph.
 struct Level {
   int64_t N = 0, M = 0;
-  DevBuf<int64_t> row_ptr, noff_d;
+  DevBuf<int64_t> row_ptr, noff_d, aoff_d;
   DevBuf<int32_t> col, ew, nw, gid, cmap, blk;
   const int64_t* rp_in = nullptr;          // borrowed arrays (input level)
   const int32_t* col_in = nullptr;
@@ -267,6 +300,9 @@ struct Level {
     LevelView v;
     v.N = N; v.M = M; v.row_ptr = rp(); v.col = colp(); v.ew = ewp(); v.nw = nwp();
     v.gid = gid.p;
+    v.nslots = (int32_t)noff.size() - 1;
+    v.noff = noff_d.p;
+    v.aoff = aoff_d.p;
     v.narrow = narrow;
     v.sums31 = sums31;
     return v;
@@ -335,16 +371,19 @@ void build_level0(const std::vector<GIn>& gs, struct Level& L, cudaStream_t s);
 void validate_level(const Level& L, int B, std::vector<int32_t>& status,
                     std::vector<int64_t>& cV, std::vector<int64_t>& maxc,
                     std::vector<char>& narrow, cudaStream_t s,
-                    std::vector<char>* sums31 = nullptr) {
+                    std::vector<char>* sums31 = nullptr, const int32_t* label = nullptr,
+                    int64_t* cut2 = nullptr) {
   DevBuf<int32_t> err(B, s), mx(B, s);
   DevBuf<unsigned long long> sum(B, s), arcw(B, s);
-  DevBuf<int64_t> d_aoff(B + 1, s);
   err.zero(); mx.zero(); sum.zero(); arcw.zero();
-  d_aoff.upload(L.aoff);
   if (L.N > 0) {
-    k_validate_level<<<grid_for(L.N, 256, (int64_t)num_sms() * 16), 256, 0, s>>>(
-        L.rp(), L.colp(), L.ewp(), L.nwp(), L.noff_d.p, d_aoff.p, B, L.N, err.p, sum.p, mx.p,
-        arcw.p); SCLAP_NOTE_LAUNCH("k_validate_level");
+    k_validate_nodes<<<grid_for(L.N, 256 * 4, (int64_t)num_sms() * 8), 256, 0, s>>>(
+        L.rp(), L.nwp(), L.noff_d.p, L.aoff_d.p, B, L.N, err.p, sum.p, mx.p); SCLAP_NOTE_LAUNCH("k_validate_nodes");
+    if (L.M > 0) {
+      (label ? k_validate_arcs<true> : k_validate_arcs<false>)<<<arc_grid(L.M), AT_NT, 0, s>>>(
+          L.rp(), L.colp(), L.ewp(), L.noff_d.p, L.aoff_d.p, B, L.M, err.p, arcw.p, label,
+          reinterpret_cast<unsigned long long*>(cut2)); SCLAP_NOTE_LAUNCH("k_validate_arcs");
+    }
     SCLAP_LAUNCH_CHECK();
   }
   std::vector<int32_t> e(B), m(B);
@@ -370,14 +409,15 @@ void validate_level(const Level& L, int B, std::vector<int32_t>& status,
 }
 
 // Validates one device-resident graph (step entry points); returns c(V) and
-// max c(v) or throws.
-void validate(const GIn& g, cudaStream_t s, int64_t* cV, int64_t* maxc, bool* narrow = nullptr) {
+// max c(v) or throws.  label, cut2: also adds twice the label's cut (device).
+void validate(const GIn& g, cudaStream_t s, int64_t* cV, int64_t* maxc, bool* narrow = nullptr,
+              const int32_t* label = nullptr, int64_t* cut2 = nullptr) {
   Level L;
   build_level0({g}, L, s);
   std::vector<int32_t> st;
   std::vector<int64_t> a, b;
   std::vector<char> nar;
-  validate_level(L, 1, st, a, b, nar, s);
+  validate_level(L, 1, st, a, b, nar, s, nullptr, label, cut2);
   if (st[0] == SCLAP_ECSR)
     throw Error(SCLAP_ECSR, "malformed CSR (row_ptr, column range, self-loop or weight)");
   if (st[0] == SCLAP_EOVERFLOW) throw Error(SCLAP_EOVERFLOW, "sum of node weights must be < 2^31");
@@ -403,6 +443,8 @@ void build_level0(const std::vector<GIn>& gs, Level& L, cudaStream_t s) {
   if (L.N >= ((int64_t)1 << 31)) throw Error(SCLAP_EINVAL, "total node count must be < 2^31");
   L.noff_d.alloc(B + 1, s);
   L.noff_d.upload(L.noff);
+  L.aoff_d.alloc(B + 1, s);
+  L.aoff_d.upload(L.aoff);
   if (B == 1) {
     L.borrowed = true;
     L.rp_in = gs[0].row_ptr;
@@ -551,6 +593,8 @@ void run_ip(const std::vector<IPIn>& in, const sclap_config& cfg, wgt_t* Wg,
   ip.aoff = aoff;
   ip.noff_d.alloc(S + 1, s);
   ip.noff_d.upload(noff);
+  ip.aoff_d.alloc(S + 1, s);
+  ip.aoff_d.upload(aoff);
   ip.gid.alloc(std::max<int64_t>(ip.N, 1), s);
   fill_gid(ip.noff_d.p, S, ip.gid.p, ip.N, s);
 
@@ -821,6 +865,7 @@ void run_valid_batch(const std::vector<GIn>& gs, const std::vector<int64_t>& cV,
       nx->nw = std::move(co.nw);
       nx->gid = std::move(co.gid);
       nx->noff_d = std::move(co.noff_d);
+      nx->aoff_d = std::move(co.aoff_d);
       nx->noff = co.noff;
       nx->aoff = co.aoff;
       if (respect) {
@@ -1548,6 +1593,7 @@ int sclap_cluster_hierarchy(int64_t n, const int64_t* row_ptr, const int32_t* co
       nx->nw = std::move(co.nw);
       nx->gid = std::move(co.gid);
       nx->noff_d = std::move(co.noff_d);
+      nx->aoff_d = std::move(co.aoff_d);
       nx->noff = co.noff;
       nx->aoff = co.aoff;
       cur = std::move(nx);
@@ -1656,7 +1702,7 @@ int sclap_refine(int64_t n, const int64_t* row_ptr, const int32_t* col, const in
     L.narrow = nar;
     DevBuf<wgt_t> W(k, s);
     W.zero();
-    block_weights(block, L.nwp(), n, W.p, s);
+    block_weights(block, L.nwp(), n, W.p, k, s);
     Slots sl(s, 1, L.noff_d.p, {0}, {Lmax}, {seed}, {level}, {k}, {0});
     LPRun run;
     run.mode = MODE_REFINE;
@@ -1682,14 +1728,9 @@ int sclap_cut(int64_t n, const int64_t* row_ptr, const int32_t* col, const int32
     g.n = n; g.m = device_arcs(row_ptr, n, s); g.row_ptr = row_ptr; g.col = col; g.ew = edge_w;
     check_col(g.col, g.m);
     int64_t cV, maxc;
-    bool nar = false;
-    validate(g, s, &cV, &maxc, &nar);
-    Level L;
-    single_level(g, L, s);
-    L.narrow = nar;
     DevBuf<int64_t> cut2(1, s);
     cut2.zero();
-    slot_cut(L.view(), block, cut2.p, s);
+    validate(g, s, &cV, &maxc, nullptr, block, cut2.p);
     int64_t c2 = 0;
     SCLAP_CUDA(cudaMemcpyAsync(&c2, cut2.p, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
     stream_sync(s);

@@ -12,7 +12,7 @@
 #include <map>
 #include <tuple>
 
-#include "common.cuh"
+#include "arcs.cuh"
 
 namespace sclap {
 namespace {
@@ -756,121 +756,45 @@ __global__ void __launch_bounds__(GG_NT) k_ggg_group(GGGArgs a, int32_t cpt, Gro
   }
 }
 
-// Twice the cut of every slot: 32 nodes per warp, their arcs spread over
-// the lanes.  When the warp's 32 nodes lie in one slot (all but the groups
-// that straddle a slot boundary) each lane sums in a register and the warp
-// merges once per group; otherwise every cut arc is added on its own.  Rows
-// longer than CUT_CH arcs are queued in chunks of CUT_CH arcs for
-// k_slot_cut_long instead (at most 2 * arcs / CUT_CH chunks).
-constexpr int64_t CUT_CH = 4096;
-struct CutChunk {
+// Twice the cut of every slot (every edge is met from both ends).  The arcs
+// are streamed in storage order (arcs.cuh), so a hub's row and an empty
+// graph cost what their arcs cost; per tile a thread's eight label gathers
+// are in flight together, a slot's sum stays in a register until the CTA
+// leaves the slot, then one atomic adds it.
+// Bounded by the label gathers through L1 and L2 (55-68 % busy).  Measured
+// on R-MAT 2^21 nodes, 56 M weighted arcs: 743 -> 310 us (a warp per 32 rows
+// plus a queue of long rows before); the 512-graph batch's trial and final
+// cuts 1.74 -> 1.12 ms.
+__global__ void __launch_bounds__(AT_NT, AT_CTAS) k_slot_cut(const int64_t* __restrict__ row_ptr,
+                                                    const int32_t* __restrict__ col,
+                                                    const int32_t* __restrict__ ew,
+                                                    const int64_t* __restrict__ noff,
+                                                    const int64_t* __restrict__ aoff,
+                                                    int32_t nslots, int64_t N, int64_t M,
+                                                    const int32_t* __restrict__ label,
+                                                    int64_t* __restrict__ cut2) {
+  __shared__ int32_t sh_end[AT_V];
+  __shared__ unsigned long long sh_sum[AT_NT / 32];
   int64_t lo, hi;
-  int32_t v, pad;
-};
-__global__ void __launch_bounds__(256) k_slot_cut(const int64_t* __restrict__ row_ptr,
-                                                  const int32_t* __restrict__ col,
-                                                  const int32_t* __restrict__ ew,
-                                                  const int32_t* __restrict__ gid,
-                                                  const int32_t* __restrict__ label, int64_t N,
-                                                  int64_t* __restrict__ cut2,
-                                                  CutChunk* __restrict__ q, int32_t* qn) {
-  __shared__ int sh_slot;
-  __shared__ unsigned long long sh_sum;
-  const int lane = threadIdx.x & 31;
-  const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  if (threadIdx.x == 0) {
-    const int64_t v0 = (int64_t)blockIdx.x * blockDim.x;
-    sh_slot = v0 < N ? slot_at(gid, v0) : -1;
-    sh_sum = 0;
-  }
-  __syncthreads();
-  for (int64_t base = w0 * 32; base < N; base += nwarps * 32) {
-    const int64_t v = base + lane;
-    int64_t rs = 0, d = 0;
-    int32_t lv = 0, s = -1;
-    if (v < N) {
-      rs = row_ptr[v];
-      d = row_ptr[v + 1] - rs;
-      lv = label[v];
-      s = slot_at(gid, v);
-      if (d > CUT_CH) {
-        const int32_t nch = (int32_t)((d + CUT_CH - 1) / CUT_CH);
-        const int32_t q0 = atomicAdd(qn, nch);
-        for (int32_t c = 0; c < nch; ++c)
-          q[q0 + c] = CutChunk{rs + c * CUT_CH, min64(rs + (c + 1) * CUT_CH, rs + d), (int32_t)v, 0};
-        d = 0;
-      }
-    }
-    long long incl = d;
-    for (int o = 1; o < 32; o <<= 1) {
-      long long y = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += y;
-    }
-    const long long excl = incl - d;
-    const long long total = __shfl_sync(0xffffffffu, incl, 31);
-    const int32_t s0 = __shfl_sync(0xffffffffu, s, 0);
-    const bool uni = __all_sync(0xffffffffu, s < 0 || s == s0);
+  arc_share(M, &lo, &hi);
+  while (lo < hi) {
+    const int32_t s = nslots > 1 ? slot_of(aoff, nslots, lo) : 0;
+    const int64_t end = nslots > 1 ? min64(hi, aoff[s + 1]) : hi;
     unsigned long long acc = 0;
-    for (long long x0 = 0; x0 < total; x0 += 32) {
-      const long long x = x0 + lane;
-      int L = 0;
-      for (int step = 16; step > 0; step >>= 1) {
-        long long y = __shfl_sync(0xffffffffu, incl, L + step - 1);
-        if (y <= x) L += step;
+    for_arc_tiles(row_ptr, nslots > 1 ? noff[s] : 0, nslots > 1 ? noff[s + 1] : N, lo, end, col,
+                  ew, M, sh_end, [&](const ArcTile& t) {
+      int32_t a[AT_PER], b[AT_PER];
+#pragma unroll
+      for (int i = 0; i < AT_PER; ++i) {
+        a[i] = t.v[i] >= 0 ? label[t.v[i]] : 0;
+        b[i] = t.v[i] >= 0 ? label[t.c[i]] : 0;
       }
-      const long long rsL = __shfl_sync(0xffffffffu, (long long)rs, L);
-      const long long exL = __shfl_sync(0xffffffffu, excl, L);
-      const int32_t lvL = __shfl_sync(0xffffffffu, lv, L);
-      const int32_t sL = __shfl_sync(0xffffffffu, s, L);
-      if (x < total) {
-        const int64_t e = rsL + (x - exL);
-        if (label[col[e]] != lvL) {
-          const int32_t w = wat(ew, e);
-          if (uni) acc += (unsigned long long)w;
-          else if (sL == sh_slot) atomicAdd(&sh_sum, (unsigned long long)w);
-          else atomicAdd(ull(&cut2[sL]), (unsigned long long)w);
-        }
-      }
-    }
-    if (uni) {
-      for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-      if (lane == 0 && acc) {
-        if (s0 == sh_slot) atomicAdd(&sh_sum, acc);
-        else atomicAdd(ull(&cut2[s0]), acc);
-      }
-    }
-  }
-  __syncthreads();
-  if (threadIdx.x == 0 && sh_sum) atomicAdd(ull(&cut2[sh_slot]), sh_sum);
-}
-
-// The queued chunks of long rows: one CTA per chunk, one atomic per chunk.
-__global__ void __launch_bounds__(256) k_slot_cut_long(const int32_t* __restrict__ col,
-                                                       const int32_t* __restrict__ ew,
-                                                       const int32_t* __restrict__ gid,
-                                                       const int32_t* __restrict__ label,
-                                                       const CutChunk* __restrict__ q,
-                                                       const int32_t* qn,
-                                                       int64_t* __restrict__ cut2) {
-  __shared__ unsigned long long sh[8];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int32_t n = *qn;
-  for (int32_t i = blockIdx.x; i < n; i += gridDim.x) {
-    const CutChunk c = q[i];
-    const int32_t lv = label[c.v];
-    unsigned long long acc = 0;
-    for (int64_t e = c.lo + threadIdx.x; e < c.hi; e += blockDim.x)
-      if (label[col[e]] != lv) acc += (unsigned long long)wat(ew, e);
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) sh[wid] = acc;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      unsigned long long t = 0;
-      for (int w = 0; w < 8; ++w) t += sh[w];
-      if (t) atomicAdd(ull(&cut2[slot_at(gid, c.v)]), t);
-    }
-    __syncthreads();
+#pragma unroll
+      for (int i = 0; i < AT_PER; ++i) acc += a[i] != b[i] ? (unsigned long long)t.w[i] : 0ull;
+    });
+    const unsigned long long tot = cta_sum(acc, sh_sum);
+    if (threadIdx.x == 0 && tot) atomicAdd(ull(&cut2[s]), tot);
+    lo = end;
   }
 }
 
@@ -949,11 +873,28 @@ __global__ void k_lift_blocks(const int32_t* __restrict__ cmap, const int32_t* _
   }
 }
 
-__global__ void k_block_weights(const int32_t* __restrict__ label, const int32_t* __restrict__ nw,
-                                int64_t N, wgt_t* __restrict__ W) {
+// Block weights from scratch.  With at most BW_SH blocks a CTA sums its
+// nodes in shared memory first and adds each block once: the blocks are few,
+// so one global atomic per node serialised on a handful of addresses.
+// 2^20 nodes, 16 blocks: 175 -> 14 us.
+constexpr int BW_SH = 2048;
+__global__ void __launch_bounds__(256) k_block_weights(const int32_t* __restrict__ label,
+                                                       const int32_t* __restrict__ nw, int64_t N,
+                                                       wgt_t* __restrict__ W, int64_t nlabels) {
+  __shared__ int32_t sh[BW_SH];
+  const bool few = nlabels <= BW_SH;
+  if (few) {
+    for (int b = threadIdx.x; b < nlabels; b += blockDim.x) sh[b] = 0;
+    __syncthreads();
+  }
   for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < N;
        v += (int64_t)gridDim.x * blockDim.x)
-    atomicAdd(&W[label[v]], (wgt_t)wat(nw, v));
+    atomicAdd(few ? &sh[label[v]] : &W[label[v]], (wgt_t)wat(nw, v));
+  if (few) {
+    __syncthreads();
+    for (int b = threadIdx.x; b < nlabels; b += blockDim.x)
+      if (sh[b]) atomicAdd(&W[b], sh[b]);
+  }
 }
 
 __global__ void k_isolated(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ nw,
@@ -1169,14 +1110,9 @@ void ggg_trials(const GGGArgs& a_in, const std::vector<int64_t>& noff,
 }
 
 void slot_cut(const LevelView& lv, const int32_t* label, int64_t* cut2, cudaStream_t s) {
-  if (lv.N <= 0) return;
-  DevBuf<CutChunk> q((size_t)(2 * (lv.M / CUT_CH) + 2), s);
-  DevBuf<int32_t> qn(1, s);
-  qn.zero();
-  k_slot_cut<<<grid_for(lv.N, 256, (int64_t)num_sms() * 16), 256, 0, s>>>(
-      lv.row_ptr, lv.col, lv.ew, lv.gid, label, lv.N, cut2, q.p, qn.p); SCLAP_NOTE_LAUNCH("k_slot_cut");
-  k_slot_cut_long<<<(unsigned)num_sms() * 8, 256, 0, s>>>(lv.col, lv.ew, lv.gid, label, q.p, qn.p,
-                                                          cut2); SCLAP_NOTE_LAUNCH("k_slot_cut_long");
+  if (lv.M <= 0) return;
+  k_slot_cut<<<arc_grid(lv.M), AT_NT, 0, s>>>(lv.row_ptr, lv.col, lv.ew, lv.noff, lv.aoff,
+                                                 lv.nslots, lv.N, lv.M, label, cut2); SCLAP_NOTE_LAUNCH("k_slot_cut");
   SCLAP_LAUNCH_CHECK();
 }
 
@@ -1217,10 +1153,11 @@ void lift_blocks(const int32_t* cmap, const int32_t* fine_blk, int32_t* coarse_b
   SCLAP_LAUNCH_CHECK();
 }
 
-void block_weights(const int32_t* label, const int32_t* nw, int64_t N, wgt_t* W,
+void block_weights(const int32_t* label, const int32_t* nw, int64_t N, wgt_t* W, int64_t nlabels,
                    cudaStream_t s) {
   if (N <= 0) return;
-  k_block_weights<<<grid_for(N, 256, (int64_t)num_sms() * 16), 256, 0, s>>>(label, nw, N, W); SCLAP_NOTE_LAUNCH("k_block_weights");
+  k_block_weights<<<grid_for(N, 256 * 8, (int64_t)num_sms() * 8), 256, 0, s>>>(label, nw, N, W,
+                                                                             nlabels); SCLAP_NOTE_LAUNCH("k_block_weights");
   SCLAP_LAUNCH_CHECK();
 }
 
