@@ -603,7 +603,6 @@ void ip_replicate(const std::vector<CopyTask>& tasks, int64_t* row_ptr, int32_t*
 struct GGGArgs {
   const int64_t* row_ptr;
   const int32_t* col;
-  const int32_t* ew;
   const int32_t* nw;
   const int64_t* noff;     // trial slot node offsets
   const int64_t* boff;     // trial slot block offsets
@@ -613,12 +612,12 @@ struct GGGArgs {
   const int32_t* level;    // coarsest level index per slot
   int32_t* label;          // out: global block ids
   wgt_t* W;                // out: block weights
-  int64_t* conn;           // scratch [N]
   int32_t* step;           // scratch [N]
   int32_t* front;          // scratch [N]: newly reached nodes (step alternates with it)
   int32_t* heavy;          // scratch [N]: a step's long rows (grouped growing)
   int64_t N;               // nodes of all trial slots (array lengths for bounds checks)
-  uint32_t* asg;           // scratch [N / 32 + 1]: assigned-node bitmap (grouped growing)
+  uint32_t* asg;           // assigned-node bitmap of every trial (set by ggg_trials)
+  uint32_t* seen;          // seen-node bitmap (assigned or reached; set by ggg_trials)
   int64_t* wfA;            // scratch [sum k]
   int32_t* wforder;        // scratch [sum k]
   int32_t nslots;
