@@ -230,6 +230,24 @@ void debug_inject(uint32_t wait, uint32_t probe, int32_t fail_allocs);
 // by sclap_debug_inject (the fail_allocs-th from the call on).
 bool take_injected_alloc_failure();
 
+// Thread-block clusters: rank of this CTA, the address of a shared-memory
+// object in another CTA of the cluster, and the cluster's barrier (its
+// release / acquire covers shared and global memory).
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+template <class T>
+__device__ __forceinline__ T* cluster_map(T* p, uint32_t rank) {
+  uint64_t out;
+  asm volatile("mapa.u64 %0, %1, %2;" : "=l"(out) : "l"(reinterpret_cast<uint64_t>(p)), "r"(rank));
+  return reinterpret_cast<T*>(out);
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory");
+}
+
 // Cooperative launch (all CTAs co-resident; required by grid_sync).
 template <typename... KArgs, typename... Args>
 inline void launch_coop(void (*k)(KArgs...), unsigned grid, unsigned block, size_t smem,

@@ -13,13 +13,14 @@
 //   resolve  a target whose proposals all fit admits them all; otherwise the
 //            proposals into it form a segment, and the longest prefix in
 //            (gain desc, priority asc, node asc) order that fits is admitted
-//            (one warp ranks all pairs of a segment of <= 64 entries, one CTA
-//            locates the boundary of a larger one by radix select);
+//            (one warp ranks all pairs of a segment of <= 64 entries, one CTA,
+//            or a cluster of CTAs, locates the boundary of a larger one by
+//            radix select);
 //   source   (local search) forced moves out of an overloaded block are capped
 //            at the block's excess the same way;
-//   apply    labels and label weights are updated with integer atomics
-//            (order-free, hence deterministic) and moved nodes activate their
-//            neighbours.
+//   apply    as soon as a move is admitted: labels and label weights are
+//            updated with integer atomics (order-free, hence deterministic)
+//            and moved nodes activate their neighbours.
 #include "common.cuh"
 
 namespace sclap {
@@ -49,7 +50,7 @@ struct LPArgs {
   // state
   int32_t* label;
   wgt_t* W;
-  int64_t* in_w;
+  uint64_t* in_w;        // per target: proposals << 32 | their node weight (both < 2^31)
   int32_t mode;
   int32_t S;
   // sub-round lists: for each listed node {v, own label, weight, slot} and
@@ -58,12 +59,12 @@ struct LPArgs {
   longlong2* rec2;
   int32_t* prop_t;
   uint64_t* prop_key;
-  int8_t* adm;
-  int8_t* stage;
+  wgt_t* prop_w;         // the target's weight when it was proposed to
+  int8_t* adm;           // source chain only: admitted by the target
+  int32_t* stage;        // 1 + position in its overflow segment, 0: in none
   int32_t* grp;
   // overflow segments
   int32_t* ovf_cnt;
-  int32_t* ovf_fill;
   int64_t* ovf_base;
   int64_t* ctr;          // admission segment counters (8 words, see adm_ctr)
   int32_t* seg_g;
@@ -166,7 +167,11 @@ __device__ __forceinline__ void write_prop(const LPArgs& a, int64_t i, const Nod
     const int32_t t = (int32_t)(c.loff + best.C);
     a.prop_t[i] = t;
     a.prop_key[i] = admission_key(best.conn - own_conn, (uint32_t)c.hv);
-    if (SCLAP_OK(t, a.nlabels, a.err)) atomicAdd(ull(&a.in_w[t]), (unsigned long long)c.cv);
+    // label weights stand still while proposals are made, so the target's is
+    // kept with the proposal: resolving can then apply moves at once
+    a.prop_w[i] = SCLAP_LD(a.W, t, a.nlabels, a.err);
+    if (SCLAP_OK(t, a.nlabels, a.err))
+      atomicAdd(reinterpret_cast<unsigned long long*>(&a.in_w[t]), (1ull << 32) | (uint32_t)c.cv);
   } else {
     a.prop_t[i] = -1;
   }
@@ -1267,21 +1272,158 @@ __global__ void __launch_bounds__(HUB_NT) k_hub_select(LPArgs a, int32_t sub, in
   }
 }
 
+// ------------------------------------------------------------- apply
+// Label-weight changes of the moves of a CTA, summed in a small shared hash
+// (label -> delta; a label that finds no slot within a few probes goes to
+// global memory directly), flushed with one atomic per label: in local search
+// moves concentrate on a handful of blocks, and in clustering many nodes can
+// join one cluster in a colour class (the leaves of a hub), whose global
+// counters would otherwise take one atomic per moved node each.  The clusters
+// that clustering moves leave are spread out and are updated directly.
+constexpr int APPLY_SLOTS = 1024;
+struct ApplyHash {
+  int32_t k[APPLY_SLOTS], v[APPLY_SLOTS];
+};
+__device__ __forceinline__ void apply_init(ApplyHash& h) {
+  for (int j = threadIdx.x; j < APPLY_SLOTS; j += blockDim.x) { h.k[j] = -1; h.v[j] = 0; }
+  __syncthreads();
+}
+__device__ __forceinline__ void apply_delta(const LPArgs& a, ApplyHash& h, int32_t L, int32_t d) {
+  uint32_t s = table_slot(L, 10);
+#pragma unroll 1
+  for (int p = 0; p < 8; ++p) {
+    const int32_t prev = atomicCAS(&h.k[s], -1, L);
+    if (prev == -1 || prev == L) {
+      atomicAdd(&h.v[s], d);
+      return;
+    }
+    s = (s + 1) & (APPLY_SLOTS - 1);
+  }
+  if (SCLAP_OK(L, a.nlabels, a.err)) atomicAdd(&a.W[L], (wgt_t)d);
+}
+__device__ __forceinline__ void apply_flush(const LPArgs& a, const ApplyHash& h) {
+  __syncthreads();
+  for (int j = threadIdx.x; j < APPLY_SLOTS; j += blockDim.x)
+    if (h.k[j] >= 0 && h.v[j] != 0 && SCLAP_OK(h.k[j], a.nlabels, a.err))
+      atomicAdd(&a.W[h.k[j]], (wgt_t)h.v[j]);
+}
+
+constexpr int64_t MARK_CH = 4096;     // arcs per queued chunk of a moved long row
+
+// Moves counted per slot in registers while a thread meets one slot.
+struct MovedRun {
+  int32_t slot = -1;
+  unsigned long long cnt = 0;
+};
+__device__ __forceinline__ void moved_flush(const LPArgs& a, const MovedRun& m) {
+  if (m.cnt) atomicAdd(ull(&a.moved[m.slot]), m.cnt);
+}
+
+// Node c (none: -1) becomes active in the next round.
+__device__ __forceinline__ void mark_active(const LPArgs& a, uint8_t* an, int32_t c) {
+  if (c >= 0 && SCLAP_OK(c, a.N, a.err)) an[c] = 1;
+}
+
+// Applies the move of list entry i to label t on the lanes with mv (every
+// lane of the warp calls): label, label weights, moved count, and the moved
+// node's neighbours become active (rows of <= 8 arcs by their own lane,
+// longer ones by the whole warp, the longest through the chunk queue).
+__device__ __forceinline__ void move_warp(const LPArgs& a, ApplyHash& h, MovedRun& m, int32_t sub,
+                                          bool mv, int64_t i, int32_t t) {
+  uint8_t* const an = act_next(a);
+  const int lane = threadIdx.x & 31;
+  int32_t slot = -1;
+  int64_t rs = 0, re = 0;
+  if (mv && SCLAP_OK(t, a.nlabels, a.err)) {
+    const int4 r = a.rec[i];
+    const int32_t v = r.x, own = r.y, cv = r.z;
+    slot = r.w;
+    if (an) {
+      const longlong2 r2 = a.rec2[i];
+      rs = r2.x;
+      re = r2.x + r2.y;
+    }
+    if (SCLAP_OK(v, a.N, a.err)) a.label[v] = t;
+    apply_delta(a, h, t, cv);
+    if (a.mode != MODE_CLUSTER) apply_delta(a, h, own, -cv);
+    else if (SCLAP_OK(own, a.nlabels, a.err)) atomicSub(&a.W[own], (wgt_t)cv);
+    if (re - rs <= 8) {
+      int32_t c[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) c[q] = rs + q < re ? a.col[rs + q] : -1;
+#pragma unroll
+      for (int q = 0; q < 8; ++q) mark_active(a, an, c[q]);
+      re = rs;
+    } else if (a.mark_big > 0 && re - rs > a.mark_big) {
+      const int32_t nch = (int32_t)((re - rs + MARK_CH - 1) / MARK_CH);
+      const int32_t q0 = atomicAdd(&a.mqn[sub], nch);
+      for (int32_t c = 0; c < nch; ++c)
+        a.mq[q0 + c] = make_longlong2(rs + c * MARK_CH, min64(rs + (c + 1) * MARK_CH, re));
+      re = rs;
+    }
+  }
+  // four rows at a time: their loads go out before the first store (the
+  // flags may alias the arcs as far as the compiler knows, so one row at a
+  // time was one memory latency per row)
+  unsigned big = __ballot_sync(0xffffffffu, re > rs);
+  while (big) {
+    int64_t p0[4], p1[4];
+    int32_t c[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int src = big ? __ffs(big) - 1 : 0;
+      p0[q] = __shfl_sync(0xffffffffu, (long long)rs, src);
+      p1[q] = big ? __shfl_sync(0xffffffffu, (long long)re, src) : p0[q];
+      big &= big - 1;
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) c[q] = p0[q] + lane < p1[q] ? a.col[p0[q] + lane] : -1;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) mark_active(a, an, c[q]);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      for (int64_t e = p0[q] + 32 + lane; e - lane < p1[q]; e += 128) {
+        int32_t d[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) d[u] = e + 32 * u < p1[q] ? a.col[e + 32 * u] : -1;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) mark_active(a, an, d[u]);
+      }
+    }
+  }
+  const unsigned mm = __match_any_sync(0xffffffffu, slot);
+  if (slot >= 0 && lane == __ffs(mm) - 1) {
+    if (slot != m.slot) {
+      moved_flush(a, m);
+      m.slot = slot;
+      m.cnt = 0;
+    }
+    m.cnt += __popc(mm);
+  }
+}
+
 // ------------------------------------------------------------- admission
-// Admission and application of one colour class run as ONE cooperative
-// launch (k_admit below), its phases separated by bounded grid barriers:
-//   resolve   every proposal into a target whose proposals all fit is
-//             admitted; the others are counted per target, and the first
-//             proposal into an overflowing target registers the target as a
-//             segment (with its admission threshold);
-//   alloc     each segment takes its range of the entry arrays;
-//   scatter   the overflowing proposals are written into their segments;
-//   select    each segment admits its longest fitting prefix;
-//   (source side, local search with overloaded blocks: forced moves out of
-//   an overloaded block are grouped by source the same way)
-//   apply     labels and label weights are updated.
-// When no target overflows (known to every CTA after the first barrier) the
-// kernel goes from resolve straight to apply: one barrier per colour class.
+// Admission and application of one colour class:
+//   resolve   a target whose proposals all fit takes them all, and they are
+//             applied at once: the target's weight was kept with the
+//             proposal and the sum of the proposals is complete, so nothing
+//             another proposal still needs is overwritten.  The others form
+//             segments per target: the count kept beside the incoming weight
+//             is the segment's size, so the first of them takes the whole
+//             range of the entry arrays;
+//   scatter   the overflowing proposals are written into their segments (and
+//             the incoming weights are cleared for the next class);
+//   select    each segment admits and applies its longest fitting prefix.
+// Local search with an overloaded block (source chain) also caps the forced
+// moves out of that block, and those depend on what the targets admitted:
+// there resolve and select only record the admissions, the admitted forced
+// moves are grouped by source the same way (forced, alloc, scatter, select),
+// and a last phase applies what is left.
+//
+// Three launches per colour class instead of five (resolve, alloc, scatter,
+// select, apply, each a pass over the proposals): R-MAT 2^16 nodes (80 colour
+// classes) 1.98 -> 1.57 ms of admission, R-MAT 2^22 nodes 18.5 -> 8.5 ms with
+// the cluster selection below, the 512-graph batch 7.4 -> 7.0 ms.
 //
 // Segment counters: ctr[set * 4 + side * 2 + {0: entry cursor, 1: segments}],
 // set = colour class & 1; a launch clears the other set for the next class
@@ -1290,57 +1432,77 @@ __device__ __forceinline__ int64_t* adm_ctr(const LPArgs& a, int sub, int side) 
   return a.ctr + (sub & 1) * 4 + side * 2;
 }
 
-__device__ void adm_resolve(const LPArgs& a, int64_t lbeg, int64_t cnt, int64_t* ct) {
-  for (int64_t li = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; li < cnt;
-       li += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t i = lbeg + li;
-    const int32_t t = a.prop_t[i];
-    a.stage[i] = 0;
-    if (t < 0) { a.adm[i] = 0; continue; }
-    const int64_t bound = a.bound[a.rec[i].w];
-    const int64_t Wt = SCLAP_LD(a.W, t, a.nlabels, a.err);
-    if (Wt + SCLAP_LD(a.in_w, t, a.nlabels, a.err) <= bound) {
-      a.adm[i] = 1;
-    } else {
-      a.adm[i] = 0;
-      a.grp[i] = t;
-      const int c = atomicAdd(&a.ovf_cnt[t], 1);
-      a.stage[i] = c == 0 ? 2 : 1;
-      if (c == 0) {                     // admit while the inclusive prefix <= bound - W[t]
-        const int64_t seg = (int64_t)atomicAdd(ull(&ct[1]), 1ull);
-        a.seg_g[seg] = t;
-        a.seg_thr[seg] = bound - Wt;
+template <bool APPLY>
+__device__ __forceinline__ void adm_resolve(const LPArgs& a, ApplyHash* h, int32_t sub,
+                                            int64_t lbeg, int64_t cnt, int64_t* ct) {
+  const int lane = threadIdx.x & 31;
+  const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  MovedRun m;
+  for (int64_t b0 = w0 * 32; b0 < cnt; b0 += nw * 32) {
+    const int64_t i = lbeg + b0 + lane;
+    bool mv = false;
+    int32_t t = -1;
+    if (b0 + lane < cnt) {
+      t = a.prop_t[i];
+      int32_t st = 0;
+      if (t >= 0) {
+        const int64_t bound = a.bound[a.rec[i].w];
+        const int64_t Wt = a.prop_w[i];
+        const uint64_t in = SCLAP_LD(a.in_w, t, a.nlabels, a.err);
+        if (Wt + (int64_t)(uint32_t)in <= bound) {
+          mv = true;
+        } else if (SCLAP_OK(t, a.nlabels, a.err)) {
+          a.grp[i] = t;
+          st = atomicAdd(&a.ovf_cnt[t], 1) + 1;
+          if (st == 1) {                  // admit while the inclusive prefix <= bound - W[t]
+            const int64_t seg = (int64_t)atomicAdd(ull(&ct[1]), 1ull);
+            const int32_t n = (int32_t)(in >> 32);
+            const int64_t base = (int64_t)atomicAdd(ull(&ct[0]), (unsigned long long)n);
+            a.ovf_base[t] = base;
+            a.seg_g[seg] = t;
+            a.seg_base[seg] = base;
+            a.seg_cnt[seg] = n;
+            a.seg_thr[seg] = bound - Wt;
+          }
+        }
       }
+      a.stage[i] = st;
+      if (!APPLY) a.adm[i] = mv ? 1 : 0;
     }
+    if (APPLY) move_warp(a, *h, m, sub, mv, i, t);
   }
+  if (APPLY) moved_flush(a, m);
 }
 
-// Forced moves out of overloaded blocks (local search), grouped by source;
+// Forced moves out of overloaded blocks (source chain), grouped by source;
 // admit while the exclusive prefix <= W[src] - bound - 1.
 __device__ void adm_forced(const LPArgs& a, int64_t lbeg, int64_t cnt, int64_t* ct) {
   for (int64_t li = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; li < cnt;
        li += (int64_t)gridDim.x * blockDim.x) {
     const int64_t i = lbeg + li;
-    a.stage[i] = 0;
-    if (a.adm[i] != 1) continue;
-    const int4 r = a.rec[i];
-    const int32_t own = r.y;
-    const int64_t bound = a.bound[r.w];
-    const int64_t Wo = SCLAP_LD(a.W, own, a.nlabels, a.err);
-    if (Wo > bound) {
-      a.grp[i] = own;
-      const int c = atomicAdd(&a.ovf_cnt[own], 1);
-      a.stage[i] = c == 0 ? 2 : 1;
-      if (c == 0) {
-        const int64_t seg = (int64_t)atomicAdd(ull(&ct[1]), 1ull);
-        a.seg_g[seg] = own;
-        a.seg_thr[seg] = Wo - bound - 1;
+    int32_t st = 0;
+    if (a.adm[i] == 1) {
+      const int4 r = a.rec[i];
+      const int32_t own = r.y;
+      const int64_t bound = a.bound[r.w];
+      const int64_t Wo = SCLAP_LD(a.W, own, a.nlabels, a.err);
+      if (Wo > bound && SCLAP_OK(own, a.nlabels, a.err)) {
+        a.grp[i] = own;
+        st = atomicAdd(&a.ovf_cnt[own], 1) + 1;
+        if (st == 1) {
+          const int64_t seg = (int64_t)atomicAdd(ull(&ct[1]), 1ull);
+          a.seg_g[seg] = own;
+          a.seg_thr[seg] = Wo - bound - 1;
+        }
       }
     }
+    a.stage[i] = st;
   }
 }
 
-// Each segment takes the range of its entries (order of segments is free).
+// Source chain: each segment takes the range of its entries (order of
+// segments is free).
 __device__ void adm_alloc(const LPArgs& a, int64_t nseg, int64_t* ct) {
   for (int64_t sg = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; sg < nseg;
        sg += (int64_t)gridDim.x * blockDim.x) {
@@ -1353,13 +1515,20 @@ __device__ void adm_alloc(const LPArgs& a, int64_t nseg, int64_t* ct) {
   }
 }
 
-__device__ void adm_scatter(const LPArgs& a, int64_t lbeg, int64_t cnt) {
+// Writes the staged proposals into their segments (any: there are segments)
+// and, on the target side, clears the incoming weights.
+__device__ void adm_scatter(const LPArgs& a, int64_t lbeg, int64_t cnt, bool any, int32_t source) {
+  if (!any && source) return;
   for (int64_t li = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; li < cnt;
        li += (int64_t)gridDim.x * blockDim.x) {
     const int64_t i = lbeg + li;
-    if (a.stage[i] == 0) continue;
-    const int32_t g = a.grp[i];
-    const int64_t pos = a.ovf_base[g] + atomicAdd(&a.ovf_fill[g], 1);
+    if (!source) {
+      const int32_t t = a.prop_t[i];
+      if (t >= 0 && SCLAP_OK(t, a.nlabels, a.err)) a.in_w[t] = 0;
+    }
+    const int32_t st = any ? a.stage[i] : 0;
+    if (st == 0) continue;
+    const int64_t pos = a.ovf_base[a.grp[i]] + st - 1;
     const int4 r = a.rec[i];
     a.ent_key[pos] = a.prop_key[i];
     a.ent_v[pos] = r.x;
@@ -1368,8 +1537,10 @@ __device__ void adm_scatter(const LPArgs& a, int64_t lbeg, int64_t cnt) {
   }
 }
 
-constexpr int SEL_NT = 256;
 constexpr int SEL_SMALL = 64;     // all-pairs ranking up to this many entries
+constexpr int SEL_NT = 512;       // threads of the selection launch
+constexpr int SEL_CL = 8;         // CTAs of a selection cluster
+constexpr int SEL_CTA = 4096;     // entries a single CTA selects at most (with clusters)
 
 __device__ __forceinline__ bool key_less(uint64_t k1, int32_t v1, uint64_t k2, int32_t v2) {
   return k1 < k2 || (k1 == k2 && v1 < v2);
@@ -1378,58 +1549,303 @@ __device__ __forceinline__ uint32_t digit_of(uint64_t k, int32_t v, int p) {
   return p < 8 ? (uint32_t)(k >> (56 - 8 * p)) & 0xffu
                : ((uint32_t)v >> (24 - 8 * (p - 8))) & 0xffu;
 }
+// (k, v) shares the first p digits of (PK, PV).
+__device__ __forceinline__ bool digits_match(uint64_t k, int32_t v, uint64_t PK, uint32_t PV,
+                                             int p) {
+  if (p == 0) return true;
+  if (p <= 8) return ((k ^ PK) >> (64 - 8 * p)) == 0;
+  return k == PK && (((uint32_t)v ^ PV) >> (32 - 8 * (p - 8))) == 0;
+}
 
-// Admission inside one overflowing group: entries ordered by (key, node);
+// Admission inside one overflowing segment: entries ordered by (key, node);
 // target side admits while the inclusive prefix weight <= thr, source side
-// while the exclusive prefix weight <= thr.  Groups of <= 64 entries rank
-// all pairs in shared memory.  Larger ones locate the boundary entry (the
-// first whose inclusive prefix exceeds thr) by an MSD radix select over the
-// 96-bit (key, node) order: the bytes shared by the smallest and largest
-// entry are skipped, each pass histograms the weights of the entries still
-// matching the chosen prefix, and once <= 64 candidates remain they are
-// ranked in shared memory.
-__device__ __forceinline__ void select_rank_small(const LPArgs& a, int n, int64_t thr,
-                                                  int64_t acc, uint64_t* sk, int32_t* sv,
-                                                  int32_t* sw, int32_t* si, bool write_adm,
-                                                  int32_t source, uint64_t* bk, int32_t* bv,
-                                                  int* bfound) {
-  // excl/incl prefix of every staged entry; write admissions directly, or
-  // report the boundary entry (smallest with acc + incl > thr).
+// while the exclusive prefix weight <= thr.  Segments of <= 64 entries: one
+// warp ranks all pairs through shuffles.  Larger ones locate the boundary
+// entry (the first whose inclusive prefix exceeds thr) by an MSD radix select
+// over the 96-bit (key, node) order: the bytes shared by the smallest and
+// largest entry are skipped, each pass histograms the weights of the entries
+// still matching the chosen prefix (node weights sum below 2^31, so 32-bit
+// sums do), the matching entries are copied together when they are few, and
+// once <= 64 candidates remain they are ranked in shared memory.
+//
+// A segment above SEL_CTA entries (the proposals into a block, or into a
+// hub's cluster: up to millions) is selected by a cluster of SEL_CL CTAs that
+// shares one state in the first CTA's shared memory; one CTA of 256 threads
+// read such a segment at a fraction of a percent of the memory rate while the
+// rest of the GPU waited (R-MAT 2^22 nodes, k = 8: 10.4 -> 4.5 ms, which now
+// includes applying the moves).
+struct SelState {
+  unsigned int hist[256], hcnt[256];
+  // smallest and largest key and node each warp met (64-bit atomics on
+  // another CTA's shared memory lose updates against local ones)
+  uint64_t wkmin[SEL_NT / 32], wkmax[SEL_NT / 32];
+  int32_t wvmin[SEL_NT / 32], wvmax[SEL_NT / 32];
+  uint64_t BK;
+  int32_t BV;
+  long long acc;
+  int found, done, x, nx, ncomp, bfound;
+  uint64_t sk[SEL_SMALL];
+  int32_t sv[SEL_SMALL], sw[SEL_SMALL];
+};
+
+// The boundary entry among n staged candidates: the unique one whose
+// inclusive prefix weight (acc and the smaller candidates included) first
+// exceeds thr.
+__device__ __forceinline__ void select_rank_small(SelState& S, int n, int64_t thr, int64_t acc) {
   for (int j = threadIdx.x; j < n; j += blockDim.x) {
     int64_t excl = acc;
-    const uint64_t kj = sk[j];
-    const int32_t vj = sv[j];
+    const uint64_t kj = S.sk[j];
+    const int32_t vj = S.sv[j];
     for (int l = 0; l < n; ++l)
-      if (key_less(sk[l], sv[l], kj, vj)) excl += sw[l];
-    if (write_adm) {
-      const bool ok = source ? (excl <= thr) : (excl + sw[j] <= thr);
-      a.adm[si[j]] = ok ? 1 : 0;
-    } else if (excl + sw[j] > thr && excl <= thr) {
-      *bk = kj;      // the unique entry whose inclusive prefix first exceeds thr
-      *bv = vj;
-      *bfound = 1;
+      if (key_less(S.sk[l], S.sv[l], kj, vj)) excl += S.sw[l];
+    if (excl + S.sw[j] > thr && excl <= thr) {
+      S.BK = kj;
+      S.BV = vj;
+      S.bfound = 1;
     }
   }
 }
 
-__device__ void adm_select(const LPArgs& a, int64_t nseg, int32_t source) {
-  __shared__ uint64_t sk[SEL_SMALL];
-  __shared__ int32_t sv[SEL_SMALL];
-  __shared__ int32_t sw[SEL_SMALL];
-  __shared__ int32_t si[SEL_SMALL];
-  __shared__ unsigned long long hist[256];
-  __shared__ unsigned int hcnt[256];
-  __shared__ uint64_t PK, kmin_sh, kmax_sh, BK;
-  __shared__ uint32_t PV;
-  __shared__ int32_t vmin_sh, vmax_sh, BV;
-  __shared__ long long acc_sh;
-  __shared__ int found_sh, ncand_sh, bfound_sh, done_sh, x_sh, ncomp_sh;
-  const int tid = threadIdx.x, lane = tid & 31;
-  // Phase 1: groups of <= 64 entries, one warp each (entries lane and
-  // lane + 32 in registers, every pair ranked through shuffles).
+// Segment sg, selected by CL CTAs (1: this CTA; else the cluster).  L is this
+// CTA's state, S the first CTA's.
+template <bool APPLY, int CL>
+__device__ __forceinline__ void select_large(const LPArgs& a, ApplyHash* h, MovedRun& m,
+                                             int32_t sub, int64_t sg, int32_t source,
+                                             SelState& L) {
+  const int tid = threadIdx.x, lane = tid & 31, NT = blockDim.x;
+  const int rank = CL > 1 ? (int)cluster_rank() : 0;
+  SelState& S = CL > 1 ? *cluster_map(&L, 0) : L;
+  auto sync = [&] {
+    if (CL > 1) cluster_sync();
+    else __syncthreads();
+  };
+  const int64_t base = a.seg_base[sg];
+  const int32_t n = a.seg_cnt[sg];
+  const int64_t thr = a.seg_thr[sg];
+  const int32_t g = a.seg_g[sg];
+  const int64_t j0 = (int64_t)rank * NT + tid, jstep = (int64_t)CL * NT;
+  // smallest and largest (key, node): their shared leading bytes are skipped
+  for (int j = tid; j < 256; j += NT) { L.hist[j] = 0; L.hcnt[j] = 0; }
+  if (rank == 0 && tid == 0) {
+    L.acc = 0;
+    L.found = 1;
+    L.done = 0;
+    L.ncomp = 0;
+    L.bfound = 0;
+  }
   {
-    const int64_t nw = (int64_t)gridDim.x * (SEL_NT / 32);
-    for (int64_t sg = (int64_t)blockIdx.x * (SEL_NT / 32) + (tid >> 5); sg < nseg; sg += nw) {
+    unsigned long long lmin = ~0ull, lmax = 0;
+    int32_t vmin = INT32_MAX, vmax = -1;
+    for (int64_t j = j0; j < n; j += jstep) {
+      const uint64_t k = a.ent_key[base + j];
+      const int32_t v = a.ent_v[base + j];
+      lmin = k < lmin ? k : lmin;
+      lmax = k > lmax ? k : lmax;
+      vmin = min(vmin, v);
+      vmax = max(vmax, v);
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+      const unsigned long long y = __shfl_xor_sync(0xffffffffu, lmin, o);
+      const unsigned long long z = __shfl_xor_sync(0xffffffffu, lmax, o);
+      lmin = y < lmin ? y : lmin;
+      lmax = z > lmax ? z : lmax;
+    }
+    vmin = __reduce_min_sync(0xffffffffu, vmin);
+    vmax = __reduce_max_sync(0xffffffffu, vmax);
+    if (lane == 0) {
+      L.wkmin[tid >> 5] = lmin;
+      L.wkmax[tid >> 5] = lmax;
+      L.wvmin[tid >> 5] = vmin;
+      L.wvmax[tid >> 5] = vmax;
+    }
+  }
+  sync();
+  int p0 = 0;
+  uint64_t kmin = ~0ull, kmax = 0;
+  int32_t vmin = INT32_MAX, vmax = -1;
+  for (int q = lane; q < CL * (NT >> 5); q += 32) {
+    const SelState& R = CL > 1 ? *cluster_map(&L, (uint32_t)(q / (NT >> 5))) : L;
+    const int w = q % (NT >> 5);
+    kmin = R.wkmin[w] < kmin ? R.wkmin[w] : kmin;
+    kmax = R.wkmax[w] > kmax ? R.wkmax[w] : kmax;
+    vmin = min(vmin, R.wvmin[w]);
+    vmax = max(vmax, R.wvmax[w]);
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    const uint64_t y = __shfl_xor_sync(0xffffffffu, (unsigned long long)kmin, o);
+    const uint64_t z = __shfl_xor_sync(0xffffffffu, (unsigned long long)kmax, o);
+    kmin = y < kmin ? y : kmin;
+    kmax = z > kmax ? z : kmax;
+  }
+  vmin = __reduce_min_sync(0xffffffffu, vmin);
+  vmax = __reduce_max_sync(0xffffffffu, vmax);
+  while (p0 < 8 && digit_of(kmin, 0, p0) == digit_of(kmax, 0, p0)) ++p0;
+  if (p0 == 8)
+    while (p0 < 12 && digit_of(0, vmin, p0) == digit_of(0, vmax, p0)) ++p0;
+  uint64_t PK = p0 >= 8 ? kmin : (p0 == 0 ? 0ull : (kmin >> (64 - 8 * p0)) << (64 - 8 * p0));
+  const int pv0 = p0 > 8 ? p0 - 8 : 0;
+  uint32_t PV = pv0 == 0 ? 0u : (((uint32_t)vmin >> (32 - 8 * pv0)) << (32 - 8 * pv0));
+  const uint64_t* ck = a.ent_key + base;
+  const int32_t* cv = a.ent_v + base;
+  const int32_t* cw = a.ent_w + base;
+  int64_t cn = n;
+  int buf = 0, p = p0;
+  bool found = true;
+  for (; p < 12; ++p) {
+    {
+      // runs of equal digits are summed in registers and added once: in a
+      // large segment most entries share the leading digits, and one shared
+      // atomic per entry on the same bin would serialise
+      uint32_t dc = 0xffffffffu;
+      unsigned int wacc = 0, cacc = 0;
+      for (int64_t j = j0; j < cn; j += jstep) {
+        const uint64_t k = ck[j];
+        const int32_t v = cv[j];
+        if (!digits_match(k, v, PK, PV, p)) continue;
+        const uint32_t d = digit_of(k, v, p);
+        if (d != dc) {
+          if (cacc) {
+            atomicAdd(&L.hist[dc], wacc);
+            atomicAdd(&L.hcnt[dc], cacc);
+          }
+          dc = d;
+          wacc = 0;
+          cacc = 0;
+        }
+        wacc += (unsigned int)cw[j];
+        cacc += 1;
+      }
+      if (cacc) {
+        atomicAdd(&L.hist[dc], wacc);
+        atomicAdd(&L.hcnt[dc], cacc);
+      }
+    }
+    __syncthreads();
+    if (CL > 1 && rank != 0) {
+      // this CTA's bins into the first CTA's, and clean for the next pass
+      for (int j = tid; j < 256; j += NT)
+        if (L.hcnt[j]) {
+          atomicAdd(&S.hist[j], L.hist[j]);
+          atomicAdd(&S.hcnt[j], L.hcnt[j]);
+          L.hist[j] = 0;
+          L.hcnt[j] = 0;
+        }
+    }
+    sync();
+    if (rank == 0) {
+      if (tid < 32) {
+        // first digit whose bin takes the running weight past thr: each
+        // lane owns 8 consecutive bins, a warp scan gives its offset
+        long long loc[8], sum = 0;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) { loc[q] = (long long)L.hist[tid * 8 + q]; sum += loc[q]; }
+        long long incl = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const long long y = __shfl_up_sync(0xffffffffu, incl, o);
+          if (tid >= o) incl += y;
+        }
+        long long run = L.acc + incl - sum;
+        int xq = -1;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          if (xq < 0) {
+            if (run + loc[q] > thr) xq = q;
+            else run += loc[q];
+          }
+        }
+        const unsigned fm = __ballot_sync(0xffffffffu, xq >= 0);
+        if (fm == 0) {
+          if (tid == 0) L.found = 0;     // every remaining entry fits
+        } else if (tid == __ffs(fm) - 1) {
+          const int x = tid * 8 + xq;
+          L.acc = run;
+          L.x = x;
+          L.nx = (int)L.hcnt[x];
+          L.done = L.nx <= SEL_SMALL;
+          L.ncomp = 0;
+        }
+      }
+      __syncthreads();
+      for (int j = tid; j < 256; j += NT) { L.hist[j] = 0; L.hcnt[j] = 0; }
+    }
+    sync();
+    found = S.found != 0;
+    if (!found) break;
+    const uint32_t x = (uint32_t)S.x;
+    const int nx = S.nx;
+    const bool done = S.done != 0;
+    if (p < 8) PK |= (uint64_t)x << (56 - 8 * p);
+    else PV |= x << (24 - 8 * (p - 8));
+    // the matching entries: to the shared-memory candidates when few enough,
+    // copied together when that saves the later passes most of their reading
+    const bool copy = !done && (int64_t)nx * 4 <= cn;
+    if (done || copy) {
+      uint64_t* dk = a.sel_key[buf] + base;
+      int32_t* dv = a.sel_v[buf] + base;
+      int32_t* dw = a.sel_w[buf] + base;
+      for (int64_t j = j0; j < cn; j += jstep) {
+        const uint64_t k = ck[j];
+        const int32_t v = cv[j];
+        if (!digits_match(k, v, PK, PV, p + 1)) continue;
+        const int q = atomicAdd(&S.ncomp, 1);
+        if (done) {
+          S.sk[q] = k;
+          S.sv[q] = v;
+          S.sw[q] = cw[j];
+        } else {
+          dk[q] = k;
+          dv[q] = v;
+          dw[q] = cw[j];
+        }
+      }
+      sync();
+      if (copy) {
+        ck = dk;
+        cv = dv;
+        cw = dw;
+        cn = nx;
+        buf ^= 1;
+      }
+    }
+    if (done) break;
+  }
+  if (found && p < 12) {
+    if (rank == 0) select_rank_small(L, S.ncomp, thr, L.acc);
+    sync();
+    if (S.bfound) { PK = S.BK; PV = (uint32_t)S.BV; }
+  }
+  for (int64_t b0 = 0; b0 < n; b0 += jstep) {
+    const int64_t j = b0 + j0;
+    bool ok = false;
+    int32_t i = 0;
+    if (j < n) {
+      const uint64_t k = a.ent_key[base + j];
+      const int32_t v = a.ent_v[base + j];
+      i = a.ent_i[base + j];
+      if (!found) ok = true;
+      else ok = key_less(k, v, PK, (int32_t)PV) || (source && k == PK && v == (int32_t)PV);
+      if (!APPLY) a.adm[i] = ok ? 1 : 0;
+    }
+    if (APPLY) move_warp(a, *h, m, sub, ok, i, g);
+  }
+  if (rank == 0 && tid == 0) a.ovf_cnt[g] = 0;
+  sync();                                  // the state is free again
+}
+
+// All segments of one side of a colour class.  CL > 1: the launch has
+// clusters of CL CTAs, which take the segments above SEL_CTA entries.
+template <bool APPLY, int CL>
+__device__ void adm_select(const LPArgs& a, ApplyHash* h, SelState& L, int32_t sub, int64_t nseg,
+                           int32_t source) {
+  MovedRun m;
+  const int tid = threadIdx.x, lane = tid & 31;
+  // segments of <= 64 entries, one warp each (entries lane and lane + 32 in
+  // registers, every pair ranked through shuffles)
+  {
+    const int wpc = blockDim.x >> 5;
+    const int64_t nw = (int64_t)gridDim.x * wpc;
+    for (int64_t sg = (int64_t)(tid >> 5) * gridDim.x + blockIdx.x; sg < nseg; sg += nw) {
       const int32_t n = a.seg_cnt[sg];
       if (n > SEL_SMALL) continue;
       const int64_t base = a.seg_base[sg];
@@ -1457,328 +1873,86 @@ __device__ void adm_select(const LPArgs& a, int64_t nseg, int32_t source) {
         e0 += key_less(kl, vl, k0, v0) ? wl : 0;
         e1 += key_less(kl, vl, k1, v1) ? wl : 0;
       }
-      if (h0) a.adm[a.ent_i[base + lane]] = (source ? e0 <= thr : e0 + w0 <= thr) ? 1 : 0;
-      if (h1) a.adm[a.ent_i[base + lane + 32]] = (source ? e1 <= thr : e1 + w1 <= thr) ? 1 : 0;
-      if (lane == 0) {
-        const int32_t g = a.seg_g[sg];
-        a.ovf_cnt[g] = 0;
-        a.ovf_fill[g] = 0;
-      }
-    }
-  }
-  // Phase 2: larger groups, one CTA each.
-  for (int64_t sg = blockIdx.x; sg < nseg; sg += gridDim.x) {
-    const int64_t base = a.seg_base[sg];
-    const int32_t n = a.seg_cnt[sg];
-    const int64_t thr = a.seg_thr[sg];
-    if (n <= SEL_SMALL) continue;
-    {
-      // smallest and largest (key, node): their shared leading bytes are skipped
-      if (tid == 0) { kmin_sh = ~0ull; kmax_sh = 0; vmin_sh = INT32_MAX; vmax_sh = -1; }
-      __syncthreads();
-      uint64_t lmin = ~0ull, lmax = 0;
-      for (int64_t j = tid; j < n; j += SEL_NT) {
-        const uint64_t k = a.ent_key[base + j];
-        lmin = k < lmin ? k : lmin;
-        lmax = k > lmax ? k : lmax;
-      }
-      atomicMin(reinterpret_cast<unsigned long long*>(&kmin_sh), lmin);
-      atomicMax(reinterpret_cast<unsigned long long*>(&kmax_sh), lmax);
-      __syncthreads();
-      const uint64_t kmin = kmin_sh, kmax = kmax_sh;
-      int p0 = 0;
-      while (p0 < 8 && digit_of(kmin, 0, p0) == digit_of(kmax, 0, p0)) ++p0;
-      if (p0 == 8) {
-        int32_t l1 = INT32_MAX, l2 = -1;
-        for (int64_t j = tid; j < n; j += SEL_NT) {
-          const int32_t v = a.ent_v[base + j];
-          l1 = v < l1 ? v : l1;
-          l2 = v > l2 ? v : l2;
-        }
-        atomicMin(&vmin_sh, l1);
-        atomicMax(&vmax_sh, l2);
-        __syncthreads();
-        while (p0 < 12 && digit_of(0, vmin_sh, p0) == digit_of(0, vmax_sh, p0)) ++p0;
-      }
-      if (tid == 0) {
-        PK = p0 >= 8 ? kmin : (p0 == 0 ? 0ull : (kmin >> (64 - 8 * p0)) << (64 - 8 * p0));
-        const int pv = p0 > 8 ? p0 - 8 : 0;
-        PV = pv == 0 ? 0u : (((uint32_t)vmin_sh >> (32 - 8 * pv)) << (32 - 8 * pv));
-        acc_sh = 0;
-        found_sh = 1;
-        done_sh = 0;
-        ncand_sh = 0;
-        bfound_sh = 0;
-      }
-      __syncthreads();
-      // Each pass histograms only the entries still sharing the chosen
-      // prefix: after the digit is picked, the entries of its bin are
-      // compacted into a scratch copy (two copies used in turn), so later
-      // passes read the survivors, not the whole group.
-      const uint64_t* ck = a.ent_key + base;
-      const int32_t* cv = a.ent_v + base;
-      const int32_t* cw = a.ent_w + base;
-      int64_t cn = n;
-      int buf = 0;
-      int p = p0;
-      for (; p < 12; ++p) {
-        for (int j = tid; j < 256; j += SEL_NT) { hist[j] = 0; hcnt[j] = 0; }
-        __syncthreads();
-        {
-          // runs of equal digits are summed in registers and added once: in
-          // a large group most entries share the leading digits, and one
-          // shared atomic per entry on the same bin would serialise
-          uint32_t dc = 0xffffffffu;
-          unsigned long long wacc = 0;
-          unsigned int cacc = 0;
-          for (int64_t j = tid; j < cn; j += SEL_NT) {
-            const uint32_t d = digit_of(ck[j], cv[j], p);
-            if (d != dc) {
-              if (cacc) {
-                atomicAdd(&hist[dc], wacc);
-                atomicAdd(&hcnt[dc], cacc);
-              }
-              dc = d;
-              wacc = 0;
-              cacc = 0;
-            }
-            wacc += (unsigned long long)cw[j];
-            cacc += 1;
-          }
-          if (cacc) {
-            atomicAdd(&hist[dc], wacc);
-            atomicAdd(&hcnt[dc], cacc);
-          }
-        }
-        __syncthreads();
-        if (tid < 32) {
-          // first digit whose bin takes the running weight past thr: each
-          // lane owns 8 consecutive bins, a warp scan gives its offset
-          long long loc[8], sum = 0;
-#pragma unroll
-          for (int q = 0; q < 8; ++q) { loc[q] = (long long)hist[tid * 8 + q]; sum += loc[q]; }
-          long long incl = sum;
-#pragma unroll
-          for (int o = 1; o < 32; o <<= 1) {
-            const long long y = __shfl_up_sync(0xffffffffu, incl, o);
-            if (tid >= o) incl += y;
-          }
-          long long run = acc_sh + incl - sum;
-          int xq = -1;
-#pragma unroll
-          for (int q = 0; q < 8; ++q) {
-            if (xq < 0) {
-              if (run + loc[q] > thr) xq = q;
-              else run += loc[q];
-            }
-          }
-          const unsigned fm = __ballot_sync(0xffffffffu, xq >= 0);
-          if (fm == 0) {
-            if (tid == 0) found_sh = 0;   // every remaining entry fits
-          } else if (tid == __ffs(fm) - 1) {
-            const int x = tid * 8 + xq;
-            acc_sh = run;
-            if (p < 8) PK |= (uint64_t)x << (56 - 8 * p);
-            else PV |= (uint32_t)x << (24 - 8 * (p - 8));
-            if (hcnt[x] <= SEL_SMALL) done_sh = 1;
-            x_sh = x;
-            ncomp_sh = 0;
-          }
-        }
-        __syncthreads();
-        if (!found_sh) break;
-        {
-          const uint32_t x = (uint32_t)x_sh;
-          uint64_t* dk = a.sel_key[buf] + base;
-          int32_t* dv = a.sel_v[buf] + base;
-          int32_t* dw = a.sel_w[buf] + base;
-          for (int64_t j = tid; j < cn; j += SEL_NT) {
-            const uint64_t k = ck[j];
-            const int32_t v = cv[j];
-            if (digit_of(k, v, p) == x) {
-              const int q = atomicAdd(&ncomp_sh, 1);
-              dk[q] = k;
-              dv[q] = v;
-              dw[q] = cw[j];
-            }
-          }
-          __syncthreads();
-          ck = dk;
-          cv = dv;
-          cw = dw;
-          cn = ncomp_sh;
-          buf ^= 1;
-        }
-        if (done_sh) break;
-      }
-      if (found_sh && done_sh && p < 11) {
-        // the few survivors are the candidates sharing the chosen prefix
-        for (int64_t j = tid; j < cn; j += SEL_NT) {
-          sk[j] = ck[j];
-          sv[j] = cv[j];
-          sw[j] = cw[j];
-        }
-        if (tid == 0) ncand_sh = (int)cn;
-        __syncthreads();
-        select_rank_small(a, ncand_sh, thr, acc_sh, sk, sv, sw, si, false, source, &BK, &BV,
-                          &bfound_sh);
-        __syncthreads();
-        if (tid == 0 && bfound_sh) { PK = BK; PV = (uint32_t)BV; }
-        __syncthreads();
-      }
-      const int found = found_sh;
-      const uint64_t pk = PK;
-      const int32_t pv = (int32_t)PV;
-      for (int64_t j = tid; j < n; j += SEL_NT) {
-        const uint64_t k = a.ent_key[base + j];
-        const int32_t v = a.ent_v[base + j];
-        bool ok;
-        if (!found) ok = true;
-        else if (source) ok = key_less(k, v, pk, pv) || (k == pk && v == pv);
-        else ok = key_less(k, v, pk, pv);
-        a.adm[a.ent_i[base + j]] = ok ? 1 : 0;
-      }
-      __syncthreads();
-    }
-    if (tid == 0) {
       const int32_t g = a.seg_g[sg];
-      a.ovf_cnt[g] = 0;
-      a.ovf_fill[g] = 0;
+      const bool ok0 = h0 && (source ? e0 <= thr : e0 + w0 <= thr);
+      const bool ok1 = h1 && (source ? e1 <= thr : e1 + w1 <= thr);
+      const int32_t i0 = h0 ? a.ent_i[base + lane] : 0;
+      const int32_t i1 = h1 ? a.ent_i[base + lane + 32] : 0;
+      if (APPLY) {
+        move_warp(a, *h, m, sub, ok0, i0, g);
+        if (n > 32) move_warp(a, *h, m, sub, ok1, i1, g);
+      } else {
+        if (h0) a.adm[i0] = ok0 ? 1 : 0;
+        if (h1) a.adm[i1] = ok1 ? 1 : 0;
+      }
+      if (lane == 0) a.ovf_cnt[g] = 0;
     }
   }
-}
-
-// ------------------------------------------------------------- apply
-// Admitted moves update labels and weights; moved nodes activate their
-// neighbours (small rows by their own lane, larger rows by the whole warp).
-// Label-weight changes are first summed per CTA in a small shared hash
-// (label -> delta; a label that finds no slot within a few probes goes to
-// global memory directly), then flushed with one atomic per label: in local
-// search moves concentrate on a handful of blocks, and in clustering many
-// nodes can join one cluster in a colour class (the leaves of a hub), whose
-// global counters would otherwise take one atomic per moved node each.  The
-// clusters that clustering moves leave are spread out and are updated
-// directly.
-constexpr int APPLY_SLOTS = 1024;
-__device__ __forceinline__ void apply_delta(int32_t* hk, int32_t* hv, wgt_t* W, int32_t L,
-                                            int32_t d, int64_t nW, int32_t* err) {
-  uint32_t s = table_slot(L, 10);
-#pragma unroll 1
-  for (int p = 0; p < 8; ++p) {
-    const int32_t prev = atomicCAS(&hk[s], -1, L);
-    if (prev == -1 || prev == L) {
-      atomicAdd(&hv[s], d);
-      return;
-    }
-    s = (s + 1) & (APPLY_SLOTS - 1);
-  }
-  if (SCLAP_OK(L, nW, err)) atomicAdd(&W[L], (wgt_t)d);
-}
-
-constexpr int64_t MARK_CH = 4096;     // arcs per queued chunk of a moved long row
-
-__device__ void adm_apply(const LPArgs& a, int64_t lbeg, int64_t cnt, int32_t sub) {
-  uint8_t* const an = act_next(a);
-  __shared__ int32_t hk[APPLY_SLOTS];
-  __shared__ int32_t hv[APPLY_SLOTS];
-  const bool agg_src = a.mode != MODE_CLUSTER;
-  for (int j = threadIdx.x; j < APPLY_SLOTS; j += blockDim.x) { hk[j] = -1; hv[j] = 0; }
   __syncthreads();
+  // larger ones: a CTA each
+  for (int64_t sg = blockIdx.x; sg < nseg; sg += gridDim.x) {
+    const int32_t n = a.seg_cnt[sg];
+    if (n > SEL_SMALL && (CL == 1 || n <= SEL_CTA))
+      select_large<APPLY, 1>(a, h, m, sub, sg, source, L);
+  }
+  // the largest: a cluster each
+  if (CL > 1) {
+    cluster_sync();
+    for (int64_t sg = blockIdx.x / CL; sg < nseg; sg += gridDim.x / CL)
+      if (a.seg_cnt[sg] > SEL_CTA) select_large<APPLY, CL>(a, h, m, sub, sg, source, L);
+  }
+  if (APPLY) moved_flush(a, m);
+}
+
+// Source chain: applies the proposals left admitted.
+__device__ __forceinline__ void adm_apply(const LPArgs& a, ApplyHash& h, int64_t lbeg, int64_t cnt,
+                                          int32_t sub) {
   const int lane = threadIdx.x & 31;
   const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  int32_t run_slot = -1;           // moves counted in registers per slot run
-  unsigned long long run_cnt = 0;
+  MovedRun m;
   for (int64_t b0 = w0 * 32; b0 < cnt; b0 += nw * 32) {
-    const int64_t li = b0 + lane;
-    int32_t slot = -1;
-    int64_t rs = 0, re = 0;
-    if (li < cnt) {
-      const int64_t i = lbeg + li;
-      const int32_t t = a.prop_t[i];
-      const int8_t ad = a.adm[i];
-      if (t >= 0 && SCLAP_OK(t, a.nlabels, a.err)) {
-        a.in_w[t] = 0;
-        if (ad) {
-          const int4 r = a.rec[i];
-          const int32_t v = r.x, own = r.y, cv = r.z;
-          slot = r.w;
-          if (an) {
-            const longlong2 r2 = a.rec2[i];
-            rs = r2.x;
-            re = r2.x + r2.y;
-          }
-          if (SCLAP_OK(v, a.N, a.err)) a.label[v] = t;
-          apply_delta(hk, hv, a.W, t, cv, a.nlabels, a.err);
-          if (agg_src) apply_delta(hk, hv, a.W, own, -cv, a.nlabels, a.err);
-          else if (SCLAP_OK(own, a.nlabels, a.err)) atomicSub(&a.W[own], (wgt_t)cv);
-          if (re - rs <= 8) {
-            for (int64_t e = rs; e < re; ++e)
-              if (SCLAP_OK(a.col[e], a.N, a.err)) an[a.col[e]] = 1;
-            re = rs;
-          } else if (a.mark_big > 0 && re - rs > a.mark_big) {
-            const int32_t nch = (int32_t)((re - rs + MARK_CH - 1) / MARK_CH);
-            const int32_t q0 = atomicAdd(&a.mqn[sub], nch);
-            for (int32_t c = 0; c < nch; ++c)
-              a.mq[q0 + c] = make_longlong2(rs + c * MARK_CH, min64(rs + (c + 1) * MARK_CH, re));
-            re = rs;
-          }
-        }
-      }
-    }
-    unsigned big = __ballot_sync(0xffffffffu, re > rs);
-    while (big) {
-      const int src = __ffs(big) - 1;
-      big &= big - 1;
-      const int64_t s0 = __shfl_sync(0xffffffffu, (long long)rs, src);
-      const int64_t s1 = __shfl_sync(0xffffffffu, (long long)re, src);
-      for (int64_t e = s0 + lane; e < s1; e += 32)
-        if (SCLAP_OK(a.col[e], a.N, a.err)) an[a.col[e]] = 1;
-    }
-    const unsigned mm = __match_any_sync(0xffffffffu, slot);
-    if (slot >= 0 && lane == __ffs(mm) - 1) {
-      if (slot == run_slot) {
-        run_cnt += __popc(mm);
-      } else {
-        if (run_cnt) atomicAdd(ull(&a.moved[run_slot]), run_cnt);
-        run_slot = slot;
-        run_cnt = __popc(mm);
-      }
-    }
+    const int64_t i = lbeg + b0 + lane;
+    const bool in = b0 + lane < cnt;
+    const int32_t t = in ? a.prop_t[i] : -1;
+    move_warp(a, h, m, sub, t >= 0 && a.adm[i], i, t);
   }
-  if (run_cnt) atomicAdd(ull(&a.moved[run_slot]), run_cnt);
-  __syncthreads();
-  for (int j = threadIdx.x; j < APPLY_SLOTS; j += blockDim.x)
-    if (hk[j] >= 0 && hv[j] != 0 && SCLAP_OK(hk[j], a.nlabels, a.err))
-      atomicAdd(&a.W[hk[j]], (wgt_t)hv[j]);
+  moved_flush(a, m);
 }
 
 constexpr int ADM_NT = 256;
 
-// The admission and application of colour class `sub` (see "admission"
-// above).  source_chain: local search, forced moves out of overloaded
-// blocks are possible this round.
+// The admission and application of colour class `sub` as ONE cooperative
+// launch, its phases separated by bounded grid barriers (tuning
+// fused_admission).  When no target overflows (known to every CTA after the
+// first barrier) only the incoming weights are left to clear.
+// source_chain: local search, forced moves out of overloaded blocks are
+// possible this round.
 __global__ void __launch_bounds__(ADM_NT) k_admit(LPArgs a, int32_t sub, int32_t source_chain,
                                                   GridSync* gs) {
   if (blockIdx.x == 0 && threadIdx.x < 4) a.ctr[((sub + 1) & 1) * 4 + threadIdx.x] = 0;
   // a bounded wait of an earlier launch ran out: the run is abandoned
   if (*(volatile int32_t*)a.err & DERR_TIMEOUT) return;
+  __shared__ ApplyHash h;
+  __shared__ SelState sel;
+  apply_init(h);
   int64_t lbeg, cnt;
   sub_range(a, sub, 0, NB, &lbeg, &cnt);
   const uint32_t lim = a.wait_limit;
   int64_t* ct = adm_ctr(a, sub, 0);
-  adm_resolve(a, lbeg, cnt, ct);
+  const bool chain = source_chain && *(volatile int32_t*)a.flags != 0;
+  if (chain) adm_resolve<false>(a, &h, sub, lbeg, cnt, ct);
+  else adm_resolve<true>(a, &h, sub, lbeg, cnt, ct);
   if (!grid_sync(gs, a.err, lim)) return;
   const int64_t nseg = *(volatile int64_t*)&ct[1];
+  adm_scatter(a, lbeg, cnt, nseg > 0, 0);
   if (nseg > 0) {
-    adm_alloc(a, nseg, ct);
     if (!grid_sync(gs, a.err, lim)) return;
-    adm_scatter(a, lbeg, cnt);
-    if (!grid_sync(gs, a.err, lim)) return;
-    adm_select(a, nseg, 0);
-    if (!grid_sync(gs, a.err, lim)) return;
+    if (chain) adm_select<false, 1>(a, &h, sel, sub, nseg, 0);
+    else adm_select<true, 1>(a, &h, sel, sub, nseg, 0);
   }
-  if (source_chain && *(volatile int32_t*)a.flags != 0) {
+  if (chain) {
+    if (!grid_sync(gs, a.err, lim)) return;
     int64_t* cs = adm_ctr(a, sub, 1);
     adm_forced(a, lbeg, cnt, cs);
     if (!grid_sync(gs, a.err, lim)) return;
@@ -1786,13 +1960,14 @@ __global__ void __launch_bounds__(ADM_NT) k_admit(LPArgs a, int32_t sub, int32_t
     if (nsrc > 0) {
       adm_alloc(a, nsrc, cs);
       if (!grid_sync(gs, a.err, lim)) return;
-      adm_scatter(a, lbeg, cnt);
+      adm_scatter(a, lbeg, cnt, true, 1);
       if (!grid_sync(gs, a.err, lim)) return;
-      adm_select(a, nsrc, 1);
+      adm_select<false, 1>(a, &h, sel, sub, nsrc, 1);
       if (!grid_sync(gs, a.err, lim)) return;
     }
+    adm_apply(a, h, lbeg, cnt, sub);
   }
-  adm_apply(a, lbeg, cnt, sub);
+  apply_flush(a, h);
 }
 
 // The same phases as separate launches, chained on one stream with
@@ -1800,44 +1975,71 @@ __global__ void __launch_bounds__(ADM_NT) k_admit(LPArgs a, int32_t sub, int32_t
 // chain measured faster than the cooperative kernel, whose launches also
 // slowed the propose launches that follow them).  Every kernel waits for
 // its predecessor first; the later phases read the segment counters on the
-// device and return at once when there is nothing to do.
-__global__ void __launch_bounds__(ADM_NT) k_resolve(LPArgs a, int32_t sub) {
+// device and return at once when there is nothing to do.  The source chain's
+// launches follow only when source_chain is set: the host then knows, or
+// (CUDA graph) must assume, that a listed node sits in an overloaded block,
+// and what the first launches do is decided by the flag on the device.
+__device__ __forceinline__ bool chain_on(const LPArgs& a, int32_t source_chain) {
+  return source_chain && *(volatile int32_t*)a.flags != 0;
+}
+__global__ void __launch_bounds__(ADM_NT) k_resolve(LPArgs a, int32_t sub, int32_t source_chain) {
   griddep_wait();
+  __shared__ ApplyHash h;
   if (blockIdx.x == 0 && threadIdx.x < 4) a.ctr[((sub + 1) & 1) * 4 + threadIdx.x] = 0;
   int64_t lbeg, cnt;
   sub_range(a, sub, 0, NB, &lbeg, &cnt);
-  adm_resolve(a, lbeg, cnt, adm_ctr(a, sub, 0));
+  if (chain_on(a, source_chain)) {
+    adm_resolve<false>(a, nullptr, sub, lbeg, cnt, adm_ctr(a, sub, 0));
+    return;
+  }
+  apply_init(h);
+  adm_resolve<true>(a, &h, sub, lbeg, cnt, adm_ctr(a, sub, 0));
+  apply_flush(a, h);
 }
 __global__ void __launch_bounds__(ADM_NT) k_forced(LPArgs a, int32_t sub) {
   griddep_wait();
-  if (*(volatile int32_t*)a.flags == 0) return;   // no listed node in an overloaded block
+  if (!chain_on(a, 1)) return;
   int64_t lbeg, cnt;
   sub_range(a, sub, 0, NB, &lbeg, &cnt);
   adm_forced(a, lbeg, cnt, adm_ctr(a, sub, 1));
 }
-__global__ void __launch_bounds__(ADM_NT) k_ovf_alloc(LPArgs a, int32_t sub, int32_t side) {
+__global__ void __launch_bounds__(ADM_NT) k_ovf_alloc(LPArgs a, int32_t sub) {
   griddep_wait();
-  int64_t* ct = adm_ctr(a, sub, side);
+  int64_t* ct = adm_ctr(a, sub, 1);
   const int64_t nseg = *(volatile int64_t*)&ct[1];
   if (nseg > 0) adm_alloc(a, nseg, ct);
 }
 __global__ void __launch_bounds__(ADM_NT) k_ovf_scatter(LPArgs a, int32_t sub, int32_t side) {
   griddep_wait();
-  if (*(volatile int64_t*)&adm_ctr(a, sub, side)[1] == 0) return;
+  const bool any = *(volatile int64_t*)&adm_ctr(a, sub, side)[1] > 0;
   int64_t lbeg, cnt;
   sub_range(a, sub, 0, NB, &lbeg, &cnt);
-  adm_scatter(a, lbeg, cnt);
+  adm_scatter(a, lbeg, cnt, any, side);
 }
-__global__ void __launch_bounds__(SEL_NT) k_ovf_select(LPArgs a, int32_t sub, int32_t side) {
+__global__ void __cluster_dims__(SEL_CL, 1, 1) __launch_bounds__(SEL_NT) k_ovf_select(LPArgs a, int32_t sub, int32_t side,
+                                                       int32_t source_chain) {
   griddep_wait();
+  __shared__ ApplyHash h;
+  __shared__ SelState sel;
   const int64_t nseg = *(volatile int64_t*)&adm_ctr(a, sub, side)[1];
-  if (nseg > 0) adm_select(a, nseg, side);
+  if (nseg == 0) return;
+  if (chain_on(a, source_chain)) {
+    adm_select<false, SEL_CL>(a, nullptr, sel, sub, nseg, side);
+    return;
+  }
+  apply_init(h);
+  adm_select<true, SEL_CL>(a, &h, sel, sub, nseg, side);
+  apply_flush(a, h);
 }
 __global__ void __launch_bounds__(ADM_NT) k_apply(LPArgs a, int32_t sub) {
   griddep_wait();
+  if (!chain_on(a, 1)) return;
+  __shared__ ApplyHash h;
   int64_t lbeg, cnt;
   sub_range(a, sub, 0, NB, &lbeg, &cnt);
-  adm_apply(a, lbeg, cnt, sub);
+  apply_init(h);
+  adm_apply(a, h, lbeg, cnt, sub);
+  apply_flush(a, h);
 }
 
 // Largest label count over the slots (local search: the largest k).
@@ -1858,8 +2060,13 @@ __global__ void __launch_bounds__(256) k_mark_rows(LPArgs a, int32_t sub) {
   const int32_t n = a.mqn[sub];
   for (int32_t q = blockIdx.x; q < n; q += gridDim.x) {
     const longlong2 c = a.mq[q];
-    for (int64_t e = c.x + threadIdx.x; e < c.y; e += blockDim.x)
-      if (SCLAP_OK(a.col[e], a.N, a.err)) an[a.col[e]] = 1;
+    for (int64_t e = c.x + threadIdx.x; e < c.y; e += 4 * blockDim.x) {
+      int32_t d[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) d[u] = e + u * blockDim.x < c.y ? a.col[e + u * blockDim.x] : -1;
+#pragma unroll
+      for (int u = 0; u < 4; ++u) mark_active(a, an, d[u]);
+    }
   }
 }
 
@@ -2060,14 +2267,16 @@ int64_t lp_run(const LevelView& lv, const SlotParams& sp, int32_t* label, wgt_t*
   const int nkeys = S * NB;
   const int sms = num_sms();
 
-  DevBuf<int64_t> in_w((size_t)Wsize, s), ovf_base((size_t)Wsize, s);
-  DevBuf<int32_t> ovf_cnt((size_t)Wsize, s), ovf_fill((size_t)Wsize, s);
-  in_w.zero(); ovf_cnt.zero(); ovf_fill.zero();
+  DevBuf<uint64_t> in_w((size_t)Wsize, s);
+  DevBuf<int64_t> ovf_base((size_t)Wsize, s);
+  DevBuf<int32_t> ovf_cnt((size_t)Wsize, s);
+  in_w.zero(); ovf_cnt.zero();
   DevBuf<int4> rec(N, s);
   DevBuf<longlong2> rec2(N, s);
-  DevBuf<int32_t> prop_t(N, s), grp(N, s), seg_g(N, s), seg_cnt(N, s);
+  DevBuf<int32_t> prop_t(N, s), grp(N, s), seg_g(N, s), seg_cnt(N, s), stage(N, s);
+  DevBuf<wgt_t> prop_w(N, s);
   DevBuf<uint64_t> prop_key(N, s), ent_key(N, s);
-  DevBuf<int8_t> adm(N, s), stage(N, s);
+  DevBuf<int8_t> adm(N, s);
   DevBuf<int64_t> seg_base(N, s), seg_thr(N, s);
   DevBuf<int32_t> ent_v(N, s), ent_w(N, s), ent_i(N, s);
   DevBuf<uint64_t> sel_k0(N, s), sel_k1(N, s);
@@ -2126,8 +2335,9 @@ int64_t lp_run(const LevelView& lv, const SlotParams& sp, int32_t* label, wgt_t*
   a.noff = sp.noff; a.loff = sp.loff; a.bound = sp.bound; a.rkey = sp.rkey; a.nlab = sp.nlab;
   a.done = sp.done; a.moved = sp.moved; a.rounds = sp.rounds;
   a.label = label; a.W = W; a.in_w = in_w.p; a.mode = run.mode; a.S = S;
-  a.rec = rec.p; a.rec2 = rec2.p; a.prop_t = prop_t.p; a.prop_key = prop_key.p; a.adm = adm.p; a.stage = stage.p;
-  a.grp = grp.p; a.ovf_cnt = ovf_cnt.p; a.ovf_fill = ovf_fill.p; a.ovf_base = ovf_base.p;
+  a.rec = rec.p; a.rec2 = rec2.p; a.prop_t = prop_t.p; a.prop_key = prop_key.p;
+  a.prop_w = prop_w.p; a.adm = adm.p; a.stage = stage.p;
+  a.grp = grp.p; a.ovf_cnt = ovf_cnt.p; a.ovf_base = ovf_base.p;
   a.ctr = ctr.p; a.seg_g = seg_g.p; a.seg_base = seg_base.p; a.seg_cnt = seg_cnt.p;
   a.seg_thr = seg_thr.p; a.ent_key = ent_key.p; a.ent_v = ent_v.p; a.ent_w = ent_w.p;
   a.ent_i = ent_i.p; a.bcnt = bcnt.p;
@@ -2362,7 +2572,8 @@ int64_t lp_run(const LevelView& lv, const SlotParams& sp, int32_t* label, wgt_t*
   const unsigned grid_adm_coop =
       (unsigned)std::max(1, sms * std::min<int>(adm_occ, tu.admit_ctas_per_sm));
   const unsigned grid_adm_max = (unsigned)(sms * tu.admit_ctas_per_sm);
-  const unsigned grid_sel = (unsigned)(sms * 4);
+  const unsigned grid_sel = (unsigned)(sms * 2);      // alloc; select: whole clusters
+  const unsigned grid_cl = ((unsigned)(sms * 4) + SEL_CL - 1) / SEL_CL * SEL_CL;
   auto admit = [&](cudaStream_t s, int sub, bool source_chain, int64_t cnt, bool pdl) {
     if (tu.fused_admission) {
       // one cooperative launch; it follows the propose join: plain launch
@@ -2374,17 +2585,17 @@ int64_t lp_run(const LevelView& lv, const SlotParams& sp, int32_t* label, wgt_t*
       return;
     }
     const unsigned grid_adm = cnt < 0 ? grid_adm_max : grid_for(cnt, ADM_NT, grid_adm_max);
-    launch_k(false, k_resolve, grid_adm, ADM_NT, 0, s, a, sub); SCLAP_NOTE_LAUNCH("k_resolve");
-    launch_k(pdl, k_ovf_alloc, grid_sel, ADM_NT, 0, s, a, sub, 0); SCLAP_NOTE_LAUNCH("k_ovf_alloc");
+    const int32_t ch = source_chain ? 1 : 0;
+    launch_k(false, k_resolve, grid_adm, ADM_NT, 0, s, a, sub, ch); SCLAP_NOTE_LAUNCH("k_resolve");
     launch_k(pdl, k_ovf_scatter, grid_adm, ADM_NT, 0, s, a, sub, 0); SCLAP_NOTE_LAUNCH("k_ovf_scatter");
-    launch_k(pdl, k_ovf_select, grid_sel, SEL_NT, 0, s, a, sub, 0); SCLAP_NOTE_LAUNCH("k_ovf_select");
+    launch_k(pdl, k_ovf_select, grid_cl, SEL_NT, 0, s, a, sub, 0, ch); SCLAP_NOTE_LAUNCH("k_ovf_select");
     if (source_chain) {
       launch_k(pdl, k_forced, grid_adm, ADM_NT, 0, s, a, sub); SCLAP_NOTE_LAUNCH("k_forced");
-      launch_k(pdl, k_ovf_alloc, grid_sel, ADM_NT, 0, s, a, sub, 1); SCLAP_NOTE_LAUNCH("k_ovf_alloc");
+      launch_k(pdl, k_ovf_alloc, grid_sel, ADM_NT, 0, s, a, sub); SCLAP_NOTE_LAUNCH("k_ovf_alloc");
       launch_k(pdl, k_ovf_scatter, grid_adm, ADM_NT, 0, s, a, sub, 1); SCLAP_NOTE_LAUNCH("k_ovf_scatter");
-      launch_k(pdl, k_ovf_select, grid_sel, SEL_NT, 0, s, a, sub, 1); SCLAP_NOTE_LAUNCH("k_ovf_select");
+      launch_k(pdl, k_ovf_select, grid_cl, SEL_NT, 0, s, a, sub, 1, ch); SCLAP_NOTE_LAUNCH("k_ovf_select");
+      launch_k(pdl, k_apply, grid_adm, ADM_NT, 0, s, a, sub); SCLAP_NOTE_LAUNCH("k_apply");
     }
-    launch_k(pdl, k_apply, grid_adm, ADM_NT, 0, s, a, sub); SCLAP_NOTE_LAUNCH("k_apply");
     if (a.mark_big) { launch_k(pdl, k_mark_rows, grid_mark, 256, 0, s, a, sub); SCLAP_NOTE_LAUNCH("k_mark_rows"); }
     SCLAP_LAUNCH_CHECK();
   };
