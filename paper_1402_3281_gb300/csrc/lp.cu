@@ -50,7 +50,9 @@ struct LPArgs {
   // state
   int32_t* label;
   wgt_t* W;
-  uint64_t* in_w;        // per target: proposals << 32 | their node weight (both < 2^31)
+  // per target: proposals << 32 | their node weight (both < 2^31); the
+  // persistent rounds have two sets and use them in turn (in_at)
+  uint64_t* in_w;
   int32_t mode;
   int32_t S;
   // sub-round lists: for each listed node {v, own label, weight, slot} and
@@ -93,6 +95,7 @@ struct LPArgs {
   // their neighbours through a queue of arc chunks, per colour class
   // mqn[sub] entries, read by a launch of their own
   int64_t mark_big;
+  int64_t mark_ch;       // arcs per queued chunk
   longlong2* mq;
   int32_t* mqn;
   // round state on the device, so that a level's rounds need no host
@@ -124,16 +127,21 @@ __device__ __forceinline__ void sub_range(const LPArgs& a, int sub, int b0, int 
   *cnt = a.boff[sub * NB + b1] - *beg;
 }
 
+__device__ __forceinline__ uint64_t* in_at(const LPArgs& a, int par, int32_t t) {
+  return a.in_w + (par ? a.nlabels : 0) + t;
+}
+
 struct NodeCtx {
-  int32_t v, slot, own, cv, vb;
+  int32_t v, slot, own, cv, vb, par;
   int64_t bound, loff, rs, re;
   uint64_t hv;
 };
 
-__device__ __forceinline__ NodeCtx load_node(const LPArgs& a, int64_t i) {
+__device__ __forceinline__ NodeCtx load_node(const LPArgs& a, int64_t i, int par = 0) {
   const int4 r = a.rec[i];
   const longlong2 r2 = a.rec2[i];
   NodeCtx c;
+  c.par = par;
   c.v = r.x;
   c.own = r.y;
   c.cv = r.z;
@@ -171,7 +179,8 @@ __device__ __forceinline__ void write_prop(const LPArgs& a, int64_t i, const Nod
     // kept with the proposal: resolving can then apply moves at once
     a.prop_w[i] = SCLAP_LD(a.W, t, a.nlabels, a.err);
     if (SCLAP_OK(t, a.nlabels, a.err))
-      atomicAdd(reinterpret_cast<unsigned long long*>(&a.in_w[t]), (1ull << 32) | (uint32_t)c.cv);
+      atomicAdd(reinterpret_cast<unsigned long long*>(in_at(a, c.par, t)),
+                (1ull << 32) | (uint32_t)c.cv);
   } else {
     a.prop_t[i] = -1;
   }
@@ -415,29 +424,31 @@ __device__ __forceinline__ void sorted_row_best(const LPArgs& a, const NodeCtx& 
 }
 
 template <int MAXD>
+__device__ __forceinline__ void propose_thread_node(const LPArgs& a, int64_t i, int par) {
+  const NodeCtx c = load_node(a, i, par);
+  const int deg = (int)(c.re - c.rs);
+  int32_t C[MAXD], w[MAXD];
+  int64_t total = 0;
+#pragma unroll
+  for (int j = 0; j < MAXD; ++j) {
+    const bool in = j < deg;
+    w[j] = in ? wat(a.ew, c.rs + j) : 0;
+    C[j] = in ? a.col[c.rs + j] : -1;
+    total += w[j];
+  }
+#pragma unroll
+  for (int j = 0; j < MAXD; ++j) C[j] = C[j] >= 0 ? SCLAP_LD(a.label, C[j], a.N, a.err) : INT32_MAX;
+  long long oc = 0;
+  Cand best{-1, 0, 0};
+  if (total <= INT32_MAX) sorted_row_best<MAXD, int32_t>(a, c, C, w, oc, best);
+  else sorted_row_best<MAXD, int64_t>(a, c, C, w, oc, best);
+  write_prop(a, i, c, best, oc, false);
+}
+template <int MAXD>
 __device__ __forceinline__ void propose_thread(const LPArgs& a, int64_t lbeg, int64_t cnt,
                                                int64_t blk, int64_t nblk) {
-  for (int64_t li = blk * blockDim.x + threadIdx.x; li < cnt; li += nblk * blockDim.x) {
-    const int64_t i = lbeg + li;
-    const NodeCtx c = load_node(a, i);
-    const int deg = (int)(c.re - c.rs);
-    int32_t C[MAXD], w[MAXD];
-    int64_t total = 0;
-#pragma unroll
-    for (int j = 0; j < MAXD; ++j) {
-      const bool in = j < deg;
-      w[j] = in ? wat(a.ew, c.rs + j) : 0;
-      C[j] = in ? a.col[c.rs + j] : -1;
-      total += w[j];
-    }
-#pragma unroll
-    for (int j = 0; j < MAXD; ++j) C[j] = C[j] >= 0 ? SCLAP_LD(a.label, C[j], a.N, a.err) : INT32_MAX;
-    long long oc = 0;
-    Cand best{-1, 0, 0};
-    if (total <= INT32_MAX) sorted_row_best<MAXD, int32_t>(a, c, C, w, oc, best);
-    else sorted_row_best<MAXD, int64_t>(a, c, C, w, oc, best);
-    write_prop(a, i, c, best, oc, false);
-  }
+  for (int64_t li = blk * blockDim.x + threadIdx.x; li < cnt; li += nblk * blockDim.x)
+    propose_thread_node<MAXD>(a, lbeg + li, 0);
 }
 
 // The small-degree buckets of one sub-round in one launch: block ranges
@@ -507,13 +518,28 @@ __device__ __forceinline__ int64_t table_get(const int32_t* keys, const unsigned
   return 0;
 }
 
-template <int NT>
-__device__ void block_reduce(long long& oc, Cand& cd, long long* sh_oc, Cand* sh_cd) {
-  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+// NT threads that work on one node together: a whole CTA (BAR = false), or
+// one of several teams of a CTA that meet at a named barrier (1 + team).
+template <int NT, bool BAR>
+struct Team {
+  int tid;        // 0 .. NT - 1
+  int bar;        // barrier number
+  __device__ __forceinline__ void sync() const {
+    if (BAR) asm volatile("bar.sync %0, %1;" ::"r"(bar), "n"(NT) : "memory");
+    else __syncthreads();
+  }
+};
+
+// Best candidate and own connection over the team (valid in its first warp);
+// sh_oc / sh_cd: one entry per warp.
+template <int NT, bool BAR>
+__device__ void block_reduce(const Team<NT, BAR>& tm, long long& oc, Cand& cd, long long* sh_oc,
+                             Cand* sh_cd) {
+  const int lane = tm.tid & 31, wib = tm.tid >> 5;
   oc = warp_max_ll(oc);
   cd = warp_best(cd);
   if (lane == 0) { sh_oc[wib] = oc; sh_cd[wib] = cd; }
-  __syncthreads();
+  tm.sync();
   if (wib == 0) {
     oc = lane < NT / 32 ? sh_oc[lane] : 0;
     cd = lane < NT / 32 ? sh_cd[lane] : Cand{-1, 0, 0};
@@ -521,7 +547,6 @@ __device__ void block_reduce(long long& oc, Cand& cd, long long* sh_oc, Cand* sh
     cd = warp_best(cd);
   }
 }
-
 
 // Adds an arc weight to a connection sum held in 64 bits.  When every sum of
 // the level stays below 2^32 the add is a 32-bit atomic on the low word (the
@@ -549,22 +574,12 @@ constexpr int WLOG = 8;                      // log2(WCAP)
 constexpr int WPC = 8;                       // warps per CTA
 static_assert((1 << WLOG) == WCAP, "WCAP must be 2^WLOG");
 
-__global__ void __launch_bounds__(WPC * 32) k_propose_warp(LPArgs a, int32_t sub, int32_t b0) {
-  griddep_wait();
-  int64_t lbeg, cnt;
-  sub_range(a, sub, b0, 5, &lbeg, &cnt);    // buckets b0..4 are adjacent
-  if (cnt == 0) return;
-  __shared__ unsigned long long sh_vals[WPC][WCAP];
-  __shared__ int32_t sh_keys[WPC][WCAP];
-  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  unsigned long long* vals = sh_vals[wib];
-  int32_t* keys = sh_keys[wib];
-  for (int j = lane; j < WCAP; j += 32) { keys[j] = -1; vals[j] = 0; }
-  __syncwarp();
-  const int64_t nwarps = (int64_t)gridDim.x * WPC;
-  for (int64_t li = (int64_t)blockIdx.x * WPC + wib; li < cnt; li += nwarps) {
-    const int64_t i = lbeg + li;
-    const NodeCtx c = load_node(a, i);
+// One node by one warp; its table (WCAP slots) is clean before and after.
+__device__ __forceinline__ void propose_warp_node(const LPArgs& a, int64_t i, int par,
+                                                  unsigned long long* vals, int32_t* keys) {
+  const int lane = threadIdx.x & 31;
+  {
+    const NodeCtx c = load_node(a, i, par);
     const bool ov = a.mode != MODE_CLUSTER && a.W[c.own] > c.bound;
     const int32_t nl = a.mode != MODE_CLUSTER ? a.nlab[c.slot] : 0;
     const bool direct = a.mode != MODE_CLUSTER && nl <= WCAP;
@@ -663,6 +678,23 @@ __global__ void __launch_bounds__(WPC * 32) k_propose_warp(LPArgs a, int32_t sub
   }
 }
 
+__global__ void __launch_bounds__(WPC * 32) k_propose_warp(LPArgs a, int32_t sub, int32_t b0) {
+  griddep_wait();
+  int64_t lbeg, cnt;
+  sub_range(a, sub, b0, 5, &lbeg, &cnt);    // buckets b0..4 are adjacent
+  if (cnt == 0) return;
+  __shared__ unsigned long long sh_vals[WPC][WCAP];
+  __shared__ int32_t sh_keys[WPC][WCAP];
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+  unsigned long long* vals = sh_vals[wib];
+  int32_t* keys = sh_keys[wib];
+  for (int j = lane; j < WCAP; j += 32) { keys[j] = -1; vals[j] = 0; }
+  __syncwarp();
+  const int64_t nwarps = (int64_t)gridDim.x * WPC;
+  for (int64_t li = (int64_t)blockIdx.x * WPC + wib; li < cnt; li += nwarps)
+    propose_warp_node(a, lbeg + li, 0, vals, keys);
+}
+
 // ---------------------------------------------------------------- bulk copies
 // Hub rows are staged in shared memory by the bulk-copy engine: one thread
 // issues a cp.async.bulk of a chunk of the row (col, and the weights when
@@ -736,7 +768,7 @@ __device__ __forceinline__ void hub_issue(const LPArgs& a, int64_t e0, int64_t e
 template <int SLOTS>
 constexpr size_t blk_smem_bytes() {
   return (size_t)SLOTS * (sizeof(unsigned long long) + sizeof(int32_t)) +
-         (size_t)(SLOTS / 2) * sizeof(int32_t);
+         (size_t)(SLOTS / 2) * sizeof(uint16_t);
 }
 
 // Degrees 129..8192 (buckets 5-7): one CTA of NT threads per node, a
@@ -744,6 +776,136 @@ constexpr size_t blk_smem_bytes() {
 // slots created for the current node.  The row is read four strides at a
 // time (loads first, then label gathers, then inserts), candidates are the
 // created slots only, and only those slots are cleared afterwards.
+// One node by a team; the table (tcap slots) is clean and sh.nc zero before
+// and after, clist has room for tcap / 2 slots (at most 65,536 in all).
+template <int NT>
+struct BlkShared {
+  long long oc[NT / 32];
+  Cand cd[NT / 32];
+  int nc;
+};
+template <int NT, bool BAR>
+__device__ __forceinline__ void propose_blk_node(const LPArgs& a, int64_t i, int par,
+                                                 const Team<NT, BAR>& tm, BlkShared<NT>& sh,
+                                                 unsigned long long* vals, int32_t* keys,
+                                                 uint16_t* clist, int64_t tcap) {
+  const int tid = tm.tid, lane = tid & 31;
+  const NodeCtx c = load_node(a, i, par);
+  const bool ov = a.mode != MODE_CLUSTER && a.W[c.own] > c.bound;
+  const int32_t nl = a.mode != MODE_CLUSTER ? a.nlab[c.slot] : 0;
+  const bool direct = a.mode != MODE_CLUSTER && nl <= tcap;
+  const int64_t deg = c.re - c.rs;
+  const int logcap = ceil_log2(max64(2 * deg, 32));
+  const uint32_t mask = (1u << logcap) - 1;
+  if (!direct && ((int64_t)1 << logcap) > tcap) {
+    // a launch with a smaller table than this node's hashing needs (the
+    // host only does this when every node indexes its block directly)
+    if (tid == 0) {
+      atomicOr(a.err, DERR_INTERNAL);
+      a.prop_t[i] = -1;
+    }
+    return;
+  }
+  for (int64_t e0 = c.rs; e0 < c.re; e0 += 4 * NT) {
+    int32_t C[4], w[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int64_t e = e0 + (int64_t)u * NT + tid;
+      const bool in = e < c.re;
+      w[u] = in ? wat(a.ew, e) : 0;
+      C[u] = in ? a.col[e] : -1;
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (C[u] >= 0) C[u] = SCLAP_LD(a.label, C[u], a.N, a.err);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      if (e0 + (int64_t)u * NT >= c.re) break;
+      const int32_t key = C[u] < 0 ? -1 : (direct ? (int32_t)(C[u] - c.loff) : C[u]);
+      bool cr = false;
+      uint32_t s = 0;
+      if (key >= 0) {
+        if (direct) {
+          conn_add(&vals[key], w[u], a.narrow);
+        } else {
+          s = table_slot(key, logcap);
+          const uint32_t pmax = a.probe_limit <= mask ? a.probe_limit : mask + 1;
+          bool placed = false;
+          for (uint32_t p = 0; p < pmax; ++p) {
+            const int32_t prev = atomicCAS(&keys[s], -1, key);
+            if (prev == -1 || prev == key) {
+              cr = prev == -1;
+              conn_add(&vals[s], w[u], a.narrow);
+              placed = true;
+              break;
+            }
+            s = (s + 1) & mask;
+          }
+          if (!placed) atomicOr(a.err, DERR_HASH_FULL);
+        }
+      }
+      // one list reservation per warp for the slots it created
+      const unsigned cm = __ballot_sync(0xffffffffu, cr);
+      if (cm) {
+        const int first = __ffs(cm) - 1;
+        int base = 0;
+        if (lane == first) base = atomicAdd(&sh.nc, __popc(cm));
+        base = __shfl_sync(0xffffffffu, base, first);
+        if (cr) clist[base + __popc(cm & ((1u << lane) - 1))] = (uint16_t)s;
+      }
+    }
+  }
+  tm.sync();
+  long long oc = 0;
+  Cand cd{-1, 0, 0};
+  if (direct) {
+    const int32_t own_l = (int32_t)(c.own - c.loff);
+    for (int32_t b = tid; b < nl; b += NT) {
+      const int64_t conn = (int64_t)vals[b];
+      if (b == own_l) { oc = conn; continue; }
+      if (conn == 0 && !ov) continue;
+      const int32_t Cb = (int32_t)(c.loff + b);
+      if ((int64_t)a.W[Cb] + c.cv > c.bound) continue;
+      Cand x = make_cand(c, Cb, conn);
+      if (cd.conn < 0 || cand_better(x, cd)) cd = x;
+    }
+    tm.sync();
+    for (int32_t b = tid; b < nl; b += NT) vals[b] = 0;
+  } else {
+    const int nc = sh.nc;
+    for (int j = tid; j < nc; j += NT) {
+      const int32_t s = clist[j];
+      const int32_t K = keys[s];
+      const int64_t conn = (int64_t)vals[s];
+      if (K == c.own) { oc = conn; continue; }
+      if (ov || (int64_t)a.W[K] + c.cv > c.bound) continue;
+      if (cand_block(a, c, true, K) != c.vb) continue;
+      Cand x = make_cand(c, K, conn);
+      if (cd.conn < 0 || cand_better(x, cd)) cd = x;
+    }
+    if (ov) {
+      for (int32_t b = tid; b < nl; b += NT) {
+        const int32_t Cb = (int32_t)(c.loff + b);
+        if (Cb == c.own || (int64_t)a.W[Cb] + c.cv > c.bound) continue;
+        Cand x = make_cand(c, Cb, table_get(keys, vals, logcap, Cb));
+        if (cd.conn < 0 || cand_better(x, cd)) cd = x;
+      }
+    }
+    tm.sync();
+    for (int j = tid; j < nc; j += NT) {
+      const int32_t s = clist[j];
+      keys[s] = -1;
+      vals[s] = 0;
+    }
+  }
+  block_reduce(tm, oc, cd, sh.oc, sh.cd);
+  if (tid == 0) {
+    write_prop(a, i, c, cd, oc, ov);
+    sh.nc = 0;
+  }
+  tm.sync();
+}
+
 template <int NT, int SLOTS>
 __global__ void __launch_bounds__(NT) k_propose_blk(LPArgs a, int32_t sub, int32_t bucket) {
   griddep_wait();
@@ -751,134 +913,17 @@ __global__ void __launch_bounds__(NT) k_propose_blk(LPArgs a, int32_t sub, int32
   sub_range(a, sub, bucket, bucket + 1, &lbeg, &cnt);
   if (cnt == 0) return;
   extern __shared__ unsigned long long smem_u64[];
-  __shared__ long long sh_oc[NT / 32];
-  __shared__ Cand sh_cd[NT / 32];
-  __shared__ int sh_nc;
+  __shared__ BlkShared<NT> sh;
   unsigned long long* vals = smem_u64;
   int32_t* keys = reinterpret_cast<int32_t*>(smem_u64 + SLOTS);
-  int32_t* clist = keys + SLOTS;
-  constexpr int64_t tcap = SLOTS;
-  const int tid = threadIdx.x, lane = tid & 31;
+  uint16_t* clist = reinterpret_cast<uint16_t*>(keys + SLOTS);
+  const int tid = threadIdx.x;
   for (int j = tid; j < SLOTS; j += NT) { keys[j] = -1; vals[j] = 0; }
-  if (tid == 0) sh_nc = 0;
+  if (tid == 0) sh.nc = 0;
   __syncthreads();
-  for (int64_t li = blockIdx.x; li < cnt; li += gridDim.x) {
-    const int64_t i = lbeg + li;
-    const NodeCtx c = load_node(a, i);
-    const bool ov = a.mode != MODE_CLUSTER && a.W[c.own] > c.bound;
-    const int32_t nl = a.mode != MODE_CLUSTER ? a.nlab[c.slot] : 0;
-    const bool direct = a.mode != MODE_CLUSTER && nl <= tcap;
-    const int64_t deg = c.re - c.rs;
-    const int logcap = ceil_log2(max64(2 * deg, 32));
-    const uint32_t mask = (1u << logcap) - 1;
-    if (!direct && ((int64_t)1 << logcap) > tcap) {
-      // a launch with a smaller table than this node's hashing needs (the
-      // host only does this when every node indexes its block directly)
-      if (tid == 0) {
-        atomicOr(a.err, DERR_INTERNAL);
-        a.prop_t[i] = -1;
-      }
-      continue;
-    }
-    for (int64_t e0 = c.rs; e0 < c.re; e0 += 4 * NT) {
-      int32_t C[4], w[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int64_t e = e0 + (int64_t)u * NT + tid;
-        const bool in = e < c.re;
-        w[u] = in ? wat(a.ew, e) : 0;
-        C[u] = in ? a.col[e] : -1;
-      }
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if (C[u] >= 0) C[u] = SCLAP_LD(a.label, C[u], a.N, a.err);
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        if (e0 + (int64_t)u * NT >= c.re) break;
-        const int32_t key = C[u] < 0 ? -1 : (direct ? (int32_t)(C[u] - c.loff) : C[u]);
-        bool cr = false;
-        uint32_t s = 0;
-        if (key >= 0) {
-          if (direct) {
-            conn_add(&vals[key], w[u], a.narrow);
-          } else {
-            s = table_slot(key, logcap);
-            const uint32_t pmax = a.probe_limit <= mask ? a.probe_limit : mask + 1;
-            bool placed = false;
-            for (uint32_t p = 0; p < pmax; ++p) {
-              const int32_t prev = atomicCAS(&keys[s], -1, key);
-              if (prev == -1 || prev == key) {
-                cr = prev == -1;
-                conn_add(&vals[s], w[u], a.narrow);
-                placed = true;
-                break;
-              }
-              s = (s + 1) & mask;
-            }
-            if (!placed) atomicOr(a.err, DERR_HASH_FULL);
-          }
-        }
-        // one list reservation per warp for the slots it created
-        const unsigned cm = __ballot_sync(0xffffffffu, cr);
-        if (cm) {
-          const int first = __ffs(cm) - 1;
-          int base = 0;
-          if (lane == first) base = atomicAdd(&sh_nc, __popc(cm));
-          base = __shfl_sync(0xffffffffu, base, first);
-          if (cr) clist[base + __popc(cm & ((1u << lane) - 1))] = (int32_t)s;
-        }
-      }
-    }
-    __syncthreads();
-    long long oc = 0;
-    Cand cd{-1, 0, 0};
-    if (direct) {
-      const int32_t own_l = (int32_t)(c.own - c.loff);
-      for (int32_t b = tid; b < nl; b += NT) {
-        const int64_t conn = (int64_t)vals[b];
-        if (b == own_l) { oc = conn; continue; }
-        if (conn == 0 && !ov) continue;
-        const int32_t Cb = (int32_t)(c.loff + b);
-        if ((int64_t)a.W[Cb] + c.cv > c.bound) continue;
-        Cand x = make_cand(c, Cb, conn);
-        if (cd.conn < 0 || cand_better(x, cd)) cd = x;
-      }
-      __syncthreads();
-      for (int32_t b = tid; b < nl; b += NT) vals[b] = 0;
-    } else {
-      const int nc = sh_nc;
-      for (int j = tid; j < nc; j += NT) {
-        const int32_t s = clist[j];
-        const int32_t K = keys[s];
-        const int64_t conn = (int64_t)vals[s];
-        if (K == c.own) { oc = conn; continue; }
-        if (ov || (int64_t)a.W[K] + c.cv > c.bound) continue;
-        if (cand_block(a, c, true, K) != c.vb) continue;
-        Cand x = make_cand(c, K, conn);
-        if (cd.conn < 0 || cand_better(x, cd)) cd = x;
-      }
-      if (ov) {
-        for (int32_t b = tid; b < nl; b += NT) {
-          const int32_t Cb = (int32_t)(c.loff + b);
-          if (Cb == c.own || (int64_t)a.W[Cb] + c.cv > c.bound) continue;
-          Cand x = make_cand(c, Cb, table_get(keys, vals, logcap, Cb));
-          if (cd.conn < 0 || cand_better(x, cd)) cd = x;
-        }
-      }
-      __syncthreads();
-      for (int j = tid; j < nc; j += NT) {
-        const int32_t s = clist[j];
-        keys[s] = -1;
-        vals[s] = 0;
-      }
-    }
-    block_reduce<NT>(oc, cd, sh_oc, sh_cd);
-    if (tid == 0) {
-      write_prop(a, i, c, cd, oc, ov);
-      sh_nc = 0;
-    }
-    __syncthreads();
-  }
+  const Team<NT, false> tm{tid, 0};
+  for (int64_t li = blockIdx.x; li < cnt; li += gridDim.x)
+    propose_blk_node(a, lbeg + li, 0, tm, sh, vals, keys, clist, SLOTS);
 }
 
 // ------------------------------------------------------------------ hubs
@@ -1224,7 +1269,7 @@ __global__ void __launch_bounds__(HUB_NT) k_hub_select(LPArgs a, int32_t sub, in
         }
       }
     }
-    block_reduce<HUB_NT>(oc, cd, sh_oc, sh_cd);
+    block_reduce(Team<HUB_NT, false>{tid, 0}, oc, cd, sh_oc, sh_cd);
     if (tid == 0) {
       h.pcd[q] = cd;
       h.poc[q] = oc;
@@ -1262,7 +1307,7 @@ __global__ void __launch_bounds__(HUB_NT) k_hub_select(LPArgs a, int32_t sub, in
         }
       }
       __syncthreads();                   // sh_oc / sh_cd reused
-      block_reduce<HUB_NT>(oc, cd, sh_oc, sh_cd);
+      block_reduce(Team<HUB_NT, false>{tid, 0}, oc, cd, sh_oc, sh_cd);
       if (tid == 0) {
         write_prop(a, i, c, cd, oc, ov);
         h.hdone[li] = 0;
@@ -1329,8 +1374,7 @@ __device__ __forceinline__ void mark_active(const LPArgs& a, uint8_t* an, int32_
 // node's neighbours become active (rows of <= 8 arcs by their own lane,
 // longer ones by the whole warp, the longest through the chunk queue).
 __device__ __forceinline__ void move_warp(const LPArgs& a, ApplyHash& h, MovedRun& m, int32_t sub,
-                                          bool mv, int64_t i, int32_t t) {
-  uint8_t* const an = act_next(a);
+                                          uint8_t* an, bool mv, int64_t i, int32_t t) {
   const int lane = threadIdx.x & 31;
   int32_t slot = -1;
   int64_t rs = 0, re = 0;
@@ -1355,10 +1399,10 @@ __device__ __forceinline__ void move_warp(const LPArgs& a, ApplyHash& h, MovedRu
       for (int q = 0; q < 8; ++q) mark_active(a, an, c[q]);
       re = rs;
     } else if (a.mark_big > 0 && re - rs > a.mark_big) {
-      const int32_t nch = (int32_t)((re - rs + MARK_CH - 1) / MARK_CH);
+      const int32_t nch = (int32_t)((re - rs + a.mark_ch - 1) / a.mark_ch);
       const int32_t q0 = atomicAdd(&a.mqn[sub], nch);
       for (int32_t c = 0; c < nch; ++c)
-        a.mq[q0 + c] = make_longlong2(rs + c * MARK_CH, min64(rs + (c + 1) * MARK_CH, re));
+        a.mq[q0 + c] = make_longlong2(rs + c * a.mark_ch, min64(rs + (c + 1) * a.mark_ch, re));
       re = rs;
     }
   }
@@ -1434,9 +1478,11 @@ __device__ __forceinline__ int64_t* adm_ctr(const LPArgs& a, int sub, int side) 
 
 template <bool APPLY>
 __device__ __forceinline__ void adm_resolve(const LPArgs& a, ApplyHash* h, int32_t sub,
-                                            int64_t lbeg, int64_t cnt, int64_t* ct) {
+                                            uint8_t* an, int par, int64_t lbeg, int64_t cnt,
+                                            int64_t* ct) {
   const int lane = threadIdx.x & 31;
-  const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  // 32 proposals per warp, neighbouring ones to different CTAs
+  const int64_t w0 = (int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   MovedRun m;
   for (int64_t b0 = w0 * 32; b0 < cnt; b0 += nw * 32) {
@@ -1449,7 +1495,7 @@ __device__ __forceinline__ void adm_resolve(const LPArgs& a, ApplyHash* h, int32
       if (t >= 0) {
         const int64_t bound = a.bound[a.rec[i].w];
         const int64_t Wt = a.prop_w[i];
-        const uint64_t in = SCLAP_LD(a.in_w, t, a.nlabels, a.err);
+        const uint64_t in = SCLAP_LD(in_at(a, par, 0), t, a.nlabels, a.err);
         if (Wt + (int64_t)(uint32_t)in <= bound) {
           mv = true;
         } else if (SCLAP_OK(t, a.nlabels, a.err)) {
@@ -1470,7 +1516,7 @@ __device__ __forceinline__ void adm_resolve(const LPArgs& a, ApplyHash* h, int32
       a.stage[i] = st;
       if (!APPLY) a.adm[i] = mv ? 1 : 0;
     }
-    if (APPLY) move_warp(a, *h, m, sub, mv, i, t);
+    if (APPLY) move_warp(a, *h, m, sub, an, mv, i, t);
   }
   if (APPLY) moved_flush(a, m);
 }
@@ -1517,14 +1563,17 @@ __device__ void adm_alloc(const LPArgs& a, int64_t nseg, int64_t* ct) {
 
 // Writes the staged proposals into their segments (any: there are segments)
 // and, on the target side, clears the incoming weights.
-__device__ void adm_scatter(const LPArgs& a, int64_t lbeg, int64_t cnt, bool any, int32_t source) {
+__device__ void adm_scatter(const LPArgs& a, int par, int64_t lbeg, int64_t cnt, bool any,
+                            int32_t source) {
   if (!any && source) return;
-  for (int64_t li = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; li < cnt;
-       li += (int64_t)gridDim.x * blockDim.x) {
+  const int lane = threadIdx.x & 31;
+  const int64_t w0 = (int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t li = w0 * 32 + lane; li < cnt; li += nw * 32) {
     const int64_t i = lbeg + li;
     if (!source) {
       const int32_t t = a.prop_t[i];
-      if (t >= 0 && SCLAP_OK(t, a.nlabels, a.err)) a.in_w[t] = 0;
+      if (t >= 0 && SCLAP_OK(t, a.nlabels, a.err)) *in_at(a, par, t) = 0;
     }
     const int32_t st = any ? a.stage[i] : 0;
     if (st == 0) continue;
@@ -1610,7 +1659,7 @@ __device__ __forceinline__ void select_rank_small(SelState& S, int n, int64_t th
 // CTA's state, S the first CTA's.
 template <bool APPLY, int CL>
 __device__ __forceinline__ void select_large(const LPArgs& a, ApplyHash* h, MovedRun& m,
-                                             int32_t sub, int64_t sg, int32_t source,
+                                             int32_t sub, uint8_t* an, int64_t sg, int32_t source,
                                              SelState& L) {
   const int tid = threadIdx.x, lane = tid & 31, NT = blockDim.x;
   const int rank = CL > 1 ? (int)cluster_rank() : 0;
@@ -1827,7 +1876,7 @@ __device__ __forceinline__ void select_large(const LPArgs& a, ApplyHash* h, Move
       else ok = key_less(k, v, PK, (int32_t)PV) || (source && k == PK && v == (int32_t)PV);
       if (!APPLY) a.adm[i] = ok ? 1 : 0;
     }
-    if (APPLY) move_warp(a, *h, m, sub, ok, i, g);
+    if (APPLY) move_warp(a, *h, m, sub, an, ok, i, g);
   }
   if (rank == 0 && tid == 0) a.ovf_cnt[g] = 0;
   sync();                                  // the state is free again
@@ -1836,8 +1885,8 @@ __device__ __forceinline__ void select_large(const LPArgs& a, ApplyHash* h, Move
 // All segments of one side of a colour class.  CL > 1: the launch has
 // clusters of CL CTAs, which take the segments above SEL_CTA entries.
 template <bool APPLY, int CL>
-__device__ void adm_select(const LPArgs& a, ApplyHash* h, SelState& L, int32_t sub, int64_t nseg,
-                           int32_t source) {
+__device__ void adm_select(const LPArgs& a, ApplyHash* h, SelState& L, int32_t sub, uint8_t* an,
+                           int64_t nseg, int32_t source) {
   MovedRun m;
   const int tid = threadIdx.x, lane = tid & 31;
   // segments of <= 64 entries, one warp each (entries lane and lane + 32 in
@@ -1879,8 +1928,8 @@ __device__ void adm_select(const LPArgs& a, ApplyHash* h, SelState& L, int32_t s
       const int32_t i0 = h0 ? a.ent_i[base + lane] : 0;
       const int32_t i1 = h1 ? a.ent_i[base + lane + 32] : 0;
       if (APPLY) {
-        move_warp(a, *h, m, sub, ok0, i0, g);
-        if (n > 32) move_warp(a, *h, m, sub, ok1, i1, g);
+        move_warp(a, *h, m, sub, an, ok0, i0, g);
+        if (n > 32) move_warp(a, *h, m, sub, an, ok1, i1, g);
       } else {
         if (h0) a.adm[i0] = ok0 ? 1 : 0;
         if (h1) a.adm[i1] = ok1 ? 1 : 0;
@@ -1893,20 +1942,20 @@ __device__ void adm_select(const LPArgs& a, ApplyHash* h, SelState& L, int32_t s
   for (int64_t sg = blockIdx.x; sg < nseg; sg += gridDim.x) {
     const int32_t n = a.seg_cnt[sg];
     if (n > SEL_SMALL && (CL == 1 || n <= SEL_CTA))
-      select_large<APPLY, 1>(a, h, m, sub, sg, source, L);
+      select_large<APPLY, 1>(a, h, m, sub, an, sg, source, L);
   }
   // the largest: a cluster each
   if (CL > 1) {
     cluster_sync();
     for (int64_t sg = blockIdx.x / CL; sg < nseg; sg += gridDim.x / CL)
-      if (a.seg_cnt[sg] > SEL_CTA) select_large<APPLY, CL>(a, h, m, sub, sg, source, L);
+      if (a.seg_cnt[sg] > SEL_CTA) select_large<APPLY, CL>(a, h, m, sub, an, sg, source, L);
   }
   if (APPLY) moved_flush(a, m);
 }
 
 // Source chain: applies the proposals left admitted.
-__device__ __forceinline__ void adm_apply(const LPArgs& a, ApplyHash& h, int64_t lbeg, int64_t cnt,
-                                          int32_t sub) {
+__device__ __forceinline__ void adm_apply(const LPArgs& a, ApplyHash& h, uint8_t* an, int64_t lbeg,
+                                          int64_t cnt, int32_t sub) {
   const int lane = threadIdx.x & 31;
   const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -1915,7 +1964,7 @@ __device__ __forceinline__ void adm_apply(const LPArgs& a, ApplyHash& h, int64_t
     const int64_t i = lbeg + b0 + lane;
     const bool in = b0 + lane < cnt;
     const int32_t t = in ? a.prop_t[i] : -1;
-    move_warp(a, h, m, sub, t >= 0 && a.adm[i], i, t);
+    move_warp(a, h, m, sub, an, t >= 0 && a.adm[i], i, t);
   }
   moved_flush(a, m);
 }
@@ -1941,15 +1990,16 @@ __global__ void __launch_bounds__(ADM_NT) k_admit(LPArgs a, int32_t sub, int32_t
   const uint32_t lim = a.wait_limit;
   int64_t* ct = adm_ctr(a, sub, 0);
   const bool chain = source_chain && *(volatile int32_t*)a.flags != 0;
-  if (chain) adm_resolve<false>(a, &h, sub, lbeg, cnt, ct);
-  else adm_resolve<true>(a, &h, sub, lbeg, cnt, ct);
+  uint8_t* const an = act_next(a);
+  if (chain) adm_resolve<false>(a, &h, sub, an, 0, lbeg, cnt, ct);
+  else adm_resolve<true>(a, &h, sub, an, 0, lbeg, cnt, ct);
   if (!grid_sync(gs, a.err, lim)) return;
   const int64_t nseg = *(volatile int64_t*)&ct[1];
-  adm_scatter(a, lbeg, cnt, nseg > 0, 0);
+  adm_scatter(a, 0, lbeg, cnt, nseg > 0, 0);
   if (nseg > 0) {
     if (!grid_sync(gs, a.err, lim)) return;
-    if (chain) adm_select<false, 1>(a, &h, sel, sub, nseg, 0);
-    else adm_select<true, 1>(a, &h, sel, sub, nseg, 0);
+    if (chain) adm_select<false, 1>(a, &h, sel, sub, an, nseg, 0);
+    else adm_select<true, 1>(a, &h, sel, sub, an, nseg, 0);
   }
   if (chain) {
     if (!grid_sync(gs, a.err, lim)) return;
@@ -1960,12 +2010,12 @@ __global__ void __launch_bounds__(ADM_NT) k_admit(LPArgs a, int32_t sub, int32_t
     if (nsrc > 0) {
       adm_alloc(a, nsrc, cs);
       if (!grid_sync(gs, a.err, lim)) return;
-      adm_scatter(a, lbeg, cnt, true, 1);
+      adm_scatter(a, 0, lbeg, cnt, true, 1);
       if (!grid_sync(gs, a.err, lim)) return;
-      adm_select<false, 1>(a, &h, sel, sub, nsrc, 1);
+      adm_select<false, 1>(a, &h, sel, sub, an, nsrc, 1);
       if (!grid_sync(gs, a.err, lim)) return;
     }
-    adm_apply(a, h, lbeg, cnt, sub);
+    adm_apply(a, h, an, lbeg, cnt, sub);
   }
   apply_flush(a, h);
 }
@@ -1989,11 +2039,11 @@ __global__ void __launch_bounds__(ADM_NT) k_resolve(LPArgs a, int32_t sub, int32
   int64_t lbeg, cnt;
   sub_range(a, sub, 0, NB, &lbeg, &cnt);
   if (chain_on(a, source_chain)) {
-    adm_resolve<false>(a, nullptr, sub, lbeg, cnt, adm_ctr(a, sub, 0));
+    adm_resolve<false>(a, nullptr, sub, nullptr, 0, lbeg, cnt, adm_ctr(a, sub, 0));
     return;
   }
   apply_init(h);
-  adm_resolve<true>(a, &h, sub, lbeg, cnt, adm_ctr(a, sub, 0));
+  adm_resolve<true>(a, &h, sub, act_next(a), 0, lbeg, cnt, adm_ctr(a, sub, 0));
   apply_flush(a, h);
 }
 __global__ void __launch_bounds__(ADM_NT) k_forced(LPArgs a, int32_t sub) {
@@ -2014,7 +2064,7 @@ __global__ void __launch_bounds__(ADM_NT) k_ovf_scatter(LPArgs a, int32_t sub, i
   const bool any = *(volatile int64_t*)&adm_ctr(a, sub, side)[1] > 0;
   int64_t lbeg, cnt;
   sub_range(a, sub, 0, NB, &lbeg, &cnt);
-  adm_scatter(a, lbeg, cnt, any, side);
+  adm_scatter(a, 0, lbeg, cnt, any, side);
 }
 __global__ void __cluster_dims__(SEL_CL, 1, 1) __launch_bounds__(SEL_NT) k_ovf_select(LPArgs a, int32_t sub, int32_t side,
                                                        int32_t source_chain) {
@@ -2024,11 +2074,11 @@ __global__ void __cluster_dims__(SEL_CL, 1, 1) __launch_bounds__(SEL_NT) k_ovf_s
   const int64_t nseg = *(volatile int64_t*)&adm_ctr(a, sub, side)[1];
   if (nseg == 0) return;
   if (chain_on(a, source_chain)) {
-    adm_select<false, SEL_CL>(a, nullptr, sel, sub, nseg, side);
+    adm_select<false, SEL_CL>(a, nullptr, sel, sub, nullptr, nseg, side);
     return;
   }
   apply_init(h);
-  adm_select<true, SEL_CL>(a, &h, sel, sub, nseg, side);
+  adm_select<true, SEL_CL>(a, &h, sel, sub, act_next(a), nseg, side);
   apply_flush(a, h);
 }
 __global__ void __launch_bounds__(ADM_NT) k_apply(LPArgs a, int32_t sub) {
@@ -2038,7 +2088,7 @@ __global__ void __launch_bounds__(ADM_NT) k_apply(LPArgs a, int32_t sub) {
   int64_t lbeg, cnt;
   sub_range(a, sub, 0, NB, &lbeg, &cnt);
   apply_init(h);
-  adm_apply(a, h, lbeg, cnt, sub);
+  adm_apply(a, h, act_next(a), lbeg, cnt, sub);
   apply_flush(a, h);
 }
 
@@ -2068,6 +2118,350 @@ __global__ void __launch_bounds__(256) k_mark_rows(LPArgs a, int32_t sub) {
       for (int u = 0; u < 4; ++u) mark_active(a, an, d[u]);
     }
   }
+}
+
+// ------------------------------------------------------- persistent rounds
+// All rounds of a level in ONE cooperative launch, one CTA per SM, for levels
+// small enough that launches, not work, are what a round costs (PR_MAX_N,
+// PR_MAX_M).  The phases are those of the launches above, separated by
+// grid barriers: bucketing (count, scatter), then per colour class propose,
+// resolve and, only when some target overflows, scatter and select.  No host
+// wait and no launch lies between them, so a colour class costs two to four
+// barriers and the latency of its longest chain of loads.
+//
+// Measured per colour class, R-MAT of 2^16 nodes: 22 us, with the launches 57
+// (nine launches and the events of a fork and a join); of 2^10 nodes: 12 us.
+constexpr int PR_NT = 512, PR_WARPS = PR_NT / 32, PR_TEAMS = PR_NT / 128;
+constexpr int PR_MIN_TCAP = PR_WARPS * WCAP;       // = PR_TEAMS * B5_SLOTS
+static_assert(PR_MIN_TCAP == PR_TEAMS * B5_SLOTS, "the tables of warps and teams share the CTA's");
+constexpr int64_t PR_MARK = 128, PR_MARK_CH = 512; // queued rows, arcs per queued chunk
+constexpr size_t pr_smem(int64_t tcap) {
+  return (size_t)tcap * (sizeof(unsigned long long) + sizeof(int32_t)) +
+         (size_t)(tcap / 2) * sizeof(uint16_t);
+}
+
+struct RoundsArgs {
+  int32_t nslots, phase, raw_key, tcap;
+  const uint64_t* seed;
+  const int32_t* level;
+  unsigned int* bar;             // barrier arrivals, zero at launch
+  int32_t* live;                 // two counters used in turn, zero at launch
+};
+
+// Barrier of the whole (co-resident) grid: arrivals counted up to `want`,
+// which grows by the grid size each time; at most `limit` polls.
+__device__ __forceinline__ bool round_sync(unsigned int* bar, unsigned int& want, int32_t* err,
+                                           uint32_t limit) {
+  __shared__ int ok_sh;
+  want += gridDim.x;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    atomicAdd(bar, 1u);
+    int ok = 1;
+    uint32_t it = 0;
+    while ((int)(ld_acquire_gpu(bar) - want) < 0) {
+      if (++it > limit) {
+        atomicOr(err, DERR_TIMEOUT);
+        ok = 0;
+        break;
+      }
+    }
+    __threadfence();
+    ok_sh = ok;
+  }
+  __syncthreads();
+  return ok_sh != 0;
+}
+
+// Adds the CTA's label-weight changes to the labels and leaves the hash clean.
+__device__ __forceinline__ void apply_flush_clean(const LPArgs& a, ApplyHash& h) {
+  __syncthreads();
+  for (int j = threadIdx.x; j < APPLY_SLOTS; j += blockDim.x) {
+    const int32_t L = h.k[j];
+    if (L < 0) continue;
+    const int32_t d = h.v[j];
+    h.k[j] = -1;
+    h.v[j] = 0;
+    if (d != 0 && SCLAP_OK(L, a.nlabels, a.err)) atomicAdd(&a.W[L], (wgt_t)d);
+  }
+}
+
+__global__ void __launch_bounds__(PR_NT, 1) k_lp_rounds(LPArgs a, RoundsArgs q) {
+  extern __shared__ unsigned long long smem_u64[];
+  __shared__ ApplyHash h;
+  __shared__ union {
+    SelState sel;
+    struct { int cnt[MAX_KEYS], base[MAX_KEYS]; } b;
+  } u;
+  __shared__ int32_t boff[MAX_KEYS + 1];
+  __shared__ BlkShared<PR_NT> shb;
+  __shared__ BlkShared<128> sht[PR_TEAMS];
+  __shared__ unsigned long long sh_arcs;
+  __shared__ int sh_ov;
+  unsigned long long* const vals = smem_u64;
+  int32_t* const keys = reinterpret_cast<int32_t*>(smem_u64 + q.tcap);
+  uint16_t* const clist = reinterpret_cast<uint16_t*>(keys + q.tcap);
+  const int tid = threadIdx.x, lane = tid & 31, wib = tid >> 5;
+  const int cta = blockIdx.x, G = gridDim.x;
+  const int64_t gt = (int64_t)cta * PR_NT + tid, gn = (int64_t)G * PR_NT;
+  const int nkeys = a.S * NB;
+  const uint32_t lim = a.wait_limit;
+  unsigned int want = 0;
+  auto sync = [&] { return round_sync(q.bar, want, a.err, lim); };
+  for (int j = tid; j < q.tcap; j += PR_NT) { keys[j] = -1; vals[j] = 0; }
+  if (tid == 0) shb.nc = 0;
+  if (tid < PR_TEAMS) sht[tid].nc = 0;
+  apply_init(h);
+
+  // round key and counters of slot s, or done (repair: nothing overloaded)
+  auto begin_slot = [&](int32_t s, int32_t r) {
+    if (a.mode == MODE_REPAIR) {
+      int64_t mx = 0;
+      const int64_t lo = a.loff[s];
+      for (int32_t b = 0; b < a.nlab[s]; ++b) mx = max64(mx, (int64_t)a.W[lo + b]);
+      if (mx <= a.bound[s]) { a.done[s] = 1; return; }
+    }
+    a.rkey[s] = q.raw_key ? q.seed[s]
+                          : hkey(q.seed[s], (uint64_t)q.phase, (uint64_t)q.level[s], (uint64_t)r);
+    a.moved[s] = 0;
+  };
+  for (int64_t s = gt; s < q.nslots; s += gn)
+    if (!a.done[s]) begin_slot((int32_t)s, 0);
+  if (!sync()) return;
+
+  int par = 0;
+  int32_t r = 0;
+  for (;;) {
+    const uint8_t* const ac = a.act[0] ? a.act[r & 1] : nullptr;
+    uint8_t* const an = a.act[0] ? a.act[(r + 1) & 1] : nullptr;
+    // ---- bucketing: keys and counts; the total a CTA adds its count to is
+    // also where its nodes start among the key's
+    for (int j = tid; j < nkeys; j += PR_NT) u.b.cnt[j] = 0;
+    if (tid == 0) { sh_arcs = 0; sh_ov = 0; }
+    __syncthreads();
+    {
+      unsigned long long arcs = 0;
+      bool any_ov = false;
+      for (int64_t v = gt; v < a.N; v += gn) {
+        if (an) an[v] = 0;
+        int64_t deg = 0;
+        bool ov = false;
+        const int key = node_key(a, ac, v, &deg, &ov);
+        a.nkey[v] = (int16_t)key;
+        if (key >= 0) {
+          atomicAdd(&u.b.cnt[key], 1);
+          arcs += (unsigned long long)deg;
+          any_ov = any_ov || ov;
+        }
+      }
+      for (int o = 16; o > 0; o >>= 1) arcs += __shfl_xor_sync(0xffffffffu, arcs, o);
+      if (lane == 0 && arcs) atomicAdd(&sh_arcs, arcs);
+      if (any_ov) sh_ov = 1;
+    }
+    __syncthreads();
+    for (int j = tid; j < nkeys; j += PR_NT) {
+      const int c = u.b.cnt[j];
+      u.b.base[j] = c ? atomicAdd(&a.bcnt[j], c) : 0;
+      u.b.cnt[j] = 0;                      // from here on: nodes placed
+    }
+    if (tid == 0) {
+      if (sh_arcs) atomicAdd(ull(a.arcs), sh_arcs);
+      if (sh_ov) atomicOr(&a.flags[0], 1);
+    }
+    if (!sync()) return;
+    if (wib == 0) {                        // offsets of the keys, by every CTA
+      int32_t carry = 0;
+      for (int j0 = 0; j0 < nkeys; j0 += 32) {
+        const int j = j0 + lane;
+        const int32_t c = j < nkeys ? *(volatile int32_t*)&a.bcnt[j] : 0;
+        int32_t x = c;
+        for (int o = 1; o < 32; o <<= 1) {
+          const int32_t y = __shfl_up_sync(0xffffffffu, x, o);
+          if (lane >= o) x += y;
+        }
+        if (j < nkeys) boff[j] = carry + x - c;
+        carry += __shfl_sync(0xffffffffu, x, 31);
+      }
+      if (lane == 0) boff[nkeys] = carry;
+    }
+    __syncthreads();
+    for (int64_t v = gt; v < a.N; v += gn) {
+      const int key = a.nkey[v];
+      if (key < 0) continue;
+      const int64_t pos = boff[key] + u.b.base[key] + atomicAdd(&u.b.cnt[key], 1);
+      const int64_t rs = a.row_ptr[v];
+      a.rec[pos] = make_int4((int32_t)v, a.label[v], wat(a.nw, v), slot_at(a.gid, v));
+      a.rec2[pos] = make_longlong2(rs, a.row_ptr[v + 1] - rs);
+    }
+    if (cta == 0 && tid == 0 && a.mqn) a.mqn[0] = 0;
+    if (!sync()) return;
+    if (cta == 0)                          // every CTA has read the counts
+      for (int j = tid; j < nkeys; j += PR_NT) a.bcnt[j] = 0;
+    const int32_t total = boff[nkeys];
+    const bool chain = a.mode != MODE_CLUSTER && *(volatile int32_t*)a.flags != 0;
+
+    // ---- colour classes
+    int64_t pbeg = 0, pcnt = 0;            // class whose incoming weights are still set
+    auto clear_in = [&] {                  // (of the parity not in use)
+      for (int64_t li = gt; li < pcnt; li += gn) {
+        const int32_t t = a.prop_t[pbeg + li];
+        if (t >= 0 && SCLAP_OK(t, a.nlabels, a.err)) *in_at(a, par ^ 1, t) = 0;
+      }
+      pcnt = 0;
+    };
+    for (int sub = 0; sub < a.S; ++sub) {
+      const int32_t* B = boff + sub * NB;
+      const int64_t lbeg = B[0], cnt = B[NB] - B[0];
+      if (cnt == 0) continue;
+      int64_t* const ct = a.ctr + par * 4;
+      if (cta == 0 && tid < 4) a.ctr[(par ^ 1) * 4 + tid] = 0;
+      clear_in();
+      // propose: nodes of degree above 128 as CTA items (four teams share a
+      // CTA up to 512), largest first from CTA 0 on; the others as warp tasks
+      // on the CTAs left over, or on all when those would get more than two
+      // rounds of them
+      const int32_t n7 = B[8] - B[7], n6 = B[7] - B[6], n5 = B[6] - B[5];
+      const int32_t H = n7 + n6 + (n5 + PR_TEAMS - 1) / PR_TEAMS;
+      for (int32_t it = cta; it < H; it += G) {
+        if (it < n7 + n6) {
+          const int64_t i = it < n7 ? (int64_t)B[7] + it : (int64_t)B[6] + (it - n7);
+          propose_blk_node(a, i, par, Team<PR_NT, false>{tid, 0}, shb, vals, keys, clist,
+                           (int64_t)q.tcap);
+        } else {
+          const int tm = tid >> 7;
+          const int32_t j = (it - n7 - n6) * PR_TEAMS + tm;
+          if (j < n5)
+            propose_blk_node(a, (int64_t)B[5] + j, par, Team<128, true>{tid & 127, 1 + tm},
+                             sht[tm], vals + tm * B5_SLOTS, keys + tm * B5_SLOTS,
+                             clist + tm * (B5_SLOTS / 2), (int64_t)B5_SLOTS);
+          __syncthreads();
+        }
+      }
+      // a warp per node from bucket bw on, a thread per node below: the
+      // smaller rows get a warp each, too, while warps are idle
+      int32_t F = H < G ? G - H : 0;
+      const int32_t nT[3] = {B[1] - B[0], B[2] - B[1], B[3] - B[2]};
+      int32_t L = 0;
+      auto tasks = [&](int bw) {
+        int32_t t = B[5] - B[bw];
+        for (int j = 0; j < bw; ++j) t += (nT[j] + 31) >> 5;
+        return t;
+      };
+      int bw = 3;
+      L = tasks(3);
+      if (F == 0 || L > 2 * F * PR_WARPS) F = G;
+      while (bw > 0 && tasks(bw - 1) <= F * PR_WARPS) L = tasks(--bw);
+      const int first = F == G ? 0 : H;
+      if (cta >= first) {
+        for (int32_t t = wib * F + (cta - first); t < L; t += F * PR_WARPS) {
+          int32_t x = t - (B[5] - B[bw]);
+          if (x < 0) {
+            propose_warp_node(a, (int64_t)B[bw] + t, par, vals + wib * WCAP, keys + wib * WCAP);
+            continue;
+          }
+#pragma unroll
+          for (int j = 2; j >= 0; --j) {
+            if (j >= bw) continue;
+            const int32_t n = (nT[j] + 31) >> 5;
+            if (x < n) {
+              const int32_t k = x * 32 + lane;
+              if (k < nT[j]) {
+                if (j == 2) propose_thread_node<16>(a, (int64_t)B[2] + k, par);
+                else if (j == 1) propose_thread_node<8>(a, (int64_t)B[1] + k, par);
+                else propose_thread_node<4>(a, (int64_t)B[0] + k, par);
+              }
+              break;
+            }
+            x -= n;
+          }
+          __syncwarp();
+        }
+      }
+      if (!sync()) return;
+      // admission
+      if (!chain) {
+        adm_resolve<true>(a, &h, 0, an, par, lbeg, cnt, ct);
+        apply_flush_clean(a, h);
+        if (!sync()) return;
+        const int64_t nseg = *(volatile int64_t*)&ct[1];
+        if (nseg > 0) {
+          adm_scatter(a, par, lbeg, cnt, true, 0);
+          if (!sync()) return;
+          adm_select<true, 1>(a, &h, u.sel, 0, an, nseg, 0);
+          apply_flush_clean(a, h);
+          if (!sync()) return;
+        } else {
+          pbeg = lbeg;
+          pcnt = cnt;
+        }
+      } else {
+        adm_resolve<false>(a, &h, 0, an, par, lbeg, cnt, ct);
+        if (!sync()) return;
+        const int64_t nseg = *(volatile int64_t*)&ct[1];
+        adm_scatter(a, par, lbeg, cnt, nseg > 0, 0);
+        if (!sync()) return;
+        if (nseg > 0) {
+          adm_select<false, 1>(a, &h, u.sel, 0, an, nseg, 0);
+          if (!sync()) return;
+        }
+        adm_forced(a, lbeg, cnt, ct + 2);
+        if (!sync()) return;
+        const int64_t nsrc = *(volatile int64_t*)&ct[3];
+        if (nsrc > 0) {
+          adm_alloc(a, nsrc, ct + 2);
+          if (!sync()) return;
+          adm_scatter(a, par, lbeg, cnt, true, 1);
+          if (!sync()) return;
+          adm_select<false, 1>(a, &h, u.sel, 0, an, nsrc, 1);
+          if (!sync()) return;
+        }
+        adm_apply(a, h, an, lbeg, cnt, 0);
+        apply_flush_clean(a, h);
+        if (!sync()) return;
+      }
+      par ^= 1;
+    }
+    // ---- end of the round: queued rows activate their neighbours, slots
+    // that moved little are done, the others get their next round's key
+    clear_in();
+    if (a.mark_big && an) {
+      const int32_t nq = *(volatile int32_t*)&a.mqn[0];
+      for (int32_t k = wib * G + cta; k < nq; k += G * PR_WARPS) {
+        const longlong2 c = a.mq[k];
+        for (int64_t e = c.x + lane; e - lane < c.y; e += 128) {
+          int32_t d[4];
+#pragma unroll
+          for (int w = 0; w < 4; ++w) d[w] = e + 32 * w < c.y ? a.col[e + 32 * w] : -1;
+#pragma unroll
+          for (int w = 0; w < 4; ++w) mark_active(a, an, d[w]);
+        }
+      }
+    }
+    int live = 0;
+    for (int64_t s = gt; s < q.nslots; s += gn) {
+      if (a.done[s]) continue;
+      a.rounds[s] += 1;
+      const int64_t n = a.noff[s + 1] - a.noff[s];
+      if (a.stop_rule && 20 * a.moved[s] < n) {
+        a.done[s] = 1;
+      } else {
+        ++live;
+        if (r + 1 < a.rounds_max) begin_slot((int32_t)s, r + 1);
+      }
+    }
+    if (live) atomicAdd(&q.live[r & 1], live);
+    if (cta == 0 && tid == 0) {
+      q.live[(r + 1) & 1] = 0;
+      a.flags[0] = 0;
+    }
+    if (!sync()) return;
+    const bool more = r + 1 < a.rounds_max && total > 0 &&
+                      *(volatile int32_t*)&q.live[r & 1] > 0;
+    ++r;
+    if (!more) break;
+  }
+  if (cta == 0 && tid == 0) a.rnd[0] = r;
 }
 
 }  // namespace
@@ -2258,6 +2652,16 @@ std::string timeline_dump() {
 // ---------------------------------------------------------------------------
 // Host driver of the rounds.
 // ---------------------------------------------------------------------------
+// Levels up to this size run all their rounds in one persistent launch.  A
+// colour class costs it 12-26 us of barriers and latencies where the launches
+// cost about 57 us, but its one CTA per SM keeps fewer loads in flight.
+// Measured both ways, whole calls: R-MAT 2^16 nodes 6.13 -> 4.11 ms, the
+// three lower levels of a 2^22-node mesh (1.05 M nodes and below) 18.7 ->
+// 15.8 ms, local search on a mesh of 2^20 nodes and 14.6 M arcs 0.93 -> 0.79
+// ms; with the mesh's 4.2 M-node level too 16.7 ms, and the 512-graph batch's
+// levels (8.6 M nodes) no change.
+constexpr int64_t PR_MAX_N = 1250000, PR_MAX_M = 16000000;
+
 int64_t lp_run(const LevelView& lv, const SlotParams& sp, int32_t* label, wgt_t* W,
                int64_t Wsize, const LPRun& run, int32_t* d_err, cudaStream_t s,
                const uint8_t* active_init, uint8_t* active_next_out) {
@@ -2382,6 +2786,57 @@ int64_t lp_run(const LevelView& lv, const SlotParams& sp, int32_t* label, wgt_t*
   const bool compact_blk = run.mode != MODE_CLUSTER && hstat[3] > 0 && hstat[3] <= B5_SLOTS;
   const bool refine = run.mode != MODE_CLUSTER;
   const Tuning tu = tuning_get();
+  const bool prof = profile().enabled.load();
+  const bool timeline = profile().timeline.load(std::memory_order_relaxed);
+  if (!run.graph && !prof && tu.concurrent && tu.pdl && !tu.fused_admission &&
+      maxdeg <= B7_MAXDEG && N <= PR_MAX_N && lv.M <= PR_MAX_M) {
+    int64_t tcap = PR_MIN_TCAP;
+    while (tcap < 2 * maxdeg) tcap <<= 1;
+    static std::once_flag pr_once;
+    std::call_once(pr_once, [&] {
+      SCLAP_CUDA(cudaFuncSetAttribute(k_lp_rounds, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)pr_smem(B7_SLOTS)));
+    });
+    DevBuf<uint32_t> pr(4, s);             // barrier, live counters
+    pr.zero();
+    bcnt.zero();
+    flags.zero();
+    DevBuf<uint64_t> in2((size_t)(2 * Wsize), s);
+    in2.zero();
+    a.in_w = in2.p;
+    DevBuf<longlong2> mq;
+    DevBuf<int32_t> mqn;
+    if (track_active && maxdeg > PR_MARK) {
+      mq.alloc((size_t)(lv.M / PR_MARK + lv.M / PR_MARK_CH + 2), s);
+      mqn.alloc(1, s);
+      mqn.zero();
+      a.mark_big = PR_MARK;
+      a.mark_ch = PR_MARK_CH;
+      a.mq = mq.p;
+      a.mqn = mqn.p;
+    }
+    RoundsArgs q{};
+    q.nslots = sp.nslots;
+    q.phase = run.phase;
+    q.raw_key = run.raw_key ? 1 : 0;
+    q.tcap = (int32_t)tcap;
+    q.seed = sp.seed;
+    q.level = sp.level;
+    q.bar = pr.p;
+    q.live = reinterpret_cast<int32_t*>(pr.p + 1);
+    const int64_t want = std::max<int64_t>(N / 128, lv.M / 2048);
+    const unsigned grid = (unsigned)std::max<int64_t>(8, std::min<int64_t>(sms, want));
+    launch_coop(k_lp_rounds, grid, PR_NT, pr_smem(tcap), s, a, q); SCLAP_NOTE_LAUNCH("k_lp_rounds");
+    SCLAP_LAUNCH_CHECK();
+    int32_t hr = 0;
+    int64_t h_arcs = 0;
+    SCLAP_CUDA(cudaMemcpyAsync(&hr, a.rnd, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+    SCLAP_CUDA(cudaMemcpyAsync(&h_arcs, arcs.p, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+    stream_sync(s);
+    if (active_next_out && track_active)
+      SCLAP_CUDA(cudaMemcpyAsync(active_next_out, a.act[hr & 1], N, cudaMemcpyDeviceToDevice, s));
+    return h_arcs;
+  }
   const int nsb = tu.small_max_deg >= 16 ? 3 : 2;   // buckets of the thread-per-node launch
   const bool need[NB] = {true, true, true, refine || maxdeg > (nsb == 3 ? 16 : 8), false,
                          maxdeg > B4_MAXDEG, maxdeg > B5_MAXDEG, maxdeg > B6_MAXDEG,
@@ -2412,7 +2867,7 @@ int64_t lp_run(const LevelView& lv, const SlotParams& sp, int32_t* label, wgt_t*
     mark_q.alloc((size_t)(2 * (lv.M / MARK_CH) + 2), s);
     mark_n.alloc((size_t)S, s);
     mark_n.zero();
-    a.mark_big = MARK_CH;
+    a.mark_big = a.mark_ch = MARK_CH;
     a.mq = mark_q.p;
     a.mqn = mark_n.p;
   }
@@ -2455,8 +2910,6 @@ int64_t lp_run(const LevelView& lv, const SlotParams& sp, int32_t* label, wgt_t*
   std::vector<Timed> timed;
   int64_t pn[4] = {}, pa[4] = {};
   std::vector<int64_t> hoff(nkeys + 1), hkarcs(nkeys);
-  const bool prof = profile().enabled.load();
-  const bool timeline = profile().timeline.load(std::memory_order_relaxed);
   // The propose launches of a colour class are independent of one another:
   // they run on side streams joined back by events, so latency-bound
   // launches overlap (serial when the timeline profiler is on).  With host
