@@ -1369,6 +1369,27 @@ __device__ __forceinline__ void mark_active(const LPArgs& a, uint8_t* an, int32_
   if (c >= 0 && SCLAP_OK(c, a.N, a.err)) an[c] = 1;
 }
 
+// The heads of the arcs [p0, p1) of four rows become active, by one warp.
+__device__ __forceinline__ void mark_rows4(const LPArgs& a, uint8_t* an, const int64_t (&p0)[4],
+                                           const int64_t (&p1)[4]) {
+  const int lane = threadIdx.x & 31;
+  int32_t c[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) c[q] = p0[q] + lane < p1[q] ? a.col[p0[q] + lane] : -1;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) mark_active(a, an, c[q]);
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    for (int64_t e = p0[q] + 32 + lane; e - lane < p1[q]; e += 128) {
+      int32_t d[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) d[u] = e + 32 * u < p1[q] ? a.col[e + 32 * u] : -1;
+#pragma unroll
+      for (int u = 0; u < 4; ++u) mark_active(a, an, d[u]);
+    }
+  }
+}
+
 // Applies the move of list entry i to label t on the lanes with mv (every
 // lane of the warp calls): label, label weights, moved count, and the moved
 // node's neighbours become active (rows of <= 8 arcs by their own lane,
@@ -1398,13 +1419,23 @@ __device__ __forceinline__ void move_warp(const LPArgs& a, ApplyHash& h, MovedRu
 #pragma unroll
       for (int q = 0; q < 8; ++q) mark_active(a, an, c[q]);
       re = rs;
-    } else if (a.mark_big > 0 && re - rs > a.mark_big) {
-      const int32_t nch = (int32_t)((re - rs + a.mark_ch - 1) / a.mark_ch);
-      const int32_t q0 = atomicAdd(&a.mqn[sub], nch);
-      for (int32_t c = 0; c < nch; ++c)
-        a.mq[q0 + c] = make_longlong2(rs + c * a.mark_ch, min64(rs + (c + 1) * a.mark_ch, re));
-      re = rs;
     }
+  }
+  if (a.mark_big > 0 && __any_sync(0xffffffffu, re - rs > a.mark_big)) {
+    // one reservation per warp for the chunks of its queued rows
+    const bool qd = re - rs > a.mark_big;
+    const int32_t nch = qd ? (int32_t)((re - rs + a.mark_ch - 1) / a.mark_ch) : 0;
+    int32_t incl = nch;
+    for (int o = 1; o < 32; o <<= 1) {
+      const int32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += y;
+    }
+    int32_t q0 = 0;
+    if (lane == 31) q0 = atomicAdd(&a.mqn[sub], incl);
+    q0 = __shfl_sync(0xffffffffu, q0, 31) + incl - nch;
+    for (int32_t c = 0; c < nch; ++c)
+      a.mq[q0 + c] = make_longlong2(rs + c * a.mark_ch, min64(rs + (c + 1) * a.mark_ch, re));
+    if (qd) re = rs;
   }
   // four rows at a time: their loads go out before the first store (the
   // flags may alias the arcs as far as the compiler knows, so one row at a
@@ -1412,7 +1443,6 @@ __device__ __forceinline__ void move_warp(const LPArgs& a, ApplyHash& h, MovedRu
   unsigned big = __ballot_sync(0xffffffffu, re > rs);
   while (big) {
     int64_t p0[4], p1[4];
-    int32_t c[4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const int src = big ? __ffs(big) - 1 : 0;
@@ -1420,20 +1450,7 @@ __device__ __forceinline__ void move_warp(const LPArgs& a, ApplyHash& h, MovedRu
       p1[q] = big ? __shfl_sync(0xffffffffu, (long long)re, src) : p0[q];
       big &= big - 1;
     }
-#pragma unroll
-    for (int q = 0; q < 4; ++q) c[q] = p0[q] + lane < p1[q] ? a.col[p0[q] + lane] : -1;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) mark_active(a, an, c[q]);
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      for (int64_t e = p0[q] + 32 + lane; e - lane < p1[q]; e += 128) {
-        int32_t d[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) d[u] = e + 32 * u < p1[q] ? a.col[e + 32 * u] : -1;
-#pragma unroll
-        for (int u = 0; u < 4; ++u) mark_active(a, an, d[u]);
-      }
-    }
+    mark_rows4(a, an, p0, p1);
   }
   const unsigned mm = __match_any_sync(0xffffffffu, slot);
   if (slot >= 0 && lane == __ffs(mm) - 1) {
@@ -1481,7 +1498,7 @@ __device__ __forceinline__ void adm_resolve(const LPArgs& a, ApplyHash* h, int32
                                             uint8_t* an, int par, int64_t lbeg, int64_t cnt,
                                             int64_t* ct) {
   const int lane = threadIdx.x & 31;
-  // 32 proposals per warp, neighbouring ones to different CTAs
+  // up to 32 proposals per warp, neighbouring groups to different CTAs
   const int64_t w0 = (int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   MovedRun m;
@@ -1590,6 +1607,7 @@ constexpr int SEL_SMALL = 64;     // all-pairs ranking up to this many entries
 constexpr int SEL_NT = 512;       // threads of the selection launch
 constexpr int SEL_CL = 8;         // CTAs of a selection cluster
 constexpr int SEL_CTA = 4096;     // entries a single CTA selects at most (with clusters)
+constexpr int SEL_PAIRS = 256;    // all-pairs ranking by a CTA up to this many entries
 
 __device__ __forceinline__ bool key_less(uint64_t k1, int32_t v1, uint64_t k2, int32_t v2) {
   return k1 < k2 || (k1 == k2 && v1 < v2);
@@ -1882,11 +1900,51 @@ __device__ __forceinline__ void select_large(const LPArgs& a, ApplyHash* h, Move
   sync();                                  // the state is free again
 }
 
+// Segment sg of at most SEL_PAIRS entries: a CTA ranks all pairs in shared
+// memory (scr: 2 * SEL_PAIRS words, left zero).  About 2 us where the radix
+// select's chain of passes and barriers takes 5.
+template <bool APPLY>
+__device__ __forceinline__ void select_pairs(const LPArgs& a, ApplyHash* h, MovedRun& m, int32_t sub,
+                                             uint8_t* an, int64_t sg, int32_t source,
+                                             unsigned long long* scr) {
+  const int j = threadIdx.x;
+  const int64_t base = a.seg_base[sg];
+  const int32_t n = a.seg_cnt[sg];
+  const int64_t thr = a.seg_thr[sg];
+  const int32_t g = a.seg_g[sg];
+  unsigned long long key = 0;
+  int32_t v = 0, w = 0, i = 0;
+  if (j < n) {
+    key = a.ent_key[base + j];
+    v = a.ent_v[base + j];
+    w = a.ent_w[base + j];
+    i = a.ent_i[base + j];
+    scr[j] = key;
+    scr[SEL_PAIRS + j] = ((unsigned long long)(uint32_t)v << 32) | (uint32_t)w;
+  }
+  __syncthreads();
+  bool ok = false;
+  if (j < n) {
+    int64_t excl = 0;
+    for (int l = 0; l < n; ++l) {
+      const unsigned long long kl = scr[l], vw = scr[SEL_PAIRS + l];
+      if (kl < key || (kl == key && (int32_t)(vw >> 32) < v)) excl += (int32_t)vw;
+    }
+    ok = source ? excl <= thr : excl + w <= thr;
+    if (!APPLY) a.adm[i] = ok ? 1 : 0;
+  }
+  if (APPLY && (j & ~31) < n) move_warp(a, *h, m, sub, an, ok, i, g);
+  if (j == 0) a.ovf_cnt[g] = 0;
+  __syncthreads();
+  if (j < n) scr[j] = scr[SEL_PAIRS + j] = 0;
+  __syncthreads();
+}
+
 // All segments of one side of a colour class.  CL > 1: the launch has
 // clusters of CL CTAs, which take the segments above SEL_CTA entries.
 template <bool APPLY, int CL>
-__device__ void adm_select(const LPArgs& a, ApplyHash* h, SelState& L, int32_t sub, uint8_t* an,
-                           int64_t nseg, int32_t source) {
+__device__ void adm_select(const LPArgs& a, ApplyHash* h, SelState& L, unsigned long long* scr,
+                           int32_t sub, uint8_t* an, int64_t nseg, int32_t source) {
   MovedRun m;
   const int tid = threadIdx.x, lane = tid & 31;
   // segments of <= 64 entries, one warp each (entries lane and lane + 32 in
@@ -1941,7 +1999,9 @@ __device__ void adm_select(const LPArgs& a, ApplyHash* h, SelState& L, int32_t s
   // larger ones: a CTA each
   for (int64_t sg = blockIdx.x; sg < nseg; sg += gridDim.x) {
     const int32_t n = a.seg_cnt[sg];
-    if (n > SEL_SMALL && (CL == 1 || n <= SEL_CTA))
+    if (n > SEL_SMALL && n <= SEL_PAIRS)
+      select_pairs<APPLY>(a, h, m, sub, an, sg, source, scr);
+    else if (n > SEL_SMALL && (CL == 1 || n <= SEL_CTA))
       select_large<APPLY, 1>(a, h, m, sub, an, sg, source, L);
   }
   // the largest: a cluster each
@@ -1984,6 +2044,7 @@ __global__ void __launch_bounds__(ADM_NT) k_admit(LPArgs a, int32_t sub, int32_t
   if (*(volatile int32_t*)a.err & DERR_TIMEOUT) return;
   __shared__ ApplyHash h;
   __shared__ SelState sel;
+  __shared__ unsigned long long scr[2 * SEL_PAIRS];
   apply_init(h);
   int64_t lbeg, cnt;
   sub_range(a, sub, 0, NB, &lbeg, &cnt);
@@ -1998,8 +2059,8 @@ __global__ void __launch_bounds__(ADM_NT) k_admit(LPArgs a, int32_t sub, int32_t
   adm_scatter(a, 0, lbeg, cnt, nseg > 0, 0);
   if (nseg > 0) {
     if (!grid_sync(gs, a.err, lim)) return;
-    if (chain) adm_select<false, 1>(a, &h, sel, sub, an, nseg, 0);
-    else adm_select<true, 1>(a, &h, sel, sub, an, nseg, 0);
+    if (chain) adm_select<false, 1>(a, &h, sel, scr, sub, an, nseg, 0);
+    else adm_select<true, 1>(a, &h, sel, scr, sub, an, nseg, 0);
   }
   if (chain) {
     if (!grid_sync(gs, a.err, lim)) return;
@@ -2012,7 +2073,7 @@ __global__ void __launch_bounds__(ADM_NT) k_admit(LPArgs a, int32_t sub, int32_t
       if (!grid_sync(gs, a.err, lim)) return;
       adm_scatter(a, 0, lbeg, cnt, true, 1);
       if (!grid_sync(gs, a.err, lim)) return;
-      adm_select<false, 1>(a, &h, sel, sub, an, nsrc, 1);
+      adm_select<false, 1>(a, &h, sel, scr, sub, an, nsrc, 1);
       if (!grid_sync(gs, a.err, lim)) return;
     }
     adm_apply(a, h, an, lbeg, cnt, sub);
@@ -2071,14 +2132,15 @@ __global__ void __cluster_dims__(SEL_CL, 1, 1) __launch_bounds__(SEL_NT) k_ovf_s
   griddep_wait();
   __shared__ ApplyHash h;
   __shared__ SelState sel;
+  __shared__ unsigned long long scr[2 * SEL_PAIRS];
   const int64_t nseg = *(volatile int64_t*)&adm_ctr(a, sub, side)[1];
   if (nseg == 0) return;
   if (chain_on(a, source_chain)) {
-    adm_select<false, SEL_CL>(a, nullptr, sel, sub, nullptr, nseg, side);
+    adm_select<false, SEL_CL>(a, nullptr, sel, scr, sub, nullptr, nseg, side);
     return;
   }
   apply_init(h);
-  adm_select<true, SEL_CL>(a, &h, sel, sub, act_next(a), nseg, side);
+  adm_select<true, SEL_CL>(a, &h, sel, scr, sub, act_next(a), nseg, side);
   apply_flush(a, h);
 }
 __global__ void __launch_bounds__(ADM_NT) k_apply(LPArgs a, int32_t sub) {
@@ -2134,7 +2196,7 @@ __global__ void __launch_bounds__(256) k_mark_rows(LPArgs a, int32_t sub) {
 constexpr int PR_NT = 512, PR_WARPS = PR_NT / 32, PR_TEAMS = PR_NT / 128;
 constexpr int PR_MIN_TCAP = PR_WARPS * WCAP;       // = PR_TEAMS * B5_SLOTS
 static_assert(PR_MIN_TCAP == PR_TEAMS * B5_SLOTS, "the tables of warps and teams share the CTA's");
-constexpr int64_t PR_MARK = 128, PR_MARK_CH = 512; // queued rows, arcs per queued chunk
+constexpr int64_t PR_MARK = 8, PR_MARK_CH = 512;   // queued rows, arcs per queued chunk
 constexpr size_t pr_smem(int64_t tcap) {
   return (size_t)tcap * (sizeof(unsigned long long) + sizeof(int32_t)) +
          (size_t)(tcap / 2) * sizeof(uint16_t);
@@ -2156,8 +2218,9 @@ __device__ __forceinline__ bool round_sync(unsigned int* bar, unsigned int& want
   want += gridDim.x;
   __syncthreads();
   if (threadIdx.x == 0) {
-    __threadfence();
-    atomicAdd(bar, 1u);
+    // the release orders what the CTA wrote before its barrier above, the
+    // acquire what it reads after the one below
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
     int ok = 1;
     uint32_t it = 0;
     while ((int)(ld_acquire_gpu(bar) - want) < 0) {
@@ -2167,7 +2230,6 @@ __device__ __forceinline__ bool round_sync(unsigned int* bar, unsigned int& want
         break;
       }
     }
-    __threadfence();
     ok_sh = ok;
   }
   __syncthreads();
@@ -2388,7 +2450,7 @@ __global__ void __launch_bounds__(PR_NT, 1) k_lp_rounds(LPArgs a, RoundsArgs q) 
         if (nseg > 0) {
           adm_scatter(a, par, lbeg, cnt, true, 0);
           if (!sync()) return;
-          adm_select<true, 1>(a, &h, u.sel, 0, an, nseg, 0);
+          adm_select<true, 1>(a, &h, u.sel, vals, 0, an, nseg, 0);
           apply_flush_clean(a, h);
           if (!sync()) return;
         } else {
@@ -2402,7 +2464,7 @@ __global__ void __launch_bounds__(PR_NT, 1) k_lp_rounds(LPArgs a, RoundsArgs q) 
         adm_scatter(a, par, lbeg, cnt, nseg > 0, 0);
         if (!sync()) return;
         if (nseg > 0) {
-          adm_select<false, 1>(a, &h, u.sel, 0, an, nseg, 0);
+          adm_select<false, 1>(a, &h, u.sel, vals, 0, an, nseg, 0);
           if (!sync()) return;
         }
         adm_forced(a, lbeg, cnt, ct + 2);
@@ -2413,7 +2475,7 @@ __global__ void __launch_bounds__(PR_NT, 1) k_lp_rounds(LPArgs a, RoundsArgs q) 
           if (!sync()) return;
           adm_scatter(a, par, lbeg, cnt, true, 1);
           if (!sync()) return;
-          adm_select<false, 1>(a, &h, u.sel, 0, an, nsrc, 1);
+          adm_select<false, 1>(a, &h, u.sel, vals, 0, an, nsrc, 1);
           if (!sync()) return;
         }
         adm_apply(a, h, an, lbeg, cnt, 0);
@@ -2427,15 +2489,16 @@ __global__ void __launch_bounds__(PR_NT, 1) k_lp_rounds(LPArgs a, RoundsArgs q) 
     clear_in();
     if (a.mark_big && an) {
       const int32_t nq = *(volatile int32_t*)&a.mqn[0];
-      for (int32_t k = wib * G + cta; k < nq; k += G * PR_WARPS) {
-        const longlong2 c = a.mq[k];
-        for (int64_t e = c.x + lane; e - lane < c.y; e += 128) {
-          int32_t d[4];
+      for (int32_t k0 = wib * G + cta; k0 < nq; k0 += 4 * G * PR_WARPS) {
+        int64_t p0[4], p1[4];
 #pragma unroll
-          for (int w = 0; w < 4; ++w) d[w] = e + 32 * w < c.y ? a.col[e + 32 * w] : -1;
-#pragma unroll
-          for (int w = 0; w < 4; ++w) mark_active(a, an, d[w]);
+        for (int w = 0; w < 4; ++w) {
+          const int32_t k = k0 + w * G * PR_WARPS;
+          const longlong2 c = k < nq ? a.mq[k] : make_longlong2(0, 0);
+          p0[w] = c.x;
+          p1[w] = c.y;
         }
+        mark_rows4(a, an, p0, p1);
       }
     }
     int live = 0;
@@ -2807,7 +2870,9 @@ int64_t lp_run(const LevelView& lv, const SlotParams& sp, int32_t* label, wgt_t*
     DevBuf<longlong2> mq;
     DevBuf<int32_t> mqn;
     if (track_active && maxdeg > PR_MARK) {
-      mq.alloc((size_t)(lv.M / PR_MARK + lv.M / PR_MARK_CH + 2), s);
+      // at most one chunk per node of degree above PR_MARK, and one per
+      // PR_MARK_CH arcs
+      mq.alloc((size_t)(std::min<int64_t>(N, lv.M / PR_MARK) + lv.M / PR_MARK_CH + 2), s);
       mqn.alloc(1, s);
       mqn.zero();
       a.mark_big = PR_MARK;
