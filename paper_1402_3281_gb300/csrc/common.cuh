@@ -7,6 +7,7 @@
 
 #include <atomic>
 #include <cstdio>
+#include <cstring>
 #include <mutex>
 #include <stdexcept>
 #include <string>
@@ -58,8 +59,54 @@ void timeline_mark(const char* name, cudaStream_t s);
 std::string timeline_dump();
 // cudaStreamSynchronize that also marks the timeline ("host": the copy and
 // round trip that preceded the wait).
+// Pinned memory of the calling thread that small transfers pass through, so
+// that none of them is staged by the driver (a pageable read-back is a host
+// wait of its own, and a pageable upload about 5 us).  Space is taken in
+// order and free again after the next wait for the stream; the transfers of
+// a call all go to one stream, and a call ends, or is given up, with a wait.
+struct HostRing {
+  static constexpr size_t CAP = (size_t)1 << 20;
+  char* p = nullptr;
+  size_t at = 0;
+  cudaStream_t s = nullptr;      // stream of the transfers since the last wait
+  bool failed = false;           // no pinned memory: transfers stay pageable
+  HostRing() = default;
+  HostRing(const HostRing&) = delete;
+  HostRing& operator=(const HostRing&) = delete;
+  ~HostRing() {
+    if (p) cudaFreeHost(p);
+  }
+  // room for `bytes` (NULL: none left; the caller transfers pageable memory)
+  char* take(size_t bytes, cudaStream_t st) {
+    if (failed || bytes > CAP / 4 || (at > 0 && st != s)) return nullptr;
+    if (!p && cudaHostAlloc((void**)&p, CAP, cudaHostAllocDefault) != cudaSuccess) {
+      cudaGetLastError();
+      p = nullptr;
+      failed = true;
+      return nullptr;
+    }
+    if (at + bytes > CAP) return nullptr;
+    char* r = p + at;
+    at += (bytes + 63) & ~(size_t)63;
+    s = st;
+    return r;
+  }
+  void waited(cudaStream_t st) {
+    if (st == s) at = 0;
+  }
+  // a call failed with transfers under way: they end before the space is used again
+  void give_up() {
+    if (at == 0) return;
+    cudaStreamSynchronize(s);
+    cudaGetLastError();
+    at = 0;
+  }
+};
+HostRing& host_ring();
+
 inline void stream_sync(cudaStream_t s) {
   SCLAP_CUDA(cudaStreamSynchronize(s));
+  host_ring().waited(s);
   if (profile().timeline.load(std::memory_order_relaxed)) timeline_mark("host", s);
 }
 cudaEvent_t event_from_pool();
@@ -339,6 +386,11 @@ using wgt_t = int32_t;
 // A level: one CSR holding the graphs of all slots back to back (node ids are
 // global, node range of slot s = [noff[s], noff[s+1])).
 // ---------------------------------------------------------------------------
+// Degrees of a level: the largest, and of the nodes above B7_MAXDEG (hubs)
+// their number and the table slots they need together.
+struct DegStats {
+  int64_t maxdeg = -1, nhubs = 0, hub_slots = 0;
+};
 struct LevelView {
   int64_t N = 0, M = 0;
   const int64_t* row_ptr = nullptr;
@@ -349,6 +401,9 @@ struct LevelView {
   int32_t nslots = 1;
   const int64_t* noff = nullptr;  // [nslots + 1] first node of each slot (device)
   const int64_t* aoff = nullptr;  // [nslots + 1] first arc of each slot (device)
+  // degrees of the level where the host knows them (maxdeg < 0: not); upper
+  // bounds where the level's nodes are some of another level's
+  DegStats deg;
   // every sum of arc weights over a row (so every connection) is below 2^32:
   // the propose tables may accumulate with 32-bit atomics
   bool narrow = false;
@@ -366,6 +421,7 @@ struct SlotParams {
   const uint64_t* seed = nullptr;   // seed key fed to hkey
   const int32_t* level = nullptr;   // level id fed to hkey
   const int32_t* nlab = nullptr;    // labels of the slot (k in local search)
+  int32_t max_nlab = 0;             // the largest of them (local search)
   int32_t* done = nullptr;          // 1: slot takes no part in further rounds
   int64_t* moved = nullptr;         // moves of the current round
   uint64_t* rkey = nullptr;         // key of the current round
@@ -509,9 +565,20 @@ struct DevBuf {
     if (n) SCLAP_CUDA(cudaMemsetAsync(p, v, n * sizeof(T), s));
   }
   void upload(const T* h, size_t count) {
-    if (count) SCLAP_CUDA(cudaMemcpyAsync(p, h, count * sizeof(T), cudaMemcpyHostToDevice, s));
+    if (!count) return;
+    if (char* r = host_ring().take(count * sizeof(T), s)) {
+      std::memcpy(r, h, count * sizeof(T));
+      h = reinterpret_cast<const T*>(r);
+    }
+    SCLAP_CUDA(cudaMemcpyAsync(p, h, count * sizeof(T), cudaMemcpyHostToDevice, s));
   }
-  void upload(const std::vector<T>& v) { upload(v.data(), v.size()); }
+  // (the vector may go once the call returns)
+  void upload(const std::vector<T>& v) {
+    if (v.empty()) return;
+    const size_t at = host_ring().at;
+    upload(v.data(), v.size());
+    if (host_ring().at == at) SCLAP_CUDA(cudaStreamSynchronize(s));   // not through the ring
+  }
   DevBuf(const DevBuf&) = delete;
   DevBuf& operator=(const DevBuf&) = delete;
   DevBuf(DevBuf&& o) noexcept { *this = std::move(o); }
@@ -526,6 +593,40 @@ struct DevBuf {
   ~DevBuf() { release(); }
 };
 
+// Device values read back together with one host wait.
+struct ReadBack {
+  cudaStream_t s;
+  struct Item { void* dst; const char* src; size_t bytes; };
+  std::vector<Item> items;
+  explicit ReadBack(cudaStream_t st) : s(st) {}
+  template <class T>
+  void add(T* dst, const T* dev, size_t count) {
+    const size_t bytes = count * sizeof(T);
+    if (!bytes) return;
+    char* r = host_ring().take(bytes, s);
+    SCLAP_CUDA(cudaMemcpyAsync(r ? (void*)r : (void*)dst, dev, bytes, cudaMemcpyDeviceToHost, s));
+    if (r) items.push_back(Item{dst, r, bytes});
+  }
+  void wait() {
+    stream_sync(s);
+    for (const Item& x : items) std::memcpy(x.dst, x.src, x.bytes);
+    items.clear();
+  }
+};
+
+// Lays out several arrays in one allocation: a first pass (no base) adds up
+// the sizes, a second hands out the pointers.
+struct Carve {
+  char* base = nullptr;
+  size_t at = 0;
+  template <class T>
+  void take(T*& p, size_t n) {
+    at = (at + 255) & ~(size_t)255;
+    if (base) p = reinterpret_cast<T*>(base + at);
+    at += n * sizeof(T);
+  }
+};
+
 // ---------------------------------------------------------------------------
 // Entry points of the kernel files (host side).
 // ---------------------------------------------------------------------------
@@ -535,7 +636,6 @@ void scan_excl_i64(const int64_t* in, int64_t* out, int64_t n, cudaStream_t s);
 void scan_excl_u8_to_i64(const uint8_t* in, int64_t* out, int64_t n, cudaStream_t s);
 // out[i] = number of keys[0..i) that are >= 0 (occupied hash slots).
 void scan_excl_occupied(const int32_t* keys, int64_t* out, int64_t n, cudaStream_t s);
-// largest row length (atomicMax into *out, which the caller zeroes)
 // out[0] = largest degree of the level, out[1] = nodes with degree > thr,
 // out[2] = the table slots of those nodes together (out zeroed by the caller).
 void level_degree_stats(const int64_t* row_ptr, int64_t N, int64_t thr, int64_t* out,
@@ -557,10 +657,11 @@ struct LPRun {
   const int32_t* rblk = nullptr;  // clustering: respect this partition (V-cycles)
 };
 // Runs `run.rounds` synchronous LP rounds on `lv` for every slot not marked
-// done; label/W are updated in place.  Returns the number of arcs scanned.
-int64_t lp_run(const LevelView& lv, const SlotParams& sp, int32_t* label, wgt_t* W,
-               int64_t Wsize, const LPRun& run, int32_t* d_err, cudaStream_t s,
-               const uint8_t* active_init = nullptr, uint8_t* active_next_out = nullptr);
+// done; label/W are updated in place.  Adds the arcs scanned to *d_arcs
+// (device).  The work may still be under way on return.
+void lp_run(const LevelView& lv, const SlotParams& sp, int32_t* label, wgt_t* W,
+            int64_t Wsize, const LPRun& run, int64_t* d_arcs, int32_t* d_err, cudaStream_t s,
+            const uint8_t* active_init = nullptr, uint8_t* active_next_out = nullptr);
 void lp_round_begin_host_keys(const SlotParams& sp, int phase, int r, int mode,
                               const wgt_t* W, cudaStream_t s);
 
@@ -577,6 +678,7 @@ struct CoarseLevel {
   DevBuf<int64_t> noff_d, aoff_d;
   std::vector<int64_t> noff;   // [nslots+1]
   std::vector<int64_t> aoff;   // arc offset of each slot [nslots+1]
+  DegStats deg;
 };
 // Step 1: ranks the used labels; nc_slot[s] = coarse nodes of slot s.
 // Overlay of two clusterings of a batched level (ensemble clusterings): for

@@ -289,6 +289,13 @@ __global__ void __launch_bounds__(256) k_insert_heavy(CArgs a, const int32_t* __
   });
 }
 
+__global__ void k_clear_table(unsigned long long* __restrict__ tslot,
+                              const int64_t* __restrict__ T) {
+  for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < *T;
+       j += (int64_t)gridDim.x * blockDim.x)
+    tslot[j] = ~0ull;
+}
+
 // Coarse rows: one thread per table slot; an occupied slot goes to its
 // owner's row (offsets from a scan of the claimed-slot counts) at a position
 // taken from a per-row counter.  The order of a row's arcs is therefore not
@@ -296,8 +303,9 @@ __global__ void __launch_bounds__(256) k_insert_heavy(CArgs a, const int32_t* __
 // race); nothing computed from a coarse graph depends on that order.
 __global__ void k_emit(const unsigned long long* __restrict__ tslot,
                        const int32_t* __restrict__ towner, const int64_t* __restrict__ crow,
-                       int32_t* __restrict__ fill, int64_t T, int32_t* __restrict__ ccol,
-                       int32_t* __restrict__ cew) {
+                       int32_t* __restrict__ fill, int64_t T, const int64_t* Tdev,
+                       int32_t* __restrict__ ccol, int32_t* __restrict__ cew) {
+  if (Tdev) T = min(T, *Tdev);             // the slots in use, where the host knows a bound
   for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < T;
        j += (int64_t)gridDim.x * blockDim.x) {
     const unsigned long long x = tslot[j];
@@ -807,18 +815,26 @@ __global__ void k_overlay_apply(const int32_t* __restrict__ gid, const int32_t* 
   }
 }
 
-// Node ids per slot and the arc offsets of the slots of a built level.
+// Node ids per slot, the arc offsets of the slots, the arcs and the degrees
+// of a built level (one read-back).
 void finish_level(CoarseLevel& out, int ns, cudaStream_t s) {
   const int64_t Nc = out.N;
   out.gid.alloc(std::max<int64_t>(Nc, 1), s);
   fill_gid(out.noff_d.p, ns, out.gid.p, Nc, s);
+  DevBuf<int64_t> dstat(3, s);
+  dstat.zero();
+  level_degree_stats(out.row_ptr.p, Nc, B7_MAXDEG, dstat.p, s);
   out.aoff_d.alloc(ns + 1, s);
   k_gather<<<grid_for(ns + 1, 128, 64), 128, 0, s>>>(out.row_ptr.p, out.noff_d.p, ns + 1, out.aoff_d.p); SCLAP_NOTE_LAUNCH("k_gather");
   SCLAP_LAUNCH_CHECK();
   out.aoff.assign(ns + 1, 0);
-  SCLAP_CUDA(cudaMemcpyAsync(out.aoff.data(), out.aoff_d.p, (ns + 1) * sizeof(int64_t),
-                             cudaMemcpyDeviceToHost, s));
-  stream_sync(s);
+  int64_t ds[3] = {0, 0, 0};
+  ReadBack rb(s);
+  rb.add(out.aoff.data(), out.aoff_d.p, ns + 1);
+  rb.add(ds, dstat.p, 3);
+  rb.wait();
+  out.M = out.aoff[ns];
+  out.deg = DegStats{ds[0], ds[1], ds[2]};
 }
 
 // The coarse arcs by segments (member lists and per-node merges, see the
@@ -903,9 +919,9 @@ bool contract_merge(const LevelView& lv, int64_t N, int64_t Nc, DevBuf<int32_t>&
   out.row_ptr.alloc(Nc + 1, s);
   scan_excl_i32_to_i64(cdeg.p, out.row_ptr.p, Nc, s);
   int64_t Mc = 0;
-  SCLAP_CUDA(cudaMemcpyAsync(&Mc, out.row_ptr.p + Nc, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-  stream_sync(s);
-  out.M = Mc;
+  ReadBack rb(s);
+  rb.add(&Mc, out.row_ptr.p + Nc, 1);
+  rb.wait();
   out.col.alloc(std::max<int64_t>(Mc, 1), s);
   out.ew.alloc(std::max<int64_t>(Mc, 1), s);
   k_rows_from_regions<<<grid_for(Nc * 32, 256, (int64_t)sms * 16), 256, 0, s>>>(
@@ -926,14 +942,13 @@ void contract_rank(const LevelView& lv, const std::vector<int64_t>& noff, const 
   const int sms = num_sms();
   if (N > 0) { k_mark<<<grid_for(N, 256, (int64_t)sms * 16), 256, 0, s>>>(label, N, w.flag.p); SCLAP_NOTE_LAUNCH("k_mark"); }
   scan_excl_i32_to_i64(w.flag.p, w.cid.p, N, s);
-  DevBuf<int64_t> idx(ns + 1, s), got(ns + 1, s);
-  idx.upload(noff);
-  k_gather<<<grid_for(ns + 1, 128, 64), 128, 0, s>>>(w.cid.p, idx.p, ns + 1, got.p); SCLAP_NOTE_LAUNCH("k_gather");
+  DevBuf<int64_t> got(ns + 1, s);
+  k_gather<<<grid_for(ns + 1, 128, 64), 128, 0, s>>>(w.cid.p, lv.noff, ns + 1, got.p); SCLAP_NOTE_LAUNCH("k_gather");
   SCLAP_LAUNCH_CHECK();
   w.cid_at.assign(ns + 1, 0);
-  SCLAP_CUDA(cudaMemcpyAsync(w.cid_at.data(), got.p, (ns + 1) * sizeof(int64_t),
-                             cudaMemcpyDeviceToHost, s));
-  stream_sync(s);
+  ReadBack rb(s);
+  rb.add(w.cid_at.data(), got.p, ns + 1);
+  rb.wait();
   nc_slot.assign(ns, 0);
   for (int i = 0; i < ns; ++i) nc_slot[i] = w.cid_at[i + 1] - w.cid_at[i];
 }
@@ -978,6 +993,7 @@ void contract_build(const LevelView& lv, const std::vector<int64_t>& noff, const
   const unsigned hg = (unsigned)sms * 8;                      // heavy-row chunks, grid-stride
   // rows above HEAVY_ROW arcs: listed, cut into chunks, spread over the grid
   constexpr int64_t HEAVY_ROW = 2048;
+  constexpr int64_t BOUNDED_M = 4000000;   // arcs: at most 96 MB of table
   DevBuf<int32_t> hlist(std::max<int64_t>(1, std::min<int64_t>(N, lv.M / (HEAVY_ROW + 1) + 1)), s);
   DevBuf<int64_t> hoff;
   int32_t nh = 0;
@@ -986,9 +1002,12 @@ void contract_build(const LevelView& lv, const std::vector<int64_t>& noff, const
     a.heavy = HEAVY_ROW;
     DevBuf<int32_t> hcnt(1, s);
     hcnt.zero();
-    k_heavy_list<<<ng, 256, 0, s>>>(a, N, hlist.p, hcnt.p); SCLAP_NOTE_LAUNCH("k_heavy_list");
-    SCLAP_CUDA(cudaMemcpyAsync(&nh, hcnt.p, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-    stream_sync(s);
+    if (lv.deg.maxdeg < 0 || lv.deg.maxdeg > HEAVY_ROW) {
+      k_heavy_list<<<ng, 256, 0, s>>>(a, N, hlist.p, hcnt.p); SCLAP_NOTE_LAUNCH("k_heavy_list");
+      ReadBack rb(s);
+      rb.add(&nh, hcnt.p, 1);
+      rb.wait();
+    }
     if (nh > 0) {
       DevBuf<int32_t> nch(nh, s);
       hoff.alloc(nh + 1, s);
@@ -1012,9 +1031,16 @@ void contract_build(const LevelView& lv, const std::vector<int64_t>& noff, const
     k_table_caps<<<grid_for(Nc, 256, (int64_t)sms * 16), 256, 0, s>>>(inter.p, Nc, cap.p); SCLAP_NOTE_LAUNCH("k_table_caps");
   }
   scan_excl_i64(cap.p, tbase.p, Nc, s);
-  int64_t T = 0;
-  SCLAP_CUDA(cudaMemcpyAsync(&T, tbase.p + Nc, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-  stream_sync(s);
+  // a small level takes a table and coarse arrays of the largest size they
+  // can have instead of waiting for the sizes (twice): fewer than two slots
+  // per arc, no more coarse arcs than fine ones
+  const bool bounded = lv.M <= BOUNDED_M && 2 * lv.M <= Tcap;
+  int64_t T = 2 * lv.M;
+  if (!bounded) {
+    ReadBack rb(s);
+    rb.add(&T, tbase.p + Nc, 1);
+    rb.wait();
+  }
   // the inter-arc counts have served (table sizes); the array now counts
   // claimed slots, i.e. the coarse degrees
   a.cdeg = inter.p;
@@ -1024,21 +1050,27 @@ void contract_build(const LevelView& lv, const std::vector<int64_t>& noff, const
     // one pass: the whole table at once
     DevBuf<unsigned long long> tslot(std::max<int64_t>(T, 1), s);
     DevBuf<int32_t> towner(std::max<int64_t>(T, 1), s);
-    tslot.fill_bytes(0xff);
+    if (bounded && T > 0) {
+      k_clear_table<<<grid_for(T, 1024, (int64_t)sms * 8), 256, 0, s>>>(tslot.p, tbase.p + Nc); SCLAP_NOTE_LAUNCH("k_clear_table");
+    } else {
+      tslot.fill_bytes(0xff);
+    }
     a.tslot = tslot.p;
     a.towner = towner.p;
     if (N > 0 && T > 0) insert();
     scan_excl_i32_to_i64(inter.p, out.row_ptr.p, Nc, s);
-    int64_t Mc = 0;
-    SCLAP_CUDA(cudaMemcpyAsync(&Mc, out.row_ptr.p + Nc, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-    stream_sync(s);
-    out.M = Mc;
+    int64_t Mc = lv.M;
+    if (!bounded) {
+      ReadBack rb(s);
+      rb.add(&Mc, out.row_ptr.p + Nc, 1);
+      rb.wait();
+    }
     out.col.alloc(std::max<int64_t>(Mc, 1), s);
     out.ew.alloc(std::max<int64_t>(Mc, 1), s);
     if (Nc > 0 && T > 0) {
       SCLAP_CUDA(cudaMemsetAsync(inter.p, 0, (size_t)Nc * sizeof(int32_t), s));   // row fill
-      k_emit<<<grid_for(T, 256, (int64_t)sms * 32), 256, 0, s>>>(tslot.p, towner.p, out.row_ptr.p,
-                                                                 inter.p, T, out.col.p, out.ew.p); SCLAP_NOTE_LAUNCH("k_emit");
+      k_emit<<<grid_for(T, 256, (int64_t)sms * 32), 256, 0, s>>>(
+          tslot.p, towner.p, out.row_ptr.p, inter.p, T, tbase.p + Nc, out.col.p, out.ew.p); SCLAP_NOTE_LAUNCH("k_emit");
     }
   } else {
     // Passes over ranges of coarse nodes whose table regions fit in Tcap
@@ -1077,9 +1109,9 @@ void contract_build(const LevelView& lv, const std::vector<int64_t>& noff, const
     for (size_t q = 0; q + 1 < cut_at.size(); ++q) pass(q);            // sweep 1: degrees
     scan_excl_i32_to_i64(inter.p, out.row_ptr.p, Nc, s);
     int64_t Mc = 0;
-    SCLAP_CUDA(cudaMemcpyAsync(&Mc, out.row_ptr.p + Nc, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-    stream_sync(s);
-    out.M = Mc;
+    ReadBack rb(s);
+    rb.add(&Mc, out.row_ptr.p + Nc, 1);
+    rb.wait();
     out.col.alloc(std::max<int64_t>(Mc, 1), s);
     out.ew.alloc(std::max<int64_t>(Mc, 1), s);
     a.cdeg = claims.p;                   // sweep 2 counts claims apart from the row fill
@@ -1088,7 +1120,7 @@ void contract_build(const LevelView& lv, const std::vector<int64_t>& noff, const
       const int64_t Tp = pass(q);
       k_emit<<<grid_for(Tp, 256, (int64_t)sms * 32), 256, 0, s>>>(tslot.p, towner.p,
                                                                   out.row_ptr.p, inter.p, Tp,
-                                                                  out.col.p, out.ew.p); SCLAP_NOTE_LAUNCH("k_emit");
+                                                                  nullptr, out.col.p, out.ew.p); SCLAP_NOTE_LAUNCH("k_emit");
     }
   }
   SCLAP_LAUNCH_CHECK();

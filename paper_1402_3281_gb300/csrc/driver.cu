@@ -245,29 +245,41 @@ __global__ void k_write_out(const OutTask* __restrict__ t, const int32_t* __rest
 }
 
 // ------------------------------------------------------------- slot arrays
+// Parameters of an LP run per slot: one allocation, one upload.
 struct Slots {
-  DevBuf<int64_t> loff, bound, moved;
-  DevBuf<uint64_t> seed, rkey;
-  DevBuf<int32_t> level, nlab, done, rounds;
+  DevBuf<char> buf;
   SlotParams sp;
   Slots(cudaStream_t s, int n, const int64_t* noff_d, const std::vector<int64_t>& h_loff,
         const std::vector<int64_t>& h_bound, const std::vector<uint64_t>& h_seed,
         const std::vector<int32_t>& h_level, const std::vector<int32_t>& h_nlab,
-        const std::vector<int32_t>& h_done)
-      : loff(n, s), bound(n, s), moved(n, s), seed(n, s), rkey(n, s), level(n, s), nlab(n, s),
-        done(n, s), rounds(n, s) {
-    loff.upload(h_loff); bound.upload(h_bound); seed.upload(h_seed); level.upload(h_level);
-    nlab.upload(h_nlab); done.upload(h_done); rounds.zero(); moved.zero();
-    sp.nslots = n; sp.noff = noff_d; sp.loff = loff.p; sp.bound = bound.p; sp.seed = seed.p;
-    sp.level = level.p; sp.nlab = nlab.p; sp.done = done.p; sp.moved = moved.p; sp.rkey = rkey.p;
-    sp.rounds = rounds.p;
-  }
-  std::vector<int32_t> host_rounds(cudaStream_t s) {
-    std::vector<int32_t> r(sp.nslots);
-    SCLAP_CUDA(cudaMemcpyAsync(r.data(), rounds.p, r.size() * sizeof(int32_t),
-                               cudaMemcpyDeviceToHost, s));
-    stream_sync(s);
-    return r;
+        const std::vector<int32_t>& h_done) {
+    // uploaded: loff, bound, seed, level, nlab, done, rounds and moved (zero);
+    // left as it is: rkey
+    const size_t w = (size_t)n * 8, h = (size_t)n * 4;
+    const size_t up = 4 * w + 4 * h;
+    buf.alloc(up + w, s);
+    std::vector<char> st(up, 0);
+    char* p = st.data();
+    std::memcpy(p, h_loff.data(), w);
+    std::memcpy(p + w, h_bound.data(), w);
+    std::memcpy(p + 2 * w, h_seed.data(), w);
+    std::memcpy(p + 4 * w, h_level.data(), h);
+    std::memcpy(p + 4 * w + h, h_nlab.data(), h);
+    std::memcpy(p + 4 * w + 2 * h, h_done.data(), h);
+    buf.upload(st);
+    char* d = buf.p;
+    sp.nslots = n;
+    sp.noff = noff_d;
+    sp.loff = reinterpret_cast<const int64_t*>(d);
+    sp.bound = reinterpret_cast<const int64_t*>(d + w);
+    sp.seed = reinterpret_cast<const uint64_t*>(d + 2 * w);
+    sp.moved = reinterpret_cast<int64_t*>(d + 3 * w);
+    sp.level = reinterpret_cast<const int32_t*>(d + 4 * w);
+    sp.nlab = reinterpret_cast<const int32_t*>(d + 4 * w + h);
+    sp.done = reinterpret_cast<int32_t*>(d + 4 * w + 2 * h);
+    sp.rounds = reinterpret_cast<int32_t*>(d + 4 * w + 3 * h);
+    sp.rkey = reinterpret_cast<uint64_t*>(d + up);
+    for (int32_t x : h_nlab) sp.max_nlab = std::max(sp.max_nlab, x);
   }
 };
 
@@ -285,6 +297,7 @@ struct Level {
   const int32_t* nw_in = nullptr;
   bool borrowed = false;
   std::vector<int64_t> noff, aoff;
+  DegStats deg;
   // every sum of arc weights over a row of this level fits in 32 bits: true
   // when every graph's total arc weight does (which then holds on every
   // level of its hierarchy: contraction only merges or drops arcs), and on
@@ -305,6 +318,7 @@ struct Level {
     v.aoff = aoff_d.p;
     v.narrow = narrow;
     v.sums31 = sums31;
+    v.deg = deg;
     return v;
   }
 };
@@ -338,8 +352,9 @@ void bounds(int64_t cV, int64_t maxc, int32_t k, double eps, int32_t f, int64_t*
 
 void check_err(int32_t* d_err, cudaStream_t s) {
   int32_t e = 0;
-  SCLAP_CUDA(cudaMemcpyAsync(&e, d_err, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-  stream_sync(s);
+  ReadBack rb(s);
+  rb.add(&e, d_err, 1);
+  rb.wait();
   if (e & DERR_TIMEOUT) throw Error(SCLAP_ETIMEOUT, "a bounded device-side wait ran out");
   if (e & DERR_W_OVERFLOW) throw Error(SCLAP_EOVERFLOW, "coarse edge weight above INT32_MAX");
   if (e & DERR_HASH_FULL) throw Error(SCLAP_EINTERNAL, "hash table full");
@@ -356,8 +371,9 @@ void check_range(const int32_t* a, int64_t n, int64_t lo, int64_t hi, cudaStream
   k_check_range<<<grid_for(n, 256, (int64_t)num_sms() * 8), 256, 0, s>>>(a, n, lo, hi, err.p); SCLAP_NOTE_LAUNCH("k_check_range");
   SCLAP_LAUNCH_CHECK();
   int32_t e = 0;
-  SCLAP_CUDA(cudaMemcpyAsync(&e, err.p, 4, cudaMemcpyDeviceToHost, s));
-  stream_sync(s);
+  ReadBack rb(s);
+  rb.add(&e, err.p, 1);
+  rb.wait();
   if (e) throw Error(SCLAP_EINVAL, std::string(what) + " out of range");
 }
 
@@ -368,31 +384,52 @@ void build_level0(const std::vector<GIn>& gs, struct Level& L, cudaStream_t s);
 // and whether the graph's total arc weight fits in 32 bits (every sum of arc
 // weights met later, at any level of its hierarchy, is at most that total:
 // contraction only merges or drops arcs).
-void validate_level(const Level& L, int B, std::vector<int32_t>& status,
+void validate_level(Level& L, int B, std::vector<int32_t>& status,
                     std::vector<int64_t>& cV, std::vector<int64_t>& maxc,
                     std::vector<char>& narrow, cudaStream_t s,
                     std::vector<char>* sums31 = nullptr, const int32_t* label = nullptr,
                     int64_t* cut2 = nullptr) {
-  DevBuf<int32_t> err(B, s), mx(B, s);
-  DevBuf<unsigned long long> sum(B, s), arcw(B, s);
-  err.zero(); mx.zero(); sum.zero(); arcw.zero();
+  int32_t *err = nullptr, *mx = nullptr;
+  unsigned long long *sum = nullptr, *arcw = nullptr;
+  int64_t* dstat = nullptr;
+  auto layout = [&](Carve& c) {
+    c.take(err, (size_t)B);
+    c.take(mx, (size_t)B);
+    c.take(sum, (size_t)B);
+    c.take(arcw, (size_t)B);
+    c.take(dstat, 3);
+  };
+  Carve cv;
+  layout(cv);
+  DevBuf<char> work(cv.at, s);
+  work.zero();
+  cv = Carve{work.p, 0};
+  layout(cv);
   if (L.N > 0) {
     k_validate_nodes<<<grid_for(L.N, 256 * 4, (int64_t)num_sms() * 8), 256, 0, s>>>(
-        L.rp(), L.nwp(), L.noff_d.p, L.aoff_d.p, B, L.N, err.p, sum.p, mx.p); SCLAP_NOTE_LAUNCH("k_validate_nodes");
+        L.rp(), L.nwp(), L.noff_d.p, L.aoff_d.p, B, L.N, err, sum, mx); SCLAP_NOTE_LAUNCH("k_validate_nodes");
+    level_degree_stats(L.rp(), L.N, B7_MAXDEG, dstat, s);
     if (L.M > 0) {
       (label ? k_validate_arcs<true> : k_validate_arcs<false>)<<<arc_grid(L.M), AT_NT, 0, s>>>(
-          L.rp(), L.colp(), L.ewp(), L.noff_d.p, L.aoff_d.p, B, L.M, err.p, arcw.p, label,
+          L.rp(), L.colp(), L.ewp(), L.noff_d.p, L.aoff_d.p, B, L.M, err, arcw, label,
           reinterpret_cast<unsigned long long*>(cut2)); SCLAP_NOTE_LAUNCH("k_validate_arcs");
     }
     SCLAP_LAUNCH_CHECK();
   }
   std::vector<int32_t> e(B), m(B);
   std::vector<unsigned long long> w(B), aw(B);
-  SCLAP_CUDA(cudaMemcpyAsync(e.data(), err.p, B * 4, cudaMemcpyDeviceToHost, s));
-  SCLAP_CUDA(cudaMemcpyAsync(m.data(), mx.p, B * 4, cudaMemcpyDeviceToHost, s));
-  SCLAP_CUDA(cudaMemcpyAsync(w.data(), sum.p, B * 8, cudaMemcpyDeviceToHost, s));
-  SCLAP_CUDA(cudaMemcpyAsync(aw.data(), arcw.p, B * 8, cudaMemcpyDeviceToHost, s));
-  stream_sync(s);
+  int64_t ds[3] = {0, 0, 0};
+  ReadBack rb(s);
+  rb.add(e.data(), err, B);
+  rb.add(m.data(), mx, B);
+  rb.add(w.data(), sum, B);
+  rb.add(aw.data(), arcw, B);
+  rb.add(ds, dstat, 3);
+  rb.wait();
+  // (of use only when every graph's row offsets are sound)
+  bool sound = true;
+  for (int g = 0; g < B; ++g) sound = sound && !e[g];
+  if (sound) L.deg = DegStats{ds[0], ds[1], ds[2]};
   status.assign(B, SCLAP_OK);
   cV.assign(B, 0);
   maxc.assign(B, 0);
@@ -408,11 +445,10 @@ void validate_level(const Level& L, int B, std::vector<int32_t>& status,
   }
 }
 
-// Validates one device-resident graph (step entry points); returns c(V) and
-// max c(v) or throws.  label, cut2: also adds twice the label's cut (device).
-void validate(const GIn& g, cudaStream_t s, int64_t* cV, int64_t* maxc, bool* narrow = nullptr,
+// Builds and validates the level of one device-resident graph (step entry
+// points); returns c(V) and max c(v) or throws.  label, cut2: also adds twice the label's cut (device).
+void validate(const GIn& g, Level& L, cudaStream_t s, int64_t* cV, int64_t* maxc,
               const int32_t* label = nullptr, int64_t* cut2 = nullptr) {
-  Level L;
   build_level0({g}, L, s);
   std::vector<int32_t> st;
   std::vector<int64_t> a, b;
@@ -423,7 +459,7 @@ void validate(const GIn& g, cudaStream_t s, int64_t* cV, int64_t* maxc, bool* na
   if (st[0] == SCLAP_EOVERFLOW) throw Error(SCLAP_EOVERFLOW, "sum of node weights must be < 2^31");
   *cV = a[0];
   *maxc = b[0];
-  if (narrow) *narrow = nar[0] != 0;
+  L.narrow = nar[0] != 0;
 }
 
 // Builds the level holding the graphs `gs` back to back.  One graph is used
@@ -501,7 +537,7 @@ struct IPIn {
 };
 
 void run_ip(const std::vector<IPIn>& in, const sclap_config& cfg, wgt_t* Wg,
-            std::vector<int32_t>& best, std::vector<int64_t>& ipcut, int64_t* lp_arcs,
+            std::vector<int32_t>& best, std::vector<int64_t>& ipcut, int64_t* d_arcs,
             int32_t* d_err, cudaStream_t s) {
   const int B = (int)in.size();
   const int T = cfg.ip_trials;
@@ -529,9 +565,9 @@ void run_ip(const std::vector<IPIn>& in, const sclap_config& cfg, wgt_t* Wg,
     DevBuf<int64_t> got(ns + 1, s);
     k_gather_at<<<grid_for(ns + 1, 128, 64), 128, 0, s>>>(x->rank.p, Q->noff_d.p, ns + 1, got.p); SCLAP_NOTE_LAUNCH("k_gather_at");
     SCLAP_LAUNCH_CHECK();
-    SCLAP_CUDA(cudaMemcpyAsync(x->rank_at.data(), got.p, (ns + 1) * sizeof(int64_t),
-                               cudaMemcpyDeviceToHost, s));
-    stream_sync(s);
+    ReadBack rb(s);
+    rb.add(x->rank_at.data(), got.p, ns + 1);
+    rb.wait();
     aux.emplace_back(Q, std::move(x));
     return *aux.back().second;
   };
@@ -580,7 +616,20 @@ void run_ip(const std::vector<IPIn>& in, const sclap_config& cfg, wgt_t* Wg,
   }
   Level ip;
   ip.narrow = true;
-  for (const IPIn& x : in) ip.narrow = ip.narrow && x.Q->narrow;
+  // degrees: dropping isolated nodes changes none, so the levels the graphs
+  // come from bound them (every trial may hold each level's hubs)
+  ip.deg = DegStats{0, 0, 0};
+  for (const auto& x : aux) {
+    const DegStats& d = x.first->deg;
+    ip.narrow = ip.narrow && x.first->narrow;
+    if (d.maxdeg < 0 || ip.deg.maxdeg < 0) {
+      ip.deg = DegStats{};
+      continue;
+    }
+    ip.deg.maxdeg = std::max(ip.deg.maxdeg, d.maxdeg);
+    ip.deg.nhubs += T * d.nhubs;
+    ip.deg.hub_slots += T * d.hub_slots;
+  }
   ip.N = noff[S];
   ip.M = aoff[S];
   if (ip.N >= ((int64_t)1 << 31)) throw Error(SCLAP_EINVAL, "trial batch too large");
@@ -623,8 +672,8 @@ void run_ip(const std::vector<IPIn>& in, const sclap_config& cfg, wgt_t* Wg,
 
   GGGArgs ga{};
   ga.row_ptr = ip.row_ptr.p; ga.col = ip.col.p; ga.nw = ip.nw.p;
-  ga.noff = ip.noff_d.p; ga.boff = d_boff.p; ga.nlab = sl.nlab.p; ga.avg = d_avg.p;
-  ga.tkey = sl.seed.p; ga.level = sl.level.p; ga.label = label.p; ga.W = W.p;
+  ga.noff = ip.noff_d.p; ga.boff = d_boff.p; ga.nlab = sl.sp.nlab; ga.avg = d_avg.p;
+  ga.tkey = sl.sp.seed; ga.level = sl.sp.level; ga.label = label.p; ga.W = W.p;
   ga.step = step.p; ga.front = front.p; ga.heavy = heavy.p;
   ga.wfA = wfA.p; ga.wforder = wforder.p;
   ga.nslots = S;
@@ -639,7 +688,7 @@ void run_ip(const std::vector<IPIn>& in, const sclap_config& cfg, wgt_t* Wg,
   run.sub_rounds = cfg.sub_rounds;
   run.graph = cfg.graph_rounds != 0;
   run.use_active = true;
-  *lp_arcs += lp_run(ip.view(), sl.sp, label.p, W.p, K, run, d_err, s);
+  lp_run(ip.view(), sl.sp, label.p, W.p, K, run, d_arcs, d_err, s);
 
   DevBuf<int64_t> cut2(S, s);
   cut2.zero();
@@ -668,9 +717,10 @@ void run_ip(const std::vector<IPIn>& in, const sclap_config& cfg, wgt_t* Wg,
   waterfill_isolated(fill, Wg, Kmax, s);
   best.assign(B, 0);
   ipcut.assign(B, 0);
-  SCLAP_CUDA(cudaMemcpyAsync(best.data(), d_best.p, B * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-  SCLAP_CUDA(cudaMemcpyAsync(ipcut.data(), d_cut.p, B * sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-  stream_sync(s);
+  ReadBack rb(s);
+  rb.add(best.data(), d_best.p, B);
+  rb.add(ipcut.data(), d_cut.p, B);
+  rb.wait();
 }
 
 // ---------------------------------------------------------------------------
@@ -755,8 +805,18 @@ void run_valid_batch(const std::vector<GIn>& gs, const std::vector<int64_t>& cV,
   }
   DevBuf<int32_t> d_err(1, s);
   d_err.zero();
-  int64_t lp_arcs = 0;
+  DevBuf<int64_t> d_arcs(1, s);
+  d_arcs.zero();
   const int sms = num_sms();
+  // LP rounds of each recorded run stay on the device until the end: the
+  // run's parameters, and the slots and the level they are recorded for
+  struct RunRec {
+    std::unique_ptr<Slots> sl;
+    std::vector<char> of;
+    int L;
+    bool cluster;
+  };
+  std::vector<RunRec> recs;
 
   std::vector<std::unique_ptr<Level>> lv;
   lv.push_back(std::move(level0));
@@ -785,7 +845,8 @@ void run_valid_batch(const std::vector<GIn>& gs, const std::vector<int64_t>& cV,
         h_done[g] = coarsening[g] ? 0 : 1;
       }
       std::vector<int64_t> h_loff(cur.noff.begin(), cur.noff.end() - 1);
-      Slots sl(s, B, cur.noff_d.p, h_loff, h_bound, seeds, h_level, h_nlab, h_done);
+      std::unique_ptr<Slots> sl(
+          new Slots(s, B, cur.noff_d.p, h_loff, h_bound, seeds, h_level, h_nlab, h_done));
       DevBuf<int32_t> label(std::max<int64_t>(v.N, 1), s);
       DevBuf<wgt_t> W(std::max<int64_t>(v.N, 1), s);
       k_iota<<<grid_for(v.N, 256, (int64_t)sms * 16), 256, 0, s>>>(label.p, v.N); SCLAP_NOTE_LAUNCH("k_iota");
@@ -799,11 +860,8 @@ void run_valid_batch(const std::vector<GIn>& gs, const std::vector<int64_t>& cV,
       run.graph = cfg.graph_rounds != 0;
       run.use_active = cfg.cluster_active != 0;
       run.rblk = respect ? cur.blk.p : nullptr;
-      lp_arcs += lp_run(v, sl.sp, label.p, W.p, v.N, run, d_err.p, s);
-      const std::vector<int32_t> rr = sl.host_rounds(s);
-      if (record)
-        for (int g = 0; g < B; ++g)
-          if (coarsening[g]) st[g].crounds.push_back(rr[g]);
+      lp_run(v, sl->sp, label.p, W.p, v.N, run, d_arcs.p, d_err.p, s);
+      if (record) recs.push_back(RunRec{std::move(sl), coarsening, L, true});
       if (cfg.ensemble) {
         // ensemble clusterings: clustering j >= 1 of every slot whose ensemble
         // is that large, overlaid onto the labels so far
@@ -827,7 +885,7 @@ void run_valid_batch(const std::vector<GIn>& gs, const std::vector<int64_t>& cV,
             Slots slj(s, B, cur.noff_d.p, h_loff, h_bound, sj, h_level, h_nlab, dj);
             k_iota<<<grid_for(v.N, 256, (int64_t)sms * 16), 256, 0, s>>>(C.p, v.N); SCLAP_NOTE_LAUNCH("k_iota");
             k_w_from_nw<<<grid_for(v.N, 256, (int64_t)sms * 16), 256, 0, s>>>(v.nw, v.N, W.p); SCLAP_NOTE_LAUNCH("k_w_from_nw");
-            lp_arcs += lp_run(v, slj.sp, C.p, W.p, v.N, run, d_err.p, s);
+            lp_run(v, slj.sp, C.p, W.p, v.N, run, d_arcs.p, d_err.p, s);
             part.upload(pj);
             overlay_labels(v, part.p, label.p, C.p, d_err.p, s);
           }
@@ -865,6 +923,7 @@ void run_valid_batch(const std::vector<GIn>& gs, const std::vector<int64_t>& cV,
       nx->gid = std::move(co.gid);
       nx->noff_d = std::move(co.noff_d);
       nx->aoff_d = std::move(co.aoff_d);
+      nx->deg = co.deg;
       nx->noff = co.noff;
       nx->aoff = co.aoff;
       if (respect) {
@@ -908,7 +967,7 @@ void run_valid_batch(const std::vector<GIn>& gs, const std::vector<int64_t>& cV,
     }
     std::vector<int32_t> best;
     std::vector<int64_t> ipcut;
-    run_ip(in, cfg, Wg.p, best, ipcut, &lp_arcs, d_err.p, s);
+    run_ip(in, cfg, Wg.p, best, ipcut, d_arcs.p, d_err.p, s);
     for (int g = 0; g < B; ++g) {
       res[g].st.ip_best_trial = best[g];
       res[g].st.ip_cut = ipcut[g];
@@ -944,7 +1003,8 @@ void run_valid_batch(const std::vector<GIn>& gs, const std::vector<int64_t>& cV,
         any = any || !h_done[g];
       }
       if (!any) continue;
-      Slots sl(s, B, F.noff_d.p, h_boff, h_Lmax, seeds, h_level, h_k, h_done);
+      std::unique_ptr<Slots> sl(
+          new Slots(s, B, F.noff_d.p, h_boff, h_Lmax, seeds, h_level, h_k, h_done));
       LPRun run;
       run.mode = MODE_REFINE;
       run.phase = PH_REFINE;
@@ -952,11 +1012,11 @@ void run_valid_batch(const std::vector<GIn>& gs, const std::vector<int64_t>& cV,
       run.sub_rounds = cfg.sub_rounds;
       run.graph = cfg.graph_rounds != 0;
       run.use_active = true;
-      lp_arcs += lp_run(F.view(), sl.sp, F.blk.p, Wg.p, Ktot, run, d_err.p, s);
+      lp_run(F.view(), sl->sp, F.blk.p, Wg.p, Ktot, run, d_arcs.p, d_err.p, s);
       if (record) {
-        const std::vector<int32_t> rr = sl.host_rounds(s);
-        for (int g = 0; g < B; ++g)
-          if (q[g] > L) st[g].rrounds[L] = rr[g];
+        std::vector<char> of(B);
+        for (int g = 0; g < B; ++g) of[g] = q[g] > L;
+        recs.push_back(RunRec{std::move(sl), std::move(of), L, false});
       }
     }
     lv.resize(1);
@@ -974,7 +1034,7 @@ void run_valid_batch(const std::vector<GIn>& gs, const std::vector<int64_t>& cV,
     run.sub_rounds = cfg.sub_rounds;
     run.graph = cfg.graph_rounds != 0;
     run.stop_rule = false;
-    lp_arcs += lp_run(F0.view(), sl.sp, F0.blk.p, Wg.p, Ktot, run, d_err.p, s);
+    lp_run(F0.view(), sl.sp, F0.blk.p, Wg.p, Ktot, run, d_arcs.p, d_err.p, s);
   };
   {
     std::vector<int32_t> q(B);
@@ -1019,9 +1079,20 @@ void run_valid_batch(const std::vector<GIn>& gs, const std::vector<int64_t>& cV,
   SCLAP_LAUNCH_CHECK();
   std::vector<int64_t> h_cut2(B);
   std::vector<wgt_t> h_W(Ktot);
-  SCLAP_CUDA(cudaMemcpyAsync(h_cut2.data(), cut2.p, B * sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-  SCLAP_CUDA(cudaMemcpyAsync(h_W.data(), Wg.p, Ktot * sizeof(wgt_t), cudaMemcpyDeviceToHost, s));
-  stream_sync(s);
+  int64_t lp_arcs = 0;
+  std::vector<std::vector<int32_t>> rr(recs.size(), std::vector<int32_t>(B));
+  ReadBack rb(s);
+  rb.add(h_cut2.data(), cut2.p, B);
+  rb.add(h_W.data(), Wg.p, Ktot);
+  rb.add(&lp_arcs, d_arcs.p, 1);
+  for (size_t j = 0; j < recs.size(); ++j) rb.add(rr[j].data(), recs[j].sl->sp.rounds, B);
+  rb.wait();
+  for (size_t j = 0; j < recs.size(); ++j)
+    for (int g = 0; g < B; ++g) {
+      if (!recs[j].of[g]) continue;
+      if (recs[j].cluster) st[g].crounds.push_back(rr[j][g]);
+      else st[g].rrounds[recs[j].L] = rr[j][g];
+    }
   for (int g = 0; g < B; ++g) {
     GOut& o = res[g];
     o.cut = h_cut2[g] / 2;
@@ -1046,6 +1117,12 @@ void run_valid_batch(const std::vector<GIn>& gs, const std::vector<int64_t>& cV,
 // ---------------------------------------------------------------------------
 // Helpers for the C ABI.
 // ---------------------------------------------------------------------------
+void read_rounds(const Slots& sl, int32_t* rounds, cudaStream_t s) {
+  ReadBack rb(s);
+  rb.add(rounds, sl.sp.rounds, 1);
+  rb.wait();
+}
+
 template <class F>
 int guarded(F&& f) {
   try {
@@ -1054,12 +1131,15 @@ int guarded(F&& f) {
     g_last_error.clear();
     return SCLAP_OK;
   } catch (const Error& e) {
+    host_ring().give_up();
     g_last_error = e.what();
     return e.code;
   } catch (const std::exception& e) {
+    host_ring().give_up();
     g_last_error = e.what();
     return SCLAP_EINTERNAL;
   } catch (...) {
+    host_ring().give_up();
     g_last_error = "unknown exception";
     return SCLAP_EINTERNAL;
   }
@@ -1076,8 +1156,9 @@ void check_args(int64_t n, const void* row_ptr, const void* col, int32_t k, doub
 
 int64_t device_arcs(const int64_t* row_ptr, int64_t n, cudaStream_t s) {
   int64_t m = 0;
-  SCLAP_CUDA(cudaMemcpyAsync(&m, row_ptr + n, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-  stream_sync(s);
+  ReadBack rb(s);
+  rb.add(&m, row_ptr + n, 1);
+  rb.wait();
   if (m < 0 || m >= ((int64_t)1 << 40)) throw Error(SCLAP_ECSR, "row_ptr[n] out of range");
   return m;
 }
@@ -1097,8 +1178,9 @@ std::vector<int64_t> device_arcs_many(const std::vector<const int64_t*>& ends, c
   DevBuf<int64_t> out(n, s);
   k_read_ends<<<grid_for(n, 128, 64), 128, 0, s>>>(d.p, n, out.p); SCLAP_NOTE_LAUNCH("k_read_ends");
   SCLAP_LAUNCH_CHECK();
-  SCLAP_CUDA(cudaMemcpyAsync(m.data(), out.p, n * sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-  stream_sync(s);
+  ReadBack rb(s);
+  rb.add(m.data(), out.p, n);
+  rb.wait();
   for (int64_t x : m)
     if (x < 0 || x >= ((int64_t)1 << 40)) throw Error(SCLAP_ECSR, "row_ptr[n] out of range");
   return m;
@@ -1195,12 +1277,6 @@ void parallel_copy(const std::vector<Piece>& pieces) {
   for (int t = 1; t < nt; ++t) th.emplace_back(run, total * t / nt, total * (t + 1) / nt);
   run(0, total / nt);
   for (auto& x : th) x.join();
-}
-
-// A one-slot level holding a copy of a device graph (step entry points).
-void single_level(const GIn& g, Level& L, cudaStream_t s) {
-  std::vector<GIn> v{g};
-  build_level0(v, L, s);
 }
 
 void fill_stats(sclap_stats* dst, const GOut& o) {
@@ -1467,13 +1543,10 @@ int sclap_lp_round(int32_t mode, int64_t n, const int64_t* row_ptr, const int32_
     g.ew = edge_w;
     check_col(g.col, g.m);
     int64_t cV, maxc;
-    bool nar = false;
-    validate(g, s, &cV, &maxc, &nar);
+    Level L;
+    validate(g, L, s, &cV, &maxc);
     if (mode == 0 && nlabels < n) throw Error(SCLAP_EINVAL, "clustering needs nlabels >= n");
     check_range(label, n, 0, nlabels, s, "label");
-    Level L;
-    single_level(g, L, s);
-    L.narrow = nar;
     Slots sl(s, 1, L.noff_d.p, {0}, {bound}, {rkey}, {0}, {(int32_t)nlabels}, {0});
     LPRun run;
     run.mode = mode == 0 ? MODE_CLUSTER : MODE_REFINE;
@@ -1483,15 +1556,18 @@ int sclap_lp_round(int32_t mode, int64_t n, const int64_t* row_ptr, const int32_
     run.raw_key = true;
     DevBuf<int32_t> d_err(1, s);
     d_err.zero();
+    DevBuf<int64_t> arcs(1, s);
+    arcs.zero();
     DevBuf<wgt_t> W32(nlabels, s);
     k_narrow<<<grid_for(nlabels, 256, 1024), 256, 0, s>>>(W, nlabels, W32.p, d_err.p); SCLAP_NOTE_LAUNCH("k_narrow");
     check_err(d_err.p, s);
-    lp_run(L.view(), sl.sp, label, W32.p, nlabels, run, d_err.p, s, active_cur, active_next);
+    lp_run(L.view(), sl.sp, label, W32.p, nlabels, run, arcs.p, d_err.p, s, active_cur, active_next);
     k_widen<<<grid_for(nlabels, 256, 1024), 256, 0, s>>>(W32.p, nlabels, W); SCLAP_NOTE_LAUNCH("k_widen");
     check_err(d_err.p, s);
     int64_t mv = 0;
-    SCLAP_CUDA(cudaMemcpyAsync(&mv, sl.moved.p, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-    stream_sync(s);
+    ReadBack rb(s);
+    rb.add(&mv, sl.sp.moved, 1);
+    rb.wait();
     if (moved_out) *moved_out = mv;
   });
 }
@@ -1509,11 +1585,8 @@ int sclap_cluster(int64_t n, const int64_t* row_ptr, const int32_t* col, const i
     g.ew = edge_w;
     check_col(g.col, g.m);
     int64_t cV, maxc;
-    bool nar = false;
-    validate(g, s, &cV, &maxc, &nar);
     Level L;
-    single_level(g, L, s);
-    L.narrow = nar;
+    validate(g, L, s, &cV, &maxc);
     Slots sl(s, 1, L.noff_d.p, {0}, {U}, {seed}, {level}, {0}, {0});
     DevBuf<wgt_t> W(n, s);
     k_iota<<<grid_for(n, 256, (int64_t)num_sms() * 16), 256, 0, s>>>(label_out, n); SCLAP_NOTE_LAUNCH("k_iota");
@@ -1527,9 +1600,11 @@ int sclap_cluster(int64_t n, const int64_t* row_ptr, const int32_t* col, const i
     run.use_active = c.cluster_active != 0;
     DevBuf<int32_t> d_err(1, s);
     d_err.zero();
-    lp_run(L.view(), sl.sp, label_out, W.p, n, run, d_err.p, s);
+    DevBuf<int64_t> arcs(1, s);
+    arcs.zero();
+    lp_run(L.view(), sl.sp, label_out, W.p, n, run, arcs.p, d_err.p, s);
     check_err(d_err.p, s);
-    if (rounds_out) *rounds_out = sl.host_rounds(s)[0];
+    if (rounds_out) read_rounds(sl, rounds_out, s);
   });
 }
 
@@ -1548,17 +1623,16 @@ int sclap_cluster_hierarchy(int64_t n, const int64_t* row_ptr, const int32_t* co
     g.ew = edge_w;
     check_col(g.col, g.m);
     int64_t cV, maxc;
-    bool nar = false;
-    validate(g, s, &cV, &maxc, &nar);
     const int sms = num_sms();
     std::unique_ptr<Level> cur(new Level());
-    single_level(g, *cur, s);
-    cur->narrow = nar;
+    validate(g, *cur, s, &cV, &maxc);
     k_iota<<<grid_for(n, 256, (int64_t)sms * 16), 256, 0, s>>>(comm_out, n); SCLAP_NOTE_LAUNCH("k_iota");
     int32_t levels = 0;
     if (level_n_out && cap > 0) level_n_out[0] = n;
     DevBuf<int32_t> d_err(1, s);
     d_err.zero();
+    DevBuf<int64_t> arcs(1, s);
+    arcs.zero();
     while (cur->N > stop_nodes && levels + 1 < c.max_levels) {
       const LevelView v = cur->view();
       Slots sl(s, 1, cur->noff_d.p, {0}, {U}, {seed}, {levels}, {0}, {0});
@@ -1573,7 +1647,7 @@ int sclap_cluster_hierarchy(int64_t n, const int64_t* row_ptr, const int32_t* co
       run.sub_rounds = c.sub_rounds;
       run.graph = c.graph_rounds != 0;
       run.use_active = c.cluster_active != 0;
-      lp_run(v, sl.sp, label.p, W.p, v.N, run, d_err.p, s);
+      lp_run(v, sl.sp, label.p, W.p, v.N, run, arcs.p, d_err.p, s);
       ContractWork cw;
       std::vector<int64_t> nc;
       contract_rank(v, cur->noff, label.p, cw, nc, s);
@@ -1593,6 +1667,7 @@ int sclap_cluster_hierarchy(int64_t n, const int64_t* row_ptr, const int32_t* co
       nx->gid = std::move(co.gid);
       nx->noff_d = std::move(co.noff_d);
       nx->aoff_d = std::move(co.aoff_d);
+      nx->deg = co.deg;
       nx->noff = co.noff;
       nx->aoff = co.aoff;
       cur = std::move(nx);
@@ -1619,12 +1694,9 @@ int sclap_contract(int64_t n, const int64_t* row_ptr, const int32_t* col, const 
     g.ew = edge_w;
     check_col(g.col, g.m);
     int64_t cV, maxc;
-    bool nar = false;
-    validate(g, s, &cV, &maxc, &nar);
-    check_range(label, n, 0, n, s, "label");
     Level L;
-    single_level(g, L, s);
-    L.narrow = nar;
+    validate(g, L, s, &cV, &maxc);
+    check_range(label, n, 0, n, s, "label");
     ContractWork w;
     std::vector<int64_t> nc;
     contract_rank(L.view(), L.noff, label, w, nc, s);
@@ -1661,11 +1733,8 @@ int sclap_initial_partition(int64_t n, const int64_t* row_ptr, const int32_t* co
     g.ew = edge_w;
     check_col(g.col, g.m);
     int64_t cV, maxc;
-    bool nar = false;
-    validate(g, s, &cV, &maxc, &nar);
     Level L;
-    single_level(g, L, s);
-    L.narrow = nar;
+    validate(g, L, s, &cV, &maxc);
     DevBuf<wgt_t> Wg(k, s);
     DevBuf<int32_t> d_err(1, s);
     d_err.zero();
@@ -1693,12 +1762,9 @@ int sclap_refine(int64_t n, const int64_t* row_ptr, const int32_t* col, const in
     g.ew = edge_w;
     check_col(g.col, g.m);
     int64_t cV, maxc;
-    bool nar = false;
-    validate(g, s, &cV, &maxc, &nar);
-    check_range(block, n, 0, k, s, "block");
     Level L;
-    single_level(g, L, s);
-    L.narrow = nar;
+    validate(g, L, s, &cV, &maxc);
+    check_range(block, n, 0, k, s, "block");
     DevBuf<wgt_t> W(k, s);
     W.zero();
     block_weights(block, L.nwp(), n, W.p, k, s);
@@ -1712,9 +1778,11 @@ int sclap_refine(int64_t n, const int64_t* row_ptr, const int32_t* col, const in
     run.use_active = true;
     DevBuf<int32_t> d_err(1, s);
     d_err.zero();
-    lp_run(L.view(), sl.sp, block, W.p, k, run, d_err.p, s);
+    DevBuf<int64_t> arcs(1, s);
+    arcs.zero();
+    lp_run(L.view(), sl.sp, block, W.p, k, run, arcs.p, d_err.p, s);
     check_err(d_err.p, s);
-    if (rounds_out) *rounds_out = sl.host_rounds(s)[0];
+    if (rounds_out) read_rounds(sl, rounds_out, s);
   });
 }
 
@@ -1729,10 +1797,12 @@ int sclap_cut(int64_t n, const int64_t* row_ptr, const int32_t* col, const int32
     int64_t cV, maxc;
     DevBuf<int64_t> cut2(1, s);
     cut2.zero();
-    validate(g, s, &cV, &maxc, nullptr, block, cut2.p);
+    Level L;
+    validate(g, L, s, &cV, &maxc, block, cut2.p);
     int64_t c2 = 0;
-    SCLAP_CUDA(cudaMemcpyAsync(&c2, cut2.p, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-    stream_sync(s);
+    ReadBack rb(s);
+    rb.add(&c2, cut2.p, 1);
+    rb.wait();
     if (cut_out) *cut_out = c2 / 2;
   });
 }

@@ -48,6 +48,8 @@ __global__ void k_replicate(const CopyTask* __restrict__ tasks, int64_t* __restr
   }
 }
 
+__global__ void k_set_i64(int64_t* p, int64_t v) { *p = v; }
+
 // A later copy of an already copied segment: nodes [0, nd) and arcs
 // [0, m) of the first copy (at tn0 / ta0) to dn0 / da0, row offsets shifted
 // by the arc offset difference and neighbour ids by the node offset
@@ -1088,7 +1090,6 @@ void waterfill_isolated(const std::vector<FillTask>& tasks, wgt_t* Wg, int64_t K
     k_wf_assign<<<grid, 256, 0, s>>>(d.p + t0, Wg, order.p, A.p); SCLAP_NOTE_LAUNCH("k_wf_assign");
   }
   SCLAP_LAUNCH_CHECK();
-  stream_sync(s);   // task array freed on return
 }
 
 void ip_replicate(const std::vector<CopyTask>& tasks, int64_t* row_ptr, int32_t* col,
@@ -1135,15 +1136,13 @@ void ip_replicate(const std::vector<CopyTask>& tasks, int64_t* row_ptr, int32_t*
       k_replicate_from<<<grid, 256, 0, s>>>(dl.p + t0, row_ptr, col, ew, nw); SCLAP_NOTE_LAUNCH("k_replicate_from");
     }
   }
-  int64_t endv = M_total;
   int64_t Ntot = 0;
   for (const auto& t : tasks) {
     const int64_t nd = t.rank ? 0 : t.n;   // renumbered tasks: caller passes dst end below
     Ntot = std::max(Ntot, t.dst_n0 + nd);
   }
   if (N_total_override >= 0) Ntot = N_total_override;
-  SCLAP_CUDA(cudaMemcpyAsync(row_ptr + Ntot, &endv, sizeof(int64_t), cudaMemcpyHostToDevice, s));
-  stream_sync(s);   // endv lives on the host stack
+  k_set_i64<<<1, 1, 0, s>>>(row_ptr + Ntot, M_total); SCLAP_NOTE_LAUNCH("k_set_i64");
   SCLAP_LAUNCH_CHECK();
 }
 
@@ -1236,7 +1235,6 @@ void ip_select_copy(const std::vector<SelectTask>& tasks, const int64_t* cut2,
     k_copy_best<<<grid, 256, 0, s>>>(d.p + t0, take.p + t0, ip_noff, ip_boff, ip_label, ip_W, Wg); SCLAP_NOTE_LAUNCH("k_copy_best");
   }
   SCLAP_LAUNCH_CHECK();
-  stream_sync(s);   // the task array is freed on return
 }
 
 void project(const int32_t* cmap, const int32_t* coarse_blk, int32_t* fine_blk, int64_t N,

@@ -2154,16 +2154,6 @@ __global__ void __launch_bounds__(ADM_NT) k_apply(LPArgs a, int32_t sub) {
   apply_flush(a, h);
 }
 
-// Largest label count over the slots (local search: the largest k).
-__global__ void k_max_labels(const int32_t* __restrict__ nlab, int32_t nslots, int64_t* out) {
-  int32_t m = 0;
-  for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < nslots; i += gridDim.x * blockDim.x)
-    m = max(m, nlab[i]);
-  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if ((threadIdx.x & 31) == 0 && m) atomicMax(reinterpret_cast<unsigned long long*>(out),
-                                             (unsigned long long)m);
-}
-
 // The queued chunks of moved long rows of colour class `sub`: one CTA per
 // chunk marks its heads active for the next round.
 __global__ void __launch_bounds__(256) k_mark_rows(LPArgs a, int32_t sub) {
@@ -2725,47 +2715,97 @@ std::string timeline_dump() {
 // levels (8.6 M nodes) no change.
 constexpr int64_t PR_MAX_N = 1250000, PR_MAX_M = 16000000;
 
-int64_t lp_run(const LevelView& lv, const SlotParams& sp, int32_t* label, wgt_t* W,
-               int64_t Wsize, const LPRun& run, int32_t* d_err, cudaStream_t s,
-               const uint8_t* active_init, uint8_t* active_next_out) {
+void lp_run(const LevelView& lv, const SlotParams& sp, int32_t* label, wgt_t* W, int64_t Wsize,
+            const LPRun& run, int64_t* d_arcs, int32_t* d_err, cudaStream_t s,
+            const uint8_t* active_init, uint8_t* active_next_out) {
   const int64_t N = lv.N;
-  if (N == 0 || run.rounds <= 0) return 0;
+  if (N == 0 || run.rounds <= 0) return;
   const int S = run.sub_rounds;
   const int nkeys = S * NB;
   const int sms = num_sms();
-
-  DevBuf<uint64_t> in_w((size_t)Wsize, s);
-  DevBuf<int64_t> ovf_base((size_t)Wsize, s);
-  DevBuf<int32_t> ovf_cnt((size_t)Wsize, s);
-  in_w.zero(); ovf_cnt.zero();
-  DevBuf<int4> rec(N, s);
-  DevBuf<longlong2> rec2(N, s);
-  DevBuf<int32_t> prop_t(N, s), grp(N, s), seg_g(N, s), seg_cnt(N, s), stage(N, s);
-  DevBuf<wgt_t> prop_w(N, s);
-  DevBuf<uint64_t> prop_key(N, s), ent_key(N, s);
-  DevBuf<int8_t> adm(N, s);
-  DevBuf<int64_t> seg_base(N, s), seg_thr(N, s);
-  DevBuf<int32_t> ent_v(N, s), ent_w(N, s), ent_i(N, s);
-  DevBuf<uint64_t> sel_k0(N, s), sel_k1(N, s);
-  DevBuf<int32_t> sel_v0(N, s), sel_v1(N, s), sel_w0(N, s), sel_w1(N, s);
-  DevBuf<int64_t> ctr(8, s);
-  ctr.zero();
-  DevBuf<GridSync> gsync(1, s);
-  gsync.zero();
-  DevBuf<int32_t> bcnt(nkeys, s), bfill(nkeys, s);
-  DevBuf<int64_t> boff(nkeys + 1, s), arcs(1, s), karcs(nkeys, s);
-  DevBuf<int32_t> flags(1, s);
-  DevBuf<int16_t> nkey(N, s);
-  bfill.zero(); arcs.zero();
-
   const bool track_active = run.use_active || active_init != nullptr || active_next_out != nullptr;
-  DevBuf<uint8_t> act_a, act_b;
+
+  // The level's degrees decide which propose launches can ever have work
+  // (and size the hub tables): known from the level's construction, else one
+  // read-back per run; none per round.
+  DegStats deg = lv.deg;
+  if (deg.maxdeg < 0) {
+    DevBuf<int64_t> dstat(3, s);
+    dstat.zero();
+    level_degree_stats(lv.row_ptr, N, B7_MAXDEG, dstat.p, s);
+    int64_t h[3];
+    ReadBack rb(s);
+    rb.add(h, dstat.p, 3);
+    rb.wait();
+    deg = DegStats{h[0], h[1], h[2]};
+  }
+  const int64_t maxdeg = deg.maxdeg, nhubs = deg.nhubs, hub_slots = deg.hub_slots;
+  const Tuning tu = tuning_get();
+  const bool prof = profile().enabled.load();
+  const bool timeline = profile().timeline.load(std::memory_order_relaxed);
+  const bool persistent = !run.graph && !prof && tu.concurrent && tu.pdl && !tu.fused_admission &&
+                          maxdeg <= B7_MAXDEG && N <= PR_MAX_N && lv.M <= PR_MAX_M;
+
+  // The run's working memory is one allocation; what starts zero comes first.
+  LPArgs a{};
+  RoundsArgs q{};
+  GridSync* gsync = nullptr;
+  int32_t* rstate = nullptr;            // round index, live slots, continue flag
+  auto layout = [&](Carve& c) {
+    c.take(a.in_w, (size_t)(persistent ? 2 * Wsize : Wsize));
+    c.take(a.ovf_cnt, (size_t)Wsize);
+    c.take(a.ctr, 8);
+    c.take(gsync, 1);
+    c.take(rstate, 3);
+    c.take(a.bcnt, (size_t)nkeys);
+    c.take(a.bfill, (size_t)nkeys);
+    c.take(q.bar, 1);
+    c.take(q.live, 2);
+    c.take(a.mqn, (size_t)S);
+    if (track_active) c.take(a.act[1], (size_t)N);
+    // read back together each round: bucket offsets, arcs per key, flags
+    c.take(a.boff, (size_t)(2 * nkeys + 2));
+    const size_t zero_end = c.at;
+    if (track_active) c.take(a.act[0], (size_t)N);
+    c.take(a.ovf_base, (size_t)Wsize);
+    c.take(a.rec, (size_t)N);
+    c.take(a.rec2, (size_t)N);
+    for (int32_t** x : {&a.prop_t, &a.grp, &a.seg_g, &a.seg_cnt, &a.stage, &a.prop_w, &a.ent_v,
+                        &a.ent_w, &a.ent_i, &a.sel_v[0], &a.sel_v[1], &a.sel_w[0], &a.sel_w[1]})
+      c.take(*x, (size_t)N);
+    for (uint64_t** x : {&a.prop_key, &a.ent_key, &a.sel_key[0], &a.sel_key[1]})
+      c.take(*x, (size_t)N);
+    c.take(a.seg_base, (size_t)N);
+    c.take(a.seg_thr, (size_t)N);
+    c.take(a.adm, (size_t)N);
+    c.take(a.nkey, (size_t)N);
+    if (persistent && track_active && maxdeg > PR_MARK) {
+      // at most one chunk per node of degree above PR_MARK, and one per
+      // PR_MARK_CH arcs
+      c.take(a.mq, (size_t)(std::min<int64_t>(N, lv.M / PR_MARK) + lv.M / PR_MARK_CH + 2));
+    } else if (!persistent && track_active && maxdeg > MARK_CH) {
+      // (at most arcs / 4096 chunks plus one per such row, per class)
+      c.take(a.mq, (size_t)(2 * (lv.M / MARK_CH) + 2));
+    }
+    return zero_end;
+  };
+  Carve c;
+  layout(c);
+  DevBuf<char> work(c.at, s);
+  c = Carve{work.p, 0};
+  const size_t zero_end = layout(c);
+  SCLAP_CUDA(cudaMemsetAsync(work.p, 0, zero_end, s));
+  a.karcs = a.boff + nkeys + 1;
+  a.flags = reinterpret_cast<int32_t*>(a.boff + 2 * nkeys + 1);
+  if (!a.mq) a.mqn = nullptr;
+  if (a.mq) {
+    a.mark_big = persistent ? PR_MARK : MARK_CH;
+    a.mark_ch = persistent ? PR_MARK_CH : MARK_CH;
+  }
   if (track_active) {
-    act_a.alloc(N, s);
-    act_b.alloc(N, s);
-    if (active_init) SCLAP_CUDA(cudaMemcpyAsync(act_a.p, active_init, N, cudaMemcpyDeviceToDevice, s));
-    else act_a.fill_bytes(1);
-    act_b.zero();
+    if (active_init)
+      SCLAP_CUDA(cudaMemcpyAsync(a.act[0], active_init, N, cudaMemcpyDeviceToDevice, s));
+    else SCLAP_CUDA(cudaMemsetAsync(a.act[0], 1, (size_t)N, s));
   }
 
   // Global hash tables of hub nodes: a region per hub of a colour class,
@@ -2792,7 +2832,6 @@ int64_t lp_run(const LevelView& lv, const SlotParams& sp, int32_t* label, wgt_t*
     pool_slots = slots;
   };
 
-  LPArgs a{};
   a.row_ptr = lv.row_ptr; a.col = lv.col; a.ew = lv.ew; a.nw = lv.nw; a.gid = lv.gid;
   a.narrow = lv.narrow ? 1 : 0;
   a.arcs32 = lv.M < ((int64_t)1 << 32) ? 1 : 0;
@@ -2801,58 +2840,28 @@ int64_t lp_run(const LevelView& lv, const SlotParams& sp, int32_t* label, wgt_t*
   a.nlabels = Wsize;
   a.noff = sp.noff; a.loff = sp.loff; a.bound = sp.bound; a.rkey = sp.rkey; a.nlab = sp.nlab;
   a.done = sp.done; a.moved = sp.moved; a.rounds = sp.rounds;
-  a.label = label; a.W = W; a.in_w = in_w.p; a.mode = run.mode; a.S = S;
-  a.rec = rec.p; a.rec2 = rec2.p; a.prop_t = prop_t.p; a.prop_key = prop_key.p;
-  a.prop_w = prop_w.p; a.adm = adm.p; a.stage = stage.p;
-  a.grp = grp.p; a.ovf_cnt = ovf_cnt.p; a.ovf_base = ovf_base.p;
-  a.ctr = ctr.p; a.seg_g = seg_g.p; a.seg_base = seg_base.p; a.seg_cnt = seg_cnt.p;
-  a.seg_thr = seg_thr.p; a.ent_key = ent_key.p; a.ent_v = ent_v.p; a.ent_w = ent_w.p;
-  a.ent_i = ent_i.p; a.bcnt = bcnt.p;
-  a.sel_key[0] = sel_k0.p; a.sel_key[1] = sel_k1.p;
-  a.sel_v[0] = sel_v0.p; a.sel_v[1] = sel_v1.p;
-  a.sel_w[0] = sel_w0.p; a.sel_w[1] = sel_w1.p; a.bfill = bfill.p; a.boff = boff.p; a.arcs = arcs.p;
-  a.karcs = karcs.p;
-  a.flags = flags.p;
-  a.nkey = nkey.p;
+  a.label = label; a.W = W; a.mode = run.mode; a.S = S;
+  a.arcs = d_arcs;
   a.err = d_err;
   a.wait_limit = wait_limit();
   a.probe_limit = probe_limit();
-
-  // ---- round-invariant setup ---------------------------------------------
-  DevBuf<int32_t> rstate(3, s);        // round index, live slots, continue flag
-  rstate.zero();
-  a.rnd = rstate.p;
-  a.live = rstate.p + 1;
-  int32_t* const d_cont = rstate.p + 2;
+  a.rnd = rstate;
+  a.live = rstate + 1;
+  int32_t* const d_cont = rstate + 2;
   a.rounds_max = run.rounds;
   a.stop_rule = run.stop_rule ? 1 : 0;
   a.rblk = run.mode == MODE_CLUSTER ? run.rblk : nullptr;
-  a.act[0] = track_active ? act_a.p : nullptr;
-  a.act[1] = track_active ? act_b.p : nullptr;
-
-  // The level's degrees decide which propose launches can ever have work
-  // (and size the hub tables): one read-back per run, none per round.
-  DevBuf<int64_t> dstat(4, s);
-  dstat.zero();
-  level_degree_stats(lv.row_ptr, N, B7_MAXDEG, dstat.p, s);
-  if (run.mode != MODE_CLUSTER && sp.nslots > 0) {
-    k_max_labels<<<grid_for(sp.nslots, 256, 64), 256, 0, s>>>(sp.nlab, sp.nslots, dstat.p + 3); SCLAP_NOTE_LAUNCH("k_max_labels");
-  }
-  int64_t hstat[4] = {0, 0, 0, 0};
-  SCLAP_CUDA(cudaMemcpyAsync(hstat, dstat.p, sizeof(hstat), cudaMemcpyDeviceToHost, s));
-  stream_sync(s);
-  const int64_t maxdeg = hstat[0], nhubs = hstat[1], hub_slots = hstat[2];
-  // local search where every slot has at most B5_SLOTS labels: every node of
-  // the CTA buckets indexes its block directly, so buckets 6 and 7 need only
-  // a B5_SLOTS-entry shared table (more CTAs per SM) instead of one sized
-  // for hashing 2 x degree labels
-  const bool compact_blk = run.mode != MODE_CLUSTER && hstat[3] > 0 && hstat[3] <= B5_SLOTS;
   const bool refine = run.mode != MODE_CLUSTER;
-  const Tuning tu = tuning_get();
-  const bool prof = profile().enabled.load();
-  const bool timeline = profile().timeline.load(std::memory_order_relaxed);
-  if (!run.graph && !prof && tu.concurrent && tu.pdl && !tu.fused_admission &&
-      maxdeg <= B7_MAXDEG && N <= PR_MAX_N && lv.M <= PR_MAX_M) {
+  // flags of the next round out, once the run's last round is known
+  auto write_active = [&] {
+    if (!active_next_out || !track_active) return;
+    int32_t hr = 0;
+    ReadBack rb(s);
+    rb.add(&hr, a.rnd, 1);
+    rb.wait();
+    SCLAP_CUDA(cudaMemcpyAsync(active_next_out, a.act[hr & 1], N, cudaMemcpyDeviceToDevice, s));
+  };
+  if (persistent) {
     int64_t tcap = PR_MIN_TCAP;
     while (tcap < 2 * maxdeg) tcap <<= 1;
     static std::once_flag pr_once;
@@ -2860,48 +2869,24 @@ int64_t lp_run(const LevelView& lv, const SlotParams& sp, int32_t* label, wgt_t*
       SCLAP_CUDA(cudaFuncSetAttribute(k_lp_rounds, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)pr_smem(B7_SLOTS)));
     });
-    DevBuf<uint32_t> pr(4, s);             // barrier, live counters
-    pr.zero();
-    bcnt.zero();
-    flags.zero();
-    DevBuf<uint64_t> in2((size_t)(2 * Wsize), s);
-    in2.zero();
-    a.in_w = in2.p;
-    DevBuf<longlong2> mq;
-    DevBuf<int32_t> mqn;
-    if (track_active && maxdeg > PR_MARK) {
-      // at most one chunk per node of degree above PR_MARK, and one per
-      // PR_MARK_CH arcs
-      mq.alloc((size_t)(std::min<int64_t>(N, lv.M / PR_MARK) + lv.M / PR_MARK_CH + 2), s);
-      mqn.alloc(1, s);
-      mqn.zero();
-      a.mark_big = PR_MARK;
-      a.mark_ch = PR_MARK_CH;
-      a.mq = mq.p;
-      a.mqn = mqn.p;
-    }
-    RoundsArgs q{};
     q.nslots = sp.nslots;
     q.phase = run.phase;
     q.raw_key = run.raw_key ? 1 : 0;
     q.tcap = (int32_t)tcap;
     q.seed = sp.seed;
     q.level = sp.level;
-    q.bar = pr.p;
-    q.live = reinterpret_cast<int32_t*>(pr.p + 1);
     const int64_t want = std::max<int64_t>(N / 128, lv.M / 2048);
     const unsigned grid = (unsigned)std::max<int64_t>(8, std::min<int64_t>(sms, want));
     launch_coop(k_lp_rounds, grid, PR_NT, pr_smem(tcap), s, a, q); SCLAP_NOTE_LAUNCH("k_lp_rounds");
     SCLAP_LAUNCH_CHECK();
-    int32_t hr = 0;
-    int64_t h_arcs = 0;
-    SCLAP_CUDA(cudaMemcpyAsync(&hr, a.rnd, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-    SCLAP_CUDA(cudaMemcpyAsync(&h_arcs, arcs.p, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-    stream_sync(s);
-    if (active_next_out && track_active)
-      SCLAP_CUDA(cudaMemcpyAsync(active_next_out, a.act[hr & 1], N, cudaMemcpyDeviceToDevice, s));
-    return h_arcs;
+    write_active();
+    return;
   }
+  // local search where every slot has at most B5_SLOTS labels: every node of
+  // the CTA buckets indexes its block directly, so buckets 6 and 7 need only
+  // a B5_SLOTS-entry shared table (more CTAs per SM) instead of one sized
+  // for hashing 2 x degree labels
+  const bool compact_blk = refine && sp.max_nlab > 0 && sp.max_nlab <= B5_SLOTS;
   const int nsb = tu.small_max_deg >= 16 ? 3 : 2;   // buckets of the thread-per-node launch
   const bool need[NB] = {true, true, true, refine || maxdeg > (nsb == 3 ? 16 : 8), false,
                          maxdeg > B4_MAXDEG, maxdeg > B5_MAXDEG, maxdeg > B6_MAXDEG,
@@ -2923,18 +2908,6 @@ int64_t lp_run(const LevelView& lv, const SlotParams& sp, int32_t* label, wgt_t*
     hs.pcd = hub_pcd.p;
     hs.poc = hub_poc.p;
     if (run.graph) ensure_pool(hub_slots);
-  }
-  // moved rows above 4096 arcs activate their neighbours through the chunk
-  // queue (at most arcs / 4096 chunks plus one per such row, per class)
-  DevBuf<longlong2> mark_q;
-  DevBuf<int32_t> mark_n;
-  if (track_active && maxdeg > MARK_CH) {
-    mark_q.alloc((size_t)(2 * (lv.M / MARK_CH) + 2), s);
-    mark_n.alloc((size_t)S, s);
-    mark_n.zero();
-    a.mark_big = a.mark_ch = MARK_CH;
-    a.mq = mark_q.p;
-    a.mqn = mark_n.p;
   }
   const unsigned grid_mark = (unsigned)(sms * 8);
   constexpr size_t smem5 = blk_smem_bytes<B5_SLOTS>();
@@ -2974,7 +2947,9 @@ int64_t lp_run(const LevelView& lv, const SlotParams& sp, int32_t* label, wgt_t*
   struct Timed { int family; cudaEvent_t a, b; };
   std::vector<Timed> timed;
   int64_t pn[4] = {}, pa[4] = {};
-  std::vector<int64_t> hoff(nkeys + 1), hkarcs(nkeys);
+  std::vector<int64_t> hread(2 * nkeys + 2);         // as laid out at a.boff
+  int64_t* const hoff = hread.data();
+  const int64_t* const hkarcs = hoff + nkeys + 1;
   // The propose launches of a colour class are independent of one another:
   // they run on side streams joined back by events, so latency-bound
   // launches overlap (serial when the timeline profiler is on).  With host
@@ -3096,7 +3071,7 @@ int64_t lp_run(const LevelView& lv, const SlotParams& sp, int32_t* label, wgt_t*
     if (tu.fused_admission) {
       // one cooperative launch; it follows the propose join: plain launch
       const unsigned grid = cnt < 0 ? grid_adm_coop : grid_for(cnt, ADM_NT, grid_adm_coop);
-      launch_coop(k_admit, grid, ADM_NT, 0, s, a, sub, source_chain ? 1 : 0, gsync.p);
+      launch_coop(k_admit, grid, ADM_NT, 0, s, a, sub, source_chain ? 1 : 0, gsync);
       SCLAP_NOTE_LAUNCH("k_admit");
       if (a.mark_big) { launch_k(false, k_mark_rows, grid_mark, 256, 0, s, a, sub); SCLAP_NOTE_LAUNCH("k_mark_rows"); }
       SCLAP_LAUNCH_CHECK();
@@ -3200,13 +3175,11 @@ int64_t lp_run(const LevelView& lv, const SlotParams& sp, int32_t* label, wgt_t*
     const bool pdl = tu.pdl != 0 && !timeline;
     for (int r = 0; r < run.rounds; ++r) {
       head(s, pdl);
+      ReadBack rb(s);
+      rb.add(hread.data(), a.boff, hread.size());
+      rb.wait();
       int32_t hflags = 0;
-      SCLAP_CUDA(cudaMemcpyAsync(hoff.data(), boff.p, (nkeys + 1) * sizeof(int64_t),
-                                 cudaMemcpyDeviceToHost, s));
-      SCLAP_CUDA(cudaMemcpyAsync(hkarcs.data(), karcs.p, nkeys * sizeof(int64_t),
-                                 cudaMemcpyDeviceToHost, s));
-      SCLAP_CUDA(cudaMemcpyAsync(&hflags, flags.p, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-      stream_sync(s);
+      std::memcpy(&hflags, &hread[2 * nkeys + 1], sizeof(int32_t));
       if (hoff[nkeys] == 0) {
         tail(s, 0, false, pdl);
         break;
@@ -3220,7 +3193,7 @@ int64_t lp_run(const LevelView& lv, const SlotParams& sp, int32_t* label, wgt_t*
           phase.b = event_from_pool();
           SCLAP_CUDA(cudaEventRecord(phase.a, s));
         }
-        propose(s, sub, !timeline && tu.concurrent, hoff.data(), pdl);
+        propose(s, sub, !timeline && tu.concurrent, hoff, pdl);
         if (prof) {
           SCLAP_CUDA(cudaEventRecord(phase.b, s));
           timed.push_back(phase);
@@ -3235,14 +3208,9 @@ int64_t lp_run(const LevelView& lv, const SlotParams& sp, int32_t* label, wgt_t*
       tail(s, 0, false, pdl);
     }
   }
-  int32_t hr = 0;
-  int64_t h_arcs = 0;
-  SCLAP_CUDA(cudaMemcpyAsync(&hr, a.rnd, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-  SCLAP_CUDA(cudaMemcpyAsync(&h_arcs, arcs.p, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-  stream_sync(s);
-  if (active_next_out && track_active)
-    SCLAP_CUDA(cudaMemcpyAsync(active_next_out, a.act[hr & 1], N, cudaMemcpyDeviceToDevice, s));
+  write_active();
   if (prof) {
+    stream_sync(s);
     ProfileState& P = profile();
     std::lock_guard<std::mutex> lk(P.mu);
     for (const Timed& t : timed) {
@@ -3269,7 +3237,6 @@ int64_t lp_run(const LevelView& lv, const SlotParams& sp, int32_t* label, wgt_t*
     }
     for (const Timed& t : timed) { event_to_pool(t.a); event_to_pool(t.b); }
   }
-  return h_arcs;
 }
 
 }  // namespace sclap

@@ -137,6 +137,8 @@ __global__ void k_degree_stats(const int64_t* __restrict__ row_ptr, int64_t N, i
   for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < N;
        v += (int64_t)gridDim.x * blockDim.x) {
     const int64_t d = row_ptr[v + 1] - row_ptr[v];
+    // (the row offsets may not have been validated yet)
+    if (d < 0 || d > ((int64_t)1 << 40)) continue;
     m = (unsigned long long)d > m ? (unsigned long long)d : m;
     if (d > thr) {
       c += 1;
@@ -157,6 +159,11 @@ __global__ void k_degree_stats(const int64_t* __restrict__ row_ptr, int64_t N, i
 }
 
 }  // namespace
+
+HostRing& host_ring() {
+  static thread_local HostRing r;
+  return r;
+}
 
 void level_degree_stats(const int64_t* row_ptr, int64_t N, int64_t thr, int64_t* out,
                         cudaStream_t s) {
