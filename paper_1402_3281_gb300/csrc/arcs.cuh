@@ -28,21 +28,20 @@ __device__ __forceinline__ bool arcs_aligned(const int32_t* col, const int32_t* 
   return ((reinterpret_cast<uintptr_t>(col) | reinterpret_cast<uintptr_t>(ew)) & 15) == 0;
 }
 
-// Calls f(tile) for every tile of the arcs [lo, hi); all threads of the CTA
-// call it equally often.  row_ptr is non-decreasing over [v0, v1] with
-// row_ptr[v0] <= lo and hi <= row_ptr[v1] (v0 < v1); M is the length of col
-// and ew (a 16-byte word reaching past it is read entry by entry); sh_end is
-// AT_V words of shared memory.
+// Walks the entries [lo, hi) of rows laid out back to back (arcs of nodes,
+// slots of table regions) tile by tile: calls f(lo, span, v) for the tile of
+// the entries [lo, lo + span), whose rows are v .. v + AT_V - 1 with ends
+// sh_end[j] (relative to lo).  All threads of the CTA call it equally often.
+// row_ptr is non-decreasing over [v0, v1] with row_ptr[v0] <= lo and
+// hi <= row_ptr[v1] (v0 < v1); sh_end is AT_V words of shared memory.  A tile
+// never reaches past the AT_ARCS entries from lo rounded down to 4.
 template <class F>
-__device__ __forceinline__ void for_arc_tiles(const int64_t* __restrict__ row_ptr, int64_t v0,
-                                              int64_t v1, int64_t lo, int64_t hi,
-                                              const int32_t* __restrict__ col,
-                                              const int32_t* __restrict__ ew, int64_t M,
-                                              int32_t* sh_end, F f) {
+__device__ __forceinline__ void for_tiles(const int64_t* __restrict__ row_ptr, int64_t v0,
+                                          int64_t v1, int64_t lo, int64_t hi, int32_t* sh_end,
+                                          F f) {
   if (lo >= hi) return;
   const int tid = threadIdx.x;
-  const bool vec = arcs_aligned(col, ew);
-  int64_t v = v0, b = v1 - 1;              // last node whose row starts at or before lo
+  int64_t v = v0, b = v1 - 1;              // last row that starts at or before lo
   while (v < b) {
     const int64_t mid = (v + b + 1) >> 1;
     if (row_ptr[mid] <= lo) v = mid;
@@ -50,15 +49,63 @@ __device__ __forceinline__ void for_arc_tiles(const int64_t* __restrict__ row_pt
   }
   while (lo < hi) {
     const int64_t u = v + tid + 1;
-    int32_t end = AT_ARCS + 1;             // nodes past the range: no arc of the tile
+    int32_t end = AT_ARCS + 1;             // rows past the range: no entry of the tile
     if (u <= v1) end = (int32_t)min64(row_ptr[u] - lo, AT_ARCS + 1);
     __syncthreads();                       // the previous tile's searches are done
     sh_end[tid] = end;
     __syncthreads();
-    const int head = (int)(lo & 3);        // the tile's words start on 16-byte boundaries
-    const int32_t span = (int32_t)min64(min64(AT_ARCS - head, hi - lo),
+    const int32_t span = (int32_t)min64(min64(AT_ARCS - (int)(lo & 3), hi - lo),
                                         max64(sh_end[AT_V - 1], 0));
-    const int32_t x0 = tid * AT_PER - head;   // this thread's first arc, from lo
+    f(lo, span, v);
+    // the row that holds the next entry (the staged rows ending at or before it are done)
+    int j = 0, k = AT_V;
+    while (j < k) {
+      const int mid = (j + k) >> 1;
+      if (sh_end[mid] > span) k = mid;
+      else j = mid + 1;
+    }
+    v += j;
+    lo += span;
+  }
+}
+
+// Rows (j: from the tile's first; -1: no entry) of this thread's AT_PER
+// consecutive entries, which start at x0 from the tile's first: a search for
+// the first, then forward.
+__device__ __forceinline__ void tile_rows(const int32_t* sh_end, int32_t x0, int32_t span,
+                                          int32_t (&row)[AT_PER]) {
+  const int32_t xs = x0 > 0 ? x0 : 0;
+  int j = 0, k = AT_V - 1;
+  while (j < k) {
+    const int mid = (j + k) >> 1;
+    if (sh_end[mid] > xs) k = mid;
+    else j = mid + 1;
+  }
+  int32_t ej = sh_end[j];
+#pragma unroll
+  for (int i = 0; i < AT_PER; ++i) {
+    const int32_t x = x0 + i;
+    row[i] = -1;
+    if (x >= 0 && x < span) {
+      while (ej <= x) ej = sh_end[++j];    // x < span <= sh_end[AT_V - 1]
+      row[i] = j;
+    }
+  }
+}
+
+// Calls f(tile, v) for every tile of the arcs [lo, hi) (see for_tiles; v: the
+// tile's first staged node).  M is the length of col and ew: a 16-byte word
+// reaching past it is read entry by entry.
+template <class F>
+__device__ __forceinline__ void for_arc_tiles(const int64_t* __restrict__ row_ptr, int64_t v0,
+                                              int64_t v1, int64_t lo, int64_t hi,
+                                              const int32_t* __restrict__ col,
+                                              const int32_t* __restrict__ ew, int64_t M,
+                                              int32_t* sh_end, F f) {
+  const bool vec = arcs_aligned(col, ew);
+  for_tiles(row_ptr, v0, v1, lo, hi, sh_end, [&](int64_t lo, int32_t span, int64_t v) {
+    // the tile's words start on 16-byte boundaries
+    const int32_t x0 = (int32_t)threadIdx.x * AT_PER - (int32_t)(lo & 3);
     const int64_t e0 = lo + x0;
     ArcTile t;
 #pragma unroll
@@ -86,35 +133,13 @@ __device__ __forceinline__ void for_arc_tiles(const int64_t* __restrict__ row_pt
             if (ew) t.w[i] = ew[e0 + i];
           }
       }
-      // first staged node whose row ends after the first arc, then forward
-      const int32_t xs = x0 > 0 ? x0 : 0;
-      int j = 0, k = AT_V - 1;
-      while (j < k) {
-        const int mid = (j + k) >> 1;
-        if (sh_end[mid] > xs) k = mid;
-        else j = mid + 1;
-      }
-      int32_t ej = sh_end[j];
+      tile_rows(sh_end, x0, span, t.v);
 #pragma unroll
-      for (int i = 0; i < AT_PER; ++i) {
-        const int32_t x = x0 + i;
-        if (x >= 0 && x < span) {
-          while (ej <= x) ej = sh_end[++j];   // x < span <= sh_end[AT_V - 1]
-          t.v[i] = (int32_t)v + j;
-        }
-      }
+      for (int i = 0; i < AT_PER; ++i)
+        if (t.v[i] >= 0) t.v[i] += (int32_t)v;
     }
-    f(t);
-    // the node that holds the next arc (the staged rows ending at or before it are done)
-    int j = 0, k = AT_V;
-    while (j < k) {
-      const int mid = (j + k) >> 1;
-      if (sh_end[mid] > span) k = mid;
-      else j = mid + 1;
-    }
-    v += j;
-    lo += span;
-  }
+    f(t, v);
+  });
 }
 
 // Arc range of this CTA: an even share of [0, M), whole tiles.
@@ -126,8 +151,25 @@ __device__ __forceinline__ void arc_share(int64_t M, int64_t* lo, int64_t* hi) {
 // One wave of resident CTAs: the shares are even, so a second, partial wave
 // would only add a tail.
 constexpr int AT_CTAS = 6;                 // resident CTAs per SM (launch bounds)
-inline unsigned arc_grid(int64_t M) {
-  return grid_for(M, AT_ARCS, (int64_t)num_sms() * AT_CTAS);
+inline unsigned arc_grid(int64_t M, int ctas = AT_CTAS) {
+  return grid_for(M, AT_ARCS, (int64_t)num_sms() * ctas);
+}
+
+// Exclusive prefix of x over the CTA's threads (AT_NT); sh holds AT_NT / 32
+// words, all threads call.
+__device__ __forceinline__ int32_t cta_excl(int32_t x, int32_t* sh) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  int32_t inc = x;
+  for (int o = 1; o < 32; o <<= 1) {
+    const int32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += y;
+  }
+  __syncthreads();
+  if (lane == 31) sh[wid] = inc;
+  __syncthreads();
+  int32_t before = 0;
+  for (int w = 0; w < wid; ++w) before += sh[w];
+  return before + inc - x;
 }
 
 // Last slot s with off[s] <= x (off non-decreasing, off[0] = 0): the slot of

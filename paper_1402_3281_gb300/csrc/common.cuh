@@ -132,7 +132,7 @@ struct Tuning {
 // holds unused.
 int64_t obtainable_device_bytes();
 // Slots of the contraction table one pass may use: the tuning value, or
-// (automatic) half of the obtainable memory at 12 bytes per slot.
+// (automatic) half of the obtainable memory at 8 bytes per slot.
 int64_t table_pass_slots();
 Tuning tuning_get();
 void tuning_set(const Tuning& t);

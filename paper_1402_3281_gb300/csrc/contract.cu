@@ -4,13 +4,13 @@
 // per slot); its weight is the sum of its members; two coarse nodes are
 // adjacent iff their clusters are, with the summed weight of the fine edges
 // between them.  GPU plan: rank the labels by a scan; stream the fine arcs in
-// node order (warp per 32 nodes, arcs flattened across lanes) once to count
-// each coarse node's inter-cluster arcs, size one open-addressing region per
-// coarse node from that count (next_pow2 of it: the distinct coarse
-// neighbours never outnumber the arcs, and are usually far fewer), stream the arcs again inserting (coarse
-// neighbour, weight) with one 64-bit CAS or atomic add each (a claim also
-// records the slot's owner and counts its degree), scan the degrees into row
-// offsets, and place every occupied slot in its owner's row.  The order of a
+// even tiles (arcs.cuh) once to count each coarse node's inter-cluster arcs,
+// size one open-addressing region per coarse node from that count (1.5 slots
+// per arc: the distinct coarse neighbours never outnumber the arcs, and are
+// usually far fewer), stream the arcs again inserting (coarse neighbour,
+// weight) with one 64-bit CAS or atomic add each, then stream the table in
+// the same even tiles: once to count the occupied slots of each region (the
+// coarse degrees, whose scan gives the row offsets) and once to place them.  The order of a
 // row's arcs is not fixed, which no later step depends on; all sums are
 // integer, hence deterministic.  An alternative path (tuning contract_merge)
 // replaces the global table by member lists and per-coarse-node merges in
@@ -19,7 +19,7 @@
 #include <algorithm>
 #include <mutex>
 
-#include "common.cuh"
+#include "arcs.cuh"
 
 namespace sclap {
 namespace {
@@ -51,8 +51,6 @@ struct CArgs {
   int32_t* inter;          // inter-cluster arcs per coarse node
   const int64_t* tbase;    // table region of each coarse node
   unsigned long long* tslot;   // (coarse neighbour << 32) | summed weight; ~0 = empty
-  int32_t* cdeg;           // distinct coarse neighbours per coarse node (slots claimed)
-  int32_t* towner;         // coarse node owning each claimed slot
   int32_t* err;
   // pass of the table build: only sources with coarse id in [c_lo, c_hi)
   // insert, into the table regions of that range, which start at toff
@@ -62,10 +60,7 @@ struct CArgs {
   // bounds it): adds need no overflow check, so they do not wait for the
   // old value
   bool sums31;
-  // rows longer than `heavy` arcs are left to the heavy-row kernels (split
-  // into chunks over many CTAs); 0: no split
-  int64_t heavy;
-  int64_t N, Nc;     // fine and coarse nodes (array lengths for bounds checks)
+  int64_t N, M, Nc;  // fine nodes and arcs, coarse nodes
 };
 
 __global__ void k_map(CArgs a, int64_t N) {
@@ -79,73 +74,39 @@ __global__ void k_map(CArgs a, int64_t N) {
   }
 }
 
-// Visits every arc (v, u) of the level with cmap[v] >= 0, 32 source nodes per
-// warp, the arcs of those nodes spread over the lanes; calls f(cv, cu, w) on
-// every lane (cu = -1 on lanes without an inter-cluster arc) so the warp can
-// cooperate.
-template <class F>
-__device__ __forceinline__ void for_inter_arcs(const CArgs& a, int64_t N, F f) {
-  const int lane = threadIdx.x & 31;
-  const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t base = w0 * 32; base < N; base += nwarps * 32) {
-    const int64_t v = base + lane;
-    int64_t rs = 0, d = 0;
-    int32_t cv = -1;
-    if (v < N) {
-      cv = a.cmap[v];
-      if (cv >= a.c_lo && cv < a.c_hi) {
-        rs = a.row_ptr[v];
-        d = a.row_ptr[v + 1] - rs;
-        if (a.heavy > 0 && d > a.heavy) d = 0;     // a heavy row: chunked elsewhere
+// Inter-cluster arcs per coarse node, the arcs streamed in even tiles
+// (arcs.cuh): counted per staged row in shared memory, one global atomic per
+// row and tile.
+__global__ void __launch_bounds__(AT_NT, 5) k_count_inter(CArgs a) {
+  __shared__ int32_t sh_end[AT_V], sh_cv[AT_V], sh_cnt[AT_V];
+  const int tid = threadIdx.x;
+  int64_t lo, hi;
+  arc_share(a.M, &lo, &hi);
+  for_arc_tiles(a.row_ptr, 0, a.N, lo, hi, a.col, nullptr, a.M, sh_end,
+                [&](const ArcTile& t, int64_t v0) {
+    sh_cv[tid] = v0 + tid < a.N ? a.cmap[v0 + tid] : -1;
+    sh_cnt[tid] = 0;
+    int32_t cu[AT_PER];
+#pragma unroll
+    for (int i = 0; i < AT_PER; ++i)
+      cu[i] = t.v[i] >= 0 ? SCLAP_LD(a.cmap, t.c[i], a.N, a.err) : -1;
+    __syncthreads();
+    int32_t row = -1, c = 0;               // inter-cluster arcs of the row at hand
+#pragma unroll
+    for (int i = 0; i < AT_PER; ++i) {
+      if (t.v[i] < 0) continue;
+      const int32_t j = (int32_t)(t.v[i] - v0);
+      if (j != row) {
+        if (c) atomicAdd(&sh_cnt[row], c);
+        row = j;
+        c = 0;
       }
+      c += sh_cv[j] >= 0 && cu[i] != sh_cv[j];
     }
-    long long incl = d;
-    for (int o = 1; o < 32; o <<= 1) {
-      long long y = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += y;
-    }
-    const long long excl = incl - d;
-    const long long total = __shfl_sync(0xffffffffu, incl, 31);
-    for (long long x0 = 0; x0 < total; x0 += 32) {
-      const long long x = x0 + lane;
-      int L = 0;
-      for (int step = 16; step > 0; step >>= 1) {
-        long long y = __shfl_sync(0xffffffffu, incl, L + step - 1);
-        if (y <= x) L += step;
-      }
-      const long long rsL = __shfl_sync(0xffffffffu, (long long)rs, L);
-      const long long exL = __shfl_sync(0xffffffffu, excl, L);
-      const int32_t cvL = __shfl_sync(0xffffffffu, cv, L);
-      int32_t cu = -1, w = 0;
-      if (x < total) {
-        const int64_t e = rsL + (x - exL);
-        cu = SCLAP_LD(a.cmap, a.col[e], a.N, a.err);
-        if (cu == cvL) cu = -1;
-        else w = wat(a.ew, e);
-      }
-      f(cvL, cu, w);
-    }
-  }
-}
-
-// Inter-cluster arcs per coarse node.  The lanes' arcs are in source order,
-// so lanes with the same coarse source form runs of consecutive lanes; two
-// ballots give each run's count and its last lane adds it (runs with equal
-// sources that are not adjacent simply add separately).
-__global__ void __launch_bounds__(256) k_count_inter(CArgs a, int64_t N) {
-  const int lane = threadIdx.x & 31;
-  for_inter_arcs(a, N, [&](int32_t cv, int32_t cu, int32_t) {
-    const unsigned inter = __ballot_sync(0xffffffffu, cu >= 0);
-    const int32_t prev = __shfl_up_sync(0xffffffffu, cv, 1);
-    const unsigned heads = __ballot_sync(0xffffffffu, lane == 0 || prev != cv);
-    const bool last = lane == 31 || ((heads >> (lane + 1)) & 1u);
-    if (last) {
-      const unsigned upto = lane == 31 ? 0xffffffffu : ((2u << lane) - 1u);   // lanes 0..lane
-      const int first = 31 - __clz(heads & upto);                               // run start
-      const int c = __popc(inter & upto & ~((1u << first) - 1u));
-      if (c && SCLAP_OK(cv, a.Nc, a.err)) atomicAdd(&a.inter[cv], c);
-    }
+    if (c) atomicAdd(&sh_cnt[row], c);
+    __syncthreads();
+    if (sh_cnt[tid] && SCLAP_OK(sh_cv[tid], a.Nc, a.err))
+      atomicAdd(&a.inter[sh_cv[tid]], sh_cnt[tid]);
   });
 }
 
@@ -153,7 +114,7 @@ __global__ void k_table_caps(const int32_t* __restrict__ inter, int64_t Nc, int6
   for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < Nc;
        c += (int64_t)gridDim.x * blockDim.x) {
     const int32_t x = inter[c];
-    cap[c] = x > 0 ? ((int64_t)1 << ceil_log2((int64_t)x)) : 0;
+    cap[c] = x > 0 ? (int64_t)x + x / 2 + 1 : 0;
   }
 }
 
@@ -161,131 +122,110 @@ __global__ void k_table_caps(const int32_t* __restrict__ inter, int64_t Nc, int6
 // first arc claims an empty slot with one CAS carrying its weight, later arcs
 // add to the low half with one atomicAdd.  A coarse edge weight must fit in
 // int32, so a sum reaching 2^31 is reported (and cannot carry into the key).
-__device__ __forceinline__ void insert_arc(const CArgs& a, int32_t cv, int32_t cu, int32_t w) {
-  if (!SCLAP_OK(cv, a.Nc, a.err) || !SCLAP_OK(cu, a.Nc, a.err)) return;
-  const int64_t sum = w;
-  const int64_t base = a.tbase[cv] - a.toff;
-  const int logcap = ceil_log2(a.tbase[cv + 1] - a.tbase[cv]);
-  const uint32_t mask = (1u << logcap) - 1;
-  uint32_t sl = table_slot(cu, logcap);
-  const unsigned long long mine = ((unsigned long long)(uint32_t)cu << 32) | (uint64_t)sum;
-  for (uint32_t p = 0; p <= mask; ++p) {
+// cur: the first slot's content as read before.
+__device__ __forceinline__ uint32_t region_slot(int32_t cu, uint32_t cap) {
+  return __umulhi((uint32_t)cu * 0x9E3779B1u, cap);
+}
+__device__ __forceinline__ void insert_arc(const CArgs& a, int64_t base, uint32_t cap, int32_t cu,
+                                           int32_t w, uint32_t sl, unsigned long long cur) {
+  const unsigned long long mine = ((unsigned long long)(uint32_t)cu << 32) | (uint32_t)w;
+  for (uint32_t p = 0; p < cap; ++p) {
     unsigned long long* slot = &a.tslot[base + sl];
-    unsigned long long cur = *slot;
+    if (p) cur = *slot;
     if (cur == ~0ull) {
       cur = atomicCAS(slot, ~0ull, mine);
-      if (cur == ~0ull) {            // claimed: one more coarse arc of cv
-        a.towner[base + sl] = cv;
-        atomicAdd(&a.cdeg[cv], 1);
-        return;
-      }
+      if (cur == ~0ull) return;            // claimed
     }
     if ((uint32_t)(cur >> 32) == (uint32_t)cu) {
       if (a.sums31) {
-        atomicAdd(slot, (unsigned long long)sum);
+        atomicAdd(slot, (unsigned long long)(uint32_t)w);
         return;
       }
-      const unsigned long long old = atomicAdd(slot, (unsigned long long)sum);
-      if ((old & 0xffffffffull) + (unsigned long long)sum > (unsigned long long)INT32_MAX)
+      const unsigned long long old = atomicAdd(slot, (unsigned long long)(uint32_t)w);
+      if ((old & 0xffffffffull) + (unsigned long long)(uint32_t)w > (unsigned long long)INT32_MAX)
         atomicOr(a.err, DERR_W_OVERFLOW);
       return;
     }
-    sl = (sl + 1) & mask;
+    sl = sl + 1 == cap ? 0 : sl + 1;
   }
   atomicOr(a.err, DERR_HASH_FULL);
 }
 
-__global__ void __launch_bounds__(256) k_insert(CArgs a, int64_t N) {
-  for_inter_arcs(a, N, [&](int32_t cv, int32_t cu, int32_t w) {
-    if (cu >= 0) insert_arc(a, cv, cu, w);
-  });
-}
-
-// Heavy rows (more than `heavy` arcs, cmap >= 0): listed once per level,
-// then cut into chunks of HV_CH arcs (hoff: exclusive scan of the chunks
-// per listed row) that CTAs take in turn, so that a hub's row is spread
-// over the whole grid instead of being one warp's serial job.
-constexpr int HV_CH = 2048;
-
-__global__ void k_heavy_list(CArgs a, int64_t N, int32_t* __restrict__ list, int32_t* cnt) {
-  const int lane = threadIdx.x & 31;
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t v0 = (int64_t)blockIdx.x * blockDim.x; v0 < N; v0 += stride) {
-    const int64_t v = v0 + threadIdx.x;
-    const bool h = v < N && a.cmap[v] >= 0 && a.row_ptr[v + 1] - a.row_ptr[v] > a.heavy;
-    const unsigned m = __ballot_sync(0xffffffffu, h);
-    if (!m) continue;
-    int q0 = 0;
-    if (lane == 0) q0 = atomicAdd(cnt, __popc(m));
-    q0 = __shfl_sync(0xffffffffu, q0, 0);
-    if (h) list[q0 + __popc(m & ((1u << lane) - 1))] = (int32_t)v;
-  }
-}
-__global__ void k_heavy_chunks(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ list,
-                               int32_t nh, int32_t* __restrict__ nch) {
-  for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < nh; i += gridDim.x * blockDim.x) {
-    const int32_t v = list[i];
-    nch[i] = (int32_t)((row_ptr[v + 1] - row_ptr[v] + HV_CH - 1) / HV_CH);
-  }
-}
-
-// Calls f(cv, cu, w) for every arc of every chunk this CTA takes (cu = -1
-// for an arc inside the cluster); all threads of the CTA loop alike.
-template <class F>
-__device__ __forceinline__ void for_heavy_arcs(const CArgs& a, const int32_t* __restrict__ list,
-                                               const int64_t* __restrict__ hoff, int32_t nh, F f) {
-  const int64_t total = hoff[nh];
-  for (int64_t q = blockIdx.x; q < total; q += gridDim.x) {
-    int32_t lo = 0, hi = nh - 1;           // last list position i with hoff[i] <= q
-    while (lo < hi) {
-      const int32_t mid = (lo + hi + 1) >> 1;
-      if (hoff[mid] <= q) lo = mid;
-      else hi = mid - 1;
+// Inserts the arcs, streamed in even tiles: per tile the coarse sources of
+// the staged rows and their table regions lie in shared memory, and a
+// thread's eight head gathers, then its eight slot reads, are in flight
+// together.  An arc touches one slot of the table and nothing else: who owns
+// a slot and how many are taken is read off the table afterwards.  (Before, a
+// claim also wrote the slot's owner and counted the owner's degree with an
+// atomic; the claims of a hub's cluster serialised on that one counter.)
+// Bounded by random atomics on a table beyond L2: 24 G arcs a second on R-MAT
+// 2^24 nodes, where 64-bit CAS on random words of a 2 GB table reach 23 G.
+// Inserts of both levels there 97 -> 52 ms, R-MAT 2^22 nodes 9.9 -> 6.1 ms.
+// Regions of 1.5 slots per inter-cluster arc (a power of two from 1 to 2
+// before, full to the last slot where the arcs' heads all differ) took the
+// last fifth off.  Sorting the nodes by coarse node first, so that the filled
+// regions lie in L2 and a tile's equal arcs are summed in shared memory, took
+// 74 ms: claims answered one after the other.
+__global__ void __launch_bounds__(AT_NT, 4) k_insert(CArgs a) {
+  __shared__ int32_t sh_end[AT_V], sh_cv[AT_V];
+  __shared__ int64_t sh_base[AT_V];
+  __shared__ uint32_t sh_cap[AT_V];
+  const int tid = threadIdx.x;
+  int64_t lo, hi;
+  arc_share(a.M, &lo, &hi);
+  for_arc_tiles(a.row_ptr, 0, a.N, lo, hi, a.col, a.ew, a.M, sh_end,
+                [&](const ArcTile& t, int64_t v0) {
+    int32_t cu[AT_PER];
+#pragma unroll
+    for (int i = 0; i < AT_PER; ++i)
+      cu[i] = t.v[i] >= 0 ? SCLAP_LD(a.cmap, t.c[i], a.N, a.err) : -1;
+    {
+      int32_t cv = v0 + tid < a.N ? a.cmap[v0 + tid] : -1;
+      if (cv < a.c_lo || cv >= a.c_hi || !SCLAP_OK(cv, a.Nc, a.err)) cv = -1;
+      sh_cv[tid] = cv;
+      if (cv >= 0) {
+        const int64_t b = a.tbase[cv];
+        sh_base[tid] = b - a.toff;
+        sh_cap[tid] = (uint32_t)(a.tbase[cv + 1] - b);
+      }
     }
-    const int32_t v = list[lo];
-    const int32_t cv = a.cmap[v];
-    if (cv < a.c_lo || cv >= a.c_hi) continue;
-    const int64_t e0 = a.row_ptr[v] + (q - hoff[lo]) * HV_CH;
-    const int64_t e1 = min(e0 + HV_CH, a.row_ptr[v + 1]);
-    for (int64_t e = e0 + threadIdx.x; e < e1; e += blockDim.x) {
-      int32_t cu = SCLAP_LD(a.cmap, a.col[e], a.N, a.err);
-      int32_t w = 0;
-      if (cu == cv) cu = -1;
-      else w = wat(a.ew, e);
-      f(cv, cu, w);
+    __syncthreads();
+    // arcs of this thread into the same coarse node from the same row become
+    // one (a cluster's neighbours come in bunches: the equal arcs would meet
+    // on one slot, where atomics serialise)
+    int32_t w[AT_PER];
+#pragma unroll
+    for (int i = 0; i < AT_PER; ++i) {
+      const int32_t j = t.v[i] >= 0 ? (int32_t)(t.v[i] - v0) : 0;
+      const int32_t cv = t.v[i] >= 0 ? sh_cv[j] : -1;
+      if (cv < 0 || cu[i] == cv || !SCLAP_OK(cu[i], a.Nc, a.err)) cu[i] = -1;
+      w[i] = t.w[i];
     }
-  }
-}
-
-__global__ void __launch_bounds__(256) k_count_heavy(CArgs a, const int32_t* __restrict__ list,
-                                                     const int64_t* __restrict__ hoff, int32_t nh) {
-  // a chunk belongs to one row, so one coarse source: count per thread,
-  // reduce per warp, one atomic per warp and chunk
-  const int lane = threadIdx.x & 31;
-  const int64_t total = hoff[nh];
-  for (int64_t q = blockIdx.x; q < total; q += gridDim.x) {
-    int32_t lo = 0, hi = nh - 1;
-    while (lo < hi) {
-      const int32_t mid = (lo + hi + 1) >> 1;
-      if (hoff[mid] <= q) lo = mid;
-      else hi = mid - 1;
+    if (a.sums31) {
+#pragma unroll
+      for (int i = 1; i < AT_PER; ++i) {
+#pragma unroll
+        for (int k = 0; k < i; ++k) {
+          const bool same = cu[i] >= 0 && cu[k] == cu[i] && t.v[k] == t.v[i];
+          w[k] += same ? w[i] : 0;
+          cu[i] = same ? -1 : cu[i];
+        }
+      }
     }
-    const int32_t v = list[lo];
-    const int32_t cv = a.cmap[v];
-    const int64_t e0 = a.row_ptr[v] + (q - hoff[lo]) * HV_CH;
-    const int64_t e1 = min(e0 + HV_CH, a.row_ptr[v + 1]);
-    int c = 0;
-    for (int64_t e = e0 + threadIdx.x; e < e1; e += blockDim.x)
-      c += SCLAP_LD(a.cmap, a.col[e], a.N, a.err) != cv;
-    for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-    if (lane == 0 && c && SCLAP_OK(cv, a.Nc, a.err)) atomicAdd(&a.inter[cv], c);
-  }
-}
-
-__global__ void __launch_bounds__(256) k_insert_heavy(CArgs a, const int32_t* __restrict__ list,
-                                                      const int64_t* __restrict__ hoff, int32_t nh) {
-  for_heavy_arcs(a, list, hoff, nh, [&](int32_t cv, int32_t cu, int32_t w) {
-    if (cu >= 0) insert_arc(a, cv, cu, w);
+    uint32_t sl[AT_PER];
+    unsigned long long cur[AT_PER];
+#pragma unroll
+    for (int i = 0; i < AT_PER; ++i) {
+      const int32_t j = cu[i] >= 0 ? (int32_t)(t.v[i] - v0) : 0;
+      sl[i] = cu[i] >= 0 ? region_slot(cu[i], sh_cap[j]) : 0;
+      cur[i] = cu[i] >= 0 ? a.tslot[sh_base[j] + sl[i]] : 0;
+    }
+#pragma unroll
+    for (int i = 0; i < AT_PER; ++i) {
+      if (cu[i] < 0) continue;
+      const int32_t j = (int32_t)(t.v[i] - v0);
+      insert_arc(a, sh_base[j], sh_cap[j], cu[i], w[i], sl[i], cur[i]);
+    }
   });
 }
 
@@ -296,25 +236,120 @@ __global__ void k_clear_table(unsigned long long* __restrict__ tslot,
     tslot[j] = ~0ull;
 }
 
-// Coarse rows: one thread per table slot; an occupied slot goes to its
-// owner's row (offsets from a scan of the claimed-slot counts) at a position
-// taken from a per-row counter.  The order of a row's arcs is therefore not
-// fixed, as the slot order already was not (concurrent claims in one region
-// race); nothing computed from a coarse graph depends on that order.
-__global__ void k_emit(const unsigned long long* __restrict__ tslot,
-                       const int32_t* __restrict__ towner, const int64_t* __restrict__ crow,
-                       int32_t* __restrict__ fill, int64_t T, const int64_t* Tdev,
-                       int32_t* __restrict__ ccol, int32_t* __restrict__ cew) {
-  if (Tdev) T = min(T, *Tdev);             // the slots in use, where the host knows a bound
-  for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < T;
-       j += (int64_t)gridDim.x * blockDim.x) {
-    const unsigned long long x = tslot[j];
-    if (x == ~0ull) continue;
-    const int32_t c = towner[j];
-    const int64_t p = crow[c] + atomicAdd(&fill[c], 1);
-    ccol[p] = (int32_t)(x >> 32);
-    cew[p] = (int32_t)(x & 0xffffffffull);
+// The table's slots [toff, T) (T: the table's end, *Tdev where the host knows
+// only a bound) are streamed in even tiles like arcs, the regions of the
+// coarse nodes [c_lo, c_hi) taking the place of rows.
+// k_slot_count: occupied slots per coarse node, i.e. the coarse degrees.
+struct SlotArgs {
+  const unsigned long long* tslot;
+  const int64_t* tbase;
+  const int64_t* Tdev;
+  int64_t T, toff;
+  int64_t c_lo, c_hi;
+};
+// this CTA's share of the slots [toff, T)
+__device__ __forceinline__ void slot_share(const SlotArgs& a, int64_t* lo, int64_t* hi) {
+  const int64_t T = a.Tdev ? min64(a.T, *a.Tdev) : a.T;
+  arc_share(T - a.toff, lo, hi);
+  *lo += a.toff;
+  *hi += a.toff;
+}
+// this thread's slots of a tile and their regions (j, -1: none)
+__device__ __forceinline__ void load_slots(const SlotArgs& a, int64_t lo, int32_t span,
+                                           const int32_t* sh_end,
+                                           unsigned long long (&x)[AT_PER], int32_t (&row)[AT_PER]) {
+  const int32_t x0 = (int32_t)threadIdx.x * AT_PER - (int32_t)(lo & 3);
+#pragma unroll
+  for (int i = 0; i < AT_PER; ++i) {
+    const bool in = x0 + i >= 0 && x0 + i < span;
+    x[i] = in ? a.tslot[lo - a.toff + x0 + i] : ~0ull;
+    row[i] = -1;
   }
+  if (x0 < span) tile_rows(sh_end, x0, span, row);
+}
+
+__global__ void __launch_bounds__(AT_NT, 6) k_slot_count(SlotArgs a, int32_t* __restrict__ cdeg) {
+  __shared__ int32_t sh_end[AT_V], sh_cnt[AT_V];
+  const int tid = threadIdx.x;
+  int64_t lo, hi;
+  slot_share(a, &lo, &hi);
+  for_tiles(a.tbase, a.c_lo, a.c_hi, lo, hi, sh_end, [&](int64_t lo, int32_t span, int64_t c0) {
+    unsigned long long x[AT_PER];
+    int32_t row[AT_PER];
+    sh_cnt[tid] = 0;
+    load_slots(a, lo, span, sh_end, x, row);
+    __syncthreads();
+    int32_t at = -1, c = 0;
+#pragma unroll
+    for (int i = 0; i < AT_PER; ++i) {
+      if (row[i] < 0) continue;
+      if (row[i] != at) {
+        if (c) atomicAdd(&sh_cnt[at], c);
+        at = row[i];
+        c = 0;
+      }
+      c += x[i] != ~0ull;
+    }
+    if (c) atomicAdd(&sh_cnt[at], c);
+    __syncthreads();
+    if (sh_cnt[tid]) atomicAdd(&cdeg[c0 + tid], sh_cnt[tid]);
+  });
+}
+
+// Coarse rows: an occupied slot goes to its region's row.  A tile's occupied
+// slots are numbered by a scan; one atomic per region and tile reserves their
+// places in the row.  The order of a row's arcs is therefore not fixed, as
+// the slot order already was not (concurrent claims in one region race);
+// nothing computed from a coarse graph depends on that order.
+__global__ void __launch_bounds__(AT_NT, 5) k_emit(SlotArgs a, const int64_t* __restrict__ crow,
+                                                   int32_t* __restrict__ fill,
+                                                   int32_t* __restrict__ ccol,
+                                                   int32_t* __restrict__ cew) {
+  __shared__ int32_t sh_end[AT_V], sh_cnt[AT_V], sh_first[AT_V], sh_w[AT_NT / 32];
+  __shared__ int64_t sh_at[AT_V];
+  const int tid = threadIdx.x;
+  int64_t lo, hi;
+  slot_share(a, &lo, &hi);
+  for_tiles(a.tbase, a.c_lo, a.c_hi, lo, hi, sh_end, [&](int64_t lo, int32_t span, int64_t c0) {
+    unsigned long long x[AT_PER];
+    int32_t row[AT_PER];
+    sh_cnt[tid] = 0;
+    sh_first[tid] = INT32_MAX;
+    load_slots(a, lo, span, sh_end, x, row);
+    int32_t mine = 0;
+#pragma unroll
+    for (int i = 0; i < AT_PER; ++i) mine += row[i] >= 0 && x[i] != ~0ull;
+    const int32_t before = cta_excl(mine, sh_w);   // (its barriers also order the clears)
+    int32_t at = -1, c = 0, n = before;
+#pragma unroll
+    for (int i = 0; i < AT_PER; ++i) {
+      if (row[i] < 0) continue;
+      if (row[i] != at) {
+        if (c) atomicAdd(&sh_cnt[at], c);
+        at = row[i];
+        c = 0;
+        atomicMin(&sh_first[at], n);       // occupied slots before the region's first in the tile
+      }
+      if (x[i] != ~0ull) {
+        ++c;
+        ++n;
+      }
+    }
+    if (c) atomicAdd(&sh_cnt[at], c);
+    __syncthreads();
+    if (sh_cnt[tid])
+      sh_at[tid] = crow[c0 + tid] + atomicAdd(&fill[c0 + tid], sh_cnt[tid]) - sh_first[tid];
+    __syncthreads();
+    n = before;
+#pragma unroll
+    for (int i = 0; i < AT_PER; ++i) {
+      if (row[i] < 0 || x[i] == ~0ull) continue;
+      const int64_t p = sh_at[row[i]] + n;
+      ++n;
+      ccol[p] = (int32_t)(x[i] >> 32);
+      cew[p] = (int32_t)(x[i] & 0xffffffffull);
+    }
+  });
 }
 
 // ------------------------------------------------------------------------
@@ -840,7 +875,7 @@ void finish_level(CoarseLevel& out, int ns, cudaStream_t s) {
 // The coarse arcs by segments (member lists and per-node merges, see the
 // kernels above).  Returns false, having built nothing, when the regions,
 // member lists and the table of the large nodes would take more than the
-// memory of Tcap slots of the hash table path (12 bytes each).
+// memory of Tcap slots of the hash table path (8 bytes each).
 bool contract_merge(const LevelView& lv, int64_t N, int64_t Nc, DevBuf<int32_t>& inter,
                     DevBuf<int64_t>& cap, DevBuf<int64_t>& tbase, const CArgs& ca, int64_t Tcap,
                     CoarseLevel& out, int32_t* d_err, cudaStream_t s) {
@@ -866,7 +901,7 @@ bool contract_merge(const LevelView& lv, int64_t N, int64_t Nc, DevBuf<int32_t>&
   stream_sync(s);
   const int64_t Mi = h[0], T = h[1];
   const int32_t nb = hc[0], nl = hc[1];
-  if (8 * Mi + 8 * T + 4 * N + 8 * Nc + 12 * (int64_t)nl > 12 * Tcap) return false;
+  if (8 * Mi + 8 * T + 4 * N + 8 * Nc + 12 * (int64_t)nl > 8 * Tcap) return false;
 
   // member lists: fine nodes counting-sorted by coarse id
   DevBuf<int32_t> members(N, s), cdeg(Nc, s);
@@ -986,40 +1021,19 @@ void contract_build(const LevelView& lv, const std::vector<int64_t>& noff, const
   a.label = label; a.cid = w.cid.p; a.delta = d_delta.p; a.keep = d_keep.p; a.cmap = cmap;
   a.cnw = out.nw.p; a.inter = inter.p; a.tbase = tbase.p; a.err = d_err;
   a.c_lo = 0; a.c_hi = INT32_MAX; a.toff = 0; a.sums31 = lv.sums31;
-  a.N = N; a.Nc = Nc;
+  a.N = N; a.M = lv.M; a.Nc = Nc;
 
   const unsigned ng = grid_for(N, 256, (int64_t)sms * 16);
-  const unsigned wg = grid_for(N, 256, (int64_t)sms * 16);   // 8 warps x 32 nodes per block
-  const unsigned hg = (unsigned)sms * 8;                      // heavy-row chunks, grid-stride
-  // rows above HEAVY_ROW arcs: listed, cut into chunks, spread over the grid
-  constexpr int64_t HEAVY_ROW = 2048;
-  constexpr int64_t BOUNDED_M = 4000000;   // arcs: at most 96 MB of table
-  DevBuf<int32_t> hlist(std::max<int64_t>(1, std::min<int64_t>(N, lv.M / (HEAVY_ROW + 1) + 1)), s);
-  DevBuf<int64_t> hoff;
-  int32_t nh = 0;
+  constexpr int64_t BOUNDED_M = 4000000;   // arcs: at most 80 MB of table
   if (N > 0) {
     k_map<<<ng, 256, 0, s>>>(a, N); SCLAP_NOTE_LAUNCH("k_map");
-    a.heavy = HEAVY_ROW;
-    DevBuf<int32_t> hcnt(1, s);
-    hcnt.zero();
-    if (lv.deg.maxdeg < 0 || lv.deg.maxdeg > HEAVY_ROW) {
-      k_heavy_list<<<ng, 256, 0, s>>>(a, N, hlist.p, hcnt.p); SCLAP_NOTE_LAUNCH("k_heavy_list");
-      ReadBack rb(s);
-      rb.add(&nh, hcnt.p, 1);
-      rb.wait();
+    if (lv.M > 0) {
+      k_count_inter<<<arc_grid(lv.M, 5), AT_NT, 0, s>>>(a); SCLAP_NOTE_LAUNCH("k_count_inter");
     }
-    if (nh > 0) {
-      DevBuf<int32_t> nch(nh, s);
-      hoff.alloc(nh + 1, s);
-      k_heavy_chunks<<<grid_for(nh, 256, (int64_t)sms * 4), 256, 0, s>>>(lv.row_ptr, hlist.p, nh, nch.p); SCLAP_NOTE_LAUNCH("k_heavy_chunks");
-      scan_excl_i32_to_i64(nch.p, hoff.p, nh, s);
-    }
-    k_count_inter<<<wg, 256, 0, s>>>(a, N); SCLAP_NOTE_LAUNCH("k_count_inter");
-    if (nh > 0) { k_count_heavy<<<hg, 256, 0, s>>>(a, hlist.p, hoff.p, nh); SCLAP_NOTE_LAUNCH("k_count_heavy"); }
   }
   auto insert = [&] {
-    k_insert<<<wg, 256, 0, s>>>(a, N); SCLAP_NOTE_LAUNCH("k_insert");
-    if (nh > 0) { k_insert_heavy<<<hg, 256, 0, s>>>(a, hlist.p, hoff.p, nh); SCLAP_NOTE_LAUNCH("k_insert_heavy"); }
+    if (lv.M <= 0) return;
+    k_insert<<<arc_grid(lv.M, 4), AT_NT, 0, s>>>(a); SCLAP_NOTE_LAUNCH("k_insert");
   };
   const int64_t Tcap = table_pass_slots();
   if (tuning_get().contract_merge && N > 0 && Nc > 0 &&
@@ -1032,32 +1046,44 @@ void contract_build(const LevelView& lv, const std::vector<int64_t>& noff, const
   }
   scan_excl_i64(cap.p, tbase.p, Nc, s);
   // a small level takes a table and coarse arrays of the largest size they
-  // can have instead of waiting for the sizes (twice): fewer than two slots
-  // per arc, no more coarse arcs than fine ones
-  const bool bounded = lv.M <= BOUNDED_M && 2 * lv.M <= Tcap;
-  int64_t T = 2 * lv.M;
+  // can have instead of waiting for the sizes (twice): at most five slots
+  // per two arcs, no more coarse arcs than fine ones
+  const bool bounded = lv.M <= BOUNDED_M && 5 * lv.M / 2 <= Tcap;
+  int64_t T = 5 * lv.M / 2;
   if (!bounded) {
     ReadBack rb(s);
     rb.add(&T, tbase.p + Nc, 1);
     rb.wait();
   }
-  // the inter-arc counts have served (table sizes); the array now counts
-  // claimed slots, i.e. the coarse degrees
-  a.cdeg = inter.p;
+  // the inter-arc counts have served (table sizes); the array now holds the
+  // coarse degrees, then the places taken in each row
   SCLAP_CUDA(cudaMemsetAsync(inter.p, 0, (size_t)std::max<int64_t>(Nc, 1) * sizeof(int32_t), s));
   out.row_ptr.alloc(Nc + 1, s);
+  SlotArgs sa{};
+  sa.tbase = tbase.p;
+  auto count_slots = [&] {
+    k_slot_count<<<arc_grid(sa.T - sa.toff, 6), AT_NT, 0, s>>>(sa, inter.p); SCLAP_NOTE_LAUNCH("k_slot_count");
+  };
+  auto emit = [&] {
+    k_emit<<<arc_grid(sa.T - sa.toff, 5), AT_NT, 0, s>>>(sa, out.row_ptr.p, inter.p, out.col.p,
+                                                         out.ew.p); SCLAP_NOTE_LAUNCH("k_emit");
+  };
   if (T <= Tcap) {
     // one pass: the whole table at once
     DevBuf<unsigned long long> tslot(std::max<int64_t>(T, 1), s);
-    DevBuf<int32_t> towner(std::max<int64_t>(T, 1), s);
     if (bounded && T > 0) {
       k_clear_table<<<grid_for(T, 1024, (int64_t)sms * 8), 256, 0, s>>>(tslot.p, tbase.p + Nc); SCLAP_NOTE_LAUNCH("k_clear_table");
     } else {
       tslot.fill_bytes(0xff);
     }
     a.tslot = tslot.p;
-    a.towner = towner.p;
+    sa.tslot = tslot.p;
+    sa.Tdev = bounded ? tbase.p + Nc : nullptr;
+    sa.T = T;
+    sa.c_hi = Nc;
+    const bool any = Nc > 0 && T > 0;
     if (N > 0 && T > 0) insert();
+    if (any) count_slots();
     scan_excl_i32_to_i64(inter.p, out.row_ptr.p, Nc, s);
     int64_t Mc = lv.M;
     if (!bounded) {
@@ -1067,10 +1093,9 @@ void contract_build(const LevelView& lv, const std::vector<int64_t>& noff, const
     }
     out.col.alloc(std::max<int64_t>(Mc, 1), s);
     out.ew.alloc(std::max<int64_t>(Mc, 1), s);
-    if (Nc > 0 && T > 0) {
+    if (any) {
       SCLAP_CUDA(cudaMemsetAsync(inter.p, 0, (size_t)Nc * sizeof(int32_t), s));   // row fill
-      k_emit<<<grid_for(T, 256, (int64_t)sms * 32), 256, 0, s>>>(
-          tslot.p, towner.p, out.row_ptr.p, inter.p, T, tbase.p + Nc, out.col.p, out.ew.p); SCLAP_NOTE_LAUNCH("k_emit");
+      emit();
     }
   } else {
     // Passes over ranges of coarse nodes whose table regions fit in Tcap
@@ -1095,18 +1120,22 @@ void contract_build(const LevelView& lv, const std::vector<int64_t>& noff, const
     for (size_t q = 0; q + 1 < cut_at.size(); ++q)
       Tmax = std::max<int64_t>(Tmax, htb[cut_at[q + 1]] - htb[cut_at[q]]);
     DevBuf<unsigned long long> tslot(Tmax, s);
-    DevBuf<int32_t> towner(Tmax, s), claims(std::max<int64_t>(Nc, 1), s);
     a.tslot = tslot.p;
-    a.towner = towner.p;
+    sa.tslot = tslot.p;
     auto pass = [&](size_t q) {
       a.c_lo = cut_at[q];
       a.c_hi = cut_at[q + 1];
       a.toff = htb[a.c_lo];
-      SCLAP_CUDA(cudaMemsetAsync(tslot.p, 0xff, (size_t)(htb[a.c_hi] - a.toff) * 8, s));
+      sa.c_lo = a.c_lo;
+      sa.c_hi = a.c_hi;
+      sa.toff = a.toff;
+      sa.T = htb[a.c_hi];
+      SCLAP_CUDA(cudaMemsetAsync(tslot.p, 0xff, (size_t)(sa.T - sa.toff) * 8, s));
       if (N > 0) insert();
-      return htb[a.c_hi] - a.toff;
+      return sa.T > sa.toff;
     };
-    for (size_t q = 0; q + 1 < cut_at.size(); ++q) pass(q);            // sweep 1: degrees
+    for (size_t q = 0; q + 1 < cut_at.size(); ++q)                      // sweep 1: degrees
+      if (pass(q)) count_slots();
     scan_excl_i32_to_i64(inter.p, out.row_ptr.p, Nc, s);
     int64_t Mc = 0;
     ReadBack rb(s);
@@ -1114,14 +1143,9 @@ void contract_build(const LevelView& lv, const std::vector<int64_t>& noff, const
     rb.wait();
     out.col.alloc(std::max<int64_t>(Mc, 1), s);
     out.ew.alloc(std::max<int64_t>(Mc, 1), s);
-    a.cdeg = claims.p;                   // sweep 2 counts claims apart from the row fill
     SCLAP_CUDA(cudaMemsetAsync(inter.p, 0, (size_t)Nc * sizeof(int32_t), s));   // row fill
-    for (size_t q = 0; q + 1 < cut_at.size(); ++q) {                    // sweep 2: emit
-      const int64_t Tp = pass(q);
-      k_emit<<<grid_for(Tp, 256, (int64_t)sms * 32), 256, 0, s>>>(tslot.p, towner.p,
-                                                                  out.row_ptr.p, inter.p, Tp,
-                                                                  nullptr, out.col.p, out.ew.p); SCLAP_NOTE_LAUNCH("k_emit");
-    }
+    for (size_t q = 0; q + 1 < cut_at.size(); ++q)                      // sweep 2: emit
+      if (pass(q)) emit();
   }
   SCLAP_LAUNCH_CHECK();
   finish_level(out, ns, s);

@@ -867,7 +867,7 @@ __global__ void __launch_bounds__(AT_NT, AT_CTAS) k_slot_cut(const int64_t* __re
     const int64_t end = nslots > 1 ? min64(hi, aoff[s + 1]) : hi;
     unsigned long long acc = 0;
     for_arc_tiles(row_ptr, nslots > 1 ? noff[s] : 0, nslots > 1 ? noff[s + 1] : N, lo, end, col,
-                  ew, M, sh_end, [&](const ArcTile& t) {
+                  ew, M, sh_end, [&](const ArcTile& t, int64_t) {
       int32_t a[AT_PER], b[AT_PER];
 #pragma unroll
       for (int i = 0; i < AT_PER; ++i) {

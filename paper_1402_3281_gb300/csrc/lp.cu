@@ -2576,7 +2576,7 @@ std::string alloc_failure_message(size_t bytes, cudaError_t e) {
 int64_t table_pass_slots() {
   const Tuning t = tuning_get();
   if (t.contract_table_slots > 0) return t.contract_table_slots;
-  return std::max<int64_t>((int64_t)1 << 20, obtainable_device_bytes() / 2 / 12);
+  return std::max<int64_t>((int64_t)1 << 20, obtainable_device_bytes() / 2 / 8);
 }
 
 int64_t obtainable_device_bytes() {
