@@ -163,6 +163,21 @@ __device__ __forceinline__ int32_t cand_block(const LPArgs& a, const NodeCtx& c,
   return a.rblk && need ? a.rblk[C] : c.vb;
 }
 
+// Pruning.  A node in a block that is not overloaded moves only to a label
+// connected to it more strongly than its own (write_prop), so no other label
+// is looked at: after the first round most nodes have few such labels, and a
+// label's weight is a gather as random as the arc's label itself.  CTAs, whose
+// nodes have hundreds of labels, also try the strongest label first, whether
+// or not it has room, and read one weight when it has; for threads and warps
+// the extra round trip cost more than the gathers (batch of 512 graphs, warp
+// per node 4.9 -> 5.6 ms, thread per node 4.9 -> 5.5 ms).
+__device__ __forceinline__ bool cand_fits(const LPArgs& a, const NodeCtx& c, int32_t C) {
+  if (!SCLAP_OK(C, a.nlabels, a.err)) return false;
+  const int64_t w = a.W[C];
+  const int32_t b = cand_block(a, c, true, C);
+  return w + c.cv <= c.bound && b == c.vb;
+}
+
 __device__ __forceinline__ Cand make_cand(const NodeCtx& c, int32_t C, int64_t conn) {
   const int32_t Cl = (int32_t)(C - c.loff);
   return Cand{conn, mix64(c.hv ^ (uint64_t)(uint32_t)Cl), Cl};
@@ -404,19 +419,20 @@ __device__ __forceinline__ void sorted_row_best(const LPArgs& a, const NodeCtx& 
     run[j] = (j > 0 && C[j] == C[j - 1]) ? prev + (SumT)w[j] : (SumT)w[j];
     end[j] = C[j] != INT32_MAX && (j == MAXD - 1 || C[j] != C[j + 1]);
   }
+#pragma unroll
+  for (int j = 0; j < MAXD; ++j) oc = end[j] & (C[j] == c.own) ? (long long)run[j] : oc;
+  // only labels that beat the own one are looked at (pruning, above)
+#pragma unroll
+  for (int j = 0; j < MAXD; ++j) end[j] = end[j] & (C[j] != c.own) & ((long long)run[j] > oc);
   int32_t Wl[MAXD], Bl[MAXD];
 #pragma unroll
   for (int j = 0; j < MAXD; ++j) {
-    const bool q = end[j] & (C[j] != c.own);
-    Wl[j] = q ? SCLAP_LD(a.W, C[j], a.nlabels, a.err) : 0;
-    Bl[j] = cand_block(a, c, q, C[j]);
+    Wl[j] = end[j] ? SCLAP_LD(a.W, C[j], a.nlabels, a.err) : 0;
+    Bl[j] = cand_block(a, c, end[j], C[j]);
   }
 #pragma unroll
   for (int j = 0; j < MAXD; ++j) {
-    const bool own = end[j] & (C[j] == c.own);
-    oc = own ? (long long)run[j] : oc;
-    const bool elig = end[j] & (C[j] != c.own) & ((int64_t)Wl[j] + c.cv <= c.bound) &
-                      (Bl[j] == c.vb);
+    const bool elig = end[j] & ((int64_t)Wl[j] + c.cv <= c.bound) & (Bl[j] == c.vb);
     const int32_t Cl = (int32_t)(C[j] - c.loff);
     const Cand x{(int64_t)run[j], mix64(c.hv ^ (uint64_t)(uint32_t)Cl), Cl};
     best = cand_pick(elig & cand_better(x, best), x, best);
@@ -624,14 +640,13 @@ __device__ __forceinline__ void propose_warp_node(const LPArgs& a, int64_t i, in
     }
     __syncwarp();
     long long oc = 0;
-    bool has_oc = false;
     Cand cd{-1, 0, 0};
     if (direct) {
       const int32_t own_l = (int32_t)(c.own - c.loff);
+      oc = (long long)vals[own_l];
       for (int32_t b = lane; b < nl; b += 32) {
         const int64_t conn = (int64_t)vals[b];
-        if (b == own_l) { oc = conn; has_oc = true; continue; }
-        if (conn == 0 && !ov) continue;
+        if (b == own_l || (conn <= oc && !ov)) continue;
         const int32_t Cb = (int32_t)(c.loff + b);
         if ((int64_t)a.W[Cb] + c.cv > c.bound) continue;
         const Cand x = make_cand(c, Cb, conn);
@@ -640,21 +655,23 @@ __device__ __forceinline__ void propose_warp_node(const LPArgs& a, int64_t i, in
       __syncwarp();
       for (int32_t b = lane; b < nl; b += 32) vals[b] = 0;
     } else {
-      int32_t Wk[4], Bk[4];
+      oc = table_get(keys, vals, WLOG, c.own);
+      if (!ov) {
+        int32_t Wk[4], Bk[4];
+        unsigned up = 0;                     // labels that beat the own one (pruning)
 #pragma unroll
-      for (int t = 0; t < 4; ++t) {
-        const bool q = ((created >> t) & 1u) && C[t] != c.own && !ov;
-        Wk[t] = q ? SCLAP_LD(a.W, C[t], a.nlabels, a.err) : 0;
-        Bk[t] = cand_block(a, c, q, C[t]);
-      }
+        for (int t = 0; t < 4; ++t) {
+          const bool q = ((created >> t) & 1u) && C[t] != c.own && (int64_t)vals[slot[t]] > oc;
+          up |= q ? 1u << t : 0u;
+          Wk[t] = q ? SCLAP_LD(a.W, C[t], a.nlabels, a.err) : 0;
+          Bk[t] = cand_block(a, c, q, C[t]);
+        }
 #pragma unroll
-      for (int t = 0; t < 4; ++t) {
-        if (!((created >> t) & 1u)) continue;
-        const int64_t conn = (int64_t)vals[slot[t]];
-        if (C[t] == c.own) { oc = conn; has_oc = true; continue; }
-        if (ov || (int64_t)Wk[t] + c.cv > c.bound || Bk[t] != c.vb) continue;
-        const Cand x = make_cand(c, C[t], conn);
-        if (cd.conn < 0 || cand_better(x, cd)) cd = x;
+        for (int t = 0; t < 4; ++t) {
+          if (!((up >> t) & 1u) || (int64_t)Wk[t] + c.cv > c.bound || Bk[t] != c.vb) continue;
+          const Cand x = make_cand(c, C[t], (int64_t)vals[slot[t]]);
+          if (cd.conn < 0 || cand_better(x, cd)) cd = x;
+        }
       }
       if (ov) {
         // an overloaded node may move to any block that fits, connected or not
@@ -670,9 +687,7 @@ __device__ __forceinline__ void propose_warp_node(const LPArgs& a, int64_t i, in
       for (int t = 0; t < 4; ++t)
         if ((created >> t) & 1u) { keys[slot[t]] = -1; vals[slot[t]] = 0; }
     }
-    const unsigned om = __ballot_sync(0xffffffffu, has_oc);
-    oc = om ? __shfl_sync(0xffffffffu, oc, __ffs(om) - 1) : 0;
-    cd = warp_best(cd);
+    if (__any_sync(0xffffffffu, cd.conn >= 0)) cd = warp_best(cd);
     if (lane == 0) write_prop(a, i, c, cd, oc, ov);
     __syncwarp();
   }
@@ -856,49 +871,83 @@ __device__ __forceinline__ void propose_blk_node(const LPArgs& a, int64_t i, int
     }
   }
   tm.sync();
-  long long oc = 0;
+  // the own connection is known to all before any candidate is looked at
+  const int32_t own_l = (int32_t)(c.own - c.loff);
+  long long oc = direct ? (long long)vals[own_l] : table_get(keys, vals, logcap, c.own);
   Cand cd{-1, 0, 0};
+  const int nc = sh.nc;
   if (direct) {
-    const int32_t own_l = (int32_t)(c.own - c.loff);
     for (int32_t b = tid; b < nl; b += NT) {
       const int64_t conn = (int64_t)vals[b];
-      if (b == own_l) { oc = conn; continue; }
-      if (conn == 0 && !ov) continue;
+      if (b == own_l || (conn <= oc && !ov)) continue;
       const int32_t Cb = (int32_t)(c.loff + b);
       if ((int64_t)a.W[Cb] + c.cv > c.bound) continue;
-      Cand x = make_cand(c, Cb, conn);
+      const Cand x = make_cand(c, Cb, conn);
       if (cd.conn < 0 || cand_better(x, cd)) cd = x;
     }
-    tm.sync();
-    for (int32_t b = tid; b < nl; b += NT) vals[b] = 0;
-  } else {
-    const int nc = sh.nc;
+    block_reduce(tm, oc, cd, sh.oc, sh.cd);
+  } else if (!ov) {
+    // the strongest label above the own connection (one read-back of the
+    // team), then, only if it has no room, the strongest of those that have
     for (int j = tid; j < nc; j += NT) {
       const int32_t s = clist[j];
       const int32_t K = keys[s];
       const int64_t conn = (int64_t)vals[s];
-      if (K == c.own) { oc = conn; continue; }
-      if (ov || (int64_t)a.W[K] + c.cv > c.bound) continue;
-      if (cand_block(a, c, true, K) != c.vb) continue;
-      Cand x = make_cand(c, K, conn);
+      if (conn <= oc || K == c.own) continue;
+      const Cand x = make_cand(c, K, conn);
       if (cd.conn < 0 || cand_better(x, cd)) cd = x;
     }
-    if (ov) {
-      for (int32_t b = tid; b < nl; b += NT) {
-        const int32_t Cb = (int32_t)(c.loff + b);
-        if (Cb == c.own || (int64_t)a.W[Cb] + c.cv > c.bound) continue;
-        Cand x = make_cand(c, Cb, table_get(keys, vals, logcap, Cb));
-        if (cd.conn < 0 || cand_better(x, cd)) cd = x;
-      }
-    }
+    block_reduce(tm, oc, cd, sh.oc, sh.cd);
+    if (tid == 0) sh.nc = cd.conn < 0 || cand_fits(a, c, (int32_t)(c.loff + cd.C)) ? 0 : 1;
     tm.sync();
+    if (sh.nc) {
+      cd = Cand{-1, 0, 0};
+      for (int j0 = tid; j0 < nc; j0 += 4 * NT) {
+        int32_t K[4], Wk[4], Bk[4];
+        int64_t conn[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int j = j0 + q * NT;
+          const int32_t s = j < nc ? clist[j] : 0;
+          K[q] = j < nc ? keys[s] : -1;
+          conn[q] = j < nc ? (int64_t)vals[s] : 0;
+          if (conn[q] <= oc || K[q] == c.own) K[q] = -1;
+          // (a label behind the thread's best so far needs no weight)
+          if (K[q] >= 0 && cd.conn >= 0 && !cand_better(make_cand(c, K[q], conn[q]), cd)) K[q] = -1;
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          Wk[q] = K[q] >= 0 ? SCLAP_LD(a.W, K[q], a.nlabels, a.err) : 0;
+          Bk[q] = cand_block(a, c, K[q] >= 0, K[q]);
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          if (K[q] < 0 || (int64_t)Wk[q] + c.cv > c.bound || Bk[q] != c.vb) continue;
+          const Cand x = make_cand(c, K[q], conn[q]);
+          if (cd.conn < 0 || cand_better(x, cd)) cd = x;
+        }
+      }
+      block_reduce(tm, oc, cd, sh.oc, sh.cd);
+    }
+  } else {
+    for (int32_t b = tid; b < nl; b += NT) {
+      const int32_t Cb = (int32_t)(c.loff + b);
+      if (Cb == c.own || (int64_t)a.W[Cb] + c.cv > c.bound) continue;
+      const Cand x = make_cand(c, Cb, table_get(keys, vals, logcap, Cb));
+      if (cd.conn < 0 || cand_better(x, cd)) cd = x;
+    }
+    block_reduce(tm, oc, cd, sh.oc, sh.cd);
+  }
+  // (every thread is past its reads of the table: the reduction's barrier)
+  if (direct) {
+    for (int32_t b = tid; b < nl; b += NT) vals[b] = 0;
+  } else {
     for (int j = tid; j < nc; j += NT) {
       const int32_t s = clist[j];
       keys[s] = -1;
       vals[s] = 0;
     }
   }
-  block_reduce(tm, oc, cd, sh.oc, sh.cd);
   if (tid == 0) {
     write_prop(a, i, c, cd, oc, ov);
     sh.nc = 0;
@@ -928,7 +977,8 @@ __global__ void __launch_bounds__(NT) k_propose_blk(LPArgs a, int32_t sub, int32
 
 // ------------------------------------------------------------------ hubs
 // Hubs (degree above 8192) are split over the grid in two launches.
-//   k_hub_accum   the row of each hub is cut into parts of HUB_PART arcs;
+//   k_hub_accum   the row of each hub is cut into parts of HUB_PART_MIN to
+//                 HUB_PART_MAX arcs, as many as keep the grid busy;
 //                 CTAs take parts in turn and add every arc's weight into
 //                 the hub's table in global memory (its own region of
 //                 hub_table_slots(degree) entries; in local search with few
@@ -943,11 +993,28 @@ __global__ void __launch_bounds__(NT) k_propose_blk(LPArgs a, int32_t sub, int32
 // The table pool is clean (keys -1, sums 0) before the first launch and
 // after every selection.  Results equal the per-node procedure's: the same
 // sums, the same candidates, the same order-free best.
-constexpr int64_t HUB_PART = 16384;
+//
+// When sums fit in 32 bits (narrow levels) a hashed entry is one word, label
+// << 32 | sum: an arc is one random atomic (a claim carries its weight)
+// instead of a claim and an add in two arrays, and selecting reads and
+// resets 8 bytes an entry instead of 12.  Measured, communities of a 1 M-node
+// R-MAT: accumulation 3.6 -> 1.2 ms (part size and packing), selection 1.0 ->
+// 0.8 ms; R-MAT 2^24 nodes: accumulation 70 -> 62 ms.
+constexpr int64_t HUB_PART_MIN = 2048, HUB_PART_MAX = 16384;
 constexpr int HUB_SC = 8192;
 constexpr int HUB_DACC = 1024;
 
+// The tables of the hubs of a class, a region per hub (hoff): packed words for
+// hashed entries of narrow levels, else keys and sums; direct-indexed sums
+// (local search with few labels) always in vals.
+struct HubTab {
+  int32_t* keys;
+  unsigned long long* vals;
+  unsigned long long* packed;
+};
+
 struct HubSel {
+  int64_t* part;      // arcs per accumulation part of the class
   int64_t* hoff;      // [cnt + 1] table regions (exclusive scan of table slots)
   int64_t* hpa;       // [cnt + 1] accumulation parts
   int64_t* hpb;       // [cnt + 1] selection chunks
@@ -965,15 +1032,31 @@ __device__ __forceinline__ bool hub_direct(const LPArgs& a, int32_t nl, int64_t 
 // parts and selection chunks over the class's hub list, with the totals at
 // [cnt]; the done counters are cleared.
 constexpr int HO_NT = 1024;
-__global__ void __launch_bounds__(HO_NT) k_hub_offsets(LPArgs a, int32_t sub, HubSel h) {
+__global__ void __launch_bounds__(HO_NT) k_hub_offsets(LPArgs a, int32_t sub, HubSel h,
+                                                        int32_t nblk) {
   griddep_wait();
   __shared__ int64_t sh[3][HO_NT / 32];
   __shared__ int64_t carry[3];
   int64_t lbeg, cnt;
   sub_range(a, sub, NB - 1, NB, &lbeg, &cnt);
+  __shared__ unsigned long long sh_deg;
   if (threadIdx.x < 3) carry[threadIdx.x] = 0;
+  if (threadIdx.x == 0) sh_deg = 0;
   __syncthreads();
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+  // part size: about two parts per CTA of the accumulation (a class of a
+  // middle-sized level has a few hundred thousand hub arcs: with parts of
+  // 16,384 only some twenty CTAs had any)
+  {
+    unsigned long long d = 0;
+    for (int64_t li = threadIdx.x; li < cnt; li += HO_NT) d += (unsigned long long)a.rec2[lbeg + li].y;
+    for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+    if (lane == 0 && d) atomicAdd(&sh_deg, d);
+  }
+  __syncthreads();
+  const int64_t want = (int64_t)(sh_deg / (unsigned)(2 * nblk)) / HUB_PART_MIN * HUB_PART_MIN;
+  const int64_t part = min64(max64(want, HUB_PART_MIN), HUB_PART_MAX);
+  if (threadIdx.x == 0) *h.part = part;
   int64_t* const out[3] = {h.hoff, h.hpa, h.hpb};
   for (int64_t b0 = 0; b0 < cnt; b0 += HO_NT) {
     const int64_t li = b0 + threadIdx.x;
@@ -985,7 +1068,7 @@ __global__ void __launch_bounds__(HO_NT) k_hub_offsets(LPArgs a, int32_t sub, Hu
       const int32_t nl = a.mode != MODE_CLUSTER ? a.nlab[slot] : 0;
       const int64_t range = hub_direct(a, nl, tcap) ? nl : tcap;
       x[0] = tcap;
-      x[1] = (deg + HUB_PART - 1) / HUB_PART;
+      x[1] = (deg + part - 1) / part;
       x[2] = max64((range + HUB_SC - 1) / HUB_SC, 1);
       h.hdone[li] = 0;
     }
@@ -1035,12 +1118,28 @@ __device__ __forceinline__ int64_t hub_owner(const int64_t* off, int64_t cnt, in
   return lo;
 }
 
+__device__ __forceinline__ unsigned long long hub_word(int32_t label, int32_t w) {
+  return ((unsigned long long)(uint32_t)label << 32) | (uint32_t)w;
+}
+// Sum of a label in a packed table (0: not there).
+__device__ __forceinline__ int64_t packed_get(const unsigned long long* t, int logcap, int32_t C) {
+  const uint32_t mask = (1u << logcap) - 1;
+  uint32_t s = table_slot(C, logcap);
+  for (uint32_t p = 0; p <= mask; ++p) {
+    const unsigned long long x = __ldcg(&t[s]);
+    if (x == ~0ull) return 0;
+    if ((int32_t)(x >> 32) == C) return (int64_t)(x & 0xffffffffull);
+    s = (s + 1) & mask;
+  }
+  return 0;
+}
+
 constexpr size_t hub_accum_smem() {
   return hub_smem_bytes() + (size_t)HUB_DACC * sizeof(unsigned long long);
 }
 
-__global__ void __launch_bounds__(HUB_NT) k_hub_accum(LPArgs a, int32_t sub, int32_t* gkeys,
-                                                      unsigned long long* gvals, HubSel h) {
+__global__ void __launch_bounds__(HUB_NT) k_hub_accum(LPArgs a, int32_t sub, HubTab tb,
+                                                      HubSel h) {
   griddep_wait();
   int64_t lbeg, cnt;
   sub_range(a, sub, NB - 1, NB, &lbeg, &cnt);
@@ -1069,12 +1168,14 @@ __global__ void __launch_bounds__(HUB_NT) k_hub_accum(LPArgs a, int32_t sub, int
   for (int64_t q = blockIdx.x; q < total; q += gridDim.x) {
     const int64_t li = hub_owner(h.hpa, cnt, q);
     const NodeCtx c = load_node(a, lbeg + li);
-    const int64_t p0 = c.rs + (q - h.hpa[li]) * HUB_PART;
-    const int64_t p1 = min64(p0 + HUB_PART, c.re);
+    const int64_t part = *h.part;
+    const int64_t p0 = c.rs + (q - h.hpa[li]) * part;
+    const int64_t p1 = min64(p0 + part, c.re);
     const int64_t deg = c.re - c.rs;
     const int64_t tcap = hub_table_slots(deg);
-    int32_t* keys = gkeys + h.hoff[li];
-    unsigned long long* vals = gvals + h.hoff[li];
+    int32_t* keys = tb.keys + h.hoff[li];
+    unsigned long long* vals = tb.vals + h.hoff[li];
+    unsigned long long* packed = tb.packed + h.hoff[li];
     const int32_t nl = a.mode != MODE_CLUSTER ? a.nlab[c.slot] : 0;
     const bool direct = hub_direct(a, nl, tcap);
     const bool pre = direct && nl <= HUB_DACC;
@@ -1144,6 +1245,43 @@ __global__ void __launch_bounds__(HUB_NT) k_hub_accum(LPArgs a, int32_t sub, int
           if (SCLAP_OK(key, pre ? (int64_t)HUB_DACC : tcap, a.err))
             conn_add(pre ? &sacc[key] : &vals[key], w[u], a.narrow);
         }
+      } else if (a.narrow) {
+        // the four arcs' first reads, then their claims, go out together
+        const uint32_t pmax = a.probe_limit <= mask ? a.probe_limit : mask + 1;
+        uint32_t sl[4];
+        unsigned long long cur[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          sl[u] = C[u] >= 0 ? table_slot(C[u], logcap) : 0;
+          cur[u] = C[u] >= 0 && pmax > 0 ? __ldcg(&packed[sl[u]]) : 0;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (C[u] >= 0 && cur[u] == ~0ull) {
+            cur[u] = atomicCAS(&packed[sl[u]], ~0ull, hub_word(C[u], w[u]));
+            if (cur[u] == ~0ull) C[u] = -1;          // claimed, weight and all
+          }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          if (C[u] < 0) continue;
+          uint32_t s = sl[u];
+          unsigned long long x = cur[u];
+          bool placed = false;
+          for (uint32_t p = 0; p < pmax; ++p) {
+            if (p) {
+              s = (s + 1) & mask;
+              x = __ldcg(&packed[s]);
+              if (x == ~0ull) x = atomicCAS(&packed[s], ~0ull, hub_word(C[u], w[u]));
+              if (x == ~0ull) { placed = true; break; }
+            }
+            if ((int32_t)(x >> 32) == C[u]) {
+              atomicAdd(&packed[s], (unsigned long long)(uint32_t)w[u]);
+              placed = true;
+              break;
+            }
+          }
+          if (!placed) atomicOr(a.err, DERR_HASH_FULL);
+        }
       } else {
         // the four arcs' first probes are independent: issue them together
         const uint32_t pmax = a.probe_limit <= mask ? a.probe_limit : mask + 1;
@@ -1198,8 +1336,8 @@ __device__ __forceinline__ Cand ld_cand_cg(const Cand* p) {
   return c;
 }
 
-__global__ void __launch_bounds__(HUB_NT) k_hub_select(LPArgs a, int32_t sub, int32_t* gkeys,
-                                                       unsigned long long* gvals, HubSel h) {
+__global__ void __launch_bounds__(HUB_NT) k_hub_select(LPArgs a, int32_t sub, HubTab tb,
+                                                       HubSel h) {
   griddep_wait();
   int64_t lbeg, cnt;
   sub_range(a, sub, NB - 1, NB, &lbeg, &cnt);
@@ -1215,8 +1353,9 @@ __global__ void __launch_bounds__(HUB_NT) k_hub_select(LPArgs a, int32_t sub, in
     const NodeCtx c = load_node(a, i);
     const int64_t q0 = h.hpb[li], nchunks = h.hpb[li + 1] - q0;
     const int64_t tcap = hub_table_slots(c.re - c.rs);
-    int32_t* keys = gkeys + h.hoff[li];
-    unsigned long long* vals = gvals + h.hoff[li];
+    int32_t* keys = tb.keys + h.hoff[li];
+    unsigned long long* vals = tb.vals + h.hoff[li];
+    unsigned long long* packed = tb.packed + h.hoff[li];
     const int32_t nl = a.mode != MODE_CLUSTER ? a.nlab[c.slot] : 0;
     const bool direct = hub_direct(a, nl, tcap);
     const bool ov = a.mode != MODE_CLUSTER && a.W[c.own] > c.bound;
@@ -1238,33 +1377,53 @@ __global__ void __launch_bounds__(HUB_NT) k_hub_select(LPArgs a, int32_t sub, in
       }
     } else if (!ov) {
       // four entries per thread at a time: their loads, then their label
-      // weight gathers, are in flight together
+      // weight gathers, are in flight together.  A label needs its weight only
+      // if it beats the own connection (as far as it can be seen: another
+      // chunk may already have reset that entry, which then counts as 0).
       const int64_t j1 = min64(j0 + HUB_SC, tcap);
+      const int64_t hint = a.narrow ? packed_get(packed, ceil_log2(tcap), c.own) : 0;
       for (int64_t s0 = j0; s0 < j1; s0 += 4 * HUB_NT) {
         int32_t K[4];
         int64_t conn[4];
         wgt_t WK[4];
+        bool need[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
           const int64_t sx = s0 + (int64_t)u * HUB_NT + tid;
-          K[u] = sx < j1 ? keys[sx] : -1;
+          if (a.narrow) {
+            const unsigned long long x = sx < j1 ? packed[sx] : ~0ull;
+            K[u] = x == ~0ull ? -1 : (int32_t)(x >> 32);
+            conn[u] = (int64_t)(x & 0xffffffffull);
+          } else {
+            K[u] = sx < j1 ? keys[sx] : -1;
+          }
+        }
+        if (!a.narrow) {
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const int64_t sx = s0 + (int64_t)u * HUB_NT + tid;
+            conn[u] = K[u] >= 0 ? (int64_t)vals[sx] : 0;
+          }
         }
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-          const int64_t sx = s0 + (int64_t)u * HUB_NT + tid;
-          conn[u] = K[u] >= 0 ? (int64_t)vals[sx] : 0;
-          WK[u] = K[u] >= 0 && K[u] != c.own ? SCLAP_LD(a.W, K[u], a.nlabels, a.err) : 0;
+          need[u] = K[u] >= 0 && K[u] != c.own && conn[u] > hint;
+          WK[u] = need[u] ? SCLAP_LD(a.W, K[u], a.nlabels, a.err) : 0;
         }
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
           if (K[u] < 0) continue;
           const int64_t sx = s0 + (int64_t)u * HUB_NT + tid;
-          keys[sx] = -1;
-          vals[sx] = 0;
+          if (a.narrow) {
+            packed[sx] = ~0ull;
+          } else {
+            keys[sx] = -1;
+            vals[sx] = 0;
+          }
           if (K[u] == c.own) { oc = conn[u]; continue; }
-          if ((int64_t)WK[u] + c.cv > c.bound) continue;
+          if (!need[u] || (int64_t)WK[u] + c.cv > c.bound) continue;
           if (cand_block(a, c, true, K[u]) != c.vb) continue;
-          Cand x = make_cand(c, K[u], conn[u]);
+          const Cand x = make_cand(c, K[u], conn[u]);
           if (cd.conn < 0 || cand_better(x, cd)) cd = x;
         }
       }
@@ -1286,17 +1445,24 @@ __global__ void __launch_bounds__(HUB_NT) k_hub_select(LPArgs a, int32_t sub, in
         // with more blocks than table entries): every label is a candidate,
         // its connection looked up; the chunks left the table to this CTA
         const int logcap = ceil_log2(tcap);
-        oc = table_get(keys, vals, logcap, c.own);
+        auto get = [&](int32_t C) {
+          return a.narrow ? packed_get(packed, logcap, C) : table_get(keys, vals, logcap, C);
+        };
+        oc = get(c.own);
         for (int32_t b = tid; b < nl; b += HUB_NT) {
           const int32_t Cb = (int32_t)(c.loff + b);
           if (Cb == c.own || (int64_t)a.W[Cb] + c.cv > c.bound) continue;
-          Cand x = make_cand(c, Cb, table_get(keys, vals, logcap, Cb));
+          Cand x = make_cand(c, Cb, get(Cb));
           if (cd.conn < 0 || cand_better(x, cd)) cd = x;
         }
         __syncthreads();
         for (int64_t s = tid; s < tcap; s += HUB_NT) {
-          keys[s] = -1;
-          vals[s] = 0;
+          if (a.narrow) {
+            packed[s] = ~0ull;
+          } else {
+            keys[s] = -1;
+            vals[s] = 0;
+          }
         }
       } else {
         for (int64_t k = tid; k < nchunks; k += HUB_NT) {
@@ -2815,20 +2981,33 @@ void lp_run(const LevelView& lv, const SlotParams& sp, int32_t* label, wgt_t* W,
   // level).
   int64_t pool_slots = 0;
   DevBuf<int32_t> gkeys, hub_done;
-  DevBuf<unsigned long long> gvals;
+  DevBuf<unsigned long long> gvals, gpacked;
   DevBuf<int64_t> hub_off;
   DevBuf<Cand> hub_pcd;
   DevBuf<long long> hub_poc;
   HubSel hs{};
   int gblocks = 0;
-  // the pool starts clean (keys -1, sums 0); every selection leaves it so
+  // the pool starts clean (keys -1, sums 0, packed words ~0); every selection
+  // leaves it so.  Hashed entries are needed when clustering, and in local
+  // search with more labels than the smallest hub's table has slots.
+  const bool hub_hash = run.mode == MODE_CLUSTER ||
+                        sp.max_nlab > hub_table_slots(B7_MAXDEG + 1);
   auto ensure_pool = [&](int64_t slots) {
     if (slots <= pool_slots) return;
     slots = std::max<int64_t>(slots, 1024);
-    gkeys.alloc((size_t)slots, s);
-    gvals.alloc((size_t)slots, s);
-    gkeys.fill_bytes(0xff);
-    gvals.zero();
+    if (hub_hash) {
+      if (lv.narrow) {
+        gpacked.alloc((size_t)slots, s);
+        gpacked.fill_bytes(0xff);
+      } else {
+        gkeys.alloc((size_t)slots, s);
+        gkeys.fill_bytes(0xff);
+      }
+    }
+    if (run.mode != MODE_CLUSTER || !lv.narrow) {
+      gvals.alloc((size_t)slots, s);
+      gvals.zero();
+    }
     pool_slots = slots;
   };
 
@@ -2896,7 +3075,7 @@ void lp_run(const LevelView& lv, const SlotParams& sp, int32_t* label, wgt_t* W,
     // per hub of a class: offsets of its table, parts and selection chunks
     // (three arrays), its done counter; per selection chunk (at most one per
     // HUB_SC table slots of the level's hubs, plus one per hub): its best
-    hub_off.alloc((size_t)(3 * (nhubs + 1)), s);
+    hub_off.alloc((size_t)(3 * (nhubs + 1) + 1), s);
     hub_done.alloc((size_t)nhubs, s);
     const int64_t nchunk = hub_slots / HUB_SC + nhubs + 1;
     hub_pcd.alloc((size_t)nchunk, s);
@@ -2904,6 +3083,7 @@ void lp_run(const LevelView& lv, const SlotParams& sp, int32_t* label, wgt_t* W,
     hs.hoff = hub_off.p;
     hs.hpa = hub_off.p + (nhubs + 1);
     hs.hpb = hub_off.p + 2 * (nhubs + 1);
+    hs.part = hub_off.p + 3 * (nhubs + 1);
     hs.hdone = hub_done.p;
     hs.pcd = hub_pcd.p;
     hs.poc = hub_poc.p;
@@ -3035,9 +3215,10 @@ void lp_run(const LevelView& lv, const SlotParams& sp, int32_t* label, wgt_t* W,
       SCLAP_NOTE_LAUNCH("k_propose_blk512");
     });
     if (need[8]) launch(8, 9, 3, [&](cudaStream_t ls, bool p) {
-      launch_k(p, k_hub_offsets, 1, HO_NT, 0, ls, a, sub, hs); SCLAP_NOTE_LAUNCH("k_hub_offsets");
-      launch_k(tu.pdl != 0, k_hub_accum, (unsigned)gblocks, HUB_NT, hub_accum_smem(), ls, a, sub, gkeys.p, gvals.p, hs); SCLAP_NOTE_LAUNCH("k_hub_accum");
-      launch_k(tu.pdl != 0, k_hub_select, (unsigned)gblocks, HUB_NT, 0, ls, a, sub, gkeys.p, gvals.p, hs); SCLAP_NOTE_LAUNCH("k_hub_select");
+      launch_k(p, k_hub_offsets, 1, HO_NT, 0, ls, a, sub, hs, gblocks); SCLAP_NOTE_LAUNCH("k_hub_offsets");
+      const HubTab tb{gkeys.p, gvals.p, gpacked.p};
+      launch_k(tu.pdl != 0, k_hub_accum, (unsigned)gblocks, HUB_NT, hub_accum_smem(), ls, a, sub, tb, hs); SCLAP_NOTE_LAUNCH("k_hub_accum");
+      launch_k(tu.pdl != 0, k_hub_select, (unsigned)gblocks, HUB_NT, 0, ls, a, sub, tb, hs); SCLAP_NOTE_LAUNCH("k_hub_select");
     });
     if (fork) {
       for (int j = 0; j < nside; ++j) {
