@@ -751,6 +751,11 @@ void ggg_trials(const GGGArgs& a, const std::vector<int64_t>& noff,
                 const std::vector<int32_t>& nlab, cudaStream_t s);
 // cut2[slot] += twice the cut of each slot (arcs counted from both ends).
 void slot_cut(const LevelView& lv, const int32_t* label, int64_t* cut2, cudaStream_t s);
+// The same for a level of B graphs with T trials each (slot g * T + t), which
+// all have their graph's structure; every block id is below max_k.
+void trial_cuts(const LevelView& lv, int B, int T, const std::vector<int64_t>& noff,
+                const std::vector<int64_t>& aoff, const int64_t* d_boff, int32_t max_k,
+                const int32_t* label, int64_t* cut2, cudaStream_t s);
 struct SelectTask {            // choose the best trial of one graph, copy it out
   int32_t* dst_blk;            // level array of the graph's coarsest level
   int64_t dst_n0, n;

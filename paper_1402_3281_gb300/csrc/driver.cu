@@ -692,7 +692,7 @@ void run_ip(const std::vector<IPIn>& in, const sclap_config& cfg, wgt_t* Wg,
 
   DevBuf<int64_t> cut2(S, s);
   cut2.zero();
-  slot_cut(ip.view(), label.p, cut2.p, s);
+  trial_cuts(ip.view(), B, T, noff, aoff, d_boff.p, sl.sp.max_nlab, label.p, cut2.p, s);
   std::vector<SelectTask> sel(B);
   for (int g = 0; g < B; ++g) {
     const Level& Q = *in[g].Q;

@@ -34,3 +34,37 @@ def test_growing_at_bitmap_edges(n, k, trials):
                                               cfg=P.default_config(**kw))
     assert (cut, best) == (ocut, obest)
     assert np.array_equal(tb.cpu().numpy(), ob)
+
+
+# cuts of all trials from one pass over long arc lists: 16 trials fill a word,
+# 17 take a second one; more than 256 blocks and short batches take a pass per trial
+@pytest.mark.parametrize("scale,factor,trials", [(17, 9, 2), (14, 10, 15), (14, 10, 16), (14, 10, 17),
+                                                 (13, 10, 33), (11, 8, 16)])
+@pytest.mark.parametrize("k", [2, 255, 256, 257])
+def test_best_trial_by_cut(k, scale, factor, trials):
+    import paper_1402_3281_gb300 as P
+    g = gg.random_weights(gg.rmat(scale, factor, 8), 3, max_edge_w=50)
+    cV = int(g.node_w.sum())
+    avg = -(-cV // k)
+    Lmax = O.bounds(cV, int(g.node_w.max()), k, 0.1)[0]
+    kw = dict(ip_trials=trials, lp_rounds_refine=2)
+    ob, ocut, obest = O.initial_partition(g, k, Lmax, avg, seed=3, level=1, cfg=O.config(**kw))
+    tb, cut, best = P.sclap_initial_partition(_dev(g.row_ptr), _dev(g.col), _dev(g.node_w),
+                                              _dev(g.edge_w), k, Lmax, avg, 3, 1,
+                                              cfg=P.default_config(**kw))
+    assert (cut, best) == (ocut, obest)
+    assert np.array_equal(tb.cpu().numpy(), ob)
+
+
+# two graphs of one batch: each one's arcs and packed words start inside the lists
+def test_best_trial_by_cut_batched():
+    import paper_1402_3281_gb300 as P
+    gs = [gg.random_weights(gg.rmat(14, f, s), s, max_edge_w=50) for f, s in ((9, 4), (7, 5), (8, 6))]
+    kw = dict(ip_trials=16, lp_rounds_refine=2, coarse_min_nodes=1 << 15)
+    items = [dict(row_ptr=_dev(g.row_ptr), col=_dev(g.col), node_w=_dev(g.node_w),
+                  edge_w=_dev(g.edge_w), k=k, eps=0.1, seed=k) for g, k in zip(gs, (3, 5, 16))]
+    res = P.sclap_partition_batch(items, cfg=P.default_config(**kw), device=True)
+    for g, k, r in zip(gs, (3, 5, 16), res):
+        ref = O.partition(g, k, 0.1, seed=k, cfg=O.config(**kw))
+        assert (r.status, r.cut) == (ref.status, ref.cut)
+        assert np.array_equal(r.block.cpu().numpy(), ref.block)
