@@ -698,7 +698,7 @@ void contract_build(const LevelView& lv, const std::vector<int64_t>& noff, const
 
 // ip.cu -- initial partitioning of the coarsest graphs (all trials of all
 // graphs in one batch), cut, projection.
-struct CopyTask {              // copy one graph segment (NULL weights -> unit)
+struct CopyTask {              // copies of one graph segment (NULL weights -> unit)
   const int64_t* row_ptr;
   const int32_t* col;
   const int32_t* ew;
@@ -709,12 +709,10 @@ struct CopyTask {              // copy one graph segment (NULL weights -> unit)
   // are dropped.  NULL: plain copy.
   const int64_t* rank;
   int64_t rbase;
-  int64_t nd;                  // nodes written (renumbered tasks; 0: n)
+  int64_t nd;                  // nodes written per copy
+  int64_t copies;              // laid out back to back, nd nodes and m arcs apart
 };
-// Copies graph segments; row_ptr[N_total] = M_total.  Tasks with the same
-// source segment (the trials of one graph) are copied once from the source
-// and then from that first copy, with the node and arc offsets shifted (a
-// streaming copy instead of one renumbering gather per arc).  N_total_override < 0:
+// Copies graph segments; row_ptr[N_total] = M_total.  N_total_override < 0:
 // the end of the last plain task.  ew / nw may be NULL: the destination
 // level keeps no weight array (unit weights).
 void ip_replicate(const std::vector<CopyTask>& tasks, int64_t* row_ptr, int32_t* col,

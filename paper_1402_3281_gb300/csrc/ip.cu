@@ -9,9 +9,6 @@
 // the whole trial batch).  The best trial by (overload, cut, trial) is kept.
 #include <algorithm>
 
-#include <map>
-#include <tuple>
-
 #include "arcs.cuh"
 
 namespace sclap {
@@ -25,26 +22,68 @@ constexpr int GPER = 8;   // consecutive nodes per thread in the greedy-growing 
 // wide CTAs, which have the registers and run on few trials)
 template <int GNT> struct Garc { static constexpr int value = GNT >= 512 ? 8 : 4; };
 
-__global__ void k_replicate(const CopyTask* __restrict__ tasks, int64_t* __restrict__ row_ptr,
-                            int32_t* __restrict__ col, int32_t* __restrict__ ew,
-                            int32_t* __restrict__ nw) {
+// All copies of a graph segment from one read of it: a thread holds RP_PER
+// arcs and stores them once per copy, so a graph with 16 trials moves 17
+// streams instead of 31 and its neighbours are renumbered once.  Bound by the
+// stores; four arcs in flight per thread cover the rank gather.  blockIdx.z
+// shares out the copies where a segment alone has too few tiles for the chip.
+// Two passes (copy, then copies of the copy) -> this: 16 copies of an R-MAT
+// graph of 2^22 nodes 2.35 -> 1.1 ms, of 512 small graphs 1.45 -> 0.72 ms.
+constexpr int RP_NT = 256, RP_PER = 4;
+__global__ void __launch_bounds__(RP_NT) k_replicate(const CopyTask* __restrict__ tasks,
+                                                     int64_t* __restrict__ row_ptr,
+                                                     int32_t* __restrict__ col,
+                                                     int32_t* __restrict__ ew,
+                                                     int32_t* __restrict__ nw) {
   const CopyTask t = tasks[blockIdx.y];
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < t.n; v += stride) {
-    int64_t d = v;
-    if (t.rank) {
-      const int64_t r0 = t.rank[t.src_n0 + v];
-      if (t.rank[t.src_n0 + v + 1] == r0) continue;   // isolated: dropped
-      d = r0 - t.rbase;
+  const int64_t tile = RP_NT * RP_PER, stride = (int64_t)gridDim.x * tile;
+  const int c0 = (int)blockIdx.z, cs = (int)gridDim.z;
+  for (int64_t b = (int64_t)blockIdx.x * tile; b < t.n; b += stride) {
+    int64_t d[RP_PER], r[RP_PER];
+    int32_t w[RP_PER];
+#pragma unroll
+    for (int i = 0; i < RP_PER; ++i) {
+      const int64_t v = b + i * RP_NT + threadIdx.x;
+      const bool in = v < t.n;
+      d[i] = in ? v : -1;
+      r[i] = in ? t.row_ptr[t.src_n0 + v] - t.src_a0 : 0;
+      w[i] = in && nw ? wat(t.nw, t.src_n0 + v) : 0;
+      if (in && t.rank) {
+        const int64_t x = t.rank[t.src_n0 + v];
+        d[i] = t.rank[t.src_n0 + v + 1] == x ? -1 : x - t.rbase;   // isolated: dropped
+      }
     }
-    row_ptr[t.dst_n0 + d] = t.dst_a0 + (t.row_ptr[t.src_n0 + v] - t.src_a0);
-    if (nw) nw[t.dst_n0 + d] = wat(t.nw, t.src_n0 + v);
+    for (int64_t c = c0; c < t.copies; c += cs) {
+      const int64_t n0 = t.dst_n0 + c * t.nd, a0 = t.dst_a0 + c * t.m;
+#pragma unroll
+      for (int i = 0; i < RP_PER; ++i)
+        if (d[i] >= 0) {
+          row_ptr[n0 + d[i]] = a0 + r[i];
+          if (nw) nw[n0 + d[i]] = w[i];
+        }
+    }
   }
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < t.m; e += stride) {
-    const int64_t u = t.col[t.src_a0 + e];
-    const int64_t du = t.rank ? t.rank[u] - t.rbase : u - t.src_n0;
-    col[t.dst_a0 + e] = (int32_t)(du + t.dst_n0);
-    if (ew) ew[t.dst_a0 + e] = wat(t.ew, t.src_a0 + e);
+  for (int64_t b = (int64_t)blockIdx.x * tile; b < t.m; b += stride) {
+    int64_t u[RP_PER];
+    int32_t w[RP_PER];
+#pragma unroll
+    for (int i = 0; i < RP_PER; ++i) {
+      const int64_t e = b + i * RP_NT + threadIdx.x;
+      u[i] = e < t.m ? (int64_t)t.col[t.src_a0 + e] : t.src_n0;
+      w[i] = e < t.m && ew ? wat(t.ew, t.src_a0 + e) : 0;
+    }
+#pragma unroll
+    for (int i = 0; i < RP_PER; ++i)
+      u[i] = t.rank ? t.rank[u[i]] - t.rbase : u[i] - t.src_n0;   // (unchecked input: any int32)
+    for (int64_t c = c0; c < t.copies; c += cs) {
+      const int64_t n0 = t.dst_n0 + c * t.nd, a0 = t.dst_a0 + c * t.m + b + threadIdx.x;
+#pragma unroll
+      for (int i = 0; i < RP_PER; ++i)
+        if (b + i * RP_NT + threadIdx.x < t.m) {
+          col[a0 + i * RP_NT] = (int32_t)(u[i] + n0);
+          if (ew) ew[a0 + i * RP_NT] = w[i];
+        }
+    }
   }
 }
 
@@ -888,9 +927,9 @@ __global__ void __launch_bounds__(AT_NT, AT_CTAS) k_slot_cut(const int64_t* __re
 // block ids of a node in TC of the trials lie side by side in one 16-byte word
 // (blocks fit a byte): an arc gathers one word for all of them instead of one
 // label per trial.  Bound by streaming the arcs (8 bytes each, once per TC
-// trials).  16 trials, per-trial streams -> one: 16.8 M nodes (the whole web
-// graph of the benchmark cut to its coarsest level) 28.0 -> 3.2 ms, an R-MAT
-// graph of 2^22 nodes 2.54 -> 0.34 ms, 512 small graphs 0.73 -> 0.19 ms.
+// trials).  16 trials, per-trial streams -> one: a web graph of 2^24 nodes
+// 28.0 -> 3.2 ms, an R-MAT graph of 2^22 nodes 2.54 -> 0.34 ms, 512 small
+// graphs 0.73 -> 0.19 ms.
 constexpr int TC = 16;
 constexpr int64_t TC_MIN_ARCS = (int64_t)4 << 20;   // over all trials
 struct TrialCut {
@@ -1189,45 +1228,21 @@ void ip_replicate(const std::vector<CopyTask>& tasks, int64_t* row_ptr, int32_t*
                   int32_t* ew, int32_t* nw, int64_t M_total, cudaStream_t s,
                   int64_t N_total_override) {
   if (tasks.empty()) return;
-  // the first task of each source segment copies from the source, the
-  // others from that copy
-  std::vector<CopyTask> first;
-  std::vector<CopyFrom> later;
-  std::map<std::tuple<const void*, int64_t, int64_t, int64_t, const void*, int64_t>, size_t> seen;
+  DevBuf<CopyTask> d(tasks.size(), s);
+  d.upload(tasks);
+  int64_t mx = 1, copies = 1;
   for (const auto& t : tasks) {
-    const auto key = std::make_tuple((const void*)t.col, t.src_n0, t.src_a0, t.m,
-                                     (const void*)t.rank, t.rbase);
-    const auto it = seen.find(key);
-    if (it == seen.end()) {
-      seen.emplace(key, first.size());
-      first.push_back(t);
-    } else {
-      const CopyTask& f = first[it->second];
-      later.push_back(CopyFrom{t.dst_n0, t.dst_a0, f.dst_n0, f.dst_a0, t.nd ? t.nd : t.n, t.m});
-    }
+    mx = std::max(mx, std::max(t.n, t.m));
+    copies = std::max<int64_t>(copies, t.copies);
   }
-  DevBuf<CopyTask> d(first.size(), s);
-  d.upload(first);
-  int64_t mx = 1;
-  for (const auto& t : first) mx = std::max(mx, std::max(t.n, t.m));
-  // at least 64 CTAs per task, more when few tasks would leave SMs idle
-  const int64_t per_task = std::max<int64_t>(64, (int64_t)num_sms() * 8 / (int64_t)first.size());
-  for (size_t t0 = 0; t0 < first.size(); t0 += 65535) {
-    const unsigned ny = (unsigned)std::min<size_t>(65535, first.size() - t0);
-    dim3 grid(grid_for(mx, 256, per_task), ny);
-    k_replicate<<<grid, 256, 0, s>>>(d.p + t0, row_ptr, col, ew, nw); SCLAP_NOTE_LAUNCH("k_replicate");
-  }
-  DevBuf<CopyFrom> dl(std::max<size_t>(later.size(), 1), s);
-  if (!later.empty()) {
-    dl.upload(later);
-    int64_t ml = 1;
-    for (const auto& t : later) ml = std::max(ml, std::max(t.nd, t.m));
-    const int64_t per_l = std::max<int64_t>(64, (int64_t)num_sms() * 8 / (int64_t)later.size());
-    for (size_t t0 = 0; t0 < later.size(); t0 += 65535) {
-      const unsigned ny = (unsigned)std::min<size_t>(65535, later.size() - t0);
-      dim3 grid(grid_for(ml, 256, per_l), ny);
-      k_replicate_from<<<grid, 256, 0, s>>>(dl.p + t0, row_ptr, col, ew, nw); SCLAP_NOTE_LAUNCH("k_replicate_from");
-    }
+  // at least 64 CTAs per task, more when few tasks would leave SMs idle; short
+  // segments share out the copies until the chip has eight CTAs per SM
+  const int64_t want = (int64_t)num_sms() * 8, nt = (int64_t)tasks.size();
+  const int gx = grid_for(mx, RP_NT * RP_PER, std::max<int64_t>(64, want / nt));
+  const unsigned nz = (unsigned)std::min<int64_t>(copies, std::max<int64_t>(1, want / (gx * nt)));
+  for (size_t t0 = 0; t0 < tasks.size(); t0 += 65535) {
+    const unsigned ny = (unsigned)std::min<size_t>(65535, tasks.size() - t0);
+    k_replicate<<<dim3(gx, ny, nz), RP_NT, 0, s>>>(d.p + t0, row_ptr, col, ew, nw); SCLAP_NOTE_LAUNCH("k_replicate");
   }
   int64_t Ntot = 0;
   for (const auto& t : tasks) {

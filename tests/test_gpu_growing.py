@@ -68,3 +68,38 @@ def test_best_trial_by_cut_batched():
         ref = O.partition(g, k, 0.1, seed=k, cfg=O.config(**kw))
         assert (r.status, r.cut) == (ref.status, ref.cut)
         assert np.array_equal(r.block.cpu().numpy(), ref.block)
+
+
+# copies of a segment: its own weights and offsets, tiles of 1024 arcs, one or many trials
+@pytest.mark.parametrize("trials", [1, 2, 5, 16])
+def test_copies_of_graphs_that_share_arrays(trials):
+    import paper_1402_3281_gb300 as P
+    base = gg.rmat(10, 6, 2)
+    rp, col = _dev(base.row_ptr), _dev(base.col)
+    gs = [gg.random_weights(base, s, max_edge_w=40) for s in (1, 2, 3)]
+    kw = dict(ip_trials=trials)
+    items = [dict(row_ptr=rp, col=col, node_w=_dev(g.node_w), edge_w=_dev(g.edge_w), k=k,
+                  eps=0.1, seed=k) for g, k in zip(gs, (2, 3, 4))]
+    items.append(dict(row_ptr=rp, col=col, k=5, eps=0.1, seed=5))
+    res = P.sclap_partition_batch(items, cfg=P.default_config(**kw), device=True)
+    for g, k, r in zip(gs + [base], (2, 3, 4, 5), res):
+        ref = O.partition(g, k, 0.1, seed=k, cfg=O.config(**kw))
+        assert (r.status, r.cut) == (ref.status, ref.cut)
+        assert np.array_equal(r.block.cpu().numpy(), ref.block)
+
+
+@pytest.mark.parametrize("n", [1023, 1024, 1025])
+@pytest.mark.parametrize("trials", [1, 3, 40])
+def test_copies_at_tile_edges(n, trials):
+    import paper_1402_3281_gb300 as P
+    g = gg.random_weights(gg.rgg2d(n, seed=4), 5)
+    k = 3
+    cV = int(g.node_w.sum())
+    Lmax = O.bounds(cV, int(g.node_w.max()), k, 0.2)[0]
+    ob, ocut, obest = O.initial_partition(g, k, Lmax, -(-cV // k), seed=3, level=1,
+                                          cfg=O.config(ip_trials=trials))
+    tb, cut, best = P.sclap_initial_partition(_dev(g.row_ptr), _dev(g.col), _dev(g.node_w),
+                                              _dev(g.edge_w), k, Lmax, -(-cV // k), 3, 1,
+                                              cfg=P.default_config(ip_trials=trials))
+    assert (cut, best) == (ocut, obest)
+    assert np.array_equal(tb.cpu().numpy(), ob)
