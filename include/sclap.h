@@ -35,9 +35,11 @@
  *
  * Errors: every function returns SCLAP_OK (0) or a negative SCLAP_E* code;
  * sclap_error_string() describes it.  No exception crosses the ABI.  The only
- * device-side waits are the grid barriers of the cooperative admission kernel
- * (tuning field fused_admission); they are bounded, and one that runs out
- * ends the call with SCLAP_ETIMEOUT.  Every other device loop is bounded by
+ * device-side waits are the grid barriers of the cooperative kernels (the
+ * persistent rounds of small levels, grouped greedy growing, the admission
+ * with the tuning field fused_admission) and the arrival of a hub row's bulk
+ * copies; they are bounded, and one that runs out ends the call with
+ * SCLAP_ETIMEOUT.  Every other device loop is bounded by
  * its data size.
  */
 #ifndef SCLAP_H
@@ -72,7 +74,9 @@ enum {
  * at the end of the round, so the host neither waits nor decides between
  * rounds (it then launches every bucket's kernel; empty ones exit at once).
  * 0 (default) drives the rounds from the host, which reads the bucket sizes
- * once per round and skips empty launches.  Results are identical.
+ * once per round and skips empty launches; a level of at most 1.25 M nodes
+ * and 16 M arcs without rows above 8192 runs all its rounds in one
+ * persistent launch instead.  Results are identical.
  * ensemble = 1 turns on ensemble clusterings during coarsening (Sec. 4
  * "Ensemble Clusterings", configuration E): every level computes l
  * clusterings (the first with the run's seed, clustering j >= 1 with the key
@@ -342,7 +346,7 @@ int sclap_cut_static(int64_t n, const int64_t* row_ptr, const int32_t* col,
 /* ---- Host-side fault injection for tests (no counterpart in the paper).
  * Makes the library's own failure paths run without faulting the GPU:
  *   wait_limit   iteration limit of every bounded device-side wait (the grid
- *                barriers of the admission kernel, ~0.5 us per iteration);
+ *                barriers of the cooperative kernels, ~0.5 us per iteration);
  *                0 restores the default (2^22, about two seconds).  A small
  *                value makes the waits run out: the call returns
  *                SCLAP_ETIMEOUT, and the library stays usable.
@@ -389,7 +393,9 @@ int sclap_check_selftest(void* stream);
  *                      run as one cooperative launch whose phases are
  *                      separated by bounded grid-wide barriers (a barrier
  *                      that waits too long ends the call with
- *                      SCLAP_ETIMEOUT); 0: a chain of six launches
+ *                      SCLAP_ETIMEOUT); 0: a chain of launches, three
+ *                      per colour class (eight where a block may be
+ *                      above its bound)
  *   contract_table_slots  slots of the contraction table per pass: a level
  *                      whose table is larger is contracted in passes over
  *                      ranges of coarse nodes (same result); 0: automatic,
@@ -404,6 +410,8 @@ int sclap_check_selftest(void* stream);
  *                      memory of one contraction pass falls back to the
  *                      hash tables); 0: hash tables (same result up to the
  *                      order of each coarse row's arcs)
+ * The persistent rounds of small levels run with concurrent = 1, pdl = 1 and
+ * fused_admission = 0; any other choice launches every phase.
  * The setting is process-wide; defaults 16, 8, 8, 16, 1, 1, 0, 0, 0, 0. ---- */
 typedef struct sclap_tuning {
   int32_t small_max_deg;

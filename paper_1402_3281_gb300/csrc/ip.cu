@@ -89,30 +89,6 @@ __global__ void __launch_bounds__(RP_NT) k_replicate(const CopyTask* __restrict_
 
 __global__ void k_set_i64(int64_t* p, int64_t v) { *p = v; }
 
-// A later copy of an already copied segment: nodes [0, nd) and arcs
-// [0, m) of the first copy (at tn0 / ta0) to dn0 / da0, row offsets shifted
-// by the arc offset difference and neighbour ids by the node offset
-// difference.
-struct CopyFrom {
-  int64_t dn0, da0, tn0, ta0, nd, m;
-};
-__global__ void k_replicate_from(const CopyFrom* __restrict__ tasks, int64_t* __restrict__ row_ptr,
-                                 int32_t* __restrict__ col, int32_t* __restrict__ ew,
-                                 int32_t* __restrict__ nw) {
-  const CopyFrom t = tasks[blockIdx.y];
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  const int64_t da = t.da0 - t.ta0;
-  const int32_t dn = (int32_t)(t.dn0 - t.tn0);
-  for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < t.nd; v += stride) {
-    row_ptr[t.dn0 + v] = row_ptr[t.tn0 + v] + da;
-    if (nw) nw[t.dn0 + v] = nw[t.tn0 + v];
-  }
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < t.m; e += stride) {
-    col[t.da0 + e] = col[t.ta0 + e] + dn;
-    if (ew) ew[t.da0 + e] = ew[t.ta0 + e];
-  }
-}
-
 // Block-wide inclusive scan of an int64 (all GNT threads call it).
 template <int GNT>
 __device__ int64_t block_incl_scan(int64_t x, int64_t* sh, int64_t* total) {
