@@ -29,6 +29,9 @@ template <int GNT> struct Garc { static constexpr int value = GNT >= 512 ? 8 : 4
 // shares out the copies where a segment alone has too few tiles for the chip.
 // Two passes (copy, then copies of the copy) -> this: 16 copies of an R-MAT
 // graph of 2^22 nodes 2.35 -> 1.1 ms, of 512 small graphs 1.45 -> 0.72 ms.
+// (5 TB/s of stores at 2^22 nodes; 54 GB of copies of a 2^24-node graph take
+// 33 ms either way, 1.6 TB/s: streaming stores, a copy per CTA row, longer
+// tiles and renumbering in a pass of its own gave 28 to 36 ms.)
 constexpr int RP_NT = 256, RP_PER = 4;
 __global__ void __launch_bounds__(RP_NT) k_replicate(const CopyTask* __restrict__ tasks,
                                                      int64_t* __restrict__ row_ptr,
