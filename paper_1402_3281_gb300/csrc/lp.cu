@@ -1652,11 +1652,13 @@ __device__ __forceinline__ void move_warp(const LPArgs& a, ApplyHash& h, MovedRu
 // classes) 1.98 -> 1.57 ms of admission, R-MAT 2^22 nodes 18.5 -> 8.5 ms with
 // the cluster selection below, the 512-graph batch 7.4 -> 7.0 ms.
 //
-// Segment counters: ctr[set * 4 + side * 2 + {0: entry cursor, 1: segments}],
-// set = colour class & 1; a launch clears the other set for the next class
-// (k_round_begin clears both at the start of a round).
-__device__ __forceinline__ int64_t* adm_ctr(const LPArgs& a, int sub, int side) {
-  return a.ctr + (sub & 1) * 4 + side * 2;
+// Segment counters: ctr[set * 4 + side * 2 + {0: entry cursor, 1: segments}].
+// The set alternates from one admitted class to the next (classes without
+// nodes are skipped, so it is not the class number's parity); admitting a
+// class clears the other set for the next (k_round_begin clears both at the
+// start of a round).
+__device__ __forceinline__ int64_t* adm_ctr(const LPArgs& a, int set, int side) {
+  return a.ctr + set * 4 + side * 2;
 }
 
 template <bool APPLY>
@@ -2203,9 +2205,9 @@ constexpr int ADM_NT = 256;
 // first barrier) only the incoming weights are left to clear.
 // source_chain: local search, forced moves out of overloaded blocks are
 // possible this round.
-__global__ void __launch_bounds__(ADM_NT) k_admit(LPArgs a, int32_t sub, int32_t source_chain,
-                                                  GridSync* gs) {
-  if (blockIdx.x == 0 && threadIdx.x < 4) a.ctr[((sub + 1) & 1) * 4 + threadIdx.x] = 0;
+__global__ void __launch_bounds__(ADM_NT) k_admit(LPArgs a, int32_t sub, int32_t set,
+                                                  int32_t source_chain, GridSync* gs) {
+  if (blockIdx.x == 0 && threadIdx.x < 4) a.ctr[(set ^ 1) * 4 + threadIdx.x] = 0;
   // a bounded wait of an earlier launch ran out: the run is abandoned
   if (*(volatile int32_t*)a.err & DERR_TIMEOUT) return;
   __shared__ ApplyHash h;
@@ -2215,7 +2217,7 @@ __global__ void __launch_bounds__(ADM_NT) k_admit(LPArgs a, int32_t sub, int32_t
   int64_t lbeg, cnt;
   sub_range(a, sub, 0, NB, &lbeg, &cnt);
   const uint32_t lim = a.wait_limit;
-  int64_t* ct = adm_ctr(a, sub, 0);
+  int64_t* ct = adm_ctr(a, set, 0);
   const bool chain = source_chain && *(volatile int32_t*)a.flags != 0;
   uint8_t* const an = act_next(a);
   if (chain) adm_resolve<false>(a, &h, sub, an, 0, lbeg, cnt, ct);
@@ -2230,7 +2232,7 @@ __global__ void __launch_bounds__(ADM_NT) k_admit(LPArgs a, int32_t sub, int32_t
   }
   if (chain) {
     if (!grid_sync(gs, a.err, lim)) return;
-    int64_t* cs = adm_ctr(a, sub, 1);
+    int64_t* cs = adm_ctr(a, set, 1);
     adm_forced(a, lbeg, cnt, cs);
     if (!grid_sync(gs, a.err, lim)) return;
     const int64_t nsrc = *(volatile int64_t*)&cs[1];
@@ -2259,47 +2261,49 @@ __global__ void __launch_bounds__(ADM_NT) k_admit(LPArgs a, int32_t sub, int32_t
 __device__ __forceinline__ bool chain_on(const LPArgs& a, int32_t source_chain) {
   return source_chain && *(volatile int32_t*)a.flags != 0;
 }
-__global__ void __launch_bounds__(ADM_NT) k_resolve(LPArgs a, int32_t sub, int32_t source_chain) {
+__global__ void __launch_bounds__(ADM_NT) k_resolve(LPArgs a, int32_t sub, int32_t set,
+                                                    int32_t source_chain) {
   griddep_wait();
   __shared__ ApplyHash h;
-  if (blockIdx.x == 0 && threadIdx.x < 4) a.ctr[((sub + 1) & 1) * 4 + threadIdx.x] = 0;
+  if (blockIdx.x == 0 && threadIdx.x < 4) a.ctr[(set ^ 1) * 4 + threadIdx.x] = 0;
   int64_t lbeg, cnt;
   sub_range(a, sub, 0, NB, &lbeg, &cnt);
   if (chain_on(a, source_chain)) {
-    adm_resolve<false>(a, nullptr, sub, nullptr, 0, lbeg, cnt, adm_ctr(a, sub, 0));
+    adm_resolve<false>(a, nullptr, sub, nullptr, 0, lbeg, cnt, adm_ctr(a, set, 0));
     return;
   }
   apply_init(h);
-  adm_resolve<true>(a, &h, sub, act_next(a), 0, lbeg, cnt, adm_ctr(a, sub, 0));
+  adm_resolve<true>(a, &h, sub, act_next(a), 0, lbeg, cnt, adm_ctr(a, set, 0));
   apply_flush(a, h);
 }
-__global__ void __launch_bounds__(ADM_NT) k_forced(LPArgs a, int32_t sub) {
+__global__ void __launch_bounds__(ADM_NT) k_forced(LPArgs a, int32_t sub, int32_t set) {
   griddep_wait();
   if (!chain_on(a, 1)) return;
   int64_t lbeg, cnt;
   sub_range(a, sub, 0, NB, &lbeg, &cnt);
-  adm_forced(a, lbeg, cnt, adm_ctr(a, sub, 1));
+  adm_forced(a, lbeg, cnt, adm_ctr(a, set, 1));
 }
-__global__ void __launch_bounds__(ADM_NT) k_ovf_alloc(LPArgs a, int32_t sub) {
+__global__ void __launch_bounds__(ADM_NT) k_ovf_alloc(LPArgs a, int32_t set) {
   griddep_wait();
-  int64_t* ct = adm_ctr(a, sub, 1);
+  int64_t* ct = adm_ctr(a, set, 1);
   const int64_t nseg = *(volatile int64_t*)&ct[1];
   if (nseg > 0) adm_alloc(a, nseg, ct);
 }
-__global__ void __launch_bounds__(ADM_NT) k_ovf_scatter(LPArgs a, int32_t sub, int32_t side) {
+__global__ void __launch_bounds__(ADM_NT) k_ovf_scatter(LPArgs a, int32_t sub, int32_t set,
+                                                        int32_t side) {
   griddep_wait();
-  const bool any = *(volatile int64_t*)&adm_ctr(a, sub, side)[1] > 0;
+  const bool any = *(volatile int64_t*)&adm_ctr(a, set, side)[1] > 0;
   int64_t lbeg, cnt;
   sub_range(a, sub, 0, NB, &lbeg, &cnt);
   adm_scatter(a, 0, lbeg, cnt, any, side);
 }
-__global__ void __cluster_dims__(SEL_CL, 1, 1) __launch_bounds__(SEL_NT) k_ovf_select(LPArgs a, int32_t sub, int32_t side,
-                                                       int32_t source_chain) {
+__global__ void __cluster_dims__(SEL_CL, 1, 1) __launch_bounds__(SEL_NT)
+k_ovf_select(LPArgs a, int32_t sub, int32_t set, int32_t side, int32_t source_chain) {
   griddep_wait();
   __shared__ ApplyHash h;
   __shared__ SelState sel;
   __shared__ unsigned long long scr[2 * SEL_PAIRS];
-  const int64_t nseg = *(volatile int64_t*)&adm_ctr(a, sub, side)[1];
+  const int64_t nseg = *(volatile int64_t*)&adm_ctr(a, set, side)[1];
   if (nseg == 0) return;
   if (chain_on(a, source_chain)) {
     adm_select<false, SEL_CL>(a, nullptr, sel, scr, sub, nullptr, nseg, side);
@@ -3248,11 +3252,13 @@ void lp_run(const LevelView& lv, const SlotParams& sp, int32_t* label, wgt_t* W,
   const unsigned grid_adm_max = (unsigned)(sms * tu.admit_ctas_per_sm);
   const unsigned grid_sel = (unsigned)(sms * 2);      // alloc; select: whole clusters
   const unsigned grid_cl = ((unsigned)(sms * 4) + SEL_CL - 1) / SEL_CL * SEL_CL;
-  auto admit = [&](cudaStream_t s, int sub, bool source_chain, int64_t cnt, bool pdl) {
+  // set: the segment counters of the class (adm_ctr), of the last one at first
+  auto admit = [&](cudaStream_t s, int sub, int& set, bool source_chain, int64_t cnt, bool pdl) {
+    set ^= 1;
     if (tu.fused_admission) {
       // one cooperative launch; it follows the propose join: plain launch
       const unsigned grid = cnt < 0 ? grid_adm_coop : grid_for(cnt, ADM_NT, grid_adm_coop);
-      launch_coop(k_admit, grid, ADM_NT, 0, s, a, sub, source_chain ? 1 : 0, gsync);
+      launch_coop(k_admit, grid, ADM_NT, 0, s, a, sub, set, source_chain ? 1 : 0, gsync);
       SCLAP_NOTE_LAUNCH("k_admit");
       if (a.mark_big) { launch_k(false, k_mark_rows, grid_mark, 256, 0, s, a, sub); SCLAP_NOTE_LAUNCH("k_mark_rows"); }
       SCLAP_LAUNCH_CHECK();
@@ -3260,14 +3266,14 @@ void lp_run(const LevelView& lv, const SlotParams& sp, int32_t* label, wgt_t* W,
     }
     const unsigned grid_adm = cnt < 0 ? grid_adm_max : grid_for(cnt, ADM_NT, grid_adm_max);
     const int32_t ch = source_chain ? 1 : 0;
-    launch_k(false, k_resolve, grid_adm, ADM_NT, 0, s, a, sub, ch); SCLAP_NOTE_LAUNCH("k_resolve");
-    launch_k(pdl, k_ovf_scatter, grid_adm, ADM_NT, 0, s, a, sub, 0); SCLAP_NOTE_LAUNCH("k_ovf_scatter");
-    launch_k(pdl, k_ovf_select, grid_cl, SEL_NT, 0, s, a, sub, 0, ch); SCLAP_NOTE_LAUNCH("k_ovf_select");
+    launch_k(false, k_resolve, grid_adm, ADM_NT, 0, s, a, sub, set, ch); SCLAP_NOTE_LAUNCH("k_resolve");
+    launch_k(pdl, k_ovf_scatter, grid_adm, ADM_NT, 0, s, a, sub, set, 0); SCLAP_NOTE_LAUNCH("k_ovf_scatter");
+    launch_k(pdl, k_ovf_select, grid_cl, SEL_NT, 0, s, a, sub, set, 0, ch); SCLAP_NOTE_LAUNCH("k_ovf_select");
     if (source_chain) {
-      launch_k(pdl, k_forced, grid_adm, ADM_NT, 0, s, a, sub); SCLAP_NOTE_LAUNCH("k_forced");
-      launch_k(pdl, k_ovf_alloc, grid_sel, ADM_NT, 0, s, a, sub); SCLAP_NOTE_LAUNCH("k_ovf_alloc");
-      launch_k(pdl, k_ovf_scatter, grid_adm, ADM_NT, 0, s, a, sub, 1); SCLAP_NOTE_LAUNCH("k_ovf_scatter");
-      launch_k(pdl, k_ovf_select, grid_cl, SEL_NT, 0, s, a, sub, 1, ch); SCLAP_NOTE_LAUNCH("k_ovf_select");
+      launch_k(pdl, k_forced, grid_adm, ADM_NT, 0, s, a, sub, set); SCLAP_NOTE_LAUNCH("k_forced");
+      launch_k(pdl, k_ovf_alloc, grid_sel, ADM_NT, 0, s, a, set); SCLAP_NOTE_LAUNCH("k_ovf_alloc");
+      launch_k(pdl, k_ovf_scatter, grid_adm, ADM_NT, 0, s, a, sub, set, 1); SCLAP_NOTE_LAUNCH("k_ovf_scatter");
+      launch_k(pdl, k_ovf_select, grid_cl, SEL_NT, 0, s, a, sub, set, 1, ch); SCLAP_NOTE_LAUNCH("k_ovf_select");
       launch_k(pdl, k_apply, grid_adm, ADM_NT, 0, s, a, sub); SCLAP_NOTE_LAUNCH("k_apply");
     }
     if (a.mark_big) { launch_k(pdl, k_mark_rows, grid_mark, 256, 0, s, a, sub); SCLAP_NOTE_LAUNCH("k_mark_rows"); }
@@ -3321,9 +3327,10 @@ void lp_run(const LevelView& lv, const SlotParams& sp, int32_t* label, wgt_t* W,
         // programmatic launches are captured as programmatic edges
         const bool pdl = tu.pdl != 0;
         head(cs, pdl);
+        int set = 0;
         for (int sub = 0; sub < S; ++sub) {
           propose(cs, sub, tu.concurrent != 0, nullptr, pdl);
-          admit(cs, sub, refine, -1, pdl);
+          admit(cs, sub, set, refine, -1, pdl);
         }
         tail(cs, h, true, pdl);
       } catch (...) {
@@ -3365,6 +3372,7 @@ void lp_run(const LevelView& lv, const SlotParams& sp, int32_t* label, wgt_t* W,
         tail(s, 0, false, pdl);
         break;
       }
+      int set = 0;
       for (int sub = 0; sub < S; ++sub) {
         const int64_t cnt = hoff[(sub + 1) * NB] - hoff[sub * NB];
         if (cnt == 0) continue;
@@ -3383,7 +3391,7 @@ void lp_run(const LevelView& lv, const SlotParams& sp, int32_t* label, wgt_t* W,
           precs.push_back(PhaseRec{run.phase, r, sub, cnt, sub_arcs, phase.a, phase.b,
                                    event_from_pool()});
         }
-        admit(s, sub, refine && hflags != 0, cnt, pdl);
+        admit(s, sub, set, refine && hflags != 0, cnt, pdl);
         if (prof) SCLAP_CUDA(cudaEventRecord(precs.back().c, s));
       }
       tail(s, 0, false, pdl);
