@@ -657,10 +657,10 @@ struct LPRun {
   const int32_t* rblk = nullptr;  // clustering: respect this partition (V-cycles)
 };
 // Runs `run.rounds` synchronous LP rounds on `lv` for every slot not marked
-// done; label/W are updated in place.  Adds the arcs scanned to *d_arcs
-// (device).  The work may still be under way on return.
+// done; label/W are updated in place.  Adds the arcs scanned to
+// arcs[0].  The work may still be under way on return.
 void lp_run(const LevelView& lv, const SlotParams& sp, int32_t* label, wgt_t* W,
-            int64_t Wsize, const LPRun& run, int64_t* d_arcs, int32_t* d_err, cudaStream_t s,
+            int64_t Wsize, const LPRun& run, DevBuf<int64_t>& arcs, int32_t* d_err, cudaStream_t s,
             const uint8_t* active_init = nullptr, uint8_t* active_next_out = nullptr);
 void lp_round_begin_host_keys(const SlotParams& sp, int phase, int r, int mode,
                               const wgt_t* W, cudaStream_t s);

@@ -537,7 +537,7 @@ struct IPIn {
 };
 
 void run_ip(const std::vector<IPIn>& in, const sclap_config& cfg, wgt_t* Wg,
-            std::vector<int32_t>& best, std::vector<int64_t>& ipcut, int64_t* d_arcs,
+            std::vector<int32_t>& best, std::vector<int64_t>& ipcut, DevBuf<int64_t>& arcs,
             int32_t* d_err, cudaStream_t s) {
   const int B = (int)in.size();
   const int T = cfg.ip_trials;
@@ -688,7 +688,7 @@ void run_ip(const std::vector<IPIn>& in, const sclap_config& cfg, wgt_t* Wg,
   run.sub_rounds = cfg.sub_rounds;
   run.graph = cfg.graph_rounds != 0;
   run.use_active = true;
-  lp_run(ip.view(), sl.sp, label.p, W.p, K, run, d_arcs, d_err, s);
+  lp_run(ip.view(), sl.sp, label.p, W.p, K, run, arcs, d_err, s);
 
   DevBuf<int64_t> cut2(S, s);
   cut2.zero();
@@ -860,7 +860,7 @@ void run_valid_batch(const std::vector<GIn>& gs, const std::vector<int64_t>& cV,
       run.graph = cfg.graph_rounds != 0;
       run.use_active = cfg.cluster_active != 0;
       run.rblk = respect ? cur.blk.p : nullptr;
-      lp_run(v, sl->sp, label.p, W.p, v.N, run, d_arcs.p, d_err.p, s);
+      lp_run(v, sl->sp, label.p, W.p, v.N, run, d_arcs, d_err.p, s);
       if (record) recs.push_back(RunRec{std::move(sl), coarsening, L, true});
       if (cfg.ensemble) {
         // ensemble clusterings: clustering j >= 1 of every slot whose ensemble
@@ -885,7 +885,7 @@ void run_valid_batch(const std::vector<GIn>& gs, const std::vector<int64_t>& cV,
             Slots slj(s, B, cur.noff_d.p, h_loff, h_bound, sj, h_level, h_nlab, dj);
             k_iota<<<grid_for(v.N, 256, (int64_t)sms * 16), 256, 0, s>>>(C.p, v.N); SCLAP_NOTE_LAUNCH("k_iota");
             k_w_from_nw<<<grid_for(v.N, 256, (int64_t)sms * 16), 256, 0, s>>>(v.nw, v.N, W.p); SCLAP_NOTE_LAUNCH("k_w_from_nw");
-            lp_run(v, slj.sp, C.p, W.p, v.N, run, d_arcs.p, d_err.p, s);
+            lp_run(v, slj.sp, C.p, W.p, v.N, run, d_arcs, d_err.p, s);
             part.upload(pj);
             overlay_labels(v, part.p, label.p, C.p, d_err.p, s);
           }
@@ -967,7 +967,7 @@ void run_valid_batch(const std::vector<GIn>& gs, const std::vector<int64_t>& cV,
     }
     std::vector<int32_t> best;
     std::vector<int64_t> ipcut;
-    run_ip(in, cfg, Wg.p, best, ipcut, d_arcs.p, d_err.p, s);
+    run_ip(in, cfg, Wg.p, best, ipcut, d_arcs, d_err.p, s);
     for (int g = 0; g < B; ++g) {
       res[g].st.ip_best_trial = best[g];
       res[g].st.ip_cut = ipcut[g];
@@ -1012,7 +1012,7 @@ void run_valid_batch(const std::vector<GIn>& gs, const std::vector<int64_t>& cV,
       run.sub_rounds = cfg.sub_rounds;
       run.graph = cfg.graph_rounds != 0;
       run.use_active = true;
-      lp_run(F.view(), sl->sp, F.blk.p, Wg.p, Ktot, run, d_arcs.p, d_err.p, s);
+      lp_run(F.view(), sl->sp, F.blk.p, Wg.p, Ktot, run, d_arcs, d_err.p, s);
       if (record) {
         std::vector<char> of(B);
         for (int g = 0; g < B; ++g) of[g] = q[g] > L;
@@ -1034,7 +1034,7 @@ void run_valid_batch(const std::vector<GIn>& gs, const std::vector<int64_t>& cV,
     run.sub_rounds = cfg.sub_rounds;
     run.graph = cfg.graph_rounds != 0;
     run.stop_rule = false;
-    lp_run(F0.view(), sl.sp, F0.blk.p, Wg.p, Ktot, run, d_arcs.p, d_err.p, s);
+    lp_run(F0.view(), sl.sp, F0.blk.p, Wg.p, Ktot, run, d_arcs, d_err.p, s);
   };
   {
     std::vector<int32_t> q(B);
@@ -1561,7 +1561,7 @@ int sclap_lp_round(int32_t mode, int64_t n, const int64_t* row_ptr, const int32_
     DevBuf<wgt_t> W32(nlabels, s);
     k_narrow<<<grid_for(nlabels, 256, 1024), 256, 0, s>>>(W, nlabels, W32.p, d_err.p); SCLAP_NOTE_LAUNCH("k_narrow");
     check_err(d_err.p, s);
-    lp_run(L.view(), sl.sp, label, W32.p, nlabels, run, arcs.p, d_err.p, s, active_cur, active_next);
+    lp_run(L.view(), sl.sp, label, W32.p, nlabels, run, arcs, d_err.p, s, active_cur, active_next);
     k_widen<<<grid_for(nlabels, 256, 1024), 256, 0, s>>>(W32.p, nlabels, W); SCLAP_NOTE_LAUNCH("k_widen");
     check_err(d_err.p, s);
     int64_t mv = 0;
@@ -1602,7 +1602,7 @@ int sclap_cluster(int64_t n, const int64_t* row_ptr, const int32_t* col, const i
     d_err.zero();
     DevBuf<int64_t> arcs(1, s);
     arcs.zero();
-    lp_run(L.view(), sl.sp, label_out, W.p, n, run, arcs.p, d_err.p, s);
+    lp_run(L.view(), sl.sp, label_out, W.p, n, run, arcs, d_err.p, s);
     check_err(d_err.p, s);
     if (rounds_out) read_rounds(sl, rounds_out, s);
   });
@@ -1647,7 +1647,7 @@ int sclap_cluster_hierarchy(int64_t n, const int64_t* row_ptr, const int32_t* co
       run.sub_rounds = c.sub_rounds;
       run.graph = c.graph_rounds != 0;
       run.use_active = c.cluster_active != 0;
-      lp_run(v, sl.sp, label.p, W.p, v.N, run, arcs.p, d_err.p, s);
+      lp_run(v, sl.sp, label.p, W.p, v.N, run, arcs, d_err.p, s);
       ContractWork cw;
       std::vector<int64_t> nc;
       contract_rank(v, cur->noff, label.p, cw, nc, s);
@@ -1741,8 +1741,9 @@ int sclap_initial_partition(int64_t n, const int64_t* row_ptr, const int32_t* co
     std::vector<IPIn> in{IPIn{&L, 0, k, Lmax, avg, seed, level, 0, block_out}};
     std::vector<int32_t> best;
     std::vector<int64_t> ipcut;
-    int64_t arcs = 0;
-    run_ip(in, c, Wg.p, best, ipcut, &arcs, d_err.p, s);
+    DevBuf<int64_t> arcs(1, s);
+    arcs.zero();
+    run_ip(in, c, Wg.p, best, ipcut, arcs, d_err.p, s);
     check_err(d_err.p, s);
     if (cut_out) *cut_out = ipcut[0];
     if (best_trial_out) *best_trial_out = best[0];
@@ -1780,7 +1781,7 @@ int sclap_refine(int64_t n, const int64_t* row_ptr, const int32_t* col, const in
     d_err.zero();
     DevBuf<int64_t> arcs(1, s);
     arcs.zero();
-    lp_run(L.view(), sl.sp, block, W.p, k, run, arcs.p, d_err.p, s);
+    lp_run(L.view(), sl.sp, block, W.p, k, run, arcs, d_err.p, s);
     check_err(d_err.p, s);
     if (rounds_out) read_rounds(sl, rounds_out, s);
   });

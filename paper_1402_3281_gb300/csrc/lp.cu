@@ -2886,7 +2886,7 @@ std::string timeline_dump() {
 constexpr int64_t PR_MAX_N = 1250000, PR_MAX_M = 16000000;
 
 void lp_run(const LevelView& lv, const SlotParams& sp, int32_t* label, wgt_t* W, int64_t Wsize,
-            const LPRun& run, int64_t* d_arcs, int32_t* d_err, cudaStream_t s,
+            const LPRun& run, DevBuf<int64_t>& arcs, int32_t* d_err, cudaStream_t s,
             const uint8_t* active_init, uint8_t* active_next_out) {
   const int64_t N = lv.N;
   if (N == 0 || run.rounds <= 0) return;
@@ -3024,7 +3024,7 @@ void lp_run(const LevelView& lv, const SlotParams& sp, int32_t* label, wgt_t* W,
   a.noff = sp.noff; a.loff = sp.loff; a.bound = sp.bound; a.rkey = sp.rkey; a.nlab = sp.nlab;
   a.done = sp.done; a.moved = sp.moved; a.rounds = sp.rounds;
   a.label = label; a.W = W; a.mode = run.mode; a.S = S;
-  a.arcs = d_arcs;
+  a.arcs = arcs.p;
   a.err = d_err;
   a.wait_limit = wait_limit();
   a.probe_limit = probe_limit();
