@@ -452,7 +452,8 @@ __global__ void __launch_bounds__(GNT) k_ggg(GGGArgs a) {
 // trial slot g), with the same rules as k_ggg.  The group shares the
 // trial's step and front lists and a few counters in global memory and
 // meets at a barrier of its own (bounded wait: a wait that runs out sets
-// DERR_TIMEOUT and the group leaves).  Each CTA owns a contiguous range of
+// DERR_TIMEOUT and the group leaves; the labels are valid blocks from the
+// start, k_first_blocks).  Each CTA owns a contiguous range of
 // the trial's nodes for the scans (seed search, ordered candidates,
 // water-filling); id-ordered prefixes over the whole trial are the CTAs'
 // partial sums in rank order plus the CTA's own scan.  The step nodes'
@@ -483,6 +484,19 @@ constexpr int64_t GG_HEAVY = 8 * GG_NT;
 // the bitmaps, 43 ms with consecutive arcs; 2^22 nodes 14.1 -> 6.1 ms.
 constexpr int GG_ARC = 8;                  // arcs per thread and pass
 
+// Every node of the trials in its trial's first block, and empty blocks: a
+// group whose wait runs out leaves nodes that it never reached, and what
+// follows indexes block arrays by the labels until the host reads the error.
+__global__ void __launch_bounds__(256) k_first_blocks(GGGArgs a) {
+  const int32_t s = (int32_t)blockIdx.y;
+  const int64_t base = a.noff[s], n = a.noff[s + 1] - base, bo = a.boff[s];
+  for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n;
+       v += (int64_t)gridDim.x * blockDim.x)
+    a.label[base + v] = (int32_t)bo;
+  if (blockIdx.x == 0)
+    for (int32_t b = threadIdx.x; b < a.nlab[s]; b += blockDim.x) a.W[bo + b] = 0;
+}
+
 __global__ void __launch_bounds__(GG_NT) k_ggg_group(GGGArgs a, int32_t cpt, GroupState* gst,
                                                      uint64_t* ph, int32_t* pv, int64_t* pw,
                                                      uint32_t lim) {
@@ -495,6 +509,8 @@ __global__ void __launch_bounds__(GG_NT) k_ggg_group(GGGArgs a, int32_t cpt, Gro
   __shared__ int64_t st_off[GG_NT];
   __shared__ int64_t pre_sh, tot_sh;
   __shared__ int32_t seed_sh;
+  // a bounded wait of an earlier launch ran out: the call is abandoned
+  if (*(volatile int32_t*)a.err & DERR_TIMEOUT) return;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int32_t s = (int32_t)(blockIdx.x / cpt);
   const int r = (int)(blockIdx.x % cpt);
@@ -532,8 +548,6 @@ __global__ void __launch_bounds__(GG_NT) k_ggg_group(GGGArgs a, int32_t cpt, Gro
     __syncthreads();
   };
   for (int64_t w = wr0 + tid; w < wr1; w += GG_NT) asg[w] = 0;
-  if (r == 0)
-    for (int32_t b = tid; b < k; b += GG_NT) a.W[bo + b] = 0;
   if (!sync()) return;
   int32_t* stp = a.step + base;
   int32_t* frt = a.front + base;
@@ -1284,6 +1298,7 @@ void ggg_trials(const GGGArgs& a_in, const std::vector<int64_t>& noff,
     DevBuf<int32_t> pv(S * cpt, s);
     DevBuf<int64_t> pw(S * cpt, s);
     gs.zero();
+    k_first_blocks<<<dim3(grid_for(noff[S] / S, 256 * 4, 256), (unsigned)S), 256, 0, s>>>(a); SCLAP_NOTE_LAUNCH("k_first_blocks");
     launch_coop(k_ggg_group, (unsigned)(S * cpt), GG_NT, 0, s, a, (int32_t)cpt, gs.p, ph.p, pv.p,
                 pw.p, wait_limit()); SCLAP_NOTE_LAUNCH("k_ggg_group");
     SCLAP_LAUNCH_CHECK();

@@ -2429,6 +2429,8 @@ __global__ void __launch_bounds__(PR_NT, 1) k_lp_rounds(LPArgs a, RoundsArgs q) 
   const int64_t gt = (int64_t)cta * PR_NT + tid, gn = (int64_t)G * PR_NT;
   const int nkeys = a.S * NB;
   const uint32_t lim = a.wait_limit;
+  // a bounded wait of an earlier launch ran out: the call is abandoned
+  if (*(volatile int32_t*)a.err & DERR_TIMEOUT) return;
   unsigned int want = 0;
   auto sync = [&] { return round_sync(q.bar, want, a.err, lim); };
   for (int j = tid; j < q.tcap; j += PR_NT) { keys[j] = -1; vals[j] = 0; }
