@@ -265,8 +265,9 @@ __device__ __forceinline__ bool grid_sync(GridSync* gs, int32_t* err, uint32_t l
 }
 
 // Iteration limit of every bounded device-side wait (about 2 s at the
-// default); a host-side fault-injection setting (sclap_debug_inject) may
+// default, WAIT_LIMIT); a host-side fault-injection setting (sclap_debug_inject) may
 // lower it to make waits run out on purpose.
+constexpr uint32_t WAIT_LIMIT = 1u << 22;
 uint32_t wait_limit();
 // Probe limit of the open-addressing tables of the LP sweep (default: the
 // table size, i.e. no limit); lowered only by sclap_debug_inject.

@@ -1843,7 +1843,7 @@ int sclap_debug_inject(int64_t wait, int64_t probe, int32_t fail_allocs) {
   return guarded([&] {
     if (wait < 0 || probe < 0 || fail_allocs < 0 || wait > 0xffffffffll || probe > 0xffffffffll)
       throw Error(SCLAP_EINVAL, "fault-injection value out of range");
-    debug_inject(wait == 0 ? (1u << 22) : (uint32_t)wait,
+    debug_inject(wait == 0 ? WAIT_LIMIT : (uint32_t)wait,
                  probe == 0 ? 0xffffffffu : (uint32_t)probe, fail_allocs);
   });
 }

@@ -1201,10 +1201,12 @@ __global__ void __launch_bounds__(HUB_NT) k_hub_accum(LPArgs a, int32_t sub, Hub
         const bool ok = mbar_wait(&hub_bar[b], phs[b], a.wait_limit);
         if (__syncthreads_or(!ok)) {
           // the copy did not complete in time: report, let the copies in
-          // flight land (bounded), leave
+          // flight land (bounded, by the full limit even where the limit of
+          // the waits is lowered: the shared memory they write is given back
+          // when the CTA leaves), leave
           if (tid == 0) atomicOr(a.err, DERR_TIMEOUT);
-          mbar_wait(&hub_bar[b], phs[b], a.wait_limit);
-          if (nx < p1) mbar_wait(&hub_bar[b ^ 1], phs[b ^ 1], a.wait_limit);
+          mbar_wait(&hub_bar[b], phs[b], WAIT_LIMIT);
+          if (nx < p1) mbar_wait(&hub_bar[b ^ 1], phs[b ^ 1], WAIT_LIMIT);
           return;
         }
         phs[b] ^= 1u;
@@ -2693,7 +2695,7 @@ __global__ void __launch_bounds__(PR_NT, 1) k_lp_rounds(LPArgs a, RoundsArgs q) 
 
 // Limits of the bounded device-side loops, process-wide; changed only by the
 // host-side fault injection of sclap_debug_inject (tests).
-std::atomic<uint32_t> g_wait_limit{1u << 22};
+std::atomic<uint32_t> g_wait_limit{WAIT_LIMIT};
 std::atomic<uint32_t> g_probe_limit{0xffffffffu};
 std::atomic<int32_t> g_fail_allocs{0};
 uint32_t wait_limit() { return g_wait_limit.load(); }
