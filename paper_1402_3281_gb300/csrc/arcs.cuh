@@ -14,7 +14,7 @@ namespace sclap {
 // held 32 rows and took their arcs 32 at a time: one gather in flight per
 // lane, and a hub's row was one warp's serial job.)
 constexpr int AT_NT = 256;                 // threads per CTA
-constexpr int AT_V = AT_NT;                // nodes staged per tile, one per thread
+constexpr int AT_V = AT_NT;                // rows staged per tile, one per thread (R of them: R * AT_V)
 constexpr int AT_PER = 8;                  // arcs per thread and tile
 constexpr int AT_ARCS = AT_NT * AT_PER;
 
@@ -28,37 +28,66 @@ __device__ __forceinline__ bool arcs_aligned(const int32_t* col, const int32_t* 
   return ((reinterpret_cast<uintptr_t>(col) | reinterpret_cast<uintptr_t>(ew)) & 15) == 0;
 }
 
+// Last row of [v, v1) that starts at or before lo, by a search in doubling
+// steps from v (row_ptr[v] <= lo < row_ptr[v1]).
+static __device__ __noinline__ int32_t row_after_gap(const int64_t* row_ptr, int32_t v, int32_t v1,
+                                                     int64_t lo) {
+  int32_t step = AT_V;
+  while (step < v1 - v && row_ptr[v + step] <= lo) {
+    v += step;
+    step = step < (1 << 29) ? 2 * step : step;
+  }
+  for (; step > 0; step /= 2)              // the row is less than step rows on
+    if (step < v1 - v && row_ptr[v + step] <= lo) v += step;
+  return v;
+}
+
 // Walks the entries [lo, hi) of rows laid out back to back (arcs of nodes,
 // slots of table regions) tile by tile: calls f(lo, span, v) for the tile of
-// the entries [lo, lo + span), whose rows are v .. v + AT_V - 1 with ends
-// sh_end[j] (relative to lo).  All threads of the CTA call it equally often.
+// the entries [lo, lo + span), whose rows are v .. v + R * AT_V - 1 with ends
+// sh_end[j] (relative to lo; R * AT_V rows, R per thread).  All threads of the CTA call it equally often.
 // row_ptr is non-decreasing over [v0, v1] with row_ptr[v0] <= lo and
-// hi <= row_ptr[v1] (v0 < v1); sh_end is AT_V words of shared memory.  A tile
+// hi <= row_ptr[v1] (v0 < v1); sh_end is R * AT_V words of shared memory.  A tile
 // never reaches past the AT_ARCS entries from lo rounded down to 4.
-template <class F>
+//
+// A run of rows without entries is passed over by a search in doubling steps:
+// staging it 256 rows at a time was a serial job of the one CTA that met it
+// while the rest of the grid was done (a path of 1 M nodes with ten million
+// isolated nodes in the middle: a cut 74 -> 0.18 ms, a contraction 281 -> 0.78).
+template <int R = 1, class F>
 __device__ __forceinline__ void for_tiles(const int64_t* __restrict__ row_ptr, int64_t v0,
                                           int64_t v1, int64_t lo, int64_t hi, int32_t* sh_end,
                                           F f) {
   if (lo >= hi) return;
   const int tid = threadIdx.x;
-  int64_t v = v0, b = v1 - 1;              // last row that starts at or before lo
-  while (v < b) {
-    const int64_t mid = (v + b + 1) >> 1;
+  // (rows are numbered below 2^31)
+  const int32_t vend = (int32_t)v1;
+  int32_t v = (int32_t)v0;                 // last row that starts at or before lo
+  for (int32_t b = vend - 1; v < b;) {
+    const int32_t mid = v + (b - v + 1) / 2;
     if (row_ptr[mid] <= lo) v = mid;
     else b = mid - 1;
   }
   while (lo < hi) {
-    const int64_t u = v + tid + 1;
-    int32_t end = AT_ARCS + 1;             // rows past the range: no entry of the tile
-    if (u <= v1) end = (int32_t)min64(row_ptr[u] - lo, AT_ARCS + 1);
+    int32_t end[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const int32_t j = r * AT_V + tid;
+      end[r] = AT_ARCS + 1;                // rows past the range: no entry of the tile
+      if (j < vend - v) end[r] = (int32_t)max64(min64(row_ptr[v + j + 1] - lo, AT_ARCS + 1), 0);
+    }
     __syncthreads();                       // the previous tile's searches are done
-    sh_end[tid] = end;
+#pragma unroll
+    for (int r = 0; r < R; ++r) sh_end[r * AT_V + tid] = end[r];
     __syncthreads();
-    const int32_t span = (int32_t)min64(min64(AT_ARCS - (int)(lo & 3), hi - lo),
-                                        max64(sh_end[AT_V - 1], 0));
-    f(lo, span, v);
+    if (sh_end[R * AT_V - 1] == 0) {           // none of the staged rows reaches past lo
+      v = row_after_gap(row_ptr, v + R * AT_V, vend, lo);
+      continue;
+    }
+    const int32_t span = (int32_t)min64(min64(AT_ARCS - (int)(lo & 3), hi - lo), sh_end[R * AT_V - 1]);
+    f(lo, span, (int64_t)v);
     // the row that holds the next entry (the staged rows ending at or before it are done)
-    int j = 0, k = AT_V;
+    int j = 0, k = R * AT_V;
     while (j < k) {
       const int mid = (j + k) >> 1;
       if (sh_end[mid] > span) k = mid;
@@ -72,10 +101,11 @@ __device__ __forceinline__ void for_tiles(const int64_t* __restrict__ row_ptr, i
 // Rows (j: from the tile's first; -1: no entry) of this thread's AT_PER
 // consecutive entries, which start at x0 from the tile's first: a search for
 // the first, then forward.
+template <int R = 1>
 __device__ __forceinline__ void tile_rows(const int32_t* sh_end, int32_t x0, int32_t span,
                                           int32_t (&row)[AT_PER]) {
   const int32_t xs = x0 > 0 ? x0 : 0;
-  int j = 0, k = AT_V - 1;
+  int j = 0, k = R * AT_V - 1;
   while (j < k) {
     const int mid = (j + k) >> 1;
     if (sh_end[mid] > xs) k = mid;
@@ -87,7 +117,7 @@ __device__ __forceinline__ void tile_rows(const int32_t* sh_end, int32_t x0, int
     const int32_t x = x0 + i;
     row[i] = -1;
     if (x >= 0 && x < span) {
-      while (ej <= x) ej = sh_end[++j];    // x < span <= sh_end[AT_V - 1]
+      while (ej <= x) ej = sh_end[++j];    // x < span <= the last sh_end
       row[i] = j;
     }
   }
@@ -96,14 +126,14 @@ __device__ __forceinline__ void tile_rows(const int32_t* sh_end, int32_t x0, int
 // Calls f(tile, v) for every tile of the arcs [lo, hi) (see for_tiles; v: the
 // tile's first staged node).  M is the length of col and ew: a 16-byte word
 // reaching past it is read entry by entry.
-template <class F>
+template <int R = 1, class F>
 __device__ __forceinline__ void for_arc_tiles(const int64_t* __restrict__ row_ptr, int64_t v0,
                                               int64_t v1, int64_t lo, int64_t hi,
                                               const int32_t* __restrict__ col,
                                               const int32_t* __restrict__ ew, int64_t M,
                                               int32_t* sh_end, F f) {
   const bool vec = arcs_aligned(col, ew);
-  for_tiles(row_ptr, v0, v1, lo, hi, sh_end, [&](int64_t lo, int32_t span, int64_t v) {
+  for_tiles<R>(row_ptr, v0, v1, lo, hi, sh_end, [&](int64_t lo, int32_t span, int64_t v) {
     // the tile's words start on 16-byte boundaries
     const int32_t x0 = (int32_t)threadIdx.x * AT_PER - (int32_t)(lo & 3);
     const int64_t e0 = lo + x0;
@@ -133,7 +163,7 @@ __device__ __forceinline__ void for_arc_tiles(const int64_t* __restrict__ row_pt
             if (ew) t.w[i] = ew[e0 + i];
           }
       }
-      tile_rows(sh_end, x0, span, t.v);
+      tile_rows<R>(sh_end, x0, span, t.v);
 #pragma unroll
       for (int i = 0; i < AT_PER; ++i)
         if (t.v[i] >= 0) t.v[i] += (int32_t)v;
@@ -142,18 +172,29 @@ __device__ __forceinline__ void for_arc_tiles(const int64_t* __restrict__ row_pt
   });
 }
 
-// Arc range of this CTA: an even share of [0, M), whole tiles.
+// Arc range of this CTA: an even share of [0, M), whole tiles, or on levels
+// with fewer arcs than that (arc_grid) a part of one.
 __device__ __forceinline__ void arc_share(int64_t M, int64_t* lo, int64_t* hi) {
-  const int64_t per = ((M + gridDim.x - 1) / gridDim.x + AT_ARCS - 1) / AT_ARCS * AT_ARCS;
+  int64_t per = (M + gridDim.x - 1) / gridDim.x;
+  const int64_t unit = per < AT_ARCS ? 4 : AT_ARCS;
+  per = (per + unit - 1) / unit * unit;
   *lo = min64((int64_t)blockIdx.x * per, M);
   *hi = min64(*lo + per, M);
 }
 // One wave of resident CTAs: the shares are even, so a second, partial wave
-// would only add a tail.
+// would only add a tail.  A CTA per tile of arcs or per eight staged blocks of
+// rows, whichever are more: with far fewer arcs than rows the steps over the
+// rows are the work (10 M nodes, 20,000 arcs: a cut 6.7 -> 0.23 ms, a
+// contraction 24.7 -> 0.9).
 constexpr int AT_CTAS = 6;                 // resident CTAs per SM (launch bounds)
-inline unsigned arc_grid(int64_t M, int ctas = AT_CTAS) {
-  return grid_for(M, AT_ARCS, (int64_t)num_sms() * ctas);
+inline unsigned arc_grid(int64_t M, int64_t rows, int ctas = AT_CTAS) {
+  return grid_for(M > rows ? M : rows, AT_ARCS, (int64_t)num_sms() * ctas);
 }
+
+// Rows staged per thread on levels with fewer arcs than rows: there the steps
+// over the rows are the work (10 M nodes, 2 M arcs: a cut 0.48 -> 0.25 ms, a
+// contraction 1.56 -> 0.98; one row per thread before, two barriers a step).
+constexpr int SPARSE_ROWS = 4;
 
 // Exclusive prefix of x over the CTA's threads (AT_NT); sh holds AT_NT / 32
 // words, all threads call.

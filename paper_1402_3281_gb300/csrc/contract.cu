@@ -74,18 +74,29 @@ __global__ void k_map(CArgs a, int64_t N) {
   }
 }
 
+// On levels with fewer arcs than nodes (SPARSE_ROWS) only rows with arcs look
+// their coarse node up.
+__device__ __forceinline__ bool has_entries(const int32_t* sh_end, int j) {
+  return sh_end[j] > (j > 0 ? sh_end[j - 1] : 0);
+}
+
 // Inter-cluster arcs per coarse node, the arcs streamed in even tiles
 // (arcs.cuh): counted per staged row in shared memory, one global atomic per
 // row and tile.
+template <int R>
 __global__ void __launch_bounds__(AT_NT, 5) k_count_inter(CArgs a) {
-  __shared__ int32_t sh_end[AT_V], sh_cv[AT_V], sh_cnt[AT_V];
+  __shared__ int32_t sh_end[R * AT_V], sh_cv[R * AT_V], sh_cnt[R * AT_V];
   const int tid = threadIdx.x;
   int64_t lo, hi;
   arc_share(a.M, &lo, &hi);
-  for_arc_tiles(a.row_ptr, 0, a.N, lo, hi, a.col, nullptr, a.M, sh_end,
-                [&](const ArcTile& t, int64_t v0) {
-    sh_cv[tid] = v0 + tid < a.N ? a.cmap[v0 + tid] : -1;
-    sh_cnt[tid] = 0;
+  for_arc_tiles<R>(a.row_ptr, 0, a.N, lo, hi, a.col, nullptr, a.M, sh_end,
+                   [&](const ArcTile& t, int64_t v0) {
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const int j = r * AT_V + tid;
+      sh_cv[j] = v0 + j < a.N && (R == 1 || has_entries(sh_end, j)) ? a.cmap[v0 + j] : -1;
+      sh_cnt[j] = 0;
+    }
     int32_t cu[AT_PER];
 #pragma unroll
     for (int i = 0; i < AT_PER; ++i)
@@ -105,8 +116,11 @@ __global__ void __launch_bounds__(AT_NT, 5) k_count_inter(CArgs a) {
     }
     if (c) atomicAdd(&sh_cnt[row], c);
     __syncthreads();
-    if (sh_cnt[tid] && SCLAP_OK(sh_cv[tid], a.Nc, a.err))
-      atomicAdd(&a.inter[sh_cv[tid]], sh_cnt[tid]);
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const int j = r * AT_V + tid;
+      if (sh_cnt[j] && SCLAP_OK(sh_cv[j], a.Nc, a.err)) atomicAdd(&a.inter[sh_cv[j]], sh_cnt[j]);
+    }
   });
 }
 
@@ -167,27 +181,30 @@ __device__ __forceinline__ void insert_arc(const CArgs& a, int64_t base, uint32_
 // regions lie in L2, gained nothing: 57 -> 48 ms plus 8 ms for the sort, and
 // 6.0 -> 6.3 ms plus 0.6 ms on 2^22 nodes (74 ms with a tile's equal arcs
 // summed in shared memory: claims answered one after the other).
+template <int R>
 __global__ void __launch_bounds__(AT_NT, 4) k_insert(CArgs a) {
-  __shared__ int32_t sh_end[AT_V], sh_cv[AT_V];
-  __shared__ int64_t sh_base[AT_V];
-  __shared__ uint32_t sh_cap[AT_V];
+  __shared__ int32_t sh_end[R * AT_V], sh_cv[R * AT_V];
+  __shared__ int64_t sh_base[R * AT_V];
+  __shared__ uint32_t sh_cap[R * AT_V];
   const int tid = threadIdx.x;
   int64_t lo, hi;
   arc_share(a.M, &lo, &hi);
-  for_arc_tiles(a.row_ptr, 0, a.N, lo, hi, a.col, a.ew, a.M, sh_end,
-                [&](const ArcTile& t, int64_t v0) {
+  for_arc_tiles<R>(a.row_ptr, 0, a.N, lo, hi, a.col, a.ew, a.M, sh_end,
+                   [&](const ArcTile& t, int64_t v0) {
     int32_t cu[AT_PER];
 #pragma unroll
     for (int i = 0; i < AT_PER; ++i)
       cu[i] = t.v[i] >= 0 ? SCLAP_LD(a.cmap, t.c[i], a.N, a.err) : -1;
-    {
-      int32_t cv = v0 + tid < a.N ? a.cmap[v0 + tid] : -1;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const int j = r * AT_V + tid;
+      int32_t cv = v0 + j < a.N && (R == 1 || has_entries(sh_end, j)) ? a.cmap[v0 + j] : -1;
       if (cv < a.c_lo || cv >= a.c_hi || !SCLAP_OK(cv, a.Nc, a.err)) cv = -1;
-      sh_cv[tid] = cv;
+      sh_cv[j] = cv;
       if (cv >= 0) {
         const int64_t b = a.tbase[cv];
-        sh_base[tid] = b - a.toff;
-        sh_cap[tid] = (uint32_t)(a.tbase[cv + 1] - b);
+        sh_base[j] = b - a.toff;
+        sh_cap[j] = (uint32_t)(a.tbase[cv + 1] - b);
       }
     }
     __syncthreads();
@@ -1025,16 +1042,17 @@ void contract_build(const LevelView& lv, const std::vector<int64_t>& noff, const
   a.N = N; a.M = lv.M; a.Nc = Nc;
 
   const unsigned ng = grid_for(N, 256, (int64_t)sms * 16);
+  const bool sparse = lv.M < N;
   constexpr int64_t BOUNDED_M = 4000000;   // arcs: at most 80 MB of table
   if (N > 0) {
     k_map<<<ng, 256, 0, s>>>(a, N); SCLAP_NOTE_LAUNCH("k_map");
     if (lv.M > 0) {
-      k_count_inter<<<arc_grid(lv.M, 5), AT_NT, 0, s>>>(a); SCLAP_NOTE_LAUNCH("k_count_inter");
+      (sparse ? k_count_inter<SPARSE_ROWS> : k_count_inter<1>)<<<arc_grid(lv.M, N, 5), AT_NT, 0, s>>>(a); SCLAP_NOTE_LAUNCH("k_count_inter");
     }
   }
   auto insert = [&] {
     if (lv.M <= 0) return;
-    k_insert<<<arc_grid(lv.M, 4), AT_NT, 0, s>>>(a); SCLAP_NOTE_LAUNCH("k_insert");
+    (sparse ? k_insert<SPARSE_ROWS> : k_insert<1>)<<<arc_grid(lv.M, N, 4), AT_NT, 0, s>>>(a); SCLAP_NOTE_LAUNCH("k_insert");
   };
   const int64_t Tcap = table_pass_slots();
   if (tuning_get().contract_merge && N > 0 && Nc > 0 &&
@@ -1063,10 +1081,10 @@ void contract_build(const LevelView& lv, const std::vector<int64_t>& noff, const
   SlotArgs sa{};
   sa.tbase = tbase.p;
   auto count_slots = [&] {
-    k_slot_count<<<arc_grid(sa.T - sa.toff, 6), AT_NT, 0, s>>>(sa, inter.p); SCLAP_NOTE_LAUNCH("k_slot_count");
+    k_slot_count<<<arc_grid(sa.T - sa.toff, sa.c_hi - sa.c_lo, 6), AT_NT, 0, s>>>(sa, inter.p); SCLAP_NOTE_LAUNCH("k_slot_count");
   };
   auto emit = [&] {
-    k_emit<<<arc_grid(sa.T - sa.toff, 5), AT_NT, 0, s>>>(sa, out.row_ptr.p, inter.p, out.col.p,
+    k_emit<<<arc_grid(sa.T - sa.toff, sa.c_hi - sa.c_lo, 5), AT_NT, 0, s>>>(sa, out.row_ptr.p, inter.p, out.col.p,
                                                          out.ew.p); SCLAP_NOTE_LAUNCH("k_emit");
   };
   if (T <= Tcap) {

@@ -122,13 +122,13 @@ __global__ void __launch_bounds__(256) k_validate_nodes(
 // CUT: also adds twice the cut of `label` to cut2 (sclap_cut: one pass over
 // the arcs instead of two); a head is used as an index only once it was
 // found to lie in the slot.
-template <bool CUT>
+template <bool CUT, int R>
 __global__ void __launch_bounds__(AT_NT, AT_CTAS) k_validate_arcs(
     const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
     const int32_t* __restrict__ ew, const int64_t* __restrict__ noff,
     const int64_t* __restrict__ aoff, int32_t nslots, int64_t M, int32_t* gerr,
     unsigned long long* arcw, const int32_t* __restrict__ label, unsigned long long* cut2) {
-  __shared__ int32_t sh_end[AT_V];
+  __shared__ int32_t sh_end[R * AT_V];
   __shared__ unsigned long long sh_sum[AT_NT / 32];
   __shared__ int32_t sh_bad;
   int64_t lo, hi;
@@ -143,7 +143,7 @@ __global__ void __launch_bounds__(AT_NT, AT_CTAS) k_validate_arcs(
       const int64_t v0 = noff[s], v1 = noff[s + 1];
       unsigned long long acc = 0, cut = 0;
       bool bad = false;
-      for_arc_tiles(row_ptr, v0, v1, lo, end, col, ew, M, sh_end, [&](const ArcTile& t, int64_t) {
+      for_arc_tiles<R>(row_ptr, v0, v1, lo, end, col, ew, M, sh_end, [&](const ArcTile& t, int64_t) {
 #pragma unroll
         for (int i = 0; i < AT_PER; ++i) {
           const bool in = t.v[i] >= 0;
@@ -410,7 +410,9 @@ void validate_level(Level& L, int B, std::vector<int32_t>& status,
         L.rp(), L.nwp(), L.noff_d.p, L.aoff_d.p, B, L.N, err, sum, mx); SCLAP_NOTE_LAUNCH("k_validate_nodes");
     level_degree_stats(L.rp(), L.N, B7_MAXDEG, dstat, s);
     if (L.M > 0) {
-      (label ? k_validate_arcs<true> : k_validate_arcs<false>)<<<arc_grid(L.M), AT_NT, 0, s>>>(
+      const bool sparse = L.M < L.N;
+      (label ? sparse ? k_validate_arcs<true, SPARSE_ROWS> : k_validate_arcs<true, 1>
+             : sparse ? k_validate_arcs<false, SPARSE_ROWS> : k_validate_arcs<false, 1>)<<<arc_grid(L.M, L.N), AT_NT, 0, s>>>(
           L.rp(), L.colp(), L.ewp(), L.noff_d.p, L.aoff_d.p, B, L.M, err, arcw, label,
           reinterpret_cast<unsigned long long*>(cut2)); SCLAP_NOTE_LAUNCH("k_validate_arcs");
     }

@@ -881,8 +881,11 @@ __global__ void __launch_bounds__(GG_NT) k_ggg_group(GGGArgs a, int32_t cpt, Gro
 // Bounded by the label gathers through L1 and L2 (55-68 % busy).  Measured
 // on R-MAT 2^21 nodes, 56 M weighted arcs: 743 -> 310 us (a warp per 32 rows
 // plus a queue of long rows before); the 512-graph batch's trial and final
-// cuts 1.74 -> 1.12 ms.
-__global__ void __launch_bounds__(AT_NT, AT_CTAS) k_slot_cut(const int64_t* __restrict__ row_ptr,
+// cuts 1.74 -> 1.12 ms.  Five CTAs per SM: for six it spills 72 bytes a thread
+// (R-MAT 2^24 nodes 3.76 ms, five 3.16, four 3.38).
+constexpr int CUT_CTAS = 5;
+template <int R>
+__global__ void __launch_bounds__(AT_NT, CUT_CTAS) k_slot_cut(const int64_t* __restrict__ row_ptr,
                                                     const int32_t* __restrict__ col,
                                                     const int32_t* __restrict__ ew,
                                                     const int64_t* __restrict__ noff,
@@ -890,7 +893,7 @@ __global__ void __launch_bounds__(AT_NT, AT_CTAS) k_slot_cut(const int64_t* __re
                                                     int32_t nslots, int64_t N, int64_t M,
                                                     const int32_t* __restrict__ label,
                                                     int64_t* __restrict__ cut2) {
-  __shared__ int32_t sh_end[AT_V];
+  __shared__ int32_t sh_end[R * AT_V];
   __shared__ unsigned long long sh_sum[AT_NT / 32];
   int64_t lo, hi;
   arc_share(M, &lo, &hi);
@@ -898,8 +901,8 @@ __global__ void __launch_bounds__(AT_NT, AT_CTAS) k_slot_cut(const int64_t* __re
     const int32_t s = nslots > 1 ? slot_of(aoff, nslots, lo) : 0;
     const int64_t end = nslots > 1 ? min64(hi, aoff[s + 1]) : hi;
     unsigned long long acc = 0;
-    for_arc_tiles(row_ptr, nslots > 1 ? noff[s] : 0, nslots > 1 ? noff[s + 1] : N, lo, end, col,
-                  ew, M, sh_end, [&](const ArcTile& t, int64_t) {
+    for_arc_tiles<R>(row_ptr, nslots > 1 ? noff[s] : 0, nslots > 1 ? noff[s + 1] : N, lo, end, col,
+                     ew, M, sh_end, [&](const ArcTile& t, int64_t) {
       int32_t a[AT_PER], b[AT_PER];
 #pragma unroll
       for (int i = 0; i < AT_PER; ++i) {
@@ -1314,7 +1317,7 @@ void ggg_trials(const GGGArgs& a_in, const std::vector<int64_t>& noff,
 
 void slot_cut(const LevelView& lv, const int32_t* label, int64_t* cut2, cudaStream_t s) {
   if (lv.M <= 0) return;
-  k_slot_cut<<<arc_grid(lv.M), AT_NT, 0, s>>>(lv.row_ptr, lv.col, lv.ew, lv.noff, lv.aoff,
+  (lv.M < lv.N ? k_slot_cut<SPARSE_ROWS> : k_slot_cut<1>)<<<arc_grid(lv.M, lv.N, CUT_CTAS), AT_NT, 0, s>>>(lv.row_ptr, lv.col, lv.ew, lv.noff, lv.aoff,
                                                  lv.nslots, lv.N, lv.M, label, cut2); SCLAP_NOTE_LAUNCH("k_slot_cut");
   SCLAP_LAUNCH_CHECK();
 }
@@ -1345,7 +1348,7 @@ void trial_cuts(const LevelView& lv, int B, int T, const std::vector<int64_t>& n
   for (a.t0 = 0; a.t0 < T; a.t0 += TC) {
     a.tn = std::min(TC, T - a.t0);
     k_pack_trials<<<grid_for(n, 256, (int64_t)num_sms() * 16), 256, 0, s>>>(a, label, pk.p); SCLAP_NOTE_LAUNCH("k_pack_trials");
-    k_trial_cut<<<arc_grid(m, 2), AT_NT, 0, s>>>(a, lv.row_ptr, lv.col, lv.ew, lv.M, pk.p, cut2); SCLAP_NOTE_LAUNCH("k_trial_cut");
+    k_trial_cut<<<arc_grid(m, n, 2), AT_NT, 0, s>>>(a, lv.row_ptr, lv.col, lv.ew, lv.M, pk.p, cut2); SCLAP_NOTE_LAUNCH("k_trial_cut");
   }
   SCLAP_LAUNCH_CHECK();
 }
