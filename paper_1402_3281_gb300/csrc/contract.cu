@@ -1043,7 +1043,7 @@ void contract_build(const LevelView& lv, const std::vector<int64_t>& noff, const
 
   const unsigned ng = grid_for(N, 256, (int64_t)sms * 16);
   const bool sparse = lv.M < N;
-  constexpr int64_t BOUNDED_M = 4000000;   // arcs: at most 80 MB of table
+  constexpr int64_t BOUNDED_M = 4000000;   // arcs: at most 64 MB of table
   if (N > 0) {
     k_map<<<ng, 256, 0, s>>>(a, N); SCLAP_NOTE_LAUNCH("k_map");
     if (lv.M > 0) {
@@ -1065,10 +1065,11 @@ void contract_build(const LevelView& lv, const std::vector<int64_t>& noff, const
   }
   scan_excl_i64(cap.p, tbase.p, Nc, s);
   // a small level takes a table and coarse arrays of the largest size they
-  // can have instead of waiting for the sizes (twice): at most five slots
-  // per two arcs, no more coarse arcs than fine ones
-  const bool bounded = lv.M <= BOUNDED_M && 5 * lv.M / 2 <= Tcap;
-  int64_t T = 5 * lv.M / 2;
+  // can have instead of waiting for the sizes (twice): at most two slots
+  // per arc (k_table_caps: x + x/2 + 1 <= 2x for x >= 1), no more coarse arcs
+  // than fine ones
+  const bool bounded = lv.M <= BOUNDED_M && 2 * lv.M <= Tcap;
+  int64_t T = 2 * lv.M;
   if (!bounded) {
     ReadBack rb(s);
     rb.add(&T, tbase.p + Nc, 1);

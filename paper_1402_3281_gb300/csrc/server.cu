@@ -45,7 +45,7 @@ struct Request {
 
 // Device bytes a request may hold while it runs: its level-0 graph, the
 // coarse levels (at most as large again), per-node LP and contraction
-// scratch, and the contraction table (8 B per slot, at most 4 slots per arc).
+// scratch, and the contraction table (8 B per slot, at most 2 slots per arc).
 int64_t estimate_bytes(int64_t n, int64_t m) {
   return 320 * n + 64 * m + (1 << 16);
 }
