@@ -445,7 +445,10 @@ int sclap_autotune(int32_t count, sclap_graph* graphs, const sclap_config* cfg,
  * events on its stream and its nodes/arcs are tallied per kernel family
  * (0: one thread per node, degree <= 16; 1: one warp per node, degree
  * 17..128, and CTAs of 128 threads per node, degree <= 512; 2: CTAs of
- * 256/512 threads, degree <= 8192; 3: one CTA per node with a global table).
+ * 256/512 threads, degree <= 8192; 3: rows above that, split over the grid).
+ * A profiled call launches the rounds of every level: small levels, whose
+ * rounds otherwise run in one persistent launch, take longer than without
+ * profiling.  The timeline mode below leaves them as they are.
  * Times are device milliseconds. ---- */
 typedef struct sclap_profile {
   int64_t kernel_launches;

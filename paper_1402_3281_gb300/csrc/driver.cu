@@ -67,7 +67,7 @@ sclap_config resolve_cfg(const sclap_config* c) {
 // (65 % busy: finding each arc's source), reading 2.6 TB/s; the even split of
 // the arcs is what matters: with a warp per 32 rows the longest row was one
 // warp's serial job (R-MAT 2^21 nodes, 56 M weighted arcs: 3.51 ms before,
-// 0.04 ms for the nodes and 0.20 ms for the arcs now; 0.32 ms with the cut).
+// 0.04 ms for the nodes and 0.20 ms for the arcs now; 0.29 ms with the cut).
 __device__ __forceinline__ void val_flush(int32_t s, unsigned long long sum, int32_t mx,
                                           unsigned long long* cV, int32_t* maxc) {
   if (s < 0) return;

@@ -2886,7 +2886,13 @@ std::string timeline_dump() {
 // three lower levels of a 2^22-node mesh (1.05 M nodes and below) 18.7 ->
 // 15.8 ms, local search on a mesh of 2^20 nodes and 14.6 M arcs 0.93 -> 0.79
 // ms; with the mesh's 4.2 M-node level too 16.7 ms, and the 512-graph batch's
-// levels (8.6 M nodes) no change.
+// levels (8.6 M nodes) no change.  Skewed levels without a row above 8,192
+// (power laws of 2^16 to 1.2 M nodes, 2 to 15 M arcs, up to 16,000 rows above
+// 128; launched -> persistent): partitions 9.4 -> 6.6 ms at 2 M arcs, 16.8 ->
+// 14.2 at 8 M, 24.6 -> 22.0 at 15 M, local search 1.8 -> 1.1, 3.1 -> 2.5 and
+// 3.6 -> 3.6 ms; only clustering alone loses on the longest of them (15 M
+// arcs, 15,000 such rows: 2.1 -> 2.3 ms).  Batches of R-MAT graphs of 2^12 to
+// 2^15 nodes, 1.8 to 9 M arcs in all: 5.6 -> 3.7 to 8.1 -> 7.2 ms.
 constexpr int64_t PR_MAX_N = 1250000, PR_MAX_M = 16000000;
 
 void lp_run(const LevelView& lv, const SlotParams& sp, int32_t* label, wgt_t* W, int64_t Wsize,
