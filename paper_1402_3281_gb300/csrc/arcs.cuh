@@ -14,7 +14,7 @@ namespace sclap {
 // held 32 rows and took their arcs 32 at a time: one gather in flight per
 // lane, and a hub's row was one warp's serial job.)
 constexpr int AT_NT = 256;                 // threads per CTA
-constexpr int AT_V = AT_NT;                // rows staged per tile, one per thread (R of them: R * AT_V)
+constexpr int AT_V = AT_NT;                // rows staged per tile by one row per thread
 constexpr int AT_PER = 8;                  // arcs per thread and tile
 constexpr int AT_ARCS = AT_NT * AT_PER;
 
@@ -191,10 +191,15 @@ inline unsigned arc_grid(int64_t M, int64_t rows, int ctas = AT_CTAS) {
   return grid_for(M > rows ? M : rows, AT_ARCS, (int64_t)num_sms() * ctas);
 }
 
-// Rows staged per thread on levels with fewer arcs than rows: there the steps
-// over the rows are the work (10 M nodes, 2 M arcs: a cut 0.48 -> 0.25 ms, a
-// contraction 1.56 -> 0.98; one row per thread before, two barriers a step).
-constexpr int SPARSE_ROWS = 4;
+// Rows staged per thread where rows are short: one row per thread holds fewer
+// entries than a tile when rows average below AT_ARCS / AT_V, and then the
+// steps over the rows (two barriers each) are the work.  Staging four:
+// contraction of a mesh of 4 M nodes and degree 4 1.39 -> 1.11 ms, of R-MAT
+// 2^22 nodes and 8.3 M arcs 2.61 -> 1.44, of 10 M nodes and 2 M arcs 1.56 ->
+// 0.98; cuts of the three 0.21 -> 0.17, 0.27 -> 0.18 and 0.47 -> 0.25 ms.  At
+// degree 6 5 to 7 % faster, at 8 and above no different.
+constexpr int SHORT_ROWS = 4;
+inline bool rows_short(int64_t entries, int64_t rows) { return entries < AT_ARCS / AT_V * rows; }
 
 // Exclusive prefix of x over the CTA's threads (AT_NT); sh holds AT_NT / 32
 // words, all threads call.

@@ -74,8 +74,8 @@ __global__ void k_map(CArgs a, int64_t N) {
   }
 }
 
-// On levels with fewer arcs than nodes (SPARSE_ROWS) only rows with arcs look
-// their coarse node up.
+// Where rows are short (SHORT_ROWS) only rows with arcs look their coarse node
+// up.
 __device__ __forceinline__ bool has_entries(const int32_t* sh_end, int j) {
   return sh_end[j] > (j > 0 ? sh_end[j - 1] : 0);
 }
@@ -273,6 +273,7 @@ __device__ __forceinline__ void slot_share(const SlotArgs& a, int64_t* lo, int64
   *hi += a.toff;
 }
 // this thread's slots of a tile and their regions (j, -1: none)
+template <int R>
 __device__ __forceinline__ void load_slots(const SlotArgs& a, int64_t lo, int32_t span,
                                            const int32_t* sh_end,
                                            unsigned long long (&x)[AT_PER], int32_t (&row)[AT_PER]) {
@@ -283,19 +284,21 @@ __device__ __forceinline__ void load_slots(const SlotArgs& a, int64_t lo, int32_
     x[i] = in ? a.tslot[lo - a.toff + x0 + i] : ~0ull;
     row[i] = -1;
   }
-  if (x0 < span) tile_rows(sh_end, x0, span, row);
+  if (x0 < span) tile_rows<R>(sh_end, x0, span, row);
 }
 
+template <int R>
 __global__ void __launch_bounds__(AT_NT, 6) k_slot_count(SlotArgs a, int32_t* __restrict__ cdeg) {
-  __shared__ int32_t sh_end[AT_V], sh_cnt[AT_V];
+  __shared__ int32_t sh_end[R * AT_V], sh_cnt[R * AT_V];
   const int tid = threadIdx.x;
   int64_t lo, hi;
   slot_share(a, &lo, &hi);
-  for_tiles(a.tbase, a.c_lo, a.c_hi, lo, hi, sh_end, [&](int64_t lo, int32_t span, int64_t c0) {
+  for_tiles<R>(a.tbase, a.c_lo, a.c_hi, lo, hi, sh_end, [&](int64_t lo, int32_t span, int64_t c0) {
     unsigned long long x[AT_PER];
     int32_t row[AT_PER];
-    sh_cnt[tid] = 0;
-    load_slots(a, lo, span, sh_end, x, row);
+#pragma unroll
+    for (int r = 0; r < R; ++r) sh_cnt[r * AT_V + tid] = 0;
+    load_slots<R>(a, lo, span, sh_end, x, row);
     __syncthreads();
     int32_t at = -1, c = 0;
 #pragma unroll
@@ -310,7 +313,11 @@ __global__ void __launch_bounds__(AT_NT, 6) k_slot_count(SlotArgs a, int32_t* __
     }
     if (c) atomicAdd(&sh_cnt[at], c);
     __syncthreads();
-    if (sh_cnt[tid]) atomicAdd(&cdeg[c0 + tid], sh_cnt[tid]);
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const int j = r * AT_V + tid;
+      if (sh_cnt[j]) atomicAdd(&cdeg[c0 + j], sh_cnt[j]);
+    }
   });
 }
 
@@ -319,21 +326,25 @@ __global__ void __launch_bounds__(AT_NT, 6) k_slot_count(SlotArgs a, int32_t* __
 // places in the row.  The order of a row's arcs is therefore not fixed, as
 // the slot order already was not (concurrent claims in one region race);
 // nothing computed from a coarse graph depends on that order.
+template <int R>
 __global__ void __launch_bounds__(AT_NT, 5) k_emit(SlotArgs a, const int64_t* __restrict__ crow,
                                                    int32_t* __restrict__ fill,
                                                    int32_t* __restrict__ ccol,
                                                    int32_t* __restrict__ cew) {
-  __shared__ int32_t sh_end[AT_V], sh_cnt[AT_V], sh_first[AT_V], sh_w[AT_NT / 32];
-  __shared__ int64_t sh_at[AT_V];
+  __shared__ int32_t sh_end[R * AT_V], sh_cnt[R * AT_V], sh_first[R * AT_V], sh_w[AT_NT / 32];
+  __shared__ int64_t sh_at[R * AT_V];
   const int tid = threadIdx.x;
   int64_t lo, hi;
   slot_share(a, &lo, &hi);
-  for_tiles(a.tbase, a.c_lo, a.c_hi, lo, hi, sh_end, [&](int64_t lo, int32_t span, int64_t c0) {
+  for_tiles<R>(a.tbase, a.c_lo, a.c_hi, lo, hi, sh_end, [&](int64_t lo, int32_t span, int64_t c0) {
     unsigned long long x[AT_PER];
     int32_t row[AT_PER];
-    sh_cnt[tid] = 0;
-    sh_first[tid] = INT32_MAX;
-    load_slots(a, lo, span, sh_end, x, row);
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      sh_cnt[r * AT_V + tid] = 0;
+      sh_first[r * AT_V + tid] = INT32_MAX;
+    }
+    load_slots<R>(a, lo, span, sh_end, x, row);
     int32_t mine = 0;
 #pragma unroll
     for (int i = 0; i < AT_PER; ++i) mine += row[i] >= 0 && x[i] != ~0ull;
@@ -355,8 +366,11 @@ __global__ void __launch_bounds__(AT_NT, 5) k_emit(SlotArgs a, const int64_t* __
     }
     if (c) atomicAdd(&sh_cnt[at], c);
     __syncthreads();
-    if (sh_cnt[tid])
-      sh_at[tid] = crow[c0 + tid] + atomicAdd(&fill[c0 + tid], sh_cnt[tid]) - sh_first[tid];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const int j = r * AT_V + tid;
+      if (sh_cnt[j]) sh_at[j] = crow[c0 + j] + atomicAdd(&fill[c0 + j], sh_cnt[j]) - sh_first[j];
+    }
     __syncthreads();
     n = before;
 #pragma unroll
@@ -1042,17 +1056,17 @@ void contract_build(const LevelView& lv, const std::vector<int64_t>& noff, const
   a.N = N; a.M = lv.M; a.Nc = Nc;
 
   const unsigned ng = grid_for(N, 256, (int64_t)sms * 16);
-  const bool sparse = lv.M < N;
+  const bool brief = rows_short(lv.M, N);
   constexpr int64_t BOUNDED_M = 4000000;   // arcs: at most 64 MB of table
   if (N > 0) {
     k_map<<<ng, 256, 0, s>>>(a, N); SCLAP_NOTE_LAUNCH("k_map");
     if (lv.M > 0) {
-      (sparse ? k_count_inter<SPARSE_ROWS> : k_count_inter<1>)<<<arc_grid(lv.M, N, 5), AT_NT, 0, s>>>(a); SCLAP_NOTE_LAUNCH("k_count_inter");
+      (brief ? k_count_inter<SHORT_ROWS> : k_count_inter<1>)<<<arc_grid(lv.M, N, 5), AT_NT, 0, s>>>(a); SCLAP_NOTE_LAUNCH("k_count_inter");
     }
   }
   auto insert = [&] {
     if (lv.M <= 0) return;
-    (sparse ? k_insert<SPARSE_ROWS> : k_insert<1>)<<<arc_grid(lv.M, N, 4), AT_NT, 0, s>>>(a); SCLAP_NOTE_LAUNCH("k_insert");
+    (brief ? k_insert<SHORT_ROWS> : k_insert<1>)<<<arc_grid(lv.M, N, 4), AT_NT, 0, s>>>(a); SCLAP_NOTE_LAUNCH("k_insert");
   };
   const int64_t Tcap = table_pass_slots();
   if (tuning_get().contract_merge && N > 0 && Nc > 0 &&
@@ -1082,10 +1096,10 @@ void contract_build(const LevelView& lv, const std::vector<int64_t>& noff, const
   SlotArgs sa{};
   sa.tbase = tbase.p;
   auto count_slots = [&] {
-    k_slot_count<<<arc_grid(sa.T - sa.toff, sa.c_hi - sa.c_lo, 6), AT_NT, 0, s>>>(sa, inter.p); SCLAP_NOTE_LAUNCH("k_slot_count");
+    (rows_short(sa.T - sa.toff, sa.c_hi - sa.c_lo) ? k_slot_count<SHORT_ROWS> : k_slot_count<1>)<<<arc_grid(sa.T - sa.toff, sa.c_hi - sa.c_lo, 6), AT_NT, 0, s>>>(sa, inter.p); SCLAP_NOTE_LAUNCH("k_slot_count");
   };
   auto emit = [&] {
-    k_emit<<<arc_grid(sa.T - sa.toff, sa.c_hi - sa.c_lo, 5), AT_NT, 0, s>>>(sa, out.row_ptr.p, inter.p, out.col.p,
+    (rows_short(sa.T - sa.toff, sa.c_hi - sa.c_lo) ? k_emit<SHORT_ROWS> : k_emit<1>)<<<arc_grid(sa.T - sa.toff, sa.c_hi - sa.c_lo, 5), AT_NT, 0, s>>>(sa, out.row_ptr.p, inter.p, out.col.p,
                                                          out.ew.p); SCLAP_NOTE_LAUNCH("k_emit");
   };
   if (T <= Tcap) {

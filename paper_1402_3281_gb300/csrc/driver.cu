@@ -410,9 +410,9 @@ void validate_level(Level& L, int B, std::vector<int32_t>& status,
         L.rp(), L.nwp(), L.noff_d.p, L.aoff_d.p, B, L.N, err, sum, mx); SCLAP_NOTE_LAUNCH("k_validate_nodes");
     level_degree_stats(L.rp(), L.N, B7_MAXDEG, dstat, s);
     if (L.M > 0) {
-      const bool sparse = L.M < L.N;
-      (label ? sparse ? k_validate_arcs<true, SPARSE_ROWS> : k_validate_arcs<true, 1>
-             : sparse ? k_validate_arcs<false, SPARSE_ROWS> : k_validate_arcs<false, 1>)<<<arc_grid(L.M, L.N), AT_NT, 0, s>>>(
+      const bool brief = rows_short(L.M, L.N);
+      (label ? brief ? k_validate_arcs<true, SHORT_ROWS> : k_validate_arcs<true, 1>
+             : brief ? k_validate_arcs<false, SHORT_ROWS> : k_validate_arcs<false, 1>)<<<arc_grid(L.M, L.N), AT_NT, 0, s>>>(
           L.rp(), L.colp(), L.ewp(), L.noff_d.p, L.aoff_d.p, B, L.M, err, arcw, label,
           reinterpret_cast<unsigned long long*>(cut2)); SCLAP_NOTE_LAUNCH("k_validate_arcs");
     }

@@ -1317,7 +1317,7 @@ void ggg_trials(const GGGArgs& a_in, const std::vector<int64_t>& noff,
 
 void slot_cut(const LevelView& lv, const int32_t* label, int64_t* cut2, cudaStream_t s) {
   if (lv.M <= 0) return;
-  (lv.M < lv.N ? k_slot_cut<SPARSE_ROWS> : k_slot_cut<1>)<<<arc_grid(lv.M, lv.N, CUT_CTAS), AT_NT, 0, s>>>(lv.row_ptr, lv.col, lv.ew, lv.noff, lv.aoff,
+  (rows_short(lv.M, lv.N) ? k_slot_cut<SHORT_ROWS> : k_slot_cut<1>)<<<arc_grid(lv.M, lv.N, CUT_CTAS), AT_NT, 0, s>>>(lv.row_ptr, lv.col, lv.ew, lv.noff, lv.aoff,
                                                  lv.nslots, lv.N, lv.M, label, cut2); SCLAP_NOTE_LAUNCH("k_slot_cut");
   SCLAP_LAUNCH_CHECK();
 }

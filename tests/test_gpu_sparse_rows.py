@@ -32,10 +32,23 @@ def _spread(n, step):
     return gg.from_edges(n, s, s + 1)
 
 
+def _ring(n, d):
+    """Every node joined to the next d / 2, for odd d every other node to one more."""
+    i = np.arange(n)
+    src, dst = [np.tile(i, d // 2)], [(i + q) % n for q in range(1, d // 2 + 1)]
+    if d % 2:
+        src.append(i[::2])
+        dst.append((i[::2] + d // 2 + 1) % n)
+    return gg.from_edges(n, np.concatenate(src), np.concatenate(dst))
+
+
 GRAPHS = {f"run_{q}": (lambda q=q: _gaps(700, -q, 900)) for q in (254, 256, 257, 511, 512, 513, 767, 768, 70001)}
 # four rows per thread: 1,024 rows a tile
 GRAPHS.update({f"quad_{q}": (lambda q=q: _gaps(2, -q, 2, -q, 3, -(q + 1), 2, -4 * q, 5))
                for q in range(1019, 1026)})
+# rows of 7, 8 and 9 arcs on average: four rows per thread below 8
+GRAPHS.update({f"ring_{d}_{n}": (lambda n=n, d=d: _ring(n, d)) for n in (1023, 1024, 1025, 5000)
+               for d in (7, 8, 9)})
 GRAPHS.update({
     "run_first": lambda: _gaps(-70001, 3000),
     "run_last": lambda: _gaps(3000, -70001),
