@@ -123,8 +123,8 @@ __device__ __forceinline__ void tile_rows(const int32_t* sh_end, int32_t x0, int
   }
 }
 
-// Calls f(tile, v) for every tile of the arcs [lo, hi) (see for_tiles; v: the
-// tile's first staged node).  M is the length of col and ew: a 16-byte word
+// Calls f(tile, v, span) for every tile of the arcs [lo, hi) (see for_tiles; v:
+// the tile's first staged node).  M is the length of col and ew: a 16-byte word
 // reaching past it is read entry by entry.
 template <int R = 1, class F>
 __device__ __forceinline__ void for_arc_tiles(const int64_t* __restrict__ row_ptr, int64_t v0,
@@ -168,7 +168,7 @@ __device__ __forceinline__ void for_arc_tiles(const int64_t* __restrict__ row_pt
       for (int i = 0; i < AT_PER; ++i)
         if (t.v[i] >= 0) t.v[i] += (int32_t)v;
     }
-    f(t, v);
+    f(t, v, span);
   });
 }
 

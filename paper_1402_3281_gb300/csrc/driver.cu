@@ -143,7 +143,7 @@ __global__ void __launch_bounds__(AT_NT, AT_CTAS) k_validate_arcs(
       const int64_t v0 = noff[s], v1 = noff[s + 1];
       unsigned long long acc = 0, cut = 0;
       bool bad = false;
-      for_arc_tiles<R>(row_ptr, v0, v1, lo, end, col, ew, M, sh_end, [&](const ArcTile& t, int64_t) {
+      for_arc_tiles<R>(row_ptr, v0, v1, lo, end, col, ew, M, sh_end, [&](const ArcTile& t, int64_t, int32_t) {
 #pragma unroll
         for (int i = 0; i < AT_PER; ++i) {
           const bool in = t.v[i] >= 0;

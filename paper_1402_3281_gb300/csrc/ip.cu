@@ -902,7 +902,7 @@ __global__ void __launch_bounds__(AT_NT, CUT_CTAS) k_slot_cut(const int64_t* __r
     const int64_t end = nslots > 1 ? min64(hi, aoff[s + 1]) : hi;
     unsigned long long acc = 0;
     for_arc_tiles<R>(row_ptr, nslots > 1 ? noff[s] : 0, nslots > 1 ? noff[s + 1] : N, lo, end, col,
-                     ew, M, sh_end, [&](const ArcTile& t, int64_t) {
+                     ew, M, sh_end, [&](const ArcTile& t, int64_t, int32_t) {
       int32_t a[AT_PER], b[AT_PER];
 #pragma unroll
       for (int i = 0; i < AT_PER; ++i) {
@@ -978,7 +978,7 @@ __global__ void __launch_bounds__(AT_NT, 2) k_trial_cut(TrialCut a, const int64_
     for (int t = 0; t < TC; ++t) acc[t] = 0;
     if (tid < TC) sh_sum[tid] = 0;
     for_arc_tiles(row_ptr, n0, a.noff[s0 + 1], lo + first, end + first, col, ew, M, sh_end,
-                  [&](const ArcTile& t, int64_t) {
+                  [&](const ArcTile& t, int64_t, int32_t) {
 #pragma unroll
       for (int h = 0; h < AT_PER; h += 4) {
         uint4 x[4], y[4];
