@@ -448,20 +448,22 @@ void validate_level(Level& L, int B, std::vector<int32_t>& status,
 }
 
 // Builds and validates the level of one device-resident graph (step entry
-// points); returns c(V) and max c(v) or throws.  label, cut2: also adds twice the label's cut (device).
+// points); returns c(V) and max c(v) or throws.  label, cut2: also adds twice
+// the label's cut (device).
 void validate(const GIn& g, Level& L, cudaStream_t s, int64_t* cV, int64_t* maxc,
               const int32_t* label = nullptr, int64_t* cut2 = nullptr) {
   build_level0({g}, L, s);
   std::vector<int32_t> st;
   std::vector<int64_t> a, b;
-  std::vector<char> nar;
-  validate_level(L, 1, st, a, b, nar, s, nullptr, label, cut2);
+  std::vector<char> nar, small;
+  validate_level(L, 1, st, a, b, nar, s, &small, label, cut2);
   if (st[0] == SCLAP_ECSR)
     throw Error(SCLAP_ECSR, "malformed CSR (row_ptr, column range, self-loop or weight)");
   if (st[0] == SCLAP_EOVERFLOW) throw Error(SCLAP_EOVERFLOW, "sum of node weights must be < 2^31");
   *cV = a[0];
   *maxc = b[0];
   L.narrow = nar[0] != 0;
+  L.sums31 = small[0] != 0;
 }
 
 // Builds the level holding the graphs `gs` back to back.  One graph is used
@@ -1660,6 +1662,7 @@ int sclap_cluster_hierarchy(int64_t n, const int64_t* row_ptr, const int32_t* co
       k_compose<<<grid_for(n, 256, (int64_t)sms * 16), 256, 0, s>>>(comm_out, cur->cmap.p, n); SCLAP_NOTE_LAUNCH("k_compose");
       std::unique_ptr<Level> nx(new Level());
       nx->narrow = cur->narrow;
+      nx->sums31 = cur->sums31;
       nx->N = co.N;
       nx->M = co.M;
       nx->row_ptr = std::move(co.row_ptr);
