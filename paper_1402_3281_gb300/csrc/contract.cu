@@ -176,7 +176,7 @@ __device__ __forceinline__ void insert_arc(const CArgs& a, int64_t base, uint32_
 // atomic; the claims of a hub's cluster serialised on that one counter.)
 // Bounded by random atomics on a table beyond L2: 24 G arcs a second on R-MAT
 // 2^24 nodes, where 64-bit CAS on random words of a 2 GB table reach 23 G.
-// Inserts of both levels there 97 -> 52 ms, R-MAT 2^22 nodes 9.9 -> 6.1 ms.
+// Inserts of both levels there 97 -> 57 ms, R-MAT 2^22 nodes 9.9 -> 5.9 ms.
 // Regions of 1.5 slots per inter-cluster arc (a power of two from 1 to 2
 // before, full to the last slot where the arcs' heads all differ) took the
 // last fifth off.  Sorting the nodes by coarse node first, so that the filled
